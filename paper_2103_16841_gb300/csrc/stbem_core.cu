@@ -18,6 +18,7 @@
 #include <mutex>
 #include <vector>
 
+#include "stbem_block.cuh"
 #include "stbem_internal.h"
 
 namespace stbem {
@@ -116,6 +117,35 @@ __global__ void k_tet_ball(int64_t n_tet, const double* tet_vx, TetDev* tets) {
   tets[i].ball[4] = mx;
 }
 
+// FP32 images of the columns and panels for the sparsity filter
+__global__ void k_col_f32(int64_t n_col, const ColGeom* cols, ColF* out) {
+  int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= n_col) return;
+  const ColGeom& G = cols[c];
+  ColF F;
+  for (int k = 0; k < 3; ++k)
+    for (int i = 0; i < 3; ++i) F.Xh[k][i] = (float)G.X[k][i];
+  for (int i = 0; i < 3; ++i) F.ctr[i] = (float)G.ctr[i];
+  F.rad = (float)G.rad;
+  out[c] = F;
+}
+__global__ void k_panel_f32(int64_t n_tet, const TetDev* tets, const int32_t* col_surf_begin, PanelF* out) {
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n_tet) return;
+  const TetDev& D = tets[i];
+  const int s0 = col_surf_begin[D.col];
+  PanelF F;
+  for (int k = 0; k < 4; ++k) F.vt[k] = (float)D.vt[k];
+  for (int k = 0; k < 5; ++k) F.ball[k] = (float)D.ball[k];
+  F.tmin = (float)D.tmin;
+  F.pmax = (float)D.pmax;
+  F.lo = (uint8_t)(D.lo - s0);
+  F.hi = (uint8_t)(D.hi - s0);
+  F.dup = (uint8_t)D.dup;
+  F.pad = 0;
+  out[i] = F;
+}
+
 bem_status mesh_device_geometry(bem_mesh* m, const double* d_sv_xyz, const int32_t* d_col_corner_sv,
                                 const double* d_tet_vx, const int32_t* d_surf_col, const double* d_surf_p) {
   cudaStream_t s = m->ctx->stream;
@@ -124,6 +154,11 @@ bem_status mesh_device_geometry(bem_mesh* m, const double* d_sv_xyz, const int32
   k_surf_geom<<<(unsigned)((m->n_surf + th - 1) / th), th, 0, s>>>(m->n_surf, m->d_col, d_surf_p, d_surf_col,
                                                                    m->d_surf);
   k_tet_ball<<<(unsigned)((m->n_tet + th - 1) / th), th, 0, s>>>(m->n_tet, d_tet_vx, m->d_tet);
+  STBEM_CUDA(cudaMalloc(&m->d_colf, sizeof(ColF) * m->n_col));
+  STBEM_CUDA(cudaMalloc(&m->d_panf, sizeof(PanelF) * m->n_tet));
+  k_col_f32<<<(unsigned)((m->n_col + th - 1) / th), th, 0, s>>>(m->n_col, m->d_col, static_cast<ColF*>(m->d_colf));
+  k_panel_f32<<<(unsigned)((m->n_tet + th - 1) / th), th, 0, s>>>(m->n_tet, m->d_tet, m->d_col_surf_begin,
+                                                                  static_cast<PanelF*>(m->d_panf));
   STBEM_CUDA(cudaGetLastError());
   return BEM_OK;
 }
@@ -182,16 +217,7 @@ bem_status op_outer_points(bem_operator* op, cudaStream_t s) {
 // FP64 values with the contract's operation order decide; an FP32 estimate
 // with a rigorous error margin settles the clear cases first.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double dist3x(const double* a, const double* b) {
-  double dx = __dsub_rn(a[0], b[0]), dy = __dsub_rn(a[1], b[1]), dz = __dsub_rn(a[2], b[2]);
-  return __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
-}
-// (IEEE square roots here whatever the unit's FP32 flags: the filter's margin
-// is set against the correctly rounded operations)
-__device__ __forceinline__ float dist3f(const float* a, const float* b) {
-  float dx = a[0] - b[0], dy = a[1] - b[1], dz = a[2] - b[2];
-  return __fsqrt_rn(dx * dx + dy * dy + dz * dz);
-}
+__device__ __forceinline__ float dist3f(const float* a, const float* b) { return dist3f(a[0], a[1], a[2], b); }
 
 struct TetSm {       // panel data kept in shared memory for a block
   double tmin, pmax;
@@ -286,40 +312,6 @@ __device__ inline void col_pair_bounds(const ColGeom& GI, const ColGeom& GJ, dou
   Dmin_lo = fmax(0.0, sqrt(dx * dx + dy * dy + dz * dz) - GI.rad - GJ.rad);
 }
 
-struct BlockCtx {
-  int64_t n_col;
-  int mq, nq, n_theta, prec;
-  ArcRule rule;
-  float margin;
-  double S;
-  const ColGeom* cols;
-  const int32_t* col_tet_begin;
-  const int32_t* col_surf_begin;
-  const SurfDev* surf;
-  const TetDev* tets;
-  const double* pts;
-  const float* ptsf;
-  const double* trange;
-  int32_t* bw;
-  int64_t* bnnz;
-  const int64_t* boff;
-  const int64_t* rsoff;
-  int32_t* rs;
-  double* val;
-  float* val32;
-  double* uscratch;     // [gridDim][max_surf][max_tet]
-  int max_surf, max_tet;
-  unsigned long long* counter;
-  int64_t end;                 // blocks [0, end) of the dense (I, J) order are processed
-  unsigned long long* inner;   // pattern pass: inner integrals m_Q^2 x (test face, trial panel) (null: not counted)
-  // matrix-free product: when mf_y is set the entries are not stored but
-  // y[k][i] += A_ij x[k][j] is accumulated (x, y: [mf_nrhs][mf_ld], internal order)
-  const double* mf_x;
-  double* mf_y;
-  int mf_nrhs;
-  int64_t mf_ld;
-};
-
 // cooperative load of column J into shared memory
 __device__ void load_column(const BlockCtx& B, int64_t J, ColSm& C, TetSm* T, FaceGeom* Fs) {
   if (threadIdx.x == 0) {
@@ -361,13 +353,13 @@ __device__ void face_bits(const BlockCtx& B, const ColSm& C, const TetSm* T, int
   for (int w = lane; w < words; w += 32) bits[w] = 0u;
   __syncwarp();
   const double* P = B.pts + fglob * B.nq * 4;
-  const float* Pf = B.ptsf + fglob * B.nq * 4;   // FP32 copies: no conversions in the filter
+  const float4* Pf = B.ptsf + fglob * B.nq;   // FP32 copies: no conversions in the filter
   for (int j0 = jlo; j0 < jhi; j0 += 32) {
     int j = j0 + lane;
     bool hit = false;
     if (j < jhi) {
       for (int q = 0; q < B.nq && !hit; ++q) {
-        const float4 x4 = reinterpret_cast<const float4*>(Pf)[q];
+        const float4 x4 = Pf[q];
         const float xf[4] = {x4.x, x4.y, x4.z, x4.w};
         hit = point_sees(P + 4 * q, xf, T[j], C.G, C.Xf, B.margin);
       }
@@ -391,35 +383,22 @@ __device__ inline int64_t pop_block(unsigned long long* counter) {
   return b;
 }
 
-// Pass 1: band width and pattern count of column block b.
-__device__ __forceinline__ void pattern_block(const BlockCtx& B, int64_t b, unsigned char* smem, ColSm& C, int* s_w,
+// Pass 1: band width and pattern count of block (I, J), from the bits of its
+// faces (block_bits). One row per thread, then one face per thread.
+__device__ __forceinline__ void pattern_block(const BlockCtx& B, const BlockSm& C, const BlockPtr& P, int* s_w,
                                               unsigned long long* s_n) {
-  TetSm* T = reinterpret_cast<TetSm*>(smem);
-  FaceGeom* Fs = reinterpret_cast<FaceGeom*>(T + B.max_tet);
-  uint32_t* bits = reinterpret_cast<uint32_t*>(Fs + B.max_surf);
-  const int words = (B.max_tet + 31) / 32;
-  {
-    int64_t I = b / B.n_col, J = b % B.n_col;
-    load_column(B, J, C, T, Fs);
-    const ColGeom GI = B.cols[I];
-    double Dmax, Dmin_lo;
-    col_pair_bounds(GI, C.G, Dmax, Dmin_lo);
-    int s0 = B.col_surf_begin[I], ns = B.col_surf_begin[I + 1] - s0;
-    int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int f = warp; f < ns; f += nw) {
-      int jlo, jhi;
-      face_bits(B, C, T, s0 + f, Dmax, Dmin_lo, bits + f * words, words, jlo, jhi);
-    }
-    __syncthreads();
-    int t0 = B.col_tet_begin[I], nt = B.col_tet_begin[I + 1] - t0;
-    int wmax = 0;
-    unsigned long long cnt = 0;
-    for (int r = threadIdx.x; r < nt; r += blockDim.x) {
-      const TetDev& D = B.tets[t0 + r];
-      int lo = D.lo - s0, hi = D.hi - s0;
+  const int words = bit_words(B.max_tet);
+  const int64_t b = C.I * B.n_col + C.J;
+  int wmax = 0;
+  unsigned int cnt = 0;
+  if (C.wmax > 0)
+    for (int r = threadIdx.x; r < C.ntI; r += blockDim.x) {
+      const PanelF& D = B.panf[C.tetI + r];
+      const uint32_t* lo = P.bits + D.lo * words;
+      const uint32_t* hi = P.bits + D.hi * words;
       int first = -1, last = -1;
       for (int w = 0; w < words; ++w) {
-        uint32_t m = bits[lo * words + w] | bits[hi * words + w];
+        const uint32_t m = lo[w] | hi[w];
         cnt += __popc(m);
         if (m) {
           if (first < 0) first = 32 * w + __ffs(m) - 1;
@@ -428,83 +407,74 @@ __device__ __forceinline__ void pattern_block(const BlockCtx& B, int64_t b, unsi
       }
       if (first >= 0) wmax = max(wmax, last - first + 1);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
-      cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    }
-    if ((threadIdx.x & 31) == 0) { s_w[threadIdx.x >> 5] = wmax; s_n[threadIdx.x >> 5] = cnt; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int w = 0;
-      unsigned long long n = 0;
-      for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { w = max(w, s_w[i]); n += s_n[i]; }
-      B.bw[b] = w;
-      B.bnnz[b] = (int64_t)n;
-    }
-    if (B.inner) {
-      // inner integrals of the block: every outer point of a test face against
-      // every trial panel the face's pattern bits admit
-      unsigned long long m = 0;
-      for (int f = threadIdx.x; f < ns; f += blockDim.x)
-        for (int w = 0; w < words; ++w) m += __popc(bits[f * words + w]);
-      for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-      if ((threadIdx.x & 31) == 0 && m) atomicAdd(B.inner, m * (unsigned long long)B.nq);
-    }
-    __syncthreads();
+  wmax = __reduce_max_sync(0xffffffffu, wmax);
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if ((threadIdx.x & 31) == 0) { s_w[threadIdx.x >> 5] = wmax; s_n[threadIdx.x >> 5] = cnt; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int w = 0;
+    unsigned long long n = 0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { w = max(w, s_w[i]); n += s_n[i]; }
+    B.bw[b] = w;
+    B.bnnz[b] = (int64_t)n;
   }
+  if (B.inner && C.wmax > 0) {
+    // inner integrals of the block: every outer point of a test face against
+    // every trial panel the face's pattern bits admit
+    unsigned int m = 0;
+    for (int k = threadIdx.x; k < C.nsI * words; k += blockDim.x) m += __popc(P.bits[k]);
+    m = __reduce_add_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) atomicAdd(B.inner, (unsigned long long)m * (unsigned long long)B.nq);
+  }
+  __syncthreads();
 }
 
-// segment of global work item g: prefix[seg] <= g < prefix[seg + 1]
-__device__ inline int find_seg(const int64_t* prefix, int S, int64_t g) {
-  int lo = 0, hi = S;
-  while (hi - lo > 1) {
-    int mid = (lo + hi) >> 1;
-    if (prefix[mid] <= g) lo = mid;
-    else hi = mid;
-  }
-  return lo;
-}
+// Bound by issue and latency (FP32 filter, shared memory): the level-3
+// sphere with 8 slabs takes 18.6 ms (a warp per face: 125.9), the level-2 sphere
+// with 32 slabs 6.8 ms (24.0).
+// Work items are runs of kPatternRun test columns against one trial column,
+// whose image is then loaded once; short runs on small meshes keep every SM
+// busy. The grid takes the items of all operators of a batch (S > 1; the
+// contexts share the largest column sizes, so the shared layout is uniform),
+// prefix counting items; one operator comes as the kernel argument.
+constexpr int kPatternThreads = 128;
 
-__global__ void __launch_bounds__(128) k_pattern_blocks(BlockCtx B) {
+__global__ void __launch_bounds__(kPatternThreads) k_pattern(const BlockCtx one, const BlockCtx* __restrict__ many,
+                                                             const int64_t* __restrict__ prefix, int S, int run,
+                                                             int64_t items, unsigned long long* counter) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ ColSm C;
-  __shared__ int s_w[4];
-  __shared__ unsigned long long s_n[4];
-  const int64_t nblk = B.n_col * B.n_col;
-  for (;;) {
-    int64_t b = pop_block(B.counter);
-    if (b >= nblk) break;
-    pattern_block(B, b, smem, C, s_w, s_n);
-  }
-}
-
-// The same over the blocks of a batch of operators (one work queue; the
-// contexts share the largest column sizes so the shared layout is uniform).
-__global__ void __launch_bounds__(128) k_pattern_batch(const BlockCtx* __restrict__ Bs,
-                                                       const int64_t* __restrict__ prefix, int S,
-                                                       unsigned long long* counter) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ ColSm C;
-  __shared__ int s_w[4];
-  __shared__ unsigned long long s_n[4];
-  __shared__ BlockCtx sB;
+  __shared__ BlockSm C;
+  __shared__ int s_w[kPatternThreads / 32];
+  __shared__ unsigned long long s_n[kPatternThreads / 32];
+  __shared__ BlockCtx B;
   __shared__ int s_seg;
-  int cur = -1;
-  const int64_t total = prefix[S];
+  if (threadIdx.x == 0 && S <= 1) B = one;
+  int cur = S > 1 ? -1 : 0;
+  const BlockPtr P = block_ptr(smem, one.max_tet, one.max_surf, one.nq);
   for (;;) {
     int64_t g = pop_block(counter);
-    if (g >= total) break;
-    if (threadIdx.x == 0) s_seg = find_seg(prefix, S, g);
-    __syncthreads();
-    const int seg = s_seg;
-    if (seg != cur) {
-      if (threadIdx.x == 0) sB = Bs[seg];
+    if (g >= items) break;
+    if (S > 1) {
+      if (threadIdx.x == 0) s_seg = find_seg(prefix, S, g);
+      __syncthreads();
+      const int seg = s_seg;
+      if (seg != cur && threadIdx.x == 0) B = many[seg];
       cur = seg;
+      g -= prefix[seg];
+      __syncthreads();
     }
-    __syncthreads();
-    pattern_block(sB, g - prefix[seg], smem, C, s_w, s_n);
+    const int64_t I0 = g / B.n_col * run, J = g % B.n_col;
+    load_trial(B, J, C, P.pan);
+    for (int64_t I = I0; I < min(I0 + run, B.n_col); ++I) {
+      load_test(B, I, C);
+      block_bits(B, C, P);
+      pattern_block(B, C, P, s_w, s_n);
+    }
   }
 }
+
+// test columns per work item of the pattern pass
+static int pattern_run(int64_t n_blocks) { return (int)std::max<int64_t>(1, std::min<int64_t>(8, n_blocks / 16384)); }
 
 // shared bytes per warp for the deferred arcs of the mixed kernel
 constexpr size_t ARC_WARP_BYTES = 96 * sizeof(ArcRec<float>) + 96 * sizeof(float) + 96;
@@ -799,19 +769,17 @@ __global__ void __launch_bounds__(kQuadThreads, STBEM_QUAD_MIN_CTAS) k_quad_batc
   }
 }
 
-static size_t block_smem(const bem_operator* op, bool quad) {
+static size_t block_smem(const bem_operator* op) {
   const bem_mesh* m = op->mesh;
   int words = (m->max_col_tets + 31) / 32;
   size_t s = sizeof(TetSm) * m->max_col_tets + sizeof(FaceGeom) * m->max_col_surf;
   s += sizeof(uint32_t) * ((m->max_col_surf * words + 3) & ~3);
-  if (quad) {
-    s += sizeof(PointCol) * STBEM_QUAD_WARPS * op->nq;
-    s += (op->opts.precision == BEM_PREC_MIXED ? sizeof(float) : sizeof(double)) * STBEM_QUAD_WARPS * op->nq *
-         m->max_col_surf;
-    s += sizeof(uint16_t) * (((size_t)STBEM_QUAD_WARPS * op->nq * m->max_col_surf + 7) / 8 * 8);
-    s += sizeof(FaceF) * m->max_col_surf;
-    if (op->opts.precision == BEM_PREC_MIXED) s += 16 + STBEM_QUAD_WARPS * ARC_WARP_BYTES;
-  }
+  s += sizeof(PointCol) * STBEM_QUAD_WARPS * op->nq;
+  s += (op->opts.precision == BEM_PREC_MIXED ? sizeof(float) : sizeof(double)) * STBEM_QUAD_WARPS * op->nq *
+       m->max_col_surf;
+  s += sizeof(uint16_t) * (((size_t)STBEM_QUAD_WARPS * op->nq * m->max_col_surf + 7) / 8 * 8);
+  s += sizeof(FaceF) * m->max_col_surf;
+  if (op->opts.precision == BEM_PREC_MIXED) s += 16 + STBEM_QUAD_WARPS * ARC_WARP_BYTES;
   return s;
 }
 
@@ -849,8 +817,9 @@ static BlockCtx make_ctx(bem_operator* op) {
   B.rule = make_rule(op->opts.precision, op->n_theta);
   B.S = m->coord_scale;
   B.margin = (float)(1.6e-5 * m->coord_scale);  // > 4x the FP32 error bound of C2 and C3
-  B.cols = m->d_col; B.col_tet_begin = m->d_col_tet_begin; B.col_surf_begin = m->d_col_surf_begin;
-  B.surf = m->d_surf; B.tets = m->d_tet; B.pts = op->d_pts; B.ptsf = op->d_ptsf; B.trange = op->d_pts_trange;
+  B.cols = m->d_col; B.colf = static_cast<const ColF*>(m->d_colf); B.panf = static_cast<const PanelF*>(m->d_panf);
+  B.col_tet_begin = m->d_col_tet_begin; B.col_surf_begin = m->d_col_surf_begin;
+  B.surf = m->d_surf; B.tets = m->d_tet; B.pts = op->d_pts; B.ptsf = reinterpret_cast<const float4*>(op->d_ptsf); B.trange = op->d_pts_trange;
   B.bw = op->d_bw; B.bnnz = op->d_bnnz; B.boff = op->d_boff; B.rsoff = op->d_rsoff; B.rs = op->d_rs;
   B.val = op->d_val; B.val32 = op->d_val32; B.uscratch = op->d_tmp;
   B.max_surf = m->max_col_surf; B.max_tet = m->max_col_tets;
@@ -867,19 +836,26 @@ static bem_status get_counter(const bem_operator* op, unsigned long long** out, 
   return BEM_OK;
 }
 
+static bem_status launch_pattern(const BlockCtx& one, const BlockCtx* many, const int64_t* prefix, int S, int run,
+                                 int64_t items, unsigned long long* counter, cudaStream_t s) {
+  const size_t smem = bits_smem(one.max_tet, one.max_surf, one.nq);
+  const bem_status st = ensure_smem_attr((const void*)k_pattern, smem);
+  if (st != BEM_OK) return st;
+  const int64_t grid = std::min<int64_t>(persistent_grid((const void*)k_pattern, smem, kPatternThreads), items);
+  k_pattern<<<(unsigned)grid, kPatternThreads, smem, s>>>(one, many, prefix, S, run, items, counter);
+  STBEM_CUDA(cudaGetLastError());
+  return BEM_OK;
+}
+
 bem_status op_pattern(bem_operator* op, cudaStream_t s) {
   BlockCtx B = make_ctx(op);
   bem_status st = get_counter(op, &B.counter, s);
   if (st != BEM_OK) return st;
   STBEM_CUDA(cudaMemsetAsync(op->d_counter + 1, 0, sizeof(unsigned long long), s));
   B.inner = op->d_counter + 1;
-  size_t smem = block_smem(op, false);
-  st = ensure_smem_attr((const void*)k_pattern_blocks, smem);
-  if (st != BEM_OK) return st;
-  int grid = persistent_grid((const void*)k_pattern_blocks, smem, 128);
-  k_pattern_blocks<<<grid, 128, smem, s>>>(B);
-  STBEM_CUDA(cudaGetLastError());
-  return BEM_OK;
+  const int64_t nc = op->mesh->n_col;
+  const int run = pattern_run(nc * nc);
+  return launch_pattern(B, nullptr, nullptr, 1, run, nc * ((nc + run - 1) / run), B.counter, s);
 }
 
 // quadrature kernel of a precision and register budget (variant 0: the
@@ -892,7 +868,7 @@ static const void* quad_kernel(const bem_operator* op, int variant) {
 int quad_variants(const bem_operator* op) { return op->opts.precision == BEM_PREC_MIXED ? 2 : 1; }
 
 int quad_max_per_sm(const bem_operator* op, int variant) {
-  const size_t smem = block_smem(op, true);
+  const size_t smem = block_smem(op);
   const void* kern = quad_kernel(op, variant);
   ensure_smem_attr(kern, smem);
   return std::max(1, persistent_grid(kern, smem, kQuadThreads) / std::max(1, (int)op->ctx->sm_count));
@@ -909,7 +885,7 @@ bem_status quad_launch(const bem_operator* op, int per_sm, int64_t end, const do
   B.mf_nrhs = nrhs;
   B.mf_ld = op->mesh->n_tet;
   if (variant >= quad_variants(op)) variant = 0;
-  const size_t smem = block_smem(op, true);
+  const size_t smem = block_smem(op);
   const int max_per = quad_max_per_sm(op, variant);
   const int grid = (int)op->ctx->sm_count * std::max(1, std::min(per_sm, max_per));
   if ((int64_t)grid * op->mesh->max_col_surf * op->mesh->max_col_tets > op->tmp_len) {
@@ -962,22 +938,21 @@ static void batch_dims(const std::vector<bem_operator*>& ops, int& max_tet, int&
   }
 }
 
-static size_t batch_smem(int max_tet, int max_surf, int nq, bool quad, bool fp32 = false) {
+static size_t batch_smem(int max_tet, int max_surf, int nq, bool fp32) {
   int words = (max_tet + 31) / 32;
   size_t s = sizeof(TetSm) * max_tet + sizeof(FaceGeom) * max_surf;
   s += sizeof(uint32_t) * ((max_surf * words + 3) & ~3);
-  if (quad) {
-    s += sizeof(PointCol) * STBEM_QUAD_WARPS * nq;
-    s += (fp32 ? sizeof(float) : sizeof(double)) * STBEM_QUAD_WARPS * nq * max_surf;
-    s += sizeof(uint16_t) * (((size_t)STBEM_QUAD_WARPS * nq * max_surf + 7) / 8 * 8);
-    s += sizeof(FaceF) * max_surf;
-    if (fp32) s += 16 + STBEM_QUAD_WARPS * ARC_WARP_BYTES;
-  }
+  s += sizeof(PointCol) * STBEM_QUAD_WARPS * nq;
+  s += (fp32 ? sizeof(float) : sizeof(double)) * STBEM_QUAD_WARPS * nq * max_surf;
+  s += sizeof(uint16_t) * (((size_t)STBEM_QUAD_WARPS * nq * max_surf + 7) / 8 * 8);
+  s += sizeof(FaceF) * max_surf;
+  if (fp32) s += 16 + STBEM_QUAD_WARPS * ARC_WARP_BYTES;
   return s;
 }
 
+// run > 0: the prefix counts the pattern pass's work items, else blocks
 static bem_status upload_batch(const std::vector<bem_operator*>& ops, BatchDev& dev, int max_tet, int max_surf,
-                               cudaStream_t s) {
+                               int run, int64_t* total, BlockCtx* first, cudaStream_t s) {
   const int S = (int)ops.size();
   std::vector<BlockCtx> ctx(S);
   std::vector<int64_t> prefix(S + 1, 0);
@@ -987,8 +962,11 @@ static bem_status upload_batch(const std::vector<bem_operator*>& ops, BatchDev& 
     ctx[i].max_surf = max_surf;
     ctx[i].uscratch = dev.d_uscratch;
     ctx[i].counter = dev.d_counter;
-    prefix[i + 1] = prefix[i] + ops[i]->mesh->n_col * ops[i]->mesh->n_col;
+    const int64_t nc = ops[i]->mesh->n_col;
+    prefix[i + 1] = prefix[i] + nc * (run > 0 ? (nc + run - 1) / run : nc);
   }
+  *total = prefix[S];
+  if (first) *first = ctx[0];
   STBEM_CUDA(cudaMemcpyAsync(dev.d_ctx, ctx.data(), sizeof(BlockCtx) * S, cudaMemcpyHostToDevice, s));
   STBEM_CUDA(cudaMemcpyAsync(dev.d_prefix, prefix.data(), sizeof(int64_t) * (S + 1), cudaMemcpyHostToDevice, s));
   STBEM_CUDA(cudaMemsetAsync(dev.d_counter, 0, sizeof(unsigned long long), s));
@@ -1000,22 +978,20 @@ bem_status op_pattern_batch(const std::vector<bem_operator*>& ops, BatchDev& dev
   if (ops.empty()) return BEM_OK;
   int mt, ms;
   batch_dims(ops, mt, ms);
-  bem_status st = upload_batch(ops, dev, mt, ms, s);
+  int64_t blocks = 0, items = 0;
+  for (const bem_operator* op : ops) blocks += op->mesh->n_col * op->mesh->n_col;
+  const int run = pattern_run(blocks);
+  BlockCtx first;
+  bem_status st = upload_batch(ops, dev, mt, ms, run, &items, &first, s);
   if (st != BEM_OK) return st;
-  const size_t smem = batch_smem(mt, ms, ops[0]->nq, false);
-  st = ensure_smem_attr((const void*)k_pattern_batch, smem);
-  if (st != BEM_OK) return st;
-  const int grid = persistent_grid((const void*)k_pattern_batch, smem, 128);
-  k_pattern_batch<<<grid, 128, smem, s>>>(static_cast<const BlockCtx*>(dev.d_ctx), dev.d_prefix, (int)ops.size(),
-                                          dev.d_counter);
-  STBEM_CUDA(cudaGetLastError());
-  return BEM_OK;
+  return launch_pattern(first, static_cast<const BlockCtx*>(dev.d_ctx), dev.d_prefix, (int)ops.size(), run, items,
+                        dev.d_counter, s);
 }
 
 static int quad_batch_grid(const std::vector<bem_operator*>& ops, size_t& smem) {
   int mt, ms;
   batch_dims(ops, mt, ms);
-  smem = batch_smem(mt, ms, ops[0]->nq, true, ops[0]->opts.precision == BEM_PREC_MIXED);
+  smem = batch_smem(mt, ms, ops[0]->nq, ops[0]->opts.precision == BEM_PREC_MIXED);
   if (ops[0]->opts.precision == BEM_PREC_MIXED) {
     ensure_smem_attr((const void*)k_quad_batch<true>, smem);
     return persistent_grid((const void*)k_quad_batch<true>, smem, kQuadThreads);
@@ -1045,7 +1021,8 @@ bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& 
   }
   int mt, ms;
   batch_dims(ops, mt, ms);
-  bem_status st = upload_batch(ops, dev, mt, ms, s);
+  int64_t total = 0;
+  bem_status st = upload_batch(ops, dev, mt, ms, 0, &total, nullptr, s);
   if (st != BEM_OK) return st;
   size_t smem = 0;
   const int max_grid = quad_batch_grid(ops, smem);
@@ -1062,8 +1039,6 @@ bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& 
     STBEM_CUDA(cudaGetLastError());
     return BEM_OK;
   };
-  int64_t total = 0;
-  for (const bem_operator* op : ops) total += op->mesh->n_col * op->mesh->n_col;
   int per = occ, how = 0;
   if (ops[0]->ctx->tune_mode) {
     // the batch's own shape class; sample: 1/32 of the block queue
@@ -1157,33 +1132,23 @@ bem_status op_entries(const bem_operator* op, int64_t n, const int32_t* d_ij, do
 
 // Pattern rows (internal numbering): count pass, then fill pass (columns are
 // written in internal order; the caller permutes and sorts).
-__global__ void __launch_bounds__(128) k_pattern_rows(BlockCtx B, int64_t* rowcount, const int64_t* rowptr,
-                                                      int32_t* cols, int fill, int64_t I_only) {
+__global__ void __launch_bounds__(kPatternThreads) k_pattern_rows(BlockCtx B, int64_t* rowcount, const int64_t* rowptr,
+                                                                  int32_t* cols, int fill, int64_t I_only) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ ColSm C;
-  TetSm* T = reinterpret_cast<TetSm*>(smem);
-  FaceGeom* Fs = reinterpret_cast<FaceGeom*>(T + B.max_tet);
-  uint32_t* bits = reinterpret_cast<uint32_t*>(Fs + B.max_surf);
-  const int words = (B.max_tet + 31) / 32;
+  __shared__ BlockSm C;
+  const BlockPtr P = block_ptr(smem, B.max_tet, B.max_surf, B.nq);
+  const uint32_t* bits = P.bits;
+  const int words = bit_words(B.max_tet);
   const int64_t nblk = I_only >= 0 ? B.n_col : B.n_col * B.n_col;
   for (;;) {
     int64_t b = pop_block(B.counter);
     if (b >= nblk) break;
     if (I_only >= 0) b += I_only * B.n_col;
     if (B.bw[b] == 0) continue;
-    int64_t I = b / B.n_col, J = b % B.n_col;
-    load_column(B, J, C, T, Fs);
-    const ColGeom GI = B.cols[I];
-    double Dmax, Dmin_lo;
-    col_pair_bounds(GI, C.G, Dmax, Dmin_lo);
-    int s0 = B.col_surf_begin[I], ns = B.col_surf_begin[I + 1] - s0;
-    int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int f = warp; f < ns; f += nw) {
-      int jlo, jhi;
-      face_bits(B, C, T, s0 + f, Dmax, Dmin_lo, bits + f * words, words, jlo, jhi);
-    }
-    __syncthreads();
-    int t0 = B.col_tet_begin[I], nt = B.col_tet_begin[I + 1] - t0;
+    load_trial(B, b % B.n_col, C, P.pan);
+    load_test(B, b / B.n_col, C);
+    block_bits(B, C, P);
+    const int t0 = C.tetI, nt = C.ntI, s0 = C.surfI;
     for (int r = threadIdx.x; r < nt; r += blockDim.x) {
       const TetDev& D = B.tets[t0 + r];
       int lo = D.lo - s0, hi = D.hi - s0;
@@ -1197,7 +1162,7 @@ __global__ void __launch_bounds__(128) k_pattern_rows(BlockCtx B, int64_t* rowco
           while (m) {
             int l = __ffs(m) - 1;
             m &= m - 1;
-            cols[rowptr[t0 + r] + (int64_t)pos++] = C.tet0 + 32 * w + l;
+            cols[rowptr[t0 + r] + (int64_t)pos++] = C.tetJ + 32 * w + l;
           }
         }
       }
@@ -1211,13 +1176,13 @@ bem_status op_pattern_csr(const bem_operator* op, int64_t* d_rowcount, int64_t* 
   BlockCtx B = make_ctx(const_cast<bem_operator*>(op));
   bem_status st = get_counter(op, &B.counter, s);
   if (st != BEM_OK) return st;
-  size_t smem = block_smem(op, false);
+  const size_t smem = bits_smem(B.max_tet, B.max_surf, B.nq);
   {
     bem_status sa = ensure_smem_attr((const void*)k_pattern_rows, smem);
     if (sa != BEM_OK) return sa;
   }
-  int grid = persistent_grid((const void*)k_pattern_rows, smem, 128);
-  k_pattern_rows<<<grid, 128, smem, s>>>(B, d_rowcount, d_rowptr, d_cols, fill ? 1 : 0, I_only);
+  int grid = persistent_grid((const void*)k_pattern_rows, smem, kPatternThreads);
+  k_pattern_rows<<<grid, kPatternThreads, smem, s>>>(B, d_rowcount, d_rowptr, d_cols, fill ? 1 : 0, I_only);
   STBEM_CUDA(cudaGetLastError());
   return BEM_OK;
 }

@@ -75,6 +75,8 @@ struct bem_mesh {
   stbem::SurfDev* d_surf = nullptr;
   stbem::TetDev* d_tet = nullptr;
   int32_t* d_perm = nullptr;    // internal -> caller
+  void* d_colf = nullptr;       // FP32 images of the columns and panels (ColF, PanelF)
+  void* d_panf = nullptr;
 };
 
 struct bem_operator {
