@@ -99,12 +99,12 @@ const char* bem_version(void);
  * all); synchronizes the context stream. */
 bem_status bem_alu_peaks(bem_context* ctx, double* fp32_tflops, double* fp64_tflops);
 
-/* Launch-shape autotuning of the persistent quadrature (no counterpart in the
- * paper): the number of CTAs per SM it runs with. mode 0 (default): the
+/* Launch-shape autotuning of the quadrature (no counterpart in the paper): the
+ * number of CTAs per SM its persistent stage runs with. mode 0 (default): the
  * occupancy limit of the build. mode 1: the first assembly of every shape
  * class (device, precision, m_Q^2, rule order, largest column sizes, number
  * of columns to within a factor 2) on this context times each candidate on
- * 1/32 of the block queue and keeps the fastest; choices are kept for the
+ * 1/32 of the blocks and keeps the fastest; choices are kept for the
  * process and, when cache_path is not NULL, read from and appended to that
  * text file. Values do not depend on the shape (bit-identical either way).
  * Matrix-free operators keep the default. Operators take the context's mode
@@ -196,13 +196,12 @@ bem_status bem_operator_stats(const bem_operator* op, int64_t* nnz_pattern, int6
  * (a face shared by two test panels counted once). Counted by the pattern pass. */
 bem_status bem_operator_work(const bem_operator* op, int64_t* inner_integrals);
 
-/* The quadrature's launch shape: CTAs per SM, the CTAs per SM its register
- * budget was compiled for (4: 128 registers; 2: 255, mixed precision only),
- * how it was chosen (0 default, 1 timed in this assembly, 2 taken from the
- * tuning cache) and, when timed, the sample time in ms of each candidate
- * (index = 4 x (budget == 2) + CTAs per SM - 1; 0 where not timed). Untuned,
- * the 2-CTA budget is taken where shared memory admits no more than 2 CTAs
- * per SM anyway. Any pointer may be NULL; sample_ms has 8 entries. */
+/* The quadrature's launch shape: CTAs per SM of its persistent stage (1..4),
+ * the CTAs per SM its register budget was compiled for (4), how it was chosen
+ * (0 default, 1 timed in this assembly, 2 taken from the tuning cache) and,
+ * when timed, the sample time in ms of each candidate (index = CTAs per
+ * SM - 1; 0 where not timed). Any pointer may be NULL; sample_ms has 8
+ * entries. */
 bem_status bem_operator_tuning(const bem_operator* op, int* ctas_per_sm, int* budget_ctas, int* tuned,
                                double* sample_ms);
 
@@ -437,7 +436,8 @@ void bem_batch_destroy(bem_batch* batch);
  * admitted by HBM footprint: the bytes of the operator's values, row starts,
  * quadrature scratch and solver workspace are reserved against a pool of
  * hbm_budget minus the slots' shares (max(hbm_budget / (10 max_slots),
- * 64 MiB) each, for a request's mesh and sparsity structure); reservations
+ * 64 MiB) each, for a request's mesh and sparsity structure and, while it is
+ * assembled, what the quadrature's scratch takes of the rest); reservations
  * are granted in arrival order, a request waits in its slot until its
  * reservation fits, and a request that can never fit (in the pool or in its
  * slot's share) completes with BEM_ERR_OUT_OF_MEMORY. Slots run

@@ -14,16 +14,16 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libstbem.so")
-SOURCES = ["stbem_core.cu", "stbem_matvec.cu", "stbem_solver.cu", "stbem_gmres.cu", "stbem_capi.cu", "stbem_noalloc.cu", "stbem_server.cu", "stbem_batch.cu", "stbem_peaks.cu", "stbem_spmm_tc.cu", "stbem_tune.cu", "stbem_littree.cu"]
+SOURCES = ["stbem_core.cu", "stbem_stage.cu", "stbem_matvec.cu", "stbem_solver.cu", "stbem_gmres.cu", "stbem_capi.cu", "stbem_noalloc.cu", "stbem_server.cu", "stbem_batch.cu", "stbem_peaks.cu", "stbem_spmm_tc.cu", "stbem_tune.cu", "stbem_littree.cu"]
 HEADERS = ["stbem_quad.cuh", "stbem_block.cuh", "stbem_internal.h", "stbem_tc.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-# The quadrature translation unit: FP32 division and square root to within a
+# The quadrature translation units: FP32 division and square root to within a
 # few ulp (the hardware approximations). The mixed quadrature's error target
 # is 1e-7 relative, formed from cancellation-free expressions, and the FP64
 # arithmetic (cone geometry, the FP64 path, the sparsity contract) is
 # unaffected by these flags. (Flushing FP32 denormals as well measured slower
 # for both the quadrature and the pattern kernels.)
-SOURCE_FLAGS = {"stbem_core.cu": ["-prec-div=false", "-prec-sqrt=false"]}
+SOURCE_FLAGS = {s: ["-prec-div=false", "-prec-sqrt=false"] for s in ("stbem_core.cu", "stbem_stage.cu")}
 
 
 def nvcc() -> str:

@@ -95,6 +95,8 @@ bem_status bem_batch_create(bem_context* ctx, int32_t n, const bem_mesh* const* 
     std::vector<int64_t> bnnz(nb);
     STBEM_CUDA(cudaMemcpyAsync(bw.data(), op->d_bw, sizeof(int32_t) * nb, cudaMemcpyDeviceToHost, s));
     STBEM_CUDA(cudaMemcpyAsync(bnnz.data(), op->d_bnnz, sizeof(int64_t) * nb, cudaMemcpyDeviceToHost, s));
+    op->h_gran.resize(op->n_gran());
+    STBEM_CUDA(cudaMemcpyAsync(op->h_gran.data(), op->d_gran, sizeof(uint2) * op->n_gran(), cudaMemcpyDeviceToHost, s));
     STBEM_CUDA(cudaStreamSynchronize(s));
     B_TRY(op_layout(op, bw.data(), bnnz.data(), true, false, s));
     B->nnz += op->nnz;

@@ -17,11 +17,15 @@ struct PanelF {
 };
 static_assert(sizeof(PanelF) == 48, "PanelF layout");
 
-// FP32 image of a column: corners and centroid ball
+// FP32 image of a column: corners, frame and centroid ball
 struct ColF {
-  float Xh[3][3];
+  float Xh[3][3], Xl[3][3];            // corners as FP32 pairs
+  float nh[3], nl[3], e1h[3], e1l[3], e2h[3], e2l[3];
+  ColR<float> R;
   float ctr[3], rad;
 };
+static_assert(sizeof(ColF) % 16 == 0, "ColF is copied in 16-byte pieces");
+static_assert(sizeof(FaceF) == 48, "FaceF is copied in 16-byte pieces");
 
 struct BlockCtx {
   int64_t n_col;
@@ -34,10 +38,12 @@ struct BlockCtx {
   const int32_t* col_tet_begin;
   const int32_t* col_surf_begin;
   const SurfDev* surf;
+  const FaceF* facef;
   const TetDev* tets;
   const PanelF* panf;
   const double* pts;
   const float4* ptsf;          // outer points (t, x, y, z) rounded to FP32
+  const float4* ptsl;          // and the remainders: pts = ptsf + ptsl as FP32 pairs
   const double* trange;
   int32_t* bw;
   int64_t* bnnz;
@@ -46,11 +52,10 @@ struct BlockCtx {
   int32_t* rs;
   double* val;
   float* val32;
-  double* uscratch;     // [gridDim][max_surf][max_tet]
   int max_surf, max_tet;
   unsigned long long* counter;
-  int64_t end;                 // blocks [0, end) of the dense (I, J) order are processed
   unsigned long long* inner;   // pattern pass: inner integrals m_Q^2 x (test face, trial panel) (null: not counted)
+  uint2* gran;                 // pattern pass: (apexes, potentials) of each run of GRAN blocks (null: not counted)
   // matrix-free product: when mf_y is set the entries are not stored but
   // y[k][i] += A_ij x[k][j] is accumulated (x, y: [mf_nrhs][mf_ld], internal order)
   const double* mf_x;
@@ -58,6 +63,9 @@ struct BlockCtx {
   int mf_nrhs;
   int64_t mf_ld;
 };
+
+// the quadrature takes its scratch by runs of GRAN consecutive blocks
+constexpr int GRAN = 8;
 
 // shared-memory image of a block: the trial column's panels, the distances of
 // the test column's outer points to the trial corners, the faces' windows
@@ -278,6 +286,30 @@ __device__ inline int find_seg(const int64_t* prefix, int S, int64_t g) {
   return lo;
 }
 
+// surfaces of the panels in a face's bits: first and count (0: none)
+__device__ __forceinline__ void bits_surfaces(const uint32_t* fb, int words, const PanelF* pan, int& slo, int& n) {
+  int lo = 1 << 30, hi = -1;
+  for (int w = 0; w < words; ++w) {
+    uint32_t m = fb[w];
+    while (m) {
+      const int j = 32 * w + __ffs(m) - 1;
+      m &= m - 1;
+      const int a = pan[j].lo, b = pan[j].hi;
+      lo = min(lo, min(a, b));
+      hi = max(hi, max(a, b));
+    }
+  }
+  slo = hi < 0 ? 0 : lo;
+  n = hi < 0 ? 0 : hi - lo + 1;
+}
 #endif
+
+// quadrature in stages (stbem_stage.cu)
+int stage_apex_per_sm(bool fp32, int max_tet, int max_surf, int nq);
+void stage_scratch(bool fp32, int max_tet, int max_surf, int sms, const std::vector<const std::vector<uint2>*>& gran,
+                   int64_t value_bytes, int64_t* least, int64_t* wanted);
+bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* prefix, int S, bool fp32, int sms,
+                     const std::vector<const std::vector<uint2>*>& gran, const std::vector<int64_t>& blocks, int64_t end,
+                     void* scratch, int64_t bytes, int per_sm, cudaStream_t s);
 
 }  // namespace stbem

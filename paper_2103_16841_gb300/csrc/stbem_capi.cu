@@ -343,7 +343,7 @@ void bem_mesh_destroy(bem_mesh* m) {
   if (!m) return;
   cudaFree(m->d_col); cudaFree(m->d_col_tet_begin); cudaFree(m->d_col_surf_begin);
   cudaFree(m->d_surf); cudaFree(m->d_tet); cudaFree(m->d_perm);
-  cudaFree(m->d_colf); cudaFree(m->d_panf);
+  cudaFree(m->d_colf); cudaFree(m->d_facef); cudaFree(m->d_panf);
   delete m;
 }
 
@@ -375,10 +375,16 @@ bem_status stbem::op_layout(bem_operator* op, const int32_t* bw, const int64_t* 
     op->nstored = vo; op->nrows_stored = ro; op->nnz = nnz; op->nblocks = nblk;
     op->max_bw = wmax;
     if (own_scratch) {
-      const int64_t grid = (int64_t)op->ctx->sm_count * quad_max_per_sm(op, 0);
-      op->tmp_len = std::max<int64_t>((int64_t)grid * m->max_col_surf * m->max_col_tets, 2 * m->n_tet * 8);
+      int64_t least = 0;
+      quad_scratch(op, &least, &op->tmp_len);
+      // what an admission reserves for it: U of up to four CTAs per SM
+      const int64_t smem = 44000 + 152 * m->max_col_tets + 312 * m->max_col_surf;
+      const int64_t per = std::max<int64_t>(1, std::min<int64_t>(4, 232448 / smem));
+      op->reserve_len = std::max<int64_t>((int64_t)op->ctx->sm_count * per * m->max_col_surf * m->max_col_tets,
+                                          16 * m->n_tet);
+      if (op->scratch_cap >= 0) op->tmp_len = std::max(least, std::min(op->tmp_len, op->reserve_len + op->scratch_cap / 8));
     } else {
-      op->tmp_len = 0;
+      op->tmp_len = op->reserve_len = 0;
     }
     if (op->opts.matrix_free) op->nstored = 0;
     if (op->admit) TRY(op->admit(op));
@@ -389,7 +395,13 @@ bem_status stbem::op_layout(bem_operator* op, const int32_t* bw, const int64_t* 
       if (op->opts.store_fp32 || op->opts.precision == BEM_PREC_MIXED) TRY(dalloc(&op->d_val32, (size_t)vo + 8));
       TRY(dalloc(&op->d_rs, (size_t)ro + 4));   // (tail room as for the values)
     }
-    if (own_scratch) TRY(dalloc(&op->d_tmp, (size_t)op->tmp_len));
+    if (own_scratch && op->scratch_cap < 0) TRY(dalloc(&op->d_tmp, (size_t)op->tmp_len));
+    if (own_scratch && op->scratch_cap >= 0 && cudaMallocAsync((void**)&op->d_tmp, sizeof(double) * op->tmp_len, s) != cudaSuccess) {
+      cudaGetLastError();
+      op->d_tmp = nullptr;
+      set_error("out of device memory (quadrature scratch)");
+      return BEM_ERR_OUT_OF_MEMORY;
+    }
   } else if ((!op->opts.matrix_free && vo != op->nstored) || nnz != op->nnz) {
     set_error("reassembly changed the sparsity structure");
     return BEM_ERR_INTERNAL;
@@ -425,6 +437,8 @@ bem_status stbem::op_structure_alloc(bem_context* ctx, const bem_mesh* mesh, con
   const int64_t nb = mesh->n_col * mesh->n_col;
   TRY(dalloc(&op->d_pts, (size_t)mesh->n_surf * op->nq * 4));
   TRY(dalloc(&op->d_ptsf, (size_t)mesh->n_surf * op->nq * 4));
+  TRY(dalloc(&op->d_ptsl, (size_t)mesh->n_surf * op->nq * 4));
+  TRY(dalloc(&op->d_gran, (size_t)op->n_gran()));
   TRY(dalloc(&op->d_pts_trange, (size_t)mesh->n_surf * 2));
   TRY(dalloc(&op->d_bw, (size_t)nb));
   TRY(dalloc(&op->d_bnnz, (size_t)nb));
@@ -454,6 +468,8 @@ bem_status assemble(bem_operator* op, cudaStream_t s, bool first) {
   std::vector<int64_t> bnnz(nb);
   STBEM_CUDA(cudaMemcpyAsync(bw.data(), op->d_bw, sizeof(int32_t) * nb, cudaMemcpyDeviceToHost, s));
   STBEM_CUDA(cudaMemcpyAsync(bnnz.data(), op->d_bnnz, sizeof(int64_t) * nb, cudaMemcpyDeviceToHost, s));
+  op->h_gran.resize(op->n_gran());
+  STBEM_CUDA(cudaMemcpyAsync(op->h_gran.data(), op->d_gran, sizeof(uint2) * op->n_gran(), cudaMemcpyDeviceToHost, s));
   unsigned long long n_inner = 0;
   STBEM_CUDA(cudaMemcpyAsync(&n_inner, op->d_counter + 1, sizeof(n_inner), cudaMemcpyDeviceToHost, s));
   STBEM_CUDA(cudaStreamSynchronize(s));
@@ -483,7 +499,12 @@ int64_t stbem::operator_value_bytes(const bem_operator* op) {
   int64_t b = 0;
   if (op->opts.precision == BEM_PREC_FP64) b += 8 * op->nstored;
   if (op->opts.store_fp32 || op->opts.precision == BEM_PREC_MIXED) b += 4 * op->nstored;
-  return b + 4 * op->nrows_stored + 8 * op->tmp_len;
+  return b + 4 * op->nrows_stored + 8 * op->reserve_len;
+}
+
+void stbem::operator_release_scratch(bem_operator* op, cudaStream_t s) {
+  if (op->d_tmp) cudaFreeAsync(op->d_tmp, s);
+  op->d_tmp = nullptr;
 }
 
 extern "C" {
@@ -495,7 +516,8 @@ bem_status bem_operator_create(bem_context* ctx, const bem_mesh* mesh, const bem
 }  // extern "C"
 
 bem_status stbem::operator_create(bem_context* ctx, const bem_mesh* mesh, const bem_op_opts* opts,
-                                  std::function<bem_status(const bem_operator*)> admit, bem_operator** out) {
+                                  std::function<bem_status(const bem_operator*)> admit, bem_operator** out,
+                                  int64_t scratch_cap) {
   if (!ctx || !mesh || !out) { set_error("bem_operator_create: invalid argument"); return BEM_ERR_INVALID_ARG; }
   *out = nullptr;
   bem_op_opts o{};
@@ -519,6 +541,7 @@ bem_status stbem::operator_create(bem_context* ctx, const bem_mesh* mesh, const 
   bem_status st = op_structure_alloc(ctx, mesh, &o, op);
   if (st != BEM_OK) { if (op) bem_operator_destroy(op.release()); return st; }
   op->admit = std::move(admit);
+  op->scratch_cap = scratch_cap;
   st = assemble(op.get(), ctx->stream, true);
   if (st != BEM_OK) { bem_operator_destroy(op.release()); return st; }
   int64_t nbad = 0;
@@ -584,7 +607,7 @@ bem_status bem_operator_stats(const bem_operator* op, int64_t* nnz, int64_t* sto
 
 void bem_operator_destroy(bem_operator* op) {
   if (!op) return;
-  cudaFree(op->d_pts); cudaFree(op->d_ptsf); cudaFree(op->d_pts_trange); cudaFree(op->d_bw); cudaFree(op->d_bnnz);
+  cudaFree(op->d_pts); cudaFree(op->d_ptsf); cudaFree(op->d_ptsl); cudaFree(op->d_gran); cudaFree(op->d_pts_trange); cudaFree(op->d_bw); cudaFree(op->d_bnnz);
   cudaFree(op->d_boff); cudaFree(op->d_rsoff); cudaFree(op->d_rs); cudaFree(op->d_val);
   cudaFree(op->d_val32); cudaFree(op->d_tmp); cudaFree(op->d_counter);
   cudaFree(op->d_ws); cudaFree(op->d_pv);

@@ -1,14 +1,8 @@
-// Kernels of the light-cone-clipped single-layer Galerkin assembly.
-//
-// Work decomposition: the matrix is cut into blocks (I, J) of panels over
-// spatial triangle ("column") I times panels over column J. A persistent
-// grid pops blocks from a device counter. For every face F with nu_{F,t} != 0
-// over column I and every outer point x_q on F (composite midpoint rule,
-// Fig. int_tri_mid), the kernel evaluates the potentials W of the faces over
-// column J that the backward light cone of x_q cuts, and forms
-//     U[F][j] = sum_q V 1_{sigma_j}(x_q) = sum_q (W_lo(j)(x_q) - W_hi(j)(x_q)),
-// then the entries A_ij = |K_I| / m_Q^2 * (U[F_lo(i)][j] - U[F_hi(i)][j])
-// (eq. int_bform with nu_{F,t}|F| = -|K| on the lower face, +|K| on the upper).
+// Mesh geometry, outer points, the sparsity pattern pass, right-hand sides and
+// look-ups of the light-cone-clipped single-layer Galerkin matrix. The matrix
+// is cut into blocks (I, J) of panels over spatial triangle ("column") I
+// times panels over column J; persistent grids pop blocks from a device
+// counter. The quadrature itself is in stbem_stage.cu.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -69,7 +63,7 @@ bem_status upload_gauss_tables() {
   STBEM_CUDA(cudaMemcpyToSymbol(c_gl_w, W.data(), W.size() * sizeof(double)));
   STBEM_CUDA(cudaMemcpyToSymbol(c_gl_xf, Xf.data(), Xf.size() * sizeof(float)));
   STBEM_CUDA(cudaMemcpyToSymbol(c_gl_wf, Wf.data(), Wf.size() * sizeof(float)));
-  return BEM_OK;
+  return upload_gauss_stage(X.data(), W.data(), Xf.data(), Wf.data(), X.size());
 }
 
 // ---------------------------------------------------------------------------
@@ -117,17 +111,30 @@ __global__ void k_tet_ball(int64_t n_tet, const double* tet_vx, TetDev* tets) {
   tets[i].ball[4] = mx;
 }
 
-// FP32 images of the columns and panels for the sparsity filter
+// FP32 images of the columns, faces and panels
 __global__ void k_col_f32(int64_t n_col, const ColGeom* cols, ColF* out) {
   int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (c >= n_col) return;
   const ColGeom& G = cols[c];
   ColF F;
   for (int k = 0; k < 3; ++k)
-    for (int i = 0; i < 3; ++i) F.Xh[k][i] = (float)G.X[k][i];
+    for (int i = 0; i < 3; ++i) split2(G.X[k][i], F.Xh[k][i], F.Xl[k][i]);
+  for (int i = 0; i < 3; ++i) {
+    split2(G.n[i], F.nh[i], F.nl[i]);
+    split2(G.e1[i], F.e1h[i], F.e1l[i]);
+    split2(G.e2[i], F.e2h[i], F.e2l[i]);
+  }
+  make_colr<float>(G, F.R);
   for (int i = 0; i < 3; ++i) F.ctr[i] = (float)G.ctr[i];
   F.rad = (float)G.rad;
   out[c] = F;
+}
+__global__ void k_face_f32(int64_t n_surf, const SurfDev* surf, FaceF* out) {
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n_surf) return;
+  FaceF F;
+  make_facef(surf[i].f, F);
+  out[i] = F;
 }
 __global__ void k_panel_f32(int64_t n_tet, const TetDev* tets, const int32_t* col_surf_begin, PanelF* out) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -155,7 +162,10 @@ bem_status mesh_device_geometry(bem_mesh* m, const double* d_sv_xyz, const int32
                                                                    m->d_surf);
   k_tet_ball<<<(unsigned)((m->n_tet + th - 1) / th), th, 0, s>>>(m->n_tet, d_tet_vx, m->d_tet);
   STBEM_CUDA(cudaMalloc(&m->d_colf, sizeof(ColF) * m->n_col));
+  STBEM_CUDA(cudaMalloc(&m->d_facef, sizeof(FaceF) * m->n_surf));
   STBEM_CUDA(cudaMalloc(&m->d_panf, sizeof(PanelF) * m->n_tet));
+  k_face_f32<<<(unsigned)((m->n_surf + th - 1) / th), th, 0, s>>>(m->n_surf, m->d_surf,
+                                                                  static_cast<FaceF*>(m->d_facef));
   k_col_f32<<<(unsigned)((m->n_col + th - 1) / th), th, 0, s>>>(m->n_col, m->d_col, static_cast<ColF*>(m->d_colf));
   k_panel_f32<<<(unsigned)((m->n_tet + th - 1) / th), th, 0, s>>>(m->n_tet, m->d_tet, m->d_col_surf_begin,
                                                                   static_cast<PanelF*>(m->d_panf));
@@ -168,7 +178,7 @@ bem_status mesh_device_geometry(bem_mesh* m, const double* d_sv_xyz, const int32
 // id) and x = (A + xi1 (B - A)) + xi2 (C - A) without fused operations.
 // ---------------------------------------------------------------------------
 __global__ void k_outer_points(int64_t n_surf, int mq, const ColGeom* cols, const SurfDev* surf, double* pts,
-                               float* ptsf, double* trange) {
+                               float* ptsf, float* ptsl, double* trange) {
   int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (s >= n_surf) return;
   const SurfDev S = surf[s];
@@ -189,7 +199,8 @@ __global__ void k_outer_points(int64_t n_surf, int mq, const ColGeom* cols, cons
         for (int d = 0; d < 4; ++d) {
           double p = __dadd_rn(A[d], __dmul_rn(x1, __dsub_rn(B[d], A[d])));
           out[4 * n + d] = __dadd_rn(p, __dmul_rn(x2, __dsub_rn(C[d], A[d])));
-          ptsf[(int64_t)s * nq * 4 + 4 * n + d] = (float)out[4 * n + d];
+          const int64_t o = (int64_t)s * nq * 4 + 4 * n + d;
+          split2(out[4 * n + d], ptsf[o], ptsl[o]);
         }
         tlo = fmin(tlo, out[4 * n]);
         thi = fmax(thi, out[4 * n]);
@@ -204,174 +215,9 @@ bem_status op_outer_points(bem_operator* op, cudaStream_t s) {
   const bem_mesh* m = op->mesh;
   int th = 128;
   k_outer_points<<<(unsigned)((m->n_surf + th - 1) / th), th, 0, s>>>(m->n_surf, op->mq, m->d_col, m->d_surf,
-                                                                      op->d_pts, op->d_ptsf, op->d_pts_trange);
+                                                                      op->d_pts, op->d_ptsf, op->d_ptsl, op->d_pts_trange);
   STBEM_CUDA(cudaGetLastError());
   return BEM_OK;
-}
-
-// ---------------------------------------------------------------------------
-// Sparsity predicate for one outer point and one panel (the contract):
-//   C1  tau_min(j) < t_q
-//   C2  max_b |x_q - y_b| - (t_q - tau_b) >= 0
-//   C3  not (phi_Xi(x_q - c_j) - d_r(|x_q - c_j|) > 0)     (Theorem phi_xi_sphere)
-// FP64 values with the contract's operation order decide; an FP32 estimate
-// with a rigorous error margin settles the clear cases first.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ float dist3f(const float* a, const float* b) { return dist3f(a[0], a[1], a[2], b); }
-
-struct TetSm {       // panel data kept in shared memory for a block
-  double tmin, pmax;
-  double vt[4];
-  double ball[5];
-  float vtf[4];      // FP32 copies for the filter of the sparsity predicate
-  float ballf[5];
-  int32_t lo, hi, dup, pad;
-};
-
-__device__ __noinline__ bool c2_exact(const double* x, const TetSm& T, const ColGeom& G) {
-  double mx = -INFINITY;
-  for (int b = 0; b < 4; ++b) {
-    int k = b < 3 ? b : T.dup;
-    double v = __dsub_rn(dist3x(x + 1, G.X[k]), __dsub_rn(x[0], T.vt[b]));
-    if (v > mx) mx = v;
-  }
-  return mx >= 0.0;
-}
-__device__ __noinline__ bool c3_fail_exact(const double* x, const TetSm& T) {
-  double al = dist3x(x + 1, T.ball + 1);
-  double phi = __dsub_rn(al, __dsub_rn(x[0], T.ball[0]));
-  double rj = T.ball[4];
-  double s2 = __dsqrt_rn(2.0);
-  double dr = (al < __ddiv_rn(rj, s2)) ? __dadd_rn(al, __dsqrt_rn(__dsub_rn(__dmul_rn(rj, rj), __dmul_rn(al, al))))
-                                       : __dmul_rn(rj, s2);
-  return __dsub_rn(phi, dr) > 0.0;
-}
-
-__device__ bool point_sees(const double* x, const float* xf, const TetSm& T, const ColGeom& G, const float (*Xf)[3],
-                           float margin) {
-  if (!(T.tmin < x[0])) return false;  // C1
-  // C2
-  {
-    bool sure_true = false, sure_false = true;
-    for (int b = 0; b < 4; ++b) {
-      int k = b < 3 ? b : T.dup;
-      float v = dist3f(xf + 1, Xf[k]) - (xf[0] - T.vtf[b]);
-      if (v > margin) sure_true = true;
-      if (!(v < -margin)) sure_false = false;
-    }
-    if (!sure_true) {
-      if (sure_false) return false;
-      if (!c2_exact(x, T, G)) return false;
-    }
-  }
-  // C3
-  {
-    float al = dist3f(xf + 1, T.ballf + 1);
-    float phi = al - (xf[0] - T.ballf[0]);
-    float rj = T.ballf[4];
-    float dr = (al < rj * 0.70710678f) ? al + __fsqrt_rn(fmaxf(rj * rj - al * al, 0.f)) : rj * 1.41421356f;
-    float v = phi - dr;
-    if (v > margin) return false;
-    if (!(v < -margin)) {
-      if (c3_fail_exact(x, T)) return false;
-    }
-  }
-  return true;
-}
-
-// shared-memory image of column J
-struct ColSm {
-  ColGeom G;
-  float Xf[3][3];
-  int32_t tet0, ntet, surf0, nsurf;
-  double rmax;  // max panel ball radius
-};
-
-// Trial window of column J for a face with outer-point time range [tlo, thi]:
-// panels outside [jlo, jhi) are certainly outside the pattern.
-__device__ inline void trial_window(const ColSm& C, const TetSm* T, double tlo, double thi, double Dmax,
-                                    double Dmin_lo, double S, int& jlo, int& jhi) {
-  double lim1 = tlo - Dmax * (1.0 + 1e-12) - 1e-12 * S;
-  int a = 0, b = C.ntet;  // first j with pmax >= lim1
-  while (a < b) { int m = (a + b) >> 1; if (T[m].pmax < lim1) a = m + 1; else b = m; }
-  jlo = a;
-  double lim2 = thi + fmin(0.0, C.rmax * 1.41421356237309515 * (1.0 + 1e-12) - Dmin_lo * (1.0 - 1e-12)) + 1e-12 * S;
-  a = jlo; b = C.ntet;    // first j with tmin >= lim2
-  while (a < b) { int m = (a + b) >> 1; if (T[m].tmin < lim2) a = m + 1; else b = m; }
-  jhi = a;
-}
-
-__device__ inline void col_pair_bounds(const ColGeom& GI, const ColGeom& GJ, double& Dmax, double& Dmin_lo) {
-  Dmax = 0.0;
-  for (int a = 0; a < 3; ++a)
-    for (int b = 0; b < 3; ++b) {
-      double dx = GI.X[a][0] - GJ.X[b][0], dy = GI.X[a][1] - GJ.X[b][1], dz = GI.X[a][2] - GJ.X[b][2];
-      Dmax = fmax(Dmax, sqrt(dx * dx + dy * dy + dz * dz));
-    }
-  double dx = GI.ctr[0] - GJ.ctr[0], dy = GI.ctr[1] - GJ.ctr[1], dz = GI.ctr[2] - GJ.ctr[2];
-  Dmin_lo = fmax(0.0, sqrt(dx * dx + dy * dy + dz * dz) - GI.rad - GJ.rad);
-}
-
-// cooperative load of column J into shared memory
-__device__ void load_column(const BlockCtx& B, int64_t J, ColSm& C, TetSm* T, FaceGeom* Fs) {
-  if (threadIdx.x == 0) {
-    C.G = B.cols[J];
-    for (int k = 0; k < 3; ++k)
-      for (int i = 0; i < 3; ++i) C.Xf[k][i] = (float)C.G.X[k][i];
-    C.tet0 = B.col_tet_begin[J];
-    C.ntet = B.col_tet_begin[J + 1] - C.tet0;
-    C.surf0 = B.col_surf_begin[J];
-    C.nsurf = B.col_surf_begin[J + 1] - C.surf0;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < C.ntet; j += blockDim.x) {
-    const TetDev& D = B.tets[C.tet0 + j];
-    TetSm t;
-    t.tmin = D.tmin; t.pmax = D.pmax;
-    for (int k = 0; k < 4; ++k) { t.vt[k] = D.vt[k]; t.vtf[k] = (float)D.vt[k]; }
-    for (int k = 0; k < 5; ++k) { t.ball[k] = D.ball[k]; t.ballf[k] = (float)D.ball[k]; }
-    t.lo = D.lo - C.surf0; t.hi = D.hi - C.surf0; t.dup = D.dup; t.pad = 0;
-    T[j] = t;
-  }
-  for (int s = threadIdx.x; s < C.nsurf; s += blockDim.x) Fs[s] = B.surf[C.surf0 + s].f;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int j = 0; j < C.ntet; ++j) r = fmax(r, T[j].ball[4]);
-    C.rmax = r;
-  }
-  __syncthreads();
-}
-
-// pattern bits of one face f' (global id) of column I against column J.
-// Warp-cooperative; writes bits[0..words) and returns the trial window.
-__device__ void face_bits(const BlockCtx& B, const ColSm& C, const TetSm* T, int64_t fglob, double Dmax,
-                          double Dmin_lo, uint32_t* bits, int words, int& jlo, int& jhi) {
-  int lane = threadIdx.x & 31;
-  double tlo = B.trange[2 * fglob], thi = B.trange[2 * fglob + 1];
-  trial_window(C, T, tlo, thi, Dmax, Dmin_lo, B.S, jlo, jhi);
-  for (int w = lane; w < words; w += 32) bits[w] = 0u;
-  __syncwarp();
-  const double* P = B.pts + fglob * B.nq * 4;
-  const float4* Pf = B.ptsf + fglob * B.nq;   // FP32 copies: no conversions in the filter
-  for (int j0 = jlo; j0 < jhi; j0 += 32) {
-    int j = j0 + lane;
-    bool hit = false;
-    if (j < jhi) {
-      for (int q = 0; q < B.nq && !hit; ++q) {
-        const float4 x4 = Pf[q];
-        const float xf[4] = {x4.x, x4.y, x4.z, x4.w};
-        hit = point_sees(P + 4 * q, xf, T[j], C.G, C.Xf, B.margin);
-      }
-    }
-    unsigned m = __ballot_sync(0xffffffffu, hit);
-    if (lane == 0 && m) {
-      // j0 may not be word aligned: scatter bit by bit
-      for (int l = 0; l < 32; ++l)
-        if (m & (1u << l)) bits[(j0 + l) >> 5] |= 1u << ((j0 + l) & 31);
-    }
-    __syncwarp();
-  }
 }
 
 __device__ inline int64_t pop_block(unsigned long long* counter) {
@@ -417,6 +263,22 @@ __device__ __forceinline__ void pattern_block(const BlockCtx& B, const BlockSm& 
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { w = max(w, s_w[i]); n += s_n[i]; }
     B.bw[b] = w;
     B.bnnz[b] = (int64_t)n;
+  }
+  if (B.gran && C.wmax > 0) {
+    // apexes and potentials of the quadrature (k_apex)
+    unsigned rays = 0, slots = 0;
+    for (int f = threadIdx.x; f < C.nsI; f += blockDim.x) {
+      int slo, n;
+      bits_surfaces(P.bits + f * words, words, P.pan, slo, n);
+      if (n) rays += B.nq;
+      slots += n * B.nq;
+    }
+    rays = __reduce_add_sync(0xffffffffu, rays);
+    slots = __reduce_add_sync(0xffffffffu, slots);
+    if ((threadIdx.x & 31) == 0 && rays) {
+      atomicAdd(&B.gran[b / GRAN].x, rays);
+      atomicAdd(&B.gran[b / GRAN].y, slots);
+    }
   }
   if (B.inner && C.wmax > 0) {
     // inner integrals of the block: every outer point of a test face against
@@ -476,313 +338,6 @@ __global__ void __launch_bounds__(kPatternThreads) k_pattern(const BlockCtx one,
 // test columns per work item of the pattern pass
 static int pattern_run(int64_t n_blocks) { return (int)std::max<int64_t>(1, std::min<int64_t>(8, n_blocks / 16384)); }
 
-// shared bytes per warp for the deferred arcs of the mixed kernel
-constexpr size_t ARC_WARP_BYTES = 96 * sizeof(ArcRec<float>) + 96 * sizeof(float) + 96;
-static_assert(ARC_WARP_BYTES % 16 == 0, "arc region keeps 16-byte alignment");
-
-// Pass 2: quadrature and assembly of a non-empty block.
-template <bool FP32>
-__device__ __forceinline__ void quad_block(const BlockCtx& B, int64_t b, unsigned char* smem, ColSm& C,
-                                           ColR<typename std::conditional<FP32, float, double>::type>& CR) {
-  typedef typename std::conditional<FP32, float, double>::type R;
-  TetSm* T = reinterpret_cast<TetSm*>(smem);
-  FaceGeom* Fs = reinterpret_cast<FaceGeom*>(T + B.max_tet);
-  uint32_t* bits = reinterpret_cast<uint32_t*>(Fs + B.max_surf);
-  const int words = (B.max_tet + 31) / 32;
-  PointCol* pc = reinterpret_cast<PointCol*>(bits + ((B.max_surf * words + 3) & ~3));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  PointCol* mypc = pc + warp * B.nq;
-  R* Wsc0 = reinterpret_cast<R*>(pc + nw * B.nq);
-  R* Wsc = Wsc0 + (size_t)warp * B.nq * B.max_surf;
-  uint16_t* cut0 = reinterpret_cast<uint16_t*>(Wsc0 + (size_t)nw * B.nq * B.max_surf);
-  uint16_t* mycut = cut0 + (size_t)warp * B.nq * B.max_surf;
-  FaceF* Ff = reinterpret_cast<FaceF*>(cut0 + ((size_t)nw * B.nq * B.max_surf + 7) / 8 * 8);
-  // mixed: per warp 96 deferred arcs (3 per lane), their values and the compacted order
-  unsigned char* arc0 = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(Ff + B.max_surf) + 15) & ~static_cast<uintptr_t>(15));
-  ArcRec<float>* myarc = reinterpret_cast<ArcRec<float>*>(arc0 + (size_t)warp * ARC_WARP_BYTES);
-  float* myval = reinterpret_cast<float*>(myarc + 96);
-  uint8_t* myidx = reinterpret_cast<uint8_t*>(myval + 96);
-  R* U = reinterpret_cast<R*>(B.uscratch) + (size_t)blockIdx.x * B.max_surf * B.max_tet;
-  {
-    int W = B.bw[b];
-    if (W == 0) return;
-    int64_t I = b / B.n_col, J = b % B.n_col;
-    load_column(B, J, C, T, Fs);
-    if (threadIdx.x == 0) make_colr<R>(C.G, CR);
-    if (FP32)
-      for (int s = threadIdx.x; s < C.nsurf; s += blockDim.x) make_facef(Fs[s], Ff[s]);
-    __syncthreads();
-    const ColGeom GI = B.cols[I];
-    double Dmax, Dmin_lo;
-    col_pair_bounds(GI, C.G, Dmax, Dmin_lo);
-    const int s0 = B.col_surf_begin[I], ns = B.col_surf_begin[I + 1] - s0;
-    const int ntJ = C.ntet;
-    const float fdiam = (float)C.G.diam;
-    // The warps take the phases of their surfaces in lockstep (a CTA barrier
-    // between face bits, point geometry, classification, the cut pass and the
-    // U rows): all warps of the CTA then run the same code region, and the
-    // instruction fetches they share hit (level-3 sphere, 16 slabs: 2,373 ->
-    // 1,766 ms; benchmark mesh 5.83 -> 4.11 s).
-    for (int f0 = 0; f0 < ns; f0 += nw) {
-      const int f = f0 + warp;
-      int jlo = 0, jhi = 0;
-      const int64_t fg = s0 + f;
-      R* Urow = U + (size_t)f * B.max_tet;
-      if (f < ns) {
-        face_bits(B, C, T, fg, Dmax, Dmin_lo, bits + f * words, words, jlo, jhi);
-        for (int j = lane; j < ntJ; j += 32) Urow[j] = R(0);
-      }
-      const bool skip = f >= ns || jhi <= jlo;
-      int slo = 1 << 30, shi = -1, nsw = 0, ncut = 0;
-      const double* P = B.pts + fg * B.nq * 4;
-      __syncthreads();
-      if (!skip) {
-      // surface window of the trial panels
-      for (int j = jlo + lane; j < jhi; j += 32) {
-        slo = min(slo, min(T[j].lo, T[j].hi));
-        shi = max(shi, max(T[j].lo, T[j].hi));
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        slo = min(slo, __shfl_xor_sync(0xffffffffu, slo, o));
-        shi = max(shi, __shfl_xor_sync(0xffffffffu, shi, o));
-      }
-      nsw = shi - slo + 1;
-      // per-point geometry against column J
-      if constexpr (FP32) {
-        for (int q = lane; q < B.nq; q += 32) point_col(P + 4 * q, C.G, mypc[q], true, true, &CR);
-      } else {
-        for (int q = lane; q < B.nq; q += 32) point_col(P + 4 * q, C.G, mypc[q], false);
-      }
-      if constexpr (FP32) {
-        // the whole-edge integrals of the points' fully lit triangle, lane per (point, edge)
-        __syncwarp();
-        for (int e = lane; e < 3 * B.nq; e += 32) {
-          const int q = e / 3, k = e - 3 * q;
-          mypc[q].F.Efull[k] = edge_full_mixed(mypc[q], CR, k);
-        }
-        __syncwarp();
-        for (int q = lane; q < B.nq; q += 32) point_col_finish(mypc[q]);
-      }
-      __syncwarp();
-      }
-      __syncthreads();
-      if (!skip) {
-      // pass 1: classify every (point, face) pair from the cone-function values
-      // at the corners; fully lit and dark pairs are final, cut pairs are listed
-      const int nit = B.nq * nsw;
-      for (int base = 0; base < nit; base += 32) {
-        int it = base + lane;
-        bool cut = false;
-        if (it < nit) {
-          int q = it / nsw, s = it - q * nsw;
-          int cls;
-          if (FP32) {
-            float Fv[3], cc = 0.f;
-            cls = face_class_mixed(mypc[q], Ff[slo + s], Fv, cc, fdiam);
-          } else {
-            double Fv[3], cc = 0.0;
-            cls = face_class(C.G, mypc[q], Fs[slo + s], Fv, cc);
-          }
-          if (cls == FACE_CUT) cut = true;
-          else Wsc[q * B.max_surf + s] = cls == FACE_LIT ? (FP32 ? (R)mypc[q].Wst_f : (R)mypc[q].Wst) : R(0);
-        }
-        unsigned mk = __ballot_sync(0xffffffffu, cut);
-        if (cut) mycut[ncut + __popc(mk & ((1u << lane) - 1u))] = (uint16_t)it;
-        ncut += __popc(mk);
-      }
-      __syncwarp();
-      }
-      __syncthreads();
-      if (!skip) {
-      // pass 2: the cut pairs, converged across the warp
-      if constexpr (FP32) {
-        // mixed: the geometry and edge pieces lane per cut pair; the conic
-        // arcs they need (at most 3 per pair, the larger part of the work)
-        // are collected and integrated lane per arc over the compacted list,
-        // then each pair adds its arcs in order (the same sum as in face_cut)
-        for (int base = 0; base < ncut; base += 32) {
-          const int k = base + lane;
-          int na = 0, q = 0, s = 0;
-          float et = 0.f;
-          bool need64 = false;
-          if (k < ncut) {
-            const int it = mycut[k];
-            q = it / nsw;
-            s = it - q * nsw;
-            float Fv[3], cc = 0.f;
-            face_class_mixed(mypc[q], Ff[slo + s], Fv, cc, fdiam);
-            need64 = near_singular_mixed(cc, mypc[q].F.d, fdiam);
-            if (!need64) {
-              FaceCutIn<float> in;
-              cut_in_mixed(mypc[q], Ff[slo + s], Fv, cc, Fs[slo + s], in);
-              et = (float)face_cut<float>(CR, mypc[q], in, B.rule, myarc + 3 * lane, &na);
-            }
-          }
-          int incl = na;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-          }
-          const int off = incl - na, total = __shfl_sync(0xffffffffu, incl, 31);
-          for (int i = 0; i < na; ++i) myidx[off + i] = (uint8_t)(3 * lane + i);
-          __syncwarp();
-          for (int a = lane; a < total; a += 32) {
-            const int slot = myidx[a];
-            myval[slot] = arc_value<float>(myarc[slot], B.rule);
-          }
-          __syncwarp();
-          if (k < ncut) {
-            float v = et;
-            for (int i = 0; i < na; ++i) v += myval[3 * lane + i];
-            if (need64 || !isfinite(v))   // near-singular or degenerate FP32 geometry: this face in FP64
-              v = (float)face_W_fp64(P + 4 * q, C.G, Fs[slo + s], B.n_theta);
-            Wsc[q * B.max_surf + s] = v;
-          }
-          __syncwarp();
-        }
-      } else
-      for (int k = lane; k < ncut; k += 32) {
-        int it = mycut[k];
-        int q = it / nsw, s = it - q * nsw;
-        FaceCutIn<R> in;
-        if constexpr (FP32) {
-          float Fv[3], cc = 0.f;
-          face_class_mixed(mypc[q], Ff[slo + s], Fv, cc, fdiam);
-          cut_in_mixed(mypc[q], Ff[slo + s], Fv, cc, Fs[slo + s], in);
-        } else {
-          double Fv[3], cc = 0.0;
-          face_class(C.G, mypc[q], Fs[slo + s], Fv, cc);
-          cut_in_fp64(mypc[q], Fs[slo + s], Fv, cc, in);
-        }
-        Wsc[q * B.max_surf + s] = (R)face_cut<R>(CR, mypc[q], in, B.rule);
-      }
-      __syncwarp();
-      }
-      __syncthreads();
-      if (!skip) {
-      const uint32_t* fb = bits + f * words;
-      for (int j = jlo + lane; j < jhi; j += 32) {
-        if (!((fb[j >> 5] >> (j & 31)) & 1u)) continue;
-        int lo = T[j].lo - slo, hi = T[j].hi - slo;
-        R u = R(0);
-        for (int q = 0; q < B.nq; ++q) u += Wsc[q * B.max_surf + lo] - Wsc[q * B.max_surf + hi];
-        Urow[j] = u;
-      }
-      __syncwarp();
-    }
-    }
-    __syncthreads();
-    // entries of the block rows
-    const int t0 = B.col_tet_begin[I], nt = B.col_tet_begin[I + 1] - t0;
-    const R scale = (R)(GI.area / (4.0 * STBEM_PI * B.nq));
-    const int64_t voff = B.boff[b], roff = B.rsoff[b];
-    for (int r = threadIdx.x; r < nt; r += blockDim.x) {
-      const TetDev& D = B.tets[t0 + r];
-      int lo = D.lo - s0, hi = D.hi - s0;
-      int first = -1;
-      for (int w = 0; w < words && first < 0; ++w) {
-        uint32_t m = bits[lo * words + w] | bits[hi * words + w];
-        if (m) first = 32 * w + __ffs(m) - 1;
-      }
-      if (first < 0) first = 0;
-      const R* Ulo = U + (size_t)lo * B.max_tet;
-      const R* Uhi = U + (size_t)hi * B.max_tet;
-      if (B.mf_y) {
-        // fused product: the row's band times x, one atomic add per right-hand side
-        for (int k = 0; k < B.mf_nrhs; ++k) {
-          const double* xk = B.mf_x + (int64_t)k * B.mf_ld + C.tet0;
-          double sacc = 0.0;
-          for (int w = 0; w < W; ++w) {
-            const int j = first + w;
-            if (j < ntJ) sacc += (double)(scale * (Ulo[j] - Uhi[j])) * xk[j];
-          }
-          atomicAdd(B.mf_y + (int64_t)k * B.mf_ld + t0 + r, sacc);
-        }
-        continue;
-      }
-      B.rs[roff + r] = C.tet0 + first;
-      for (int w = 0; w < W; ++w) {
-        int j = first + w;
-        R v = R(0);
-        if (j < ntJ) v = scale * (Ulo[j] - Uhi[j]);
-        if (B.val) B.val[voff + (int64_t)w * nt + r] = (double)v;
-        if (B.val32) B.val32[voff + (int64_t)w * nt + r] = (float)v;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// STBEM_QUAD_MIN_CTAS (stbem_internal.h): CTAs of 128 threads resident per
-// SM that the default register budget is cut for (quadrature of the level-3,
-// 32-slab sphere in mixed precision with an earlier build: 4 / 5 / 6 CTAs
-// took 6.83 / 6.91 / 7.56 s)
-// warps per quadrature CTA
-#ifndef STBEM_QUAD_WARPS
-#define STBEM_QUAD_WARPS 4
-#endif
-constexpr int kQuadThreads = 32 * STBEM_QUAD_WARPS;
-
-// MINB: CTAs per SM the register budget is cut for (STBEM_QUAD_MIN_CTAS: 128
-// registers; 2: up to 255, no spills, for meshes whose shared memory per CTA
-// lets no more than 2 CTAs share an SM anyway)
-template <bool FP32, int MINB>
-__global__ void __launch_bounds__(kQuadThreads, MINB) k_quad_blocks(BlockCtx B) {
-  typedef typename std::conditional<FP32, float, double>::type R;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ ColSm C;
-  __shared__ ColR<R> CR;
-  const int64_t nblk = B.end;
-  for (;;) {
-    int64_t b = pop_block(B.counter);
-    if (b >= nblk) break;
-    quad_block<FP32>(B, b, smem, C, CR);
-  }
-}
-
-template <bool FP32>
-__global__ void __launch_bounds__(kQuadThreads, STBEM_QUAD_MIN_CTAS) k_quad_batch(const BlockCtx* __restrict__ Bs,
-                                                       const int64_t* __restrict__ prefix, int S,
-                                                       unsigned long long* counter, int64_t end) {
-  typedef typename std::conditional<FP32, float, double>::type R;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ ColSm C;
-  __shared__ ColR<R> CR;
-  __shared__ BlockCtx sB;
-  __shared__ int s_seg;
-  int cur = -1;
-  const int64_t total = min(prefix[S], end);
-  for (;;) {
-    int64_t g = pop_block(counter);
-    if (g >= total) break;
-    if (threadIdx.x == 0) s_seg = find_seg(prefix, S, g);
-    __syncthreads();
-    const int seg = s_seg;
-    if (seg != cur) {
-      if (threadIdx.x == 0) sB = Bs[seg];
-      cur = seg;
-    }
-    __syncthreads();
-    quad_block<FP32>(sB, g - prefix[seg], smem, C, CR);
-  }
-}
-
-static size_t block_smem(const bem_operator* op) {
-  const bem_mesh* m = op->mesh;
-  int words = (m->max_col_tets + 31) / 32;
-  size_t s = sizeof(TetSm) * m->max_col_tets + sizeof(FaceGeom) * m->max_col_surf;
-  s += sizeof(uint32_t) * ((m->max_col_surf * words + 3) & ~3);
-  s += sizeof(PointCol) * STBEM_QUAD_WARPS * op->nq;
-  s += (op->opts.precision == BEM_PREC_MIXED ? sizeof(float) : sizeof(double)) * STBEM_QUAD_WARPS * op->nq *
-       m->max_col_surf;
-  s += sizeof(uint16_t) * (((size_t)STBEM_QUAD_WARPS * op->nq * m->max_col_surf + 7) / 8 * 8);
-  s += sizeof(FaceF) * m->max_col_surf;
-  if (op->opts.precision == BEM_PREC_MIXED) s += 16 + STBEM_QUAD_WARPS * ARC_WARP_BYTES;
-  return s;
-}
-
 // The dynamic shared-memory limit of a kernel is state of the device shared by
 // every host thread: operators of different sizes launching the same kernel
 // concurrently (server slots) must never lower it under another's launch, so
@@ -809,7 +364,7 @@ static int persistent_grid(const void* kern, size_t smem, int threads) {
   return sms * per;
 }
 
-static BlockCtx make_ctx(bem_operator* op) {
+static BlockCtx make_ctx(const bem_operator* op) {
   const bem_mesh* m = op->mesh;
   BlockCtx B;
   B.n_col = m->n_col;
@@ -818,14 +373,16 @@ static BlockCtx make_ctx(bem_operator* op) {
   B.S = m->coord_scale;
   B.margin = (float)(1.6e-5 * m->coord_scale);  // > 4x the FP32 error bound of C2 and C3
   B.cols = m->d_col; B.colf = static_cast<const ColF*>(m->d_colf); B.panf = static_cast<const PanelF*>(m->d_panf);
+  B.facef = static_cast<const FaceF*>(m->d_facef);
   B.col_tet_begin = m->d_col_tet_begin; B.col_surf_begin = m->d_col_surf_begin;
-  B.surf = m->d_surf; B.tets = m->d_tet; B.pts = op->d_pts; B.ptsf = reinterpret_cast<const float4*>(op->d_ptsf); B.trange = op->d_pts_trange;
+  B.surf = m->d_surf; B.tets = m->d_tet; B.pts = op->d_pts; B.ptsf = reinterpret_cast<const float4*>(op->d_ptsf);
+  B.ptsl = reinterpret_cast<const float4*>(op->d_ptsl); B.trange = op->d_pts_trange;
   B.bw = op->d_bw; B.bnnz = op->d_bnnz; B.boff = op->d_boff; B.rsoff = op->d_rsoff; B.rs = op->d_rs;
-  B.val = op->d_val; B.val32 = op->d_val32; B.uscratch = op->d_tmp;
+  B.val = op->d_val; B.val32 = op->d_val32;
   B.max_surf = m->max_col_surf; B.max_tet = m->max_col_tets;
   B.counter = nullptr;
-  B.end = m->n_col * m->n_col;
   B.inner = nullptr;
+  B.gran = op->d_gran;
   B.mf_x = nullptr; B.mf_y = nullptr; B.mf_nrhs = 0; B.mf_ld = m->n_tet;
   return B;
 }
@@ -853,73 +410,54 @@ bem_status op_pattern(bem_operator* op, cudaStream_t s) {
   if (st != BEM_OK) return st;
   STBEM_CUDA(cudaMemsetAsync(op->d_counter + 1, 0, sizeof(unsigned long long), s));
   B.inner = op->d_counter + 1;
+  STBEM_CUDA(cudaMemsetAsync(op->d_gran, 0, sizeof(uint2) * op->n_gran(), s));
   const int64_t nc = op->mesh->n_col;
   const int run = pattern_run(nc * nc);
   return launch_pattern(B, nullptr, nullptr, 1, run, nc * ((nc + run - 1) / run), B.counter, s);
 }
 
-// quadrature kernel of a precision and register budget (variant 0: the
-// STBEM_QUAD_MIN_CTAS budget; variant 1: the 2-CTA budget, mixed precision only)
-static const void* quad_kernel(const bem_operator* op, int variant) {
-  if (op->opts.precision != BEM_PREC_MIXED) return (const void*)k_quad_blocks<false, STBEM_QUAD_MIN_CTAS>;
-  return variant ? (const void*)k_quad_blocks<true, 2> : (const void*)k_quad_blocks<true, STBEM_QUAD_MIN_CTAS>;
+int quad_max_per_sm(const bem_operator* op) {
+  return stage_apex_per_sm(op->opts.precision == BEM_PREC_MIXED, op->mesh->max_col_tets, op->mesh->max_col_surf, op->nq);
 }
 
-int quad_variants(const bem_operator* op) { return op->opts.precision == BEM_PREC_MIXED ? 2 : 1; }
-
-int quad_max_per_sm(const bem_operator* op, int variant) {
-  const size_t smem = block_smem(op);
-  const void* kern = quad_kernel(op, variant);
-  ensure_smem_attr(kern, smem);
-  return std::max(1, persistent_grid(kern, smem, kQuadThreads) / std::max(1, (int)op->ctx->sm_count));
+void quad_scratch(const bem_operator* op, int64_t* least, int64_t* wanted) {
+  int64_t a = 0, b = 0;
+  const bool fp32 = op->opts.precision == BEM_PREC_MIXED;
+  stage_scratch(fp32, op->mesh->max_col_tets, op->mesh->max_col_surf, (int)op->ctx->sm_count, {&op->h_gran},
+                op->nstored * (fp32 ? 4 : 8), &a, &b);
+  *least = (a + 7) / 8;
+  *wanted = (b + 7) / 8;
 }
 
 bem_status quad_launch(const bem_operator* op, int per_sm, int64_t end, const double* mf_x, double* mf_y, int nrhs,
-                       cudaStream_t s, int variant) {
-  BlockCtx B = make_ctx(const_cast<bem_operator*>(op));
-  bem_status st = get_counter(op, &B.counter, s);
-  if (st != BEM_OK) return st;
-  B.end = std::min<int64_t>(end, B.end);
+                       cudaStream_t s) {
+  BlockCtx B = make_ctx(op);
+  const int64_t nb = op->mesh->n_col * op->mesh->n_col;
   B.mf_x = mf_x;
   B.mf_y = mf_y;
   B.mf_nrhs = nrhs;
-  B.mf_ld = op->mesh->n_tet;
-  if (variant >= quad_variants(op)) variant = 0;
-  const size_t smem = block_smem(op);
-  const int max_per = quad_max_per_sm(op, variant);
-  const int grid = (int)op->ctx->sm_count * std::max(1, std::min(per_sm, max_per));
-  if ((int64_t)grid * op->mesh->max_col_surf * op->mesh->max_col_tets > op->tmp_len) {
-    set_error("quadrature scratch too small");
-    return BEM_ERR_INTERNAL;
-  }
-  if (op->opts.precision != BEM_PREC_MIXED) k_quad_blocks<false, STBEM_QUAD_MIN_CTAS><<<grid, kQuadThreads, smem, s>>>(B);
-  else if (variant) k_quad_blocks<true, 2><<<grid, kQuadThreads, smem, s>>>(B);
-  else k_quad_blocks<true, STBEM_QUAD_MIN_CTAS><<<grid, kQuadThreads, smem, s>>>(B);
-  STBEM_CUDA(cudaGetLastError());
-  return BEM_OK;
+  return stage_run(B, nullptr, nullptr, 1, op->opts.precision == BEM_PREC_MIXED, (int)op->ctx->sm_count,
+                   {&op->h_gran}, {nb}, std::min(end, nb), op->d_tmp, op->tmp_len * 8, per_sm, s);
 }
 
 bem_status op_quadrature(bem_operator* op, cudaStream_t s) {
   bem_status st = choose_quad_shape(op, s);
   if (st != BEM_OK) return st;
-  return quad_launch(op, op->quad_per_sm, op->mesh->n_col * op->mesh->n_col, nullptr, nullptr, 0, s,
-                     op->quad_variant);
+  return quad_launch(op, op->quad_per_sm, op->mesh->n_col * op->mesh->n_col, nullptr, nullptr, 0, s);
 }
 
 // Matrix-free product y = A x (internal order, [nrhs][n_tet]): the quadrature
 // pass with the entries summed against x instead of stored.
 bem_status op_matvec_free(const bem_operator* op, const double* x, double* y, int nrhs, cudaStream_t s) {
   STBEM_CUDA(cudaMemsetAsync(y, 0, sizeof(double) * op->mesh->n_tet * nrhs, s));
-  int per_sm = op->quad_per_sm, variant = op->quad_variant;
-  if (per_sm <= 0) default_quad_shape(op, &per_sm, &variant);
-  return quad_launch(op, per_sm, op->mesh->n_col * op->mesh->n_col, x, y, nrhs, s, variant);
+  const int per_sm = op->quad_per_sm > 0 ? op->quad_per_sm : quad_max_per_sm(op);
+  return quad_launch(op, per_sm, op->mesh->n_col * op->mesh->n_col, x, y, nrhs, s);
 }
 
 // ---------------------------------------------------------------------------
-// Batched passes: one persistent launch over the blocks of several operators.
-// All contexts take the largest column sizes of the batch, so the shared
-// memory layout is the same for every block, and the quadrature scratch
-// (one slab per CTA) is shared.
+// Batched passes over the blocks of several operators. All contexts take the
+// largest column sizes of the batch, so the shared memory layout is the same
+// for every block, and the quadrature scratch is shared.
 // ---------------------------------------------------------------------------
 bem_status op_outer_points_all(const std::vector<bem_operator*>& ops, cudaStream_t s) {
   for (bem_operator* op : ops) {
@@ -938,18 +476,6 @@ static void batch_dims(const std::vector<bem_operator*>& ops, int& max_tet, int&
   }
 }
 
-static size_t batch_smem(int max_tet, int max_surf, int nq, bool fp32) {
-  int words = (max_tet + 31) / 32;
-  size_t s = sizeof(TetSm) * max_tet + sizeof(FaceGeom) * max_surf;
-  s += sizeof(uint32_t) * ((max_surf * words + 3) & ~3);
-  s += sizeof(PointCol) * STBEM_QUAD_WARPS * nq;
-  s += (fp32 ? sizeof(float) : sizeof(double)) * STBEM_QUAD_WARPS * nq * max_surf;
-  s += sizeof(uint16_t) * (((size_t)STBEM_QUAD_WARPS * nq * max_surf + 7) / 8 * 8);
-  s += sizeof(FaceF) * max_surf;
-  if (fp32) s += 16 + STBEM_QUAD_WARPS * ARC_WARP_BYTES;
-  return s;
-}
-
 // run > 0: the prefix counts the pattern pass's work items, else blocks
 static bem_status upload_batch(const std::vector<bem_operator*>& ops, BatchDev& dev, int max_tet, int max_surf,
                                int run, int64_t* total, BlockCtx* first, cudaStream_t s) {
@@ -960,13 +486,12 @@ static bem_status upload_batch(const std::vector<bem_operator*>& ops, BatchDev& 
     ctx[i] = make_ctx(ops[i]);
     ctx[i].max_tet = max_tet;
     ctx[i].max_surf = max_surf;
-    ctx[i].uscratch = dev.d_uscratch;
     ctx[i].counter = dev.d_counter;
     const int64_t nc = ops[i]->mesh->n_col;
     prefix[i + 1] = prefix[i] + nc * (run > 0 ? (nc + run - 1) / run : nc);
   }
   *total = prefix[S];
-  if (first) *first = ctx[0];
+  *first = ctx[0];
   STBEM_CUDA(cudaMemcpyAsync(dev.d_ctx, ctx.data(), sizeof(BlockCtx) * S, cudaMemcpyHostToDevice, s));
   STBEM_CUDA(cudaMemcpyAsync(dev.d_prefix, prefix.data(), sizeof(int64_t) * (S + 1), cudaMemcpyHostToDevice, s));
   STBEM_CUDA(cudaMemsetAsync(dev.d_counter, 0, sizeof(unsigned long long), s));
@@ -982,30 +507,33 @@ bem_status op_pattern_batch(const std::vector<bem_operator*>& ops, BatchDev& dev
   for (const bem_operator* op : ops) blocks += op->mesh->n_col * op->mesh->n_col;
   const int run = pattern_run(blocks);
   BlockCtx first;
+  for (bem_operator* op : ops) STBEM_CUDA(cudaMemsetAsync(op->d_gran, 0, sizeof(uint2) * op->n_gran(), s));
   bem_status st = upload_batch(ops, dev, mt, ms, run, &items, &first, s);
   if (st != BEM_OK) return st;
   return launch_pattern(first, static_cast<const BlockCtx*>(dev.d_ctx), dev.d_prefix, (int)ops.size(), run, items,
                         dev.d_counter, s);
 }
 
-static int quad_batch_grid(const std::vector<bem_operator*>& ops, size_t& smem) {
-  int mt, ms;
-  batch_dims(ops, mt, ms);
-  smem = batch_smem(mt, ms, ops[0]->nq, ops[0]->opts.precision == BEM_PREC_MIXED);
-  if (ops[0]->opts.precision == BEM_PREC_MIXED) {
-    ensure_smem_attr((const void*)k_quad_batch<true>, smem);
-    return persistent_grid((const void*)k_quad_batch<true>, smem, kQuadThreads);
+static void batch_grans(const std::vector<bem_operator*>& ops, std::vector<const std::vector<uint2>*>& gran,
+                        std::vector<int64_t>& blocks) {
+  for (const bem_operator* op : ops) {
+    gran.push_back(&op->h_gran);
+    blocks.push_back(op->mesh->n_col * op->mesh->n_col);
   }
-  ensure_smem_attr((const void*)k_quad_batch<false>, smem);
-  return persistent_grid((const void*)k_quad_batch<false>, smem, kQuadThreads);
 }
 
 int64_t quad_batch_scratch(const std::vector<bem_operator*>& ops) {
   if (ops.empty()) return 0;
   int mt, ms;
   batch_dims(ops, mt, ms);
-  size_t smem = 0;
-  return (int64_t)quad_batch_grid(ops, smem) * mt * ms;
+  std::vector<const std::vector<uint2>*> gran;
+  std::vector<int64_t> blocks;
+  batch_grans(ops, gran, blocks);
+  const bool fp32 = ops[0]->opts.precision == BEM_PREC_MIXED;
+  int64_t values = 0, least = 0, wanted = 0;
+  for (const bem_operator* op : ops) values += op->nstored * (fp32 ? 4 : 8);
+  stage_scratch(fp32, mt, ms, (int)ops[0]->ctx->sm_count, gran, values, &least, &wanted);
+  return (wanted + 7) / 8;
 }
 
 bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& dev, cudaStream_t s) {
@@ -1022,22 +550,18 @@ bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& 
   int mt, ms;
   batch_dims(ops, mt, ms);
   int64_t total = 0;
-  bem_status st = upload_batch(ops, dev, mt, ms, 0, &total, nullptr, s);
+  BlockCtx first;
+  bem_status st = upload_batch(ops, dev, mt, ms, 0, &total, &first, s);
   if (st != BEM_OK) return st;
-  size_t smem = 0;
-  const int max_grid = quad_batch_grid(ops, smem);
+  const bool fp32 = ops[0]->opts.precision == BEM_PREC_MIXED;
   const int sms = (int)ops[0]->ctx->sm_count;
-  const int occ = std::max(1, max_grid / std::max(1, sms));
-  const BlockCtx* d = static_cast<const BlockCtx*>(dev.d_ctx);
-  auto launch = [&](int per, int64_t end) -> bem_status {
-    STBEM_CUDA(cudaMemsetAsync(dev.d_counter, 0, sizeof(unsigned long long), s));
-    const int grid = sms * std::max(1, std::min(per, occ));
-    if (ops[0]->opts.precision == BEM_PREC_MIXED)
-      k_quad_batch<true><<<grid, kQuadThreads, smem, s>>>(d, dev.d_prefix, (int)ops.size(), dev.d_counter, end);
-    else
-      k_quad_batch<false><<<grid, kQuadThreads, smem, s>>>(d, dev.d_prefix, (int)ops.size(), dev.d_counter, end);
-    STBEM_CUDA(cudaGetLastError());
-    return BEM_OK;
+  const int occ = stage_apex_per_sm(fp32, mt, ms, ops[0]->nq);
+  std::vector<const std::vector<uint2>*> gran;
+  std::vector<int64_t> blocks;
+  batch_grans(ops, gran, blocks);
+  auto launch = [&](int per, int64_t end) {
+    return stage_run(first, static_cast<const BlockCtx*>(dev.d_ctx), dev.d_prefix, (int)ops.size(), fp32, sms, gran,
+                     blocks, end, dev.d_uscratch, dev.uscratch_len * 8, per, s);
   };
   int per = occ, how = 0;
   if (ops[0]->ctx->tune_mode) {
@@ -1173,7 +697,7 @@ __global__ void __launch_bounds__(kPatternThreads) k_pattern_rows(BlockCtx B, in
 
 bem_status op_pattern_csr(const bem_operator* op, int64_t* d_rowcount, int64_t* d_rowptr, int32_t* d_cols, bool fill,
                           cudaStream_t s, int64_t I_only) {
-  BlockCtx B = make_ctx(const_cast<bem_operator*>(op));
+  BlockCtx B = make_ctx(op);
   bem_status st = get_counter(op, &B.counter, s);
   if (st != BEM_OK) return st;
   const size_t smem = bits_smem(B.max_tet, B.max_surf, B.nq);

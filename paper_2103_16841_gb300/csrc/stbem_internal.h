@@ -28,10 +28,7 @@ void set_error(const std::string& msg);
 constexpr int MAX_COL_TETS = 192;   // panels sharing one spatial triangle
 constexpr int MAX_COL_SURF = 193;   // nu_t != 0 faces over one spatial triangle
 constexpr int MAX_NQ = 64;          // m_Q^2 outer points per face
-#ifndef STBEM_QUAD_MIN_CTAS
-#define STBEM_QUAD_MIN_CTAS 4           // CTAs per SM the quadrature's default register budget is cut for
-#endif
-constexpr int STBEM_QUAD_BUDGET_CTAS = STBEM_QUAD_MIN_CTAS;
+constexpr int STBEM_QUAD_BUDGET_CTAS = 4;   // CTAs per SM the quadrature's register budget is cut for
 
 // Per panel data on the device (internal panel order: by column, then time).
 struct TetDev {
@@ -75,7 +72,8 @@ struct bem_mesh {
   stbem::SurfDev* d_surf = nullptr;
   stbem::TetDev* d_tet = nullptr;
   int32_t* d_perm = nullptr;    // internal -> caller
-  void* d_colf = nullptr;       // FP32 images of the columns and panels (ColF, PanelF)
+  void* d_colf = nullptr;       // FP32 images of the columns, faces and panels (ColF, FaceF, PanelF)
+  void* d_facef = nullptr;
   void* d_panf = nullptr;
 };
 
@@ -86,12 +84,16 @@ struct bem_operator {
   int mq = 3, nq = 9, n_theta = 12;
   double* d_pts = nullptr;       // [n_surf][nq][4] outer points
   float* d_ptsf = nullptr;       // the same rounded to FP32 (the sparsity filter's inputs)
+  float* d_ptsl = nullptr;       // and the remainders (FP32 pairs)
   double* d_pts_trange = nullptr;// [n_surf][2] min / max time of the outer points
   int32_t* d_bw = nullptr;       // [n_col*n_col] band width per column block
   int64_t* d_bnnz = nullptr;     // [n_col*n_col] pattern entries per block
   int64_t* d_boff = nullptr;     // [n_col*n_col] value offset
   int64_t* d_rsoff = nullptr;    // [n_col*n_col] row-start offset
   int32_t* d_rs = nullptr;       // row starts (internal trial index)
+  uint2* d_gran = nullptr;       // (apexes, potentials) of the quadrature per run of 8 blocks (dense order)
+  std::vector<uint2> h_gran;     // the same on the host: they set the quadrature's chunks
+  int64_t n_gran() const { return (mesh->n_col * mesh->n_col + 7) / 8; }
   double* d_val = nullptr;       // values, per block column-major [W][R_I]
   float* d_val32 = nullptr;
   int64_t nnz = 0, nstored = 0, nblocks = 0, nrows_stored = 0;
@@ -100,13 +102,14 @@ struct bem_operator {
   double assemble_ms = 0.0;
   double phase_ms[4] = {0, 0, 0, 0};
   int quad_per_sm = 0;           // CTAs per SM of the persistent quadrature (0: not chosen yet)
-  int quad_variant = 0;          // its register budget (0: 4 CTAs per SM, 1: 2 CTAs per SM)
   int quad_tuned = 0;            // 0 default shape, 1 timed here, 2 from the tuning cache
-  double tune_ms[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // sample time per candidate: index = 4 variant + CTAs per SM - 1
+  double tune_ms[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // sample time per candidate: index = CTAs per SM - 1
   unsigned long long* d_counter = nullptr;  // work counter of the persistent kernels
   // quadrature scratch
   double* d_tmp = nullptr;
   int64_t tmp_len = 0;
+  int64_t reserve_len = 0;       // doubles an admission reserves for the scratch
+  int64_t scratch_cap = -1;      // >= 0: bytes the scratch may take beyond that, allocated stream-ordered
   // made on first use by the products (an operator is used by one host thread at a time)
   mutable float* d_ws = nullptr;        // packed operands of the FP32 / tensor-core products
   mutable int64_t ws_len = 0;
@@ -134,18 +137,16 @@ bem_status mesh_device_geometry(bem_mesh* m, const double* d_sv_xyz, const int32
 bem_status op_outer_points(bem_operator* op, cudaStream_t s);
 bem_status op_pattern(bem_operator* op, cudaStream_t s);
 bem_status op_quadrature(bem_operator* op, cudaStream_t s);
-// register-budget variants of the quadrature kernel (1 for FP64 operators;
-// 2 for mixed ones: the 4-CTA budget, and the 2-CTA budget of 255 registers)
-int quad_variants(const bem_operator* op);
-// most CTAs of a variant of the quadrature kernel resident per SM (shared memory and registers)
-int quad_max_per_sm(const bem_operator* op, int variant);
-// one persistent quadrature launch of a variant with per_sm CTAs per SM over
-// the blocks [0, end) of the dense (I, J) order (assembled, or summed against mf_x)
+// Gauss tables of the quadrature's own translation unit
+bem_status upload_gauss_stage(const double* x, const double* w, const float* xf, const float* wf, size_t n);
+// most CTAs per SM of the quadrature's persistent stage (at most 4)
+int quad_max_per_sm(const bem_operator* op);
+// least and wanted length of an operator's quadrature scratch, in doubles
+void quad_scratch(const bem_operator* op, int64_t* least, int64_t* wanted);
+// the quadrature over the blocks [0, end) of the dense (I, J) order, its
+// persistent stage with per_sm CTAs per SM (assembled, or summed against mf_x)
 bem_status quad_launch(const bem_operator* op, int per_sm, int64_t end, const double* mf_x, double* mf_y, int nrhs,
-                       cudaStream_t s, int variant);
-// the untuned shape: the 2-CTA budget where shared memory admits no more than
-// 2 CTAs per SM anyway, else the 4-CTA budget; its occupancy
-void default_quad_shape(const bem_operator* op, int* per_sm, int* variant);
+                       cudaStream_t s);
 // sets op->quad_per_sm: the context's tuning cache, a timed choice, or the default (stbem_tune.cu)
 bem_status choose_quad_shape(bem_operator* op, cudaStream_t s);
 // the tuner behind it: the fastest of the candidate launch codes of launch(code, end)
@@ -202,7 +203,10 @@ bem_status gmres_solve_layout(const SegLayout& L, const MatvecFn& mv_hi, const M
                               double* d_x, const bem_solve_opts* o, bem_solve_info* info, cudaStream_t s);
 // operator creation with an admission hook (see bem_operator::admit)
 bem_status operator_create(bem_context* ctx, const bem_mesh* mesh, const bem_op_opts* opts,
-                           std::function<bem_status(const bem_operator*)> admit, bem_operator** out);
+                           std::function<bem_status(const bem_operator*)> admit, bem_operator** out,
+                           int64_t scratch_cap = -1);
+// gives the quadrature scratch of an operator created with a scratch_cap back (stream-ordered)
+void operator_release_scratch(bem_operator* op, cudaStream_t s);
 // operator object with its structure arrays allocated (nothing assembled yet)
 bem_status op_structure_alloc(bem_context* ctx, const bem_mesh* mesh, const bem_op_opts* opts,
                               std::unique_ptr<bem_operator>& op);
@@ -211,8 +215,8 @@ bem_status op_structure_alloc(bem_context* ctx, const bem_mesh* mesh, const bem_
 // (and the quadrature scratch when own_scratch)
 bem_status op_layout(bem_operator* op, const int32_t* bw, const int64_t* bnnz, bool first, bool own_scratch,
                      cudaStream_t s);
-// batched pattern and quadrature passes over several operators (one
-// persistent launch each); the operators share `uscratch` for the quadrature
+// batched pattern and quadrature passes over several operators; the operators
+// share `uscratch` for the quadrature
 struct BatchDev {
   void* d_ctx = nullptr;                 // BlockCtx[S]
   int64_t* d_prefix = nullptr;           // [S+1] block prefix

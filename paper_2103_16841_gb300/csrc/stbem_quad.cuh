@@ -130,24 +130,28 @@ struct PtR {             // apex-against-column quantities in precision R (colum
   R C, far_rho;
 };
 
+// the apex against the cone, mixed path: times and distances as FP32 pairs
+struct ConeM {
+  float rho_hi[3], rho_lo[3];   // r_k - t
+  float nt_hi, nt_lo;           // -t
+  float rlot_hi, rlot_lo;       // rlo - t, rlo a lower bound of dist(x_s, K)
+};
+
 struct PointCol {        // apex x against one column
   double t;
   double r[3];           // |x_s - corner_k| (FP64: the cone-function values need it)
   double rlo;            // lower bound of dist(x_s, K)
   double Wst;            // 4 pi * potential of the whole triangle
-  float Wst_f;
   int inK;
   PtR<double> D;
   PtR<float> F;          // filled for the mixed-precision path
-  float rho_hi[3], rho_lo[3];   // r_k - t as an FP32 pair (mixed path)
-  float nt_hi, nt_lo;           // -t as an FP32 pair
-  float rlot_hi, rlot_lo;       // rlo - t as an FP32 pair
+  ConeM M;
 };
 
 // per face, FP32 view for the mixed path: corner times as FP32 pairs
 struct FaceF {
   float p_hi[3], p_lo[3];
-  float g[2];
+  float g[2], g_lo[2];
   float pmin_hi, pmin_lo;
 };
 
@@ -171,7 +175,7 @@ STBEM_HD inline void make_facef(const FaceGeom& F, FaceF& o) {
     if (F.p[k] < F.p[km]) km = k;
   }
   o.pmin_hi = o.p_hi[km]; o.pmin_lo = o.p_lo[km];
-  o.g[0] = (float)F.g[0]; o.g[1] = (float)F.g[1];
+  for (int i = 0; i < 2; ++i) split2(F.g[i], o.g[i], o.g_lo[i]);
 }
 
 template <typename R>
@@ -181,13 +185,6 @@ struct ColR {            // edge data of a column in precision R
 
 STBEM_HD inline void sc(float x, float* s, float* c) { sincosf(x, s, c); }
 STBEM_HD inline void sc(double x, double* s, double* c) { sincos(x, s, c); }
-
-template <typename R>
-STBEM_HD inline const PtR<R>& pt(const PointCol& P);
-template <>
-STBEM_HD inline const PtR<double>& pt<double>(const PointCol& P) { return P.D; }
-template <>
-STBEM_HD inline const PtR<float>& pt<float>(const PointCol& P) { return P.F; }
 
 struct ArcRule {
   int nmin, nmax;    // Gauss node bounds per piece
@@ -429,8 +426,7 @@ STBEM_HD inline void make_colr(const ColGeom& G, ColR<R>& C) {
 
 // whole-edge integral k of the mixed path (the fully lit triangle is the sum
 // over the three edges): the far-field form when P.far, else edge_int
-STBEM_HD inline float edge_full_mixed(const PointCol& P, const ColR<float>& CR, int k) {
-  const PtR<float>& T = P.F;
+STBEM_HD inline float edge_full_mixed(const PtR<float>& T, const ColR<float>& CR, int k) {
   const ArcRule er = make_rule(1, 0);
   if (T.far) return edge_far<float>(T, CR, k, 0.f, 1.f, er);
   return edge_int<float>(T.ws[k], CR.L[k], T.ps[k], T.d, er);
@@ -440,12 +436,7 @@ STBEM_HD inline float edge_full_mixed(const PointCol& P, const ColR<float>& CR, 
 // fully lit case). FP64 path: everything in FP64. Mixed path: the relative
 // position, the height d, the foot point and the corner distances in FP64
 // (they carry the cancellation between |x - y| and t - tau), the rest in FP32.
-// With defer_edges (mixed path only)
-// the whole-edge integrals Efull and the whole-triangle value Wst are left to
-// the caller (edge_full_mixed per edge, then point_col_finish), so that a warp
-// can spread the three edges of its points over its lanes.
-STBEM_HD inline void point_col(const double* x, const ColGeom& G, PointCol& P, bool prec_fp32,
-                               bool defer_edges = false, const ColR<float>* CRf = nullptr) {
+STBEM_HD inline void point_col(const double* x, const ColGeom& G, PointCol& P, bool prec_fp32) {
   P.t = x[0];
   double rel[3] = {x[1] - G.c0[0], x[2] - G.c0[1], x[3] - G.c0[2]};
   double d = rel[0] * G.n[0] + rel[1] * G.n[1] + rel[2] * G.n[2];
@@ -463,40 +454,36 @@ STBEM_HD inline void point_col(const double* x, const ColGeom& G, PointCol& P, b
     T.xb[1] = (float)xb1;
     int in = 1;
     float out = 0.f, W = 0.f;
-    // (the column's FP32 frame from CRf when given: no conversions per point)
     for (int k = 0; k < 3; ++k) {
-      T.q[k][0] = (CRf ? CRf->Q[k][0] : (float)G.Q[k][0]) - T.xb[0];
-      T.q[k][1] = (CRf ? CRf->Q[k][1] : (float)G.Q[k][1]) - T.xb[1];
+      T.q[k][0] = (float)G.Q[k][0] - T.xb[0];
+      T.q[k][1] = (float)G.Q[k][1] - T.xb[1];
       T.rs[k] = (float)P.r[k];
     }
     for (int k = 0; k < 3; ++k) {
-      float ux = CRf ? CRf->U[k][0] : (float)G.U[k][0], uy = CRf ? CRf->U[k][1] : (float)G.U[k][1];
+      float ux = (float)G.U[k][0], uy = (float)G.U[k][1];
       T.ps[k] = T.q[k][0] * uy - T.q[k][1] * ux;
       T.ws[k] = T.q[k][0] * ux + T.q[k][1] * uy;
       if (!(T.ps[k] > 0.f)) in = 0;
       out = fmaxf(out, -T.ps[k]);
-      split2(P.r[k] - P.t, P.rho_hi[k], P.rho_lo[k]);
+      split2(P.r[k] - P.t, P.M.rho_hi[k], P.M.rho_lo[k]);
     }
-    T.far = out >= FAR_RHO * (CRf ? CRf->diam : (float)G.diam);
+    T.far = out >= FAR_RHO * (float)G.diam;
     T.C = T.rs[0];
     T.far_rho = out;
-    if (!defer_edges) {
-      ColR<float> CR;
-      make_colr<float>(G, CR);
-      for (int k = 0; k < 3; ++k) {
-        T.Efull[k] = edge_full_mixed(P, CR, k);
-        W += T.Efull[k];
-      }
+    ColR<float> CR;
+    make_colr<float>(G, CR);
+    for (int k = 0; k < 3; ++k) {
+      T.Efull[k] = edge_full_mixed(T, CR, k);
+      W += T.Efull[k];
     }
     P.inK = in;
     P.rlo = sqrt(d * d + (double)out * (double)out);
     P.Wst = (double)W;
-    P.Wst_f = W;
     P.D.d = d;
     P.D.xb[0] = xb0;
     P.D.xb[1] = xb1;
-    split2(-P.t, P.nt_hi, P.nt_lo);
-    split2(P.rlo - P.t, P.rlot_hi, P.rlot_lo);
+    split2(-P.t, P.M.nt_hi, P.M.nt_lo);
+    split2(P.rlo - P.t, P.M.rlot_hi, P.M.rlot_lo);
     return;
   }
   PtR<double>& D = P.D;
@@ -524,14 +511,6 @@ STBEM_HD inline void point_col(const double* x, const ColGeom& G, PointCol& P, b
   P.inK = in;
   P.rlo = sqrt(d * d + out * out);
   P.Wst = W;
-  P.Wst_f = (float)W;
-}
-
-// the whole-triangle value of the mixed path from its three edge integrals
-STBEM_HD inline void point_col_finish(PointCol& P) {
-  const float W = (P.F.Efull[0] + P.F.Efull[1]) + P.F.Efull[2];
-  P.Wst = (double)W;
-  P.Wst_f = W;
 }
 
 // ---------------------------------------------------------------------------
@@ -918,33 +897,37 @@ STBEM_HD inline int face_class(const ColGeom& G, const PointCol& P, const FaceGe
 // Step 1 for the mixed path in FP32 pairs: F_k = p_k + (r_k - t) and
 // c = -((p_0 - t) + <g, xb>) keep their absolute accuracy although p_k, r_k
 // and t are O(T) and F_k, c are O(diam K) near the cone.
-STBEM_HD inline int face_class_mixed(const PointCol& P, const FaceF& Fc, float* F, float& c, float diam) {
+STBEM_HD inline float face_c_mixed(const PtR<float>& T, const ConeM& M, const FaceF& Fc, float diam) {
+  const float p0t = add2(Fc.p_hi[0], Fc.p_lo[0], M.nt_hi, M.nt_lo);
+  const float c = -(p0t + (Fc.g[0] * T.xb[0] + Fc.g[1] * T.xb[1]));
+  return fabsf(c) < 1e-6f * diam ? 0.f : c;
+}
+
+// (c is left to face_c_mixed: only cut faces need it)
+STBEM_HD inline int face_class_mixed(const PtR<float>& T, const ConeM& M, const FaceF& Fc, float* F) {
   int nlit = 0;
   for (int k = 0; k < 3; ++k) {
-    F[k] = add2(Fc.p_hi[k], Fc.p_lo[k], P.rho_hi[k], P.rho_lo[k]);
+    F[k] = add2(Fc.p_hi[k], Fc.p_lo[k], M.rho_hi[k], M.rho_lo[k]);
     if (F[k] < 0.f) ++nlit;
   }
   if (nlit == 3) return FACE_LIT;
-  if (add2(Fc.pmin_hi, Fc.pmin_lo, P.rlot_hi, P.rlot_lo) >= 0.f) return FACE_DARK;
+  if (add2(Fc.pmin_hi, Fc.pmin_lo, M.rlot_hi, M.rlot_lo) >= 0.f) return FACE_DARK;
   {
     // F = P + |x_s - y| - t is convex on K: its tangent plane at the corner m
     // of smallest F, F_m + (P(y) - P(Q_m)) + <Q_m - xb, y - Q_m> / r_m, bounds
     // it from below and is linear, so no point of K is lit when the bound is
     // positive at the three corners (margin: the FP32 error of the linear term)
     const int m = F[0] <= F[1] ? (F[0] <= F[2] ? 0 : 2) : (F[1] <= F[2] ? 1 : 2);
-    const float qx = P.F.q[m][0], qy = P.F.q[m][1], rm = P.F.rs[m];
+    const float qx = T.q[m][0], qy = T.q[m][1], rm = T.rs[m];
     float lo = F[m];
     for (int k = 0; k < 3; ++k) {
       if (k == m) continue;
       const float dp = add2(Fc.p_hi[k], Fc.p_lo[k], -Fc.p_hi[m], -Fc.p_lo[m]);
-      const float lin = (qx * (P.F.q[k][0] - qx) + qy * (P.F.q[k][1] - qy)) / rm;
+      const float lin = (qx * (T.q[k][0] - qx) + qy * (T.q[k][1] - qy)) / rm;
       lo = fminf(lo, F[m] + dp + lin);
     }
     if (lo > 4e-7f * rm) return FACE_DARK;
   }
-  float p0t = add2(Fc.p_hi[0], Fc.p_lo[0], P.nt_hi, P.nt_lo);
-  c = -(p0t + (Fc.g[0] * P.F.xb[0] + Fc.g[1] * P.F.xb[1]));
-  if (fabsf(c) < 1e-6f * diam) c = 0.f;
   return FACE_CUT;
 }
 
@@ -980,31 +963,30 @@ STBEM_HD inline void cut_in_fp64(const PointCol& P, const FaceGeom& Fc, const do
   o.D0 = c * c - P.D.d * P.D.d * (1.0 - (Fc.g[0] * Fc.g[0] + Fc.g[1] * Fc.g[1]));
 }
 
-STBEM_HD inline void cut_in_mixed(const PointCol& P, const FaceF& Fc, const float* F, float c, const FaceGeom& F64,
+// The conic's size D0 = c^2 - d^2 (1 - |g|^2) is formed in FP32 here; where
+// the cone only just reaches the face plane (d0_cancels: |D0| < c^2 / 20,
+// about 3 % of the cut faces) its two terms cancel, and c (an O(1) difference
+// formed in FP32 pairs, but with <g, xb> in FP32) loses the relative accuracy
+// D0 needs; there the caller replaces it by the value from the apex's FP64
+// geometry (d0_fp64) or from FP32 pairs (d0_pairs).
+STBEM_HD inline void cut_in_mixed(const PtR<float>& T, const ConeM& M, const FaceF& Fc, const float* F, float c,
                                   FaceCutIn<float>& o) {
   for (int k = 0; k < 3; ++k) {
     int k1 = (k + 1) % 3;
     o.F[k] = F[k];
-    o.a0[k] = -add2(Fc.p_hi[k], Fc.p_lo[k], P.nt_hi, P.nt_lo);
+    o.a0[k] = -add2(Fc.p_hi[k], Fc.p_lo[k], M.nt_hi, M.nt_lo);
     o.a1[k] = add2(Fc.p_hi[k1], Fc.p_lo[k1], -Fc.p_hi[k], -Fc.p_lo[k]);
   }
   o.g[0] = Fc.g[0]; o.g[1] = Fc.g[1];
-  o.g64[0] = F64.g[0]; o.g64[1] = F64.g[1];
+  o.g64[0] = o.g64[1] = o.c64 = 0.0;   // coplanar arcs never come here (near_singular_mixed)
   o.c = c;
-  o.c64 = (double)c;
-  // the conic's size D0 = c^2 - d^2 (1 - |g|^2): where the cone only just
-  // reaches the face plane (|D0| < c^2 / 20) its two terms cancel, and c (an
-  // O(1) difference formed in FP32 pairs, but with <g, xb> in FP32) loses the
-  // relative accuracy D0 needs; there it is formed in FP64 from the apex's
-  // FP64 geometry (about 3 % of the cut faces)
-  const float d = P.F.d;
-  float D0 = c * c - d * d * (1.f - (Fc.g[0] * Fc.g[0] + Fc.g[1] * Fc.g[1]));
-  if (fabsf(D0) < 0.05f * c * c) {
-    const double c64 = P.t - (F64.p[0] + (F64.g[0] * P.D.xb[0] + F64.g[1] * P.D.xb[1]));
-    const double d64 = P.D.d;
-    D0 = (float)(c64 * c64 - d64 * d64 * (1.0 - (F64.g[0] * F64.g[0] + F64.g[1] * F64.g[1])));
-  }
-  o.D0 = D0;
+  o.D0 = c * c - T.d * T.d * (1.f - (Fc.g[0] * Fc.g[0] + Fc.g[1] * Fc.g[1]));
+}
+STBEM_HD inline bool d0_cancels(const FaceCutIn<float>& in) { return fabsf(in.D0) < 0.05f * in.c * in.c; }
+STBEM_HD inline float d0_fp64(const PointCol& P, const FaceGeom& F64) {
+  const double c64 = P.t - (F64.p[0] + (F64.g[0] * P.D.xb[0] + F64.g[1] * P.D.xb[1]));
+  const double d64 = P.D.d;
+  return (float)(c64 * c64 - d64 * d64 * (1.0 - (F64.g[0] * F64.g[0] + F64.g[1] * F64.g[1])));
 }
 
 // A conic arc of a cut face (d != 0) recorded for evaluation later: the
@@ -1048,9 +1030,8 @@ STBEM_HD inline R arc_value(const ArcRec<R>& a, const ArcRule& rule) {
 // three) are appended to defer[*ndefer] instead of integrated, and the
 // return value holds the edge pieces (and any coplanar arc) only.
 template <typename R>
-STBEM_HD __noinline__ double face_cut(const ColR<R>& G, const PointCol& P64, const FaceCutIn<R>& in,
+STBEM_HD __noinline__ double face_cut(const ColR<R>& G, const PtR<R>& P, const FaceCutIn<R>& in,
                                       const ArcRule& rule, ArcRec<R>* defer = nullptr, int* ndefer = nullptr) {
-  const PtR<R>& P = pt<R>(P64);
   const R d = P.d, c = in.c;
   const R* g = in.g;
   const R* F = in.F;
@@ -1174,22 +1155,72 @@ STBEM_HD __noinline__ double face_cut(const ColR<R>& G, const PointCol& P64, con
   return (double)total;
 }
 
+#ifdef __CUDACC__
+// ---------------------------------------------------------------------------
+// FP32 pairs (double-float, about 2^-45 relative): the geometry of an apex
+// against a column off the FP64 pipe, which on sm_103a has 1/76 of the FP32
+// rate. Error-free sums (Knuth) and products (fma), after Dekker 1971; the
+// intrinsics keep the compiler from contracting them.
+// ---------------------------------------------------------------------------
+struct F2 { float h, l; };
+__device__ __forceinline__ F2 f2_fast(float a, float b) {   // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ F2 f2_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 s = f2_sum(a.h, b.h);
+  const F2 t = f2_sum(a.l, b.l);
+  s = f2_fast(s.h, __fadd_rn(s.l, t.h));
+  return f2_fast(s.h, __fadd_rn(s.l, t.l));
+}
+__device__ __forceinline__ F2 f2_neg(F2 a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = __fmaf_rn(a.h, b.h, -p);
+  e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e));
+  return f2_fast(p, e);
+}
+__device__ __forceinline__ F2 f2_sqrt(F2 a) {
+  if (!(a.h > 0.f)) return {0.f, 0.f};
+  const float s = __fsqrt_rn(a.h), p = __fmul_rn(s, s);
+  const float r = __fadd_rn(__fsub_rn(__fsub_rn(a.h, p), __fmaf_rn(s, s, -p)), a.l);   // a - s^2
+  return f2_fast(s, __fdividef(r, 2.f * s));
+}
+
+// D0 where it cancels (see cut_in_mixed), from FP32 pairs
+__device__ __forceinline__ float d0_pairs(F2 d, const F2* xb, F2 nt, const FaceF& Fc) {
+  const F2 g0 = {Fc.g[0], Fc.g_lo[0]}, g1 = {Fc.g[1], Fc.g_lo[1]};
+  F2 c = f2_add(F2{Fc.p_hi[0], Fc.p_lo[0]}, nt);                      // -(t - P(xb))
+  c = f2_add(c, f2_add(f2_mul(g0, xb[0]), f2_mul(g1, xb[1])));
+  const F2 gg = f2_add(f2_mul(g0, g0), f2_mul(g1, g1));
+  const F2 om = f2_add(F2{1.f, 0.f}, f2_neg(gg));
+  const F2 D = f2_add(f2_mul(c, c), f2_neg(f2_mul(f2_mul(d, d), om)));
+  return D.h + D.l;
+}
+#endif
+
 // 4 pi W_P(x) in one call (used by the kernel-level entry point and checks)
 template <bool FP32>
 STBEM_HD inline double face_W(const ColGeom& G, const PointCol& P, const FaceGeom& Fc, const ArcRule& rule) {
   if (FP32) {
     FaceF Ff;
     make_facef(Fc, Ff);
-    float F[3], c = 0.f;
-    int cls = face_class_mixed(P, Ff, F, c, (float)G.diam);
+    float F[3];
+    int cls = face_class_mixed(P.F, P.M, Ff, F);
     if (cls == FACE_LIT) return P.Wst;
     if (cls == FACE_DARK) return 0.0;
+    const float c = face_c_mixed(P.F, P.M, Ff, (float)G.diam);
     if (near_singular_mixed(c, P.F.d, (float)G.diam)) return nan("");   // the caller recomputes it in FP64
     ColR<float> CR;
     make_colr<float>(G, CR);
     FaceCutIn<float> in;
-    cut_in_mixed(P, Ff, F, c, Fc, in);
-    return face_cut<float>(CR, P, in, rule);
+    cut_in_mixed(P.F, P.M, Ff, F, c, in);
+    if (d0_cancels(in)) in.D0 = d0_fp64(P, Fc);
+    return face_cut<float>(CR, P.F, in, rule);
   }
   double F[3], c = 0.0;
   int cls = face_class(G, P, Fc, F, c);
@@ -1199,7 +1230,7 @@ STBEM_HD inline double face_W(const ColGeom& G, const PointCol& P, const FaceGeo
   make_colr<double>(G, CR);
   FaceCutIn<double> in;
   cut_in_fp64(P, Fc, F, c, in);
-  return face_cut<double>(CR, P, in, rule);
+  return face_cut<double>(CR, P.D, in, rule);
 }
 
 // 4 pi W_P(x) entirely in FP64 from the apex coordinates: the fallback of the

@@ -328,12 +328,13 @@ bem_status run_job(bem_server* S, bem_context* cx, const Job& J, Done& D, int64_
         bem_status a = acquire(S, ticket, need);
         if (a == BEM_OK) reserved = need;
         return a;
-      }, &op);
+      }, &op, S->slot_share - sbytes);
   if (st != BEM_OK) {
     if (reserved > 0) release(S, reserved, 0);
     return st;
   }
   std::unique_ptr<bem_operator, void (*)(bem_operator*)> op_guard(op, bem_operator_destroy);
+  operator_release_scratch(op, s);   // the slot's share is the next request's
   st = solve_job(S, s, op, J, D);
   if (!caching || (st != BEM_OK && st != BEM_ERR_NOT_CONVERGED)) {
     release(S, reserved, 0);

@@ -1,0 +1,753 @@
+// Quadrature and assembly of the matrix in stages (eq. int_bform).
+//
+// For every face F with nu_{F,t} != 0 over test column I and every outer
+// point x_q on F (composite midpoint rule, Fig. int_tri_mid) the potentials W
+// of the faces over trial column J are evaluated,
+//     U[F][j] = sum_q V 1_{sigma_j}(x_q) = sum_q (W_lo(j)(x_q) - W_hi(j)(x_q)),
+// and A_ij = |K_I| / m_Q^2 * (U[F_lo(i)][j] - U[F_hi(i)][j]) (eq. int_bform
+// with nu_{F,t}|F| = -|K| on the lower face, +|K| on the upper).
+//
+// The blocks (I, J) are taken in chunks whose intermediate data fit the
+// operator's scratch. Per chunk:
+//   k_apex       a CTA per block: the block's pattern bits; one thread per
+//                (face, outer point): its geometry against column J and the
+//                class of every face of its window (dark: W = 0, fully lit:
+//                the whole triangle's W, cut: queued)
+//   k_cut_far    one thread per queued pair in the far field: the edge pieces
+//                and the conic arc of the cut face
+//   k_cut_any    pairs in the near field and arcs the far form refuses
+//   k_cut_fp64   near-singular faces of the mixed path, in FP64
+//   k_assemble   a CTA per block: U and the entries (or their product with x)
+// The FP64 operator takes the same stages in FP64, with one queue.
+//
+// Why stages: the cut faces are about a third of the pairs and cost ten times
+// a dark or lit one. In one kernel with a warp per face, 14 of 32 lanes were
+// active, every warp held the registers and shared memory of the largest
+// phase (8 to 16 warps per SM), and the phases' code did not fit the
+// instruction caches. Queues fill the lanes, and each stage has its own
+// register budget and occupancy. The intermediate data are about 150 bytes
+// per (face, outer point), written and read once.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "stbem_block.cuh"
+#include "stbem_internal.h"
+
+namespace stbem {
+
+bem_status upload_gauss_stage(const double* x, const double* w, const float* xf, const float* wf, size_t n) {
+  STBEM_CUDA(cudaMemcpyToSymbol(c_gl_x, x, n * sizeof(double)));
+  STBEM_CUDA(cudaMemcpyToSymbol(c_gl_w, w, n * sizeof(double)));
+  STBEM_CUDA(cudaMemcpyToSymbol(c_gl_xf, xf, n * sizeof(float)));
+  STBEM_CUDA(cudaMemcpyToSymbol(c_gl_wf, wf, n * sizeof(float)));
+  return BEM_OK;
+}
+
+namespace {
+
+// One apex (face, outer point) against a trial column, as the cut stages need it.
+struct alignas(16) ApexF {
+  float xbh[2], xbl[2];          // foot point, FP32 pairs
+  float dh, dl, far_rho;
+  int far;
+  float rs[3], E[3];             // corner distances, whole-edge integrals
+  float rho_hi[3], rho_lo[3], nt_hi, nt_lo;
+  uint32_t slot0;                // potential of the window's first face
+  int32_t surf0;                 // and that face
+  int32_t col, pt, seg, pad;
+};
+static_assert(sizeof(ApexF) == 112, "ApexF layout");
+struct alignas(16) ApexD {
+  double t, d, xb[2], rs[3], E[3];
+  uint32_t slot0;
+  int32_t surf0, col, seg;
+};
+static_assert(sizeof(ApexD) == 96, "ApexD layout");
+
+template <typename R> struct Types;
+template <> struct Types<float> { typedef ApexF Apex; typedef FaceF Face; };
+template <> struct Types<double> { typedef ApexD Apex; typedef FaceGeom Face; };
+
+enum { CNT_APEX, CNT_ASM, CNT_SLOT, CNT_RAY, CNT_FAR, CNT_ANY, CNT_F64, CNT_N };
+
+struct StageArgs {
+  BlockCtx one;                  // the operator (S <= 1), or the sizes all operators of a batch share
+  const BlockCtx* many;
+  const int64_t* prefix;
+  int S;
+  int64_t g0, g1;                // blocks of the chunk (dense order, operators one after the other)
+  void* apex;
+  void* W;                       // potentials; a queued one holds its apex's index until it is computed
+  uint32_t *q_far, *q_any, *q_64;
+  uint2* fmeta;                  // per block and face: first potential, window (first face | faces << 16)
+  uint32_t* bits;                // per block and face
+  unsigned* cnt;
+  void* uslab;                   // per CTA of k_assemble: U where shared memory does not hold it
+  int ucap;                      // entries of U that shared memory holds
+};
+
+constexpr int kApexThreads = 256;   // >= MAX_COL_SURF: one thread per face in the window scan
+static_assert(kApexThreads >= MAX_COL_SURF, "one thread per face");
+constexpr int kCutThreads = 128;
+constexpr int kAsmThreads = 128;
+
+// exclusive sum over the CTA (kApexThreads threads); *total = the sum
+__device__ __forceinline__ unsigned cta_scan(unsigned v, unsigned* s_w, unsigned* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned u = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += u;
+  }
+  if (lane == 31) s_w[warp] = inc;
+  __syncthreads();
+  unsigned off = 0, sum = 0;
+#pragma unroll
+  for (int w = 0; w < kApexThreads / 32; ++w) {
+    const unsigned x = s_w[w];
+    if (w < warp) off += x;
+    sum += x;
+  }
+  *total = sum;
+  __syncthreads();
+  return off + inc - v;
+}
+
+// appends v to a queue; the active lanes take their places with one atomic
+__device__ __forceinline__ void push(uint32_t* q, unsigned* n, uint32_t v) {
+  const unsigned m = __activemask(), lane = threadIdx.x & 31;
+  const int leader = __ffs(m) - 1;
+  unsigned base = 0;
+  if ((int)lane == leader) base = atomicAdd(n, (unsigned)__popc(m));
+  base = __shfl_sync(m, base, leader);
+  q[base + __popc(m & ((1u << lane) - 1u))] = v;
+}
+
+// ---- geometry of an apex against the trial column ----------------------
+
+__device__ __forceinline__ void frame_points(PtR<float>& T, const ColR<float>& R) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    T.q[k][0] = R.Q[k][0] - T.xb[0];
+    T.q[k][1] = R.Q[k][1] - T.xb[1];
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    T.ps[k] = T.q[k][0] * R.U[k][1] - T.q[k][1] * R.U[k][0];
+    T.ws[k] = T.q[k][0] * R.U[k][0] + T.q[k][1] * R.U[k][1];
+  }
+}
+
+// A function of its own: inlined, its products were contracted with those of
+// the geometry around it, and the near edges came out an ulp apart from the
+// same edges integrated elsewhere.
+__device__ __noinline__ float whole_edge(const PtR<float>& T, const ColR<float>& R, int k) {
+  return edge_full_mixed(T, R, k);
+}
+
+// The mixed path: what cancels between |x - y| and t - tau (relative
+// position, height, foot point, corner distances) in FP32 pairs, the rest in
+// FP32. The same values came from FP64 before, whose pipe (1/76 of the FP32
+// rate) was the kernel's busiest unit.
+__device__ __forceinline__ void apex_geometry(const float4 xh, const float4 xl, const ColF& G, PtR<float>& T, ConeM& M,
+                                              F2& d, F2* xb, float& Wst) {
+  const F2 nt = {-xh.x, -xl.x}, x[3] = {{xh.y, xl.y}, {xh.z, xl.z}, {xh.w, xl.w}};
+  F2 rel[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) rel[i] = f2_add(x[i], F2{-G.Xh[0][i], -G.Xl[0][i]});
+  auto dot = [&](const float* h, const float* l) {
+    return f2_add(f2_add(f2_mul(rel[0], F2{h[0], l[0]}), f2_mul(rel[1], F2{h[1], l[1]})), f2_mul(rel[2], F2{h[2], l[2]}));
+  };
+  d = dot(G.nh, G.nl);
+  if (fabsf(d.h) < 1e-13f * G.R.diam) d = F2{0.f, 0.f};
+  xb[0] = dot(G.e1h, G.e1l);
+  xb[1] = dot(G.e2h, G.e2l);
+  T.d = d.h;
+  T.xb[0] = xb[0].h;
+  T.xb[1] = xb[1].h;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    F2 v[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      v[i] = k == 0 ? rel[i] : f2_add(x[i], F2{-G.Xh[k][i], -G.Xl[k][i]});
+      v[i] = f2_mul(v[i], v[i]);
+    }
+    const F2 r = f2_sqrt(f2_add(f2_add(v[0], v[1]), v[2]));
+    T.rs[k] = r.h;
+    const F2 rho = f2_add(r, nt);
+    M.rho_hi[k] = rho.h;
+    M.rho_lo[k] = rho.l;
+  }
+  frame_points(T, G.R);
+  float out = 0.f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) out = fmaxf(out, -T.ps[k]);
+  T.far = out >= FAR_RHO * G.R.diam;
+  T.C = T.rs[0];
+  T.far_rho = out;
+  const F2 o2 = {out, 0.f};
+  const F2 rl = f2_add(f2_sqrt(f2_add(f2_mul(d, d), f2_mul(o2, o2))), nt);
+  M.nt_hi = nt.h;
+  M.nt_lo = nt.l;
+  M.rlot_hi = rl.h;
+  M.rlot_lo = rl.l;
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k) T.Efull[k] = whole_edge(T, G.R, k);
+  Wst = (T.Efull[0] + T.Efull[1]) + T.Efull[2];
+}
+
+// ---- k_apex ------------------------------------------------------------
+
+template <typename R>
+size_t apex_smem(int max_tet, int max_surf, int nq) {
+  size_t s = bits_smem(max_tet, max_surf, nq);
+  s = (s + 15) / 16 * 16 + sizeof(typename Types<R>::Face) * max_surf;
+  return s + sizeof(uint2) * max_surf + sizeof(uint16_t) * ((max_surf + 7) / 8 * 8);
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(const StageArgs a) {
+  constexpr bool FP32 = sizeof(R) == 4;
+  typedef typename Types<R>::Face Face;
+  typedef typename Types<R>::Apex Apex;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ BlockSm C;
+  __shared__ BlockCtx B;
+  __shared__ __align__(16) ColF G;
+  __shared__ unsigned s_w[kApexThreads / 32], s_base[4];
+  __shared__ int s_seg, s_wmax;
+  const int tid = threadIdx.x, nq = a.one.nq, max_surf = a.one.max_surf, words = bit_words(a.one.max_tet);
+  const BlockPtr P = block_ptr(smem, a.one.max_tet, max_surf, nq);
+  Face* Fs = reinterpret_cast<Face*>(smem + (bits_smem(a.one.max_tet, max_surf, nq) + 15) / 16 * 16);
+  uint2* fm = reinterpret_cast<uint2*>(Fs + max_surf);
+  uint16_t* act = reinterpret_cast<uint16_t*>(fm + max_surf);
+  if (tid == 0 && a.S <= 1) B = a.one;
+  int cur = a.S > 1 ? -1 : 0;
+  for (;;) {
+    if (tid == 0) s_base[3] = atomicAdd(&a.cnt[CNT_APEX], 1u);
+    __syncthreads();
+    const int64_t g = a.g0 + s_base[3];
+    if (g >= a.g1) break;
+    int64_t b = g;
+    if (a.S > 1) {
+      if (tid == 0) s_seg = find_seg(a.prefix, a.S, g);
+      __syncthreads();
+      if (s_seg != cur && tid == 0) B = a.many[s_seg];
+      cur = s_seg;
+      b -= a.prefix[cur];
+    }
+    if (tid == 0) s_wmax = 0;
+    __syncthreads();
+    if (B.bw[b] == 0) continue;
+    const int64_t I = b / B.n_col, J = b % B.n_col;
+    load_trial(B, J, C, P.pan);
+    load_test(B, I, C);
+    block_bits(B, C, P);
+    // trial faces and column frame
+    if constexpr (FP32) {
+      const uint4* src = reinterpret_cast<const uint4*>(B.facef + C.surfJ);
+      for (int k = tid; k < 3 * C.nsJ; k += kApexThreads) reinterpret_cast<uint4*>(Fs)[k] = src[k];
+      const uint4* cs = reinterpret_cast<const uint4*>(B.colf + J);
+      for (int k = tid; k < (int)(sizeof(ColF) / 16); k += kApexThreads) reinterpret_cast<uint4*>(&G)[k] = cs[k];
+    } else {
+      for (int k = tid; k < C.nsJ; k += kApexThreads) Fs[k] = B.surf[C.surfJ + k].f;
+    }
+    // windows of the faces, their places among the chunk's potentials
+    int slo = 0, nsw = 0;
+    if (tid < C.nsI) bits_surfaces(P.bits + tid * words, words, P.pan, slo, nsw);
+    if (nsw) atomicMax(&s_wmax, nsw);
+    unsigned total;
+    const unsigned ex = cta_scan((unsigned)(nsw * nq) | (nsw ? 1u << 24 : 0u), s_w, &total);
+    const int nact = (int)(total >> 24);
+    if (tid == 0) {
+      s_base[0] = atomicAdd(&a.cnt[CNT_SLOT], total & 0xffffffu);
+      s_base[1] = atomicAdd(&a.cnt[CNT_RAY], (unsigned)(nact * nq));
+    }
+    __syncthreads();
+    const unsigned ray0 = s_base[1];
+    if (tid < C.nsI) {
+      const uint2 m = make_uint2(s_base[0] + (ex & 0xffffffu), (unsigned)slo | ((unsigned)nsw << 16));
+      fm[tid] = m;
+      a.fmeta[(g - a.g0) * max_surf + tid] = m;
+      if (nsw) act[ex >> 24] = (uint16_t)tid;
+    }
+    for (int k = tid; k < C.nsI * words; k += kApexThreads) a.bits[(g - a.g0) * max_surf * words + k] = P.bits[k];
+    __syncthreads();
+    const int wmax = s_wmax, nr = nact * nq;
+    R* W = static_cast<R*>(a.W);
+    for (int r0 = 0; r0 < nr; r0 += kApexThreads) {
+      const int r = r0 + tid;
+      const bool on = r < nr;
+      int n = 0, first = 0;
+      uint32_t slot0 = 0;
+      int pt = 0;
+      typename std::conditional<FP32, PtR<float>, PointCol>::type T;
+      ConeM M;
+      F2 d2 = {0.f, 0.f}, xb2[2] = {{0.f, 0.f}, {0.f, 0.f}};
+      R Wst = R(0);
+      bool far = true;
+      if (on) {
+        const int k = r / nq, q = r - k * nq, f = act[k];
+        const uint2 m = fm[f];
+        first = (int)(m.y & 0xffffu);
+        n = (int)(m.y >> 16);
+        slot0 = m.x + q;
+        pt = (C.surfI + f) * nq + q;
+        if constexpr (FP32) {
+          apex_geometry(B.ptsf[pt], B.ptsl[pt], G, T, M, d2, xb2, Wst);
+          far = T.far;
+        } else {
+          point_col(B.pts + 4 * (int64_t)pt, B.cols[J], T, false);
+          Wst = T.Wst;
+        }
+      }
+      bool any = false;
+      for (int s0 = 0; s0 < wmax; s0 += 64) {
+        unsigned long long mask = 0;
+        const int s1 = min(n, s0 + 64);
+        for (int s = s0; s < s1; ++s) {
+          int cls;
+          R F[3];
+          if constexpr (FP32) {
+            cls = face_class_mixed(T, M, Fs[first + s], F);
+          } else {
+            double c;
+            cls = face_class(B.cols[J], T, Fs[first + s], F, c);
+          }
+          if (cls == FACE_CUT) mask |= 1ull << (s - s0);
+          else W[slot0 + s * nq] = cls == FACE_LIT ? Wst : R(0);
+        }
+        any |= mask != 0;
+        const unsigned cnt = (unsigned)__popcll(mask);
+        unsigned tot;
+        const unsigned at = cta_scan(far ? cnt : cnt << 16, s_w, &tot);
+        if (tid == 0) {
+          if (tot & 0xffffu) s_base[0] = atomicAdd(&a.cnt[CNT_FAR], tot & 0xffffu);
+          if (tot >> 16) s_base[2] = atomicAdd(&a.cnt[CNT_ANY], tot >> 16);
+        }
+        __syncthreads();
+        uint32_t* q = far ? a.q_far + s_base[0] + (at & 0xffffu) : a.q_any + s_base[2] + (at >> 16);
+        while (mask) {
+          const int s = s0 + __ffsll((long long)mask) - 1;
+          mask &= mask - 1;
+          const uint32_t slot = slot0 + s * nq;
+          *q++ = slot;
+          if constexpr (FP32) W[slot] = __uint_as_float(ray0 + r);
+          else W[slot] = __hiloint2double(0, (int)(ray0 + r));
+        }
+        __syncthreads();   // s_base is rewritten by the next round
+      }
+      if (any) {
+        Apex Y;
+        if constexpr (FP32) {
+          for (int i = 0; i < 2; ++i) { Y.xbh[i] = xb2[i].h; Y.xbl[i] = xb2[i].l; }
+          Y.dh = d2.h; Y.dl = d2.l; Y.far_rho = T.far_rho; Y.far = T.far;
+          for (int k = 0; k < 3; ++k) {
+            Y.rs[k] = T.rs[k]; Y.E[k] = T.Efull[k]; Y.rho_hi[k] = M.rho_hi[k]; Y.rho_lo[k] = M.rho_lo[k];
+          }
+          Y.nt_hi = M.nt_hi; Y.nt_lo = M.nt_lo;
+          Y.pt = pt; Y.pad = 0;
+        } else {
+          Y.t = T.t; Y.d = T.D.d; Y.xb[0] = T.D.xb[0]; Y.xb[1] = T.D.xb[1];
+          for (int k = 0; k < 3; ++k) { Y.rs[k] = T.D.rs[k]; Y.E[k] = T.D.Efull[k]; }
+        }
+        Y.slot0 = slot0; Y.surf0 = C.surfJ + first; Y.col = (int32_t)J; Y.seg = cur;
+        static_cast<Apex*>(a.apex)[ray0 + r] = Y;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// ---- cut faces ---------------------------------------------------------
+
+// a queued pair of the mixed path: its apex, face and column; false: near-singular
+struct CutF {
+  PtR<float> T;
+  ColR<float> R;
+  FaceCutIn<float> in;
+};
+__device__ __forceinline__ bool load_cut(const StageArgs& a, uint32_t slot, uint32_t ray, CutF& c) {
+  const ApexF Y = static_cast<const ApexF*>(a.apex)[ray];
+  const BlockCtx& B = a.S > 1 ? a.many[Y.seg] : a.one;
+  const FaceF Fc = B.facef[Y.surf0 + (int)(slot - Y.slot0) / a.one.nq];
+  c.R = B.colf[Y.col].R;
+  PtR<float>& T = c.T;
+  ConeM M;
+  T.d = Y.dh;
+  T.xb[0] = Y.xbh[0]; T.xb[1] = Y.xbh[1];
+  T.far = Y.far;
+  T.far_rho = Y.far_rho;
+  for (int k = 0; k < 3; ++k) {
+    T.rs[k] = Y.rs[k]; T.Efull[k] = Y.E[k]; M.rho_hi[k] = Y.rho_hi[k]; M.rho_lo[k] = Y.rho_lo[k];
+  }
+  T.C = T.rs[0];
+  M.nt_hi = Y.nt_hi; M.nt_lo = Y.nt_lo;
+  frame_points(T, c.R);
+  float F[3];
+  for (int k = 0; k < 3; ++k) F[k] = add2(Fc.p_hi[k], Fc.p_lo[k], M.rho_hi[k], M.rho_lo[k]);
+  const float cc = face_c_mixed(T, M, Fc, c.R.diam);
+  if (near_singular_mixed(cc, T.d, c.R.diam)) return false;
+  cut_in_mixed(T, M, Fc, F, cc, c.in);
+  if (d0_cancels(c.in)) {
+    const F2 xb[2] = {{Y.xbh[0], Y.xbl[0]}, {Y.xbh[1], Y.xbl[1]}};
+    c.in.D0 = d0_pairs(F2{Y.dh, Y.dl}, xb, F2{Y.nt_hi, Y.nt_lo}, Fc);
+  }
+  return true;
+}
+
+// FAR: the pairs of apexes in the far field; arcs the chord form refuses go
+// on to the other queue. A value that is not finite is recomputed in FP64.
+template <bool FAR>
+__global__ void __launch_bounds__(kCutThreads) k_cut(const StageArgs a) {
+  float* W = static_cast<float*>(a.W);
+  const uint32_t* q = FAR ? a.q_far : a.q_any;
+  const unsigned n = a.cnt[FAR ? CNT_FAR : CNT_ANY];
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t slot = q[i];
+    CutF c;
+    if (!load_cut(a, slot, __float_as_uint(W[slot]), c)) {
+      push(a.q_64, &a.cnt[CNT_F64], slot);
+      continue;
+    }
+    ArcRec<float> arc[3];
+    int na = 0;
+    float v = (float)face_cut<float>(c.R, c.T, c.in, a.one.rule, arc, &na);
+    bool ok = true;
+    for (int k = 0; k < na; ++k) {
+      if (FAR) {
+        float t = 0.f;
+        ok = ok && arc[k].far && arc_far<float>(arc[k].xb, arc[k].d, arc[k].C, arc[k].far_rho, arc[k].g, arc[k].A,
+                                                arc[k].dAB, a.one.rule, t);
+        v += t;
+      } else {
+        v += arc_value<float>(arc[k], a.one.rule);
+      }
+    }
+    if (!ok) push(a.q_any, &a.cnt[CNT_ANY], slot);
+    else if (!isfinite(v)) push(a.q_64, &a.cnt[CNT_F64], slot);
+    else W[slot] = v;
+  }
+}
+
+__global__ void __launch_bounds__(kCutThreads) k_cut_fp64(const StageArgs a) {
+  float* W = static_cast<float*>(a.W);
+  const unsigned n = a.cnt[CNT_F64];
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t slot = a.q_64[i];
+    const ApexF& Y = static_cast<const ApexF*>(a.apex)[__float_as_uint(W[slot])];
+    const BlockCtx& B = a.S > 1 ? a.many[Y.seg] : a.one;
+    W[slot] = (float)face_W_fp64(B.pts + 4 * (int64_t)Y.pt, B.cols[Y.col],
+                                 B.surf[Y.surf0 + (int)(slot - Y.slot0) / a.one.nq].f, a.one.n_theta);
+  }
+}
+
+// the FP64 operator's cut faces
+__global__ void __launch_bounds__(kCutThreads) k_cut_d(const StageArgs a) {
+  double* W = static_cast<double*>(a.W);
+  const unsigned n = a.cnt[CNT_FAR];
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t slot = a.q_far[i];
+    const ApexD Y = static_cast<const ApexD*>(a.apex)[(uint32_t)__double2loint(W[slot])];
+    const BlockCtx& B = a.S > 1 ? a.many[Y.seg] : a.one;
+    const ColGeom& G = B.cols[Y.col];
+    ColR<double> R;
+    make_colr<double>(G, R);
+    PointCol P;
+    P.t = Y.t;
+    P.rlo = 0.0;                    // the class is known: the pair is cut
+    P.D.d = Y.d; P.D.xb[0] = Y.xb[0]; P.D.xb[1] = Y.xb[1];
+    P.D.far = 0; P.D.C = 0.0; P.D.far_rho = 0.0;
+    for (int k = 0; k < 3; ++k) {
+      P.r[k] = P.D.rs[k] = Y.rs[k];
+      P.D.Efull[k] = Y.E[k];
+      P.D.q[k][0] = R.Q[k][0] - Y.xb[0];
+      P.D.q[k][1] = R.Q[k][1] - Y.xb[1];
+    }
+    for (int k = 0; k < 3; ++k) {
+      P.D.ps[k] = P.D.q[k][0] * R.U[k][1] - P.D.q[k][1] * R.U[k][0];
+      P.D.ws[k] = P.D.q[k][0] * R.U[k][0] + P.D.q[k][1] * R.U[k][1];
+    }
+    const FaceGeom Fc = B.surf[Y.surf0 + (int)(slot - Y.slot0) / a.one.nq].f;
+    double F[3], c;
+    for (int k = 0; k < 3; ++k) F[k] = (Fc.p[k] - P.t) + P.r[k];
+    c = P.t - (Fc.p[0] + Fc.g[0] * P.D.xb[0] + Fc.g[1] * P.D.xb[1]);
+    if (fabs(c) < 1e-13 * G.diam) c = 0.0;
+    FaceCutIn<double> in;
+    cut_in_fp64(P, Fc, F, c, in);
+    W[slot] = face_cut<double>(R, P.D, in, a.one.rule);
+  }
+}
+
+// ---- k_assemble --------------------------------------------------------
+
+constexpr size_t kUBytes = 24576;   // shared memory for U
+
+template <typename R>
+size_t asm_smem(int max_tet, int max_surf) {
+  const int words = bit_words(max_tet);
+  return kUBytes + sizeof(uint32_t) * ((size_t)max_surf * words + 3 * max_surf + 2 * max_tet + 16);
+}
+
+// Bound by latency and L1 traffic: the entries are written once, coalesced;
+// the potentials are read twice (as the lower and the upper face of a panel).
+template <typename R>
+__global__ void __launch_bounds__(kAsmThreads) k_assemble(const StageArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ BlockCtx B;
+  __shared__ int s_seg, s_wU;
+  __shared__ unsigned s_g;
+  __shared__ R s_scale;
+  const int tid = threadIdx.x, nq = a.one.nq, max_surf = a.one.max_surf, max_tet = a.one.max_tet;
+  const int words = bit_words(max_tet);
+  R* Us = reinterpret_cast<R*>(smem);
+  uint32_t* bits = reinterpret_cast<uint32_t*>(smem + kUBytes);
+  uint2* fm = reinterpret_cast<uint2*>(bits + (max_surf * words + 1) / 2 * 2);
+  int* jf = reinterpret_cast<int*>(fm + max_surf);                        // first panel of a face's bits
+  uint32_t* lohi = reinterpret_cast<uint32_t*>(jf + max_surf);            // faces of the trial panels
+  uint32_t* row = lohi + max_tet;                                         // first panel | lo << 16 | hi << 24 of a row
+  const R* W = static_cast<const R*>(a.W);
+  if (tid == 0 && a.S <= 1) B = a.one;
+  int cur = a.S > 1 ? -1 : 0;
+  for (;;) {
+    if (tid == 0) {
+      s_g = atomicAdd(&a.cnt[CNT_ASM], 1u);
+      s_wU = 0;
+    }
+    __syncthreads();
+    const int64_t g = a.g0 + s_g;
+    if (g >= a.g1) break;
+    int64_t b = g;
+    if (a.S > 1) {
+      if (tid == 0) s_seg = find_seg(a.prefix, a.S, g);
+      __syncthreads();
+      if (s_seg != cur && tid == 0) B = a.many[s_seg];
+      cur = s_seg;
+      b -= a.prefix[cur];
+      __syncthreads();
+    }
+    const int Wd = B.bw[b];
+    __syncthreads();
+    if (Wd == 0) continue;
+    const int64_t I = b / B.n_col, J = b % B.n_col;
+    const int t0 = B.col_tet_begin[I], nt = B.col_tet_begin[I + 1] - t0;
+    const int tJ = B.col_tet_begin[J], ntJ = B.col_tet_begin[J + 1] - tJ;
+    const int ns = B.col_surf_begin[I + 1] - B.col_surf_begin[I];
+    if (tid == 0) s_scale = (R)(B.cols[I].area / (4.0 * STBEM_PI * nq));
+    for (int f = tid; f < ns; f += kAsmThreads) {
+      fm[f] = a.fmeta[(g - a.g0) * max_surf + f];
+      int lo = -1, hi = -1;
+      for (int w = 0; w < words; ++w) {
+        const uint32_t m = a.bits[((g - a.g0) * max_surf + f) * words + w];
+        bits[f * words + w] = m;
+        if (m) {
+          if (lo < 0) lo = 32 * w + __ffs(m) - 1;
+          hi = 32 * w + 31 - __clz(m);
+        }
+      }
+      jf[f] = max(lo, 0);
+      if (lo >= 0) atomicMax(&s_wU, hi - lo + 1);
+    }
+    for (int j = tid; j < ntJ; j += kAsmThreads) {
+      const PanelF& D = B.panf[tJ + j];
+      lohi[j] = (uint32_t)D.lo | ((uint32_t)D.hi << 16);
+    }
+    __syncthreads();
+    const int wU = s_wU;
+    R* U = ns * wU <= a.ucap ? Us : static_cast<R*>(a.uslab) + (size_t)blockIdx.x * max_surf * max_tet;
+    for (int it = tid; it < ns * wU; it += kAsmThreads) {
+      const int f = it / wU, j = jf[f] + it - f * wU;
+      R u = R(0);
+      if (j < ntJ && ((bits[f * words + (j >> 5)] >> (j & 31)) & 1u)) {
+        const uint2 m = fm[f];
+        const uint32_t lh = lohi[j];
+        const int slo = (int)(m.y & 0xffffu);
+        const R* lo = W + m.x + ((int)(lh & 0xffffu) - slo) * nq;
+        const R* hi = W + m.x + ((int)(lh >> 16) - slo) * nq;
+        for (int q = 0; q < nq; ++q) u += lo[q] - hi[q];
+      }
+      U[it] = u;
+    }
+    for (int r = tid; r < nt; r += kAsmThreads) {
+      const PanelF& D = B.panf[t0 + r];
+      int first = -1;
+      for (int w = 0; w < words && first < 0; ++w) {
+        const uint32_t m = bits[D.lo * words + w] | bits[D.hi * words + w];
+        if (m) first = 32 * w + __ffs(m) - 1;
+      }
+      row[r] = (uint32_t)max(first, 0) | ((uint32_t)D.lo << 16) | ((uint32_t)D.hi << 24);
+    }
+    __syncthreads();
+    const R scale = s_scale;
+    auto entry = [&](uint32_t rw, int j) {
+      const int lo = (int)((rw >> 16) & 0xffu), hi = (int)(rw >> 24);
+      const int ol = j - jf[lo], oh = j - jf[hi];
+      const R ul = (unsigned)ol < (unsigned)wU ? U[lo * wU + ol] : R(0);
+      const R uh = (unsigned)oh < (unsigned)wU ? U[hi * wU + oh] : R(0);
+      return scale * (ul - uh);
+    };
+    if (B.mf_y) {
+      // fused product: the row's band times x, one atomic add per right-hand side
+      for (int it = tid; it < nt * B.mf_nrhs; it += kAsmThreads) {
+        const int k = it / nt, r = it - k * nt;
+        const uint32_t rw = row[r];
+        const int first = (int)(rw & 0xffffu);
+        const double* xk = B.mf_x + (int64_t)k * B.mf_ld + tJ;
+        double sacc = 0.0;
+        for (int j = first; j < min(first + Wd, ntJ); ++j) sacc += (double)entry(rw, j) * xk[j];
+        atomicAdd(B.mf_y + (int64_t)k * B.mf_ld + t0 + r, sacc);
+      }
+    } else {
+      const int64_t voff = B.boff[b], roff = B.rsoff[b];
+      for (int r = tid; r < nt; r += kAsmThreads) B.rs[roff + r] = tJ + (int)(row[r] & 0xffffu);
+      for (int e = tid; e < nt * Wd; e += kAsmThreads) {
+        const int w = e / nt, r = e - w * nt;
+        const uint32_t rw = row[r];
+        const int j = (int)(rw & 0xffffu) + w;
+        const R v = j < ntJ ? entry(rw, j) : R(0);
+        if (B.val) B.val[voff + e] = (double)v;
+        if (B.val32) B.val32[voff + e] = (float)v;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+size_t up256(size_t n) { return (n + 255) / 256 * 256; }
+
+int occupancy(const void* kern, int threads, size_t smem) {
+  int per = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem) != cudaSuccess) cudaGetLastError();
+  return std::max(per, 1);
+}
+
+size_t slot_bytes(bool fp32) { return fp32 ? 4 + 3 * 4 : 8 + 4; }
+size_t apex_bytes(bool fp32) { return fp32 ? sizeof(ApexF) : sizeof(ApexD); }
+// scratch of `blocks` blocks with `rays` apexes and `slots` potentials (with the regions' alignment)
+size_t chunk_bytes(bool fp32, int max_tet, int max_surf, int64_t blocks, int64_t rays, int64_t slots) {
+  return 8 * 256 + rays * apex_bytes(fp32) + slots * slot_bytes(fp32) +
+         (size_t)blocks * max_surf * (sizeof(uint2) + sizeof(uint32_t) * bit_words(max_tet));
+}
+// fixed part: counters, and U of every CTA of k_assemble where shared memory does not hold it
+size_t fixed_bytes(bool fp32, int max_tet, int max_surf, int sms) {
+  const size_t u = (size_t)max_tet * max_surf * (fp32 ? 4 : 8);
+  return 256 + (u > kUBytes ? up256(u * sms * 4) : 0);
+}
+
+}  // namespace
+
+int stage_apex_per_sm(bool fp32, int max_tet, int max_surf, int nq) {
+  const size_t smem = fp32 ? apex_smem<float>(max_tet, max_surf, nq) : apex_smem<double>(max_tet, max_surf, nq);
+  const void* kern = fp32 ? (const void*)k_apex<float> : (const void*)k_apex<double>;
+  ensure_smem_attr(kern, smem);
+  return std::min(occupancy(kern, kApexThreads, smem), 4);
+}
+
+// Scratch of a quadrature over the blocks counted in `gran`: at most kScratch
+// bytes (a chunk), at least the largest run of GRAN blocks.
+void stage_scratch(bool fp32, int max_tet, int max_surf, int sms, const std::vector<const std::vector<uint2>*>& gran,
+                   int64_t value_bytes, int64_t* least, int64_t* wanted) {
+  size_t big = 0, all = 0;
+  for (const auto* v : gran)
+    for (const uint2& c : *v) {
+      const size_t n = chunk_bytes(fp32, max_tet, max_surf, GRAN, c.x, c.y);
+      big = std::max(big, n);
+      all += n;
+    }
+  const size_t fixed = fixed_bytes(fp32, max_tet, max_surf, sms);
+  const size_t cap = std::min<size_t>(std::max<size_t>(value_bytes / 2, (size_t)64 << 20), (size_t)1 << 30);
+  *least = (int64_t)(fixed + big);
+  *wanted = (int64_t)(fixed + std::max(big, std::min(all, cap)));
+}
+
+// All stages over the blocks [0, end) of the concatenated operators.
+bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* prefix, int S, bool fp32, int sms,
+                     const std::vector<const std::vector<uint2>*>& gran, const std::vector<int64_t>& blocks, int64_t end,
+                     void* scratch, int64_t bytes, int per_sm, cudaStream_t s) {
+  const int mt = one.max_tet, ms = one.max_surf, nq = one.nq;
+  const size_t fixed = fixed_bytes(fp32, mt, ms, sms);
+  unsigned char* base = static_cast<unsigned char*>(scratch);
+  StageArgs a;
+  a.one = one;
+  a.many = many;
+  a.prefix = prefix;
+  a.S = S;
+  a.cnt = reinterpret_cast<unsigned*>(base);
+  a.uslab = base + 256;
+  a.ucap = (int)(kUBytes / (fp32 ? 4 : 8));
+  const size_t sm_apex = fp32 ? apex_smem<float>(mt, ms, nq) : apex_smem<double>(mt, ms, nq);
+  const size_t sm_asm = fp32 ? asm_smem<float>(mt, ms) : asm_smem<double>(mt, ms);
+  const void* k_asm = fp32 ? (const void*)k_assemble<float> : (const void*)k_assemble<double>;
+  bem_status st = ensure_smem_attr(k_asm, sm_asm);
+  if (st != BEM_OK) return st;
+  const int n_apex = sms * std::max(1, std::min(per_sm, stage_apex_per_sm(fp32, mt, ms, nq)));
+  int n_asm = sms * occupancy(k_asm, kAsmThreads, sm_asm);
+  if (fixed > 256) n_asm = std::min(n_asm, sms * 4);   // one slab per CTA
+  const int n_far = sms * occupancy((const void*)(fp32 ? (const void*)k_cut<true> : (const void*)k_cut_d), kCutThreads, 0);
+  const int n_any = sms * occupancy((const void*)k_cut<false>, kCutThreads, 0);
+  const int n_64 = sms * occupancy((const void*)k_cut_fp64, kCutThreads, 0);
+
+  auto flush = [&](int64_t g0, int64_t g1, int64_t rays, int64_t slots) -> bem_status {
+    if (rays == 0) return BEM_OK;
+    const int64_t nb = g1 - g0;
+    unsigned char* p = base + fixed;
+    auto take = [&](size_t n) { unsigned char* r = p; p += up256(n); return r; };
+    a.g0 = g0;
+    a.g1 = g1;
+    a.apex = take(rays * apex_bytes(fp32));
+    a.W = take(slots * (fp32 ? 4 : 8));
+    a.q_far = reinterpret_cast<uint32_t*>(take(slots * 4));
+    a.q_any = a.q_64 = nullptr;
+    if (fp32) {
+      a.q_any = reinterpret_cast<uint32_t*>(take(slots * 4));
+      a.q_64 = reinterpret_cast<uint32_t*>(take(slots * 4));
+    }
+    a.fmeta = reinterpret_cast<uint2*>(take(nb * ms * sizeof(uint2)));
+    a.bits = reinterpret_cast<uint32_t*>(take(nb * ms * sizeof(uint32_t) * bit_words(mt)));
+    if (p - base > bytes) {
+      set_error("quadrature scratch too small");
+      return BEM_ERR_INTERNAL;
+    }
+    STBEM_CUDA(cudaMemsetAsync(a.cnt, 0, sizeof(unsigned) * CNT_N, s));
+    if (fp32) {
+      k_apex<float><<<n_apex, kApexThreads, sm_apex, s>>>(a);
+      k_cut<true><<<n_far, kCutThreads, 0, s>>>(a);
+      k_cut<false><<<n_any, kCutThreads, 0, s>>>(a);
+      k_cut_fp64<<<n_64, kCutThreads, 0, s>>>(a);
+      k_assemble<float><<<n_asm, kAsmThreads, sm_asm, s>>>(a);
+    } else {
+      k_apex<double><<<n_apex, kApexThreads, sm_apex, s>>>(a);
+      k_cut_d<<<n_far, kCutThreads, 0, s>>>(a);
+      k_assemble<double><<<n_asm, kAsmThreads, sm_asm, s>>>(a);
+    }
+    STBEM_CUDA(cudaGetLastError());
+    return BEM_OK;
+  };
+  // chunks: runs of granules that fit the scratch
+  int64_t g0 = 0, g1 = 0, rays = 0, slots = 0, off = 0;
+  for (size_t o = 0; o < gran.size(); ++o) {
+    const int64_t nb = std::min(blocks[o], end - off);
+    for (int64_t k = 0; k * GRAN < nb; ++k) {
+      const uint2 c = (*gran[o])[k];
+      const int64_t h0 = off + k * GRAN, h1 = off + std::min<int64_t>(nb, (k + 1) * GRAN);
+      if (h1 > g0 && g1 > g0 &&
+          (int64_t)(fixed + chunk_bytes(fp32, mt, ms, h1 - g0, rays + c.x, slots + c.y)) > bytes) {
+        st = flush(g0, g1, rays, slots);
+        if (st != BEM_OK) return st;
+        g0 = h0;
+        rays = slots = 0;
+      }
+      g1 = h1;
+      rays += c.x;
+      slots += c.y;
+    }
+    off += blocks[o];
+  }
+  return flush(g0, g1, rays, slots);
+}
+
+}  // namespace stbem

@@ -1,11 +1,9 @@
-// Launch-shape autotuning of the persistent quadrature (no counterpart in the
-// paper). The quadrature kernel is a persistent block queue; its free launch
-// parameters are the number of CTAs per SM it runs with (up to the occupancy
-// limit of its register and shared-memory budget) and, in mixed precision,
-// the register budget it was compiled for (128 registers for 4 CTAs per SM,
-// with spills; or 255 for 2, without). Fewer CTAs give each more L1 and issue
-// slots, more CTAs hide more latency; which wins depends on the device and
-// on the mesh's column sizes (the shared memory a CTA needs grows with them).
+// Launch-shape autotuning of the quadrature (no counterpart in the paper).
+// Its first stage is a persistent block queue whose free launch parameter is
+// the number of CTAs per SM it runs with, up to the occupancy limit: fewer
+// CTAs give each more L1 and issue slots, more CTAs hide more latency; which
+// wins depends on the device and on the mesh's column sizes (the shared
+// memory a CTA needs grows with them).
 //
 // With tuning on (bem_context_set_tuning), the first assembly of a shape
 // class times every candidate on a sample of the block queue (the first
@@ -14,10 +12,9 @@
 // (name, SM count), the precision, m_Q^2, the rule order, the largest column
 // sizes and the number of columns to within a factor of two. Choices are
 // kept for the process and, with a cache path, in a text file, one line per
-// class: "stbem-tune-v2 <class> <code>", code = 4 x budget variant + CTAs per
-// SM - 1 (variant 0: the 4-CTA budget, 1: the 2-CTA budget; a batch's code
-// is its CTAs per SM with the 4-CTA budget). The values do not depend on
-// the launch shape (every block is computed by one CTA alone), so tuned and
+// class: "stbem-tune-v2 <class> <code>", code = CTAs per SM - 1 (a batch's
+// code is its CTAs per SM). The values do not depend on the launch shape
+// (every potential and entry is computed by one thread alone), so tuned and
 // untuned assemblies give the same bits.
 #include <cuda_runtime.h>
 
@@ -143,41 +140,27 @@ bem_status tune_launch_shape(const bem_context* ctx, const std::string& key, con
   return BEM_OK;
 }
 
-void default_quad_shape(const bem_operator* op, int* per_sm, int* variant) {
-  const int occ0 = quad_max_per_sm(op, 0);
-  if (quad_variants(op) > 1 && occ0 <= 2) {
-    *variant = 1;
-    *per_sm = quad_max_per_sm(op, 1);
-  } else {
-    *variant = 0;
-    *per_sm = occ0;
-  }
-}
-
-// Candidates: each register-budget variant at its occupancy and the one or
-// two CTA counts below it; code = 4 variant + CTAs per SM - 1.
+// Candidates: the occupancy and the one or two CTA counts below it; code =
+// CTAs per SM - 1.
 bem_status choose_quad_shape(bem_operator* op, cudaStream_t s) {
   if (op->quad_per_sm > 0) return BEM_OK;
   if (op->ctx->tune_mode == 0 || op->opts.matrix_free) {
-    default_quad_shape(op, &op->quad_per_sm, &op->quad_variant);
+    op->quad_per_sm = quad_max_per_sm(op);
     op->quad_tuned = 0;
     return BEM_OK;
   }
   std::vector<int> codes;
-  for (int v = 0; v < quad_variants(op); ++v) {
-    const int occ = std::min(quad_max_per_sm(op, v), 4);
-    for (int per = std::max(1, occ - 2); per <= occ; ++per) codes.push_back(4 * v + per - 1);
-  }
+  const int occ = quad_max_per_sm(op);
+  for (int per = std::max(1, occ - 2); per <= occ; ++per) codes.push_back(per - 1);
   // sample: 1/32 of the dense block order, at least 16 test columns
   const int64_t nblk = op->mesh->n_col * op->mesh->n_col;
   const int64_t end = std::min(nblk, std::max(nblk / 32, 16 * op->mesh->n_col));
-  auto launch = [&](int code, int64_t e) { return quad_launch(op, code % 4 + 1, e, nullptr, nullptr, 0, s, code / 4); };
+  auto launch = [&](int code, int64_t e) { return quad_launch(op, code + 1, e, nullptr, nullptr, 0, s); };
   int best = 0;
   const bem_status st = tune_launch_shape(op->ctx, shape_class(op), codes, end, launch, s, &best, &op->quad_tuned,
                                           op->tune_ms);
   if (st != BEM_OK) return st;
-  op->quad_per_sm = best % 4 + 1;
-  op->quad_variant = best / 4;
+  op->quad_per_sm = best + 1;
   return BEM_OK;
 }
 
@@ -202,7 +185,7 @@ extern "C" bem_status bem_operator_tuning(const bem_operator* op, int* ctas_per_
     return BEM_ERR_INVALID_ARG;
   }
   if (ctas_per_sm) *ctas_per_sm = op->quad_per_sm;
-  if (budget_ctas) *budget_ctas = op->quad_variant ? 2 : STBEM_QUAD_BUDGET_CTAS;
+  if (budget_ctas) *budget_ctas = STBEM_QUAD_BUDGET_CTAS;
   if (tuned) *tuned = op->quad_tuned;
   if (sample_ms)
     for (int k = 0; k < 8; ++k) sample_ms[k] = op->tune_ms[k];

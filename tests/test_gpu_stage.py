@@ -1,0 +1,63 @@
+"""The staged quadrature and the pattern pass at the edges of their ranges:
+the smallest column, the largest (192 panels, 193 faces: U of the FP64
+operator leaves shared memory), word edges of the pattern bits, every m_Q,
+coplanar columns, and several test columns per work item of the pattern pass."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2103_16841_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2103_16841_gb300 as stb
+    return stb.Context(0)
+
+
+def _square(m):
+    """[0, 1]^2 in the plane z = 0, m x m squares of two triangles."""
+    v = np.array([[i / m, j / m, 0.0] for i in range(m + 1) for j in range(m + 1)])
+    f = []
+    for i in range(m):
+        for j in range(m):
+            a, b, c, d = i * (m + 1) + j, (i + 1) * (m + 1) + j, (i + 1) * (m + 1) + j + 1, i * (m + 1) + j + 1
+            f += [(a, b, c), (a, c, d)]
+    return v, np.array(f, dtype=np.int32)
+
+
+@pytest.mark.parametrize("surface,level,slabs,T,mq", [
+    ("sphere", 0, 1, 0.5, 3), ("sphere", 0, 64, 4.0, 3), ("sphere", 0, 21, 2.0, 4), ("sphere", 0, 11, 2.0, 1),
+    ("square", 1, 11, 2.0, 2), ("square", 10, 1, 0.3, 3)])
+def test_entries_and_pattern(ctx, surface, level, slabs, T, mq):
+    """Pattern bit-exact; FP64 entries within 1e-11 of the oracle's, relative
+    to the largest (the error of the parity tests); mixed entries within 1e-5
+    of the FP64 ones (FP32 face geometry, about 1e-6, with a margin of 10)."""
+    import paper_2103_16841_gb300 as stb
+    v, f = inputs.icosphere(level) if surface == "sphere" else _square(level)
+    m = inputs.prism_mesh(v, f, slabs, T, 0.2, seed=7)
+    om = oracle.Mesh.from_spacetime(m)
+    mesh = stb.Mesh.from_spacetime(ctx, m)
+    rng = np.random.default_rng(1)
+    rows = np.sort(rng.choice(m.n_tet, min(24, m.n_tet), replace=False)).astype(np.int32)
+    want = om.pattern_rows(rows, mq=mq)
+    ops = {p: stb.Operator(ctx, mesh, p, m_q=mq) for p in ("fp64", "mixed")}
+    for op in ops.values():
+        for a, b in zip(op.pattern_rows(rows), want):
+            assert np.array_equal(a, b)
+    ij = np.array([(r, c) for r, cols in zip(rows, want) for c in rng.choice(cols, min(40, len(cols)), replace=False)])
+    out = np.array([(r, c) for r, cols in zip(rows, want) for c in np.setdiff1d(np.arange(m.n_tet), cols)[:20]])
+    ref = om.entries(ij, mq=mq, nthreads=os.cpu_count())
+    scale = np.abs(ref).max()
+    assert np.abs(ops["fp64"].entries(ij) - ref).max() <= 1e-11 * scale
+    assert np.abs(ops["mixed"].entries(ij) - ref).max() <= 1e-5 * scale
+    for op in ops.values():
+        assert out.size == 0 or np.all(op.entries(out) == 0.0)
+        assert op.check()[0] == 0
