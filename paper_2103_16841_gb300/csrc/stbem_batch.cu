@@ -33,7 +33,6 @@ struct bem_batch {
     cudaFree(dev.d_ctx);
     cudaFree(dev.d_prefix);
     cudaFree(dev.d_counter);
-    cudaFree(dev.d_uscratch);
   }
 };
 
@@ -101,8 +100,6 @@ bem_status bem_batch_create(bem_context* ctx, int32_t n, const bem_mesh* const* 
     B_TRY(op_layout(op, bw.data(), bnnz.data(), true, false, s));
     B->nnz += op->nnz;
   }
-  B->dev.uscratch_len = quad_batch_scratch(B->ops);
-  B_TRY(balloc(&B->dev.d_uscratch, B->dev.uscratch_len));
   B_TRY(op_quadrature_batch(B->ops, B->dev, s));
   STBEM_CUDA(cudaEventRecord(e1, s));
   STBEM_CUDA(cudaEventSynchronize(e1));

@@ -307,9 +307,9 @@ __device__ __forceinline__ void bits_surfaces(const uint32_t* fb, int words, con
 // quadrature in stages (stbem_stage.cu)
 int stage_apex_per_sm(bool fp32, int max_tet, int max_surf, int nq);
 void stage_scratch(bool fp32, int max_tet, int max_surf, int sms, const std::vector<const std::vector<uint2>*>& gran,
-                   int64_t value_bytes, int64_t* least, int64_t* wanted);
+                   int64_t* least, int64_t* wanted);
 bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* prefix, int S, bool fp32, int sms,
                      const std::vector<const std::vector<uint2>*>& gran, const std::vector<int64_t>& blocks, int64_t end,
-                     void* scratch, int64_t bytes, int per_sm, cudaStream_t s);
+                     void* scratch, int64_t bytes, int per_sm, cudaStream_t side, cudaStream_t s);
 
 }  // namespace stbem

@@ -38,6 +38,16 @@ bem_status dalloc(T** p, size_t n) {
   return BEM_OK;
 }
 
+// the same, giving the context's quadrature scratch back when memory runs short
+template <typename T>
+bem_status dalloc_room(bem_context* ctx, T** p, size_t n) {
+  const bem_status st = dalloc(p, n);
+  if (st != BEM_ERR_OUT_OF_MEMORY) return st;
+  cudaGetLastError();
+  scratch_trim(ctx->scratch);
+  return dalloc(p, n);
+}
+
 template <typename T>
 struct DevBuf {
   T* p = nullptr;
@@ -78,6 +88,7 @@ bem_status bem_context_create(int device, bem_context** out) {
   std::unique_ptr<bem_context> ctx(new bem_context());
   ctx->device = device;
   STBEM_CUDA(cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking));
+  STBEM_CUDA(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   ctx->sm_count = sms;
@@ -92,6 +103,9 @@ bem_status bem_context_create(int device, bem_context** out) {
 void bem_context_destroy(bem_context* ctx) {
   if (!ctx) return;
   if (ctx->stream) cudaStreamDestroy(ctx->stream);
+  if (ctx->side) cudaStreamDestroy(ctx->side);
+  scratch_trim(ctx->scratch);
+  if (ctx->scratch.done) cudaEventDestroy(ctx->scratch.done);
   delete ctx;
 }
 
@@ -375,32 +389,29 @@ bem_status stbem::op_layout(bem_operator* op, const int32_t* bw, const int64_t* 
     op->nstored = vo; op->nrows_stored = ro; op->nnz = nnz; op->nblocks = nblk;
     op->max_bw = wmax;
     if (own_scratch) {
-      int64_t least = 0;
-      quad_scratch(op, &least, &op->tmp_len);
-      // what an admission reserves for it: U of up to four CTAs per SM
+      // what an admission reserves for the quadrature's scratch: U of up to four CTAs per SM
       const int64_t smem = 44000 + 152 * m->max_col_tets + 312 * m->max_col_surf;
       const int64_t per = std::max<int64_t>(1, std::min<int64_t>(4, 232448 / smem));
-      op->reserve_len = std::max<int64_t>((int64_t)op->ctx->sm_count * per * m->max_col_surf * m->max_col_tets,
-                                          16 * m->n_tet);
-      if (op->scratch_cap >= 0) op->tmp_len = std::max(least, std::min(op->tmp_len, op->reserve_len + op->scratch_cap / 8));
-    } else {
-      op->tmp_len = op->reserve_len = 0;
+      op->reserve_bytes = 8 * std::max<int64_t>((int64_t)op->ctx->sm_count * per * m->max_col_surf * m->max_col_tets,
+                                                16 * m->n_tet);
     }
     if (op->opts.matrix_free) op->nstored = 0;
     if (op->admit) TRY(op->admit(op));
     if (!op->opts.matrix_free) {
       // mixed-precision values carry FP32 accuracy: FP32 storage only
-      if (op->opts.precision == BEM_PREC_FP64) TRY(dalloc(&op->d_val, (size_t)vo));
+      if (op->opts.precision == BEM_PREC_FP64) TRY(dalloc_room(op->ctx, &op->d_val, (size_t)vo));
       // (8 floats of tail room: the tensor-core product copies whole 16-byte granules)
-      if (op->opts.store_fp32 || op->opts.precision == BEM_PREC_MIXED) TRY(dalloc(&op->d_val32, (size_t)vo + 8));
+      if (op->opts.store_fp32 || op->opts.precision == BEM_PREC_MIXED)
+        TRY(dalloc_room(op->ctx, &op->d_val32, (size_t)vo + 8));
       TRY(dalloc(&op->d_rs, (size_t)ro + 4));   // (tail room as for the values)
     }
-    if (own_scratch && op->scratch_cap < 0) TRY(dalloc(&op->d_tmp, (size_t)op->tmp_len));
-    if (own_scratch && op->scratch_cap >= 0 && cudaMallocAsync((void**)&op->d_tmp, sizeof(double) * op->tmp_len, s) != cudaSuccess) {
-      cudaGetLastError();
-      op->d_tmp = nullptr;
-      set_error("out of device memory (quadrature scratch)");
-      return BEM_ERR_OUT_OF_MEMORY;
+    if (own_scratch && op->opts.matrix_free) {
+      int64_t least = 0, wanted = 0;
+      quad_scratch(op, &least, &wanted);
+      op->tmp_bytes = std::max(least, std::min(wanted, std::max<int64_t>(4 * vo, (int64_t)64 << 20)));
+      unsigned char* p = nullptr;
+      TRY(dalloc(&p, (size_t)op->tmp_bytes));
+      op->d_tmp = p;
     }
   } else if ((!op->opts.matrix_free && vo != op->nstored) || nnz != op->nnz) {
     set_error("reassembly changed the sparsity structure");
@@ -499,12 +510,7 @@ int64_t stbem::operator_value_bytes(const bem_operator* op) {
   int64_t b = 0;
   if (op->opts.precision == BEM_PREC_FP64) b += 8 * op->nstored;
   if (op->opts.store_fp32 || op->opts.precision == BEM_PREC_MIXED) b += 4 * op->nstored;
-  return b + 4 * op->nrows_stored + 8 * op->reserve_len;
-}
-
-void stbem::operator_release_scratch(bem_operator* op, cudaStream_t s) {
-  if (op->d_tmp) cudaFreeAsync(op->d_tmp, s);
-  op->d_tmp = nullptr;
+  return b + 4 * op->nrows_stored + op->reserve_bytes;
 }
 
 extern "C" {

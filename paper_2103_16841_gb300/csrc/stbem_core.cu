@@ -421,29 +421,93 @@ int quad_max_per_sm(const bem_operator* op) {
 }
 
 void quad_scratch(const bem_operator* op, int64_t* least, int64_t* wanted) {
-  int64_t a = 0, b = 0;
-  const bool fp32 = op->opts.precision == BEM_PREC_MIXED;
-  stage_scratch(fp32, op->mesh->max_col_tets, op->mesh->max_col_surf, (int)op->ctx->sm_count, {&op->h_gran},
-                op->nstored * (fp32 ? 4 : 8), &a, &b);
-  *least = (a + 7) / 8;
-  *wanted = (b + 7) / 8;
+  stage_scratch(op->opts.precision == BEM_PREC_MIXED, op->mesh->max_col_tets, op->mesh->max_col_surf,
+                (int)op->ctx->sm_count, {&op->h_gran}, least, wanted);
 }
 
 bem_status quad_launch(const bem_operator* op, int per_sm, int64_t end, const double* mf_x, double* mf_y, int nrhs,
-                       cudaStream_t s) {
+                       void* scratch, int64_t bytes, cudaStream_t s) {
   BlockCtx B = make_ctx(op);
   const int64_t nb = op->mesh->n_col * op->mesh->n_col;
   B.mf_x = mf_x;
   B.mf_y = mf_y;
   B.mf_nrhs = nrhs;
   return stage_run(B, nullptr, nullptr, 1, op->opts.precision == BEM_PREC_MIXED, (int)op->ctx->sm_count,
-                   {&op->h_gran}, {nb}, std::min(end, nb), op->d_tmp, op->tmp_len * 8, per_sm, s);
+                   {&op->h_gran}, {nb}, std::min(end, nb), scratch, bytes, per_sm, op->ctx->side, s);
+}
+
+bem_status ScratchHold::take(Scratch& c, bool own, int64_t least, int64_t wanted, cudaStream_t stream) {
+  s = stream;
+  if (!own) {
+    std::lock_guard<std::mutex> lk(c.mu);
+    if (!c.busy) {
+      if (c.bytes < wanted) {
+        cudaFree(c.p);   // (waits for the work on it)
+        c.p = nullptr;
+        c.bytes = 0;
+        if (cudaMalloc(&c.p, wanted) == cudaSuccess) {
+          c.bytes = wanted;
+        } else {
+          cudaGetLastError();
+          c.p = nullptr;
+        }
+      }
+      if (!c.done && cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        c.done = nullptr;
+      }
+      if (c.p && c.done) {
+        STBEM_CUDA(cudaStreamWaitEvent(s, c.done, 0));
+        c.busy = true;
+        from = &c;
+        p = c.p;
+        bytes = c.bytes;
+        return BEM_OK;
+      }
+    }
+  }
+  for (int64_t n = wanted;; n = std::max(least, n / 4)) {
+    if (cudaMallocAsync(&p, n, s) == cudaSuccess) {
+      bytes = n;
+      return BEM_OK;
+    }
+    cudaGetLastError();
+    p = nullptr;
+    if (n <= least) break;
+  }
+  set_error("out of device memory (quadrature scratch)");
+  return BEM_ERR_OUT_OF_MEMORY;
+}
+
+ScratchHold::~ScratchHold() {
+  if (from) {
+    std::lock_guard<std::mutex> lk(from->mu);
+    cudaEventRecord(from->done, s);
+    from->busy = false;
+  } else if (p) {
+    cudaFreeAsync(p, s);
+  }
+}
+
+void scratch_trim(Scratch& c) {
+  std::lock_guard<std::mutex> lk(c.mu);
+  if (c.busy) return;
+  cudaFree(c.p);
+  c.p = nullptr;
+  c.bytes = 0;
 }
 
 bem_status op_quadrature(bem_operator* op, cudaStream_t s) {
-  bem_status st = choose_quad_shape(op, s);
+  int64_t least = 0, wanted = 0;
+  quad_scratch(op, &least, &wanted);
+  const bool capped = op->scratch_cap >= 0;
+  if (capped) wanted = std::max(least, std::min(wanted, op->reserve_bytes + op->scratch_cap));
+  ScratchHold h;
+  bem_status st = h.take(op->ctx->scratch, capped, least, wanted, s);
   if (st != BEM_OK) return st;
-  return quad_launch(op, op->quad_per_sm, op->mesh->n_col * op->mesh->n_col, nullptr, nullptr, 0, s);
+  st = choose_quad_shape(op, h.p, h.bytes, s);
+  if (st != BEM_OK) return st;
+  return quad_launch(op, op->quad_per_sm, op->mesh->n_col * op->mesh->n_col, nullptr, nullptr, 0, h.p, h.bytes, s);
 }
 
 // Matrix-free product y = A x (internal order, [nrhs][n_tet]): the quadrature
@@ -451,7 +515,7 @@ bem_status op_quadrature(bem_operator* op, cudaStream_t s) {
 bem_status op_matvec_free(const bem_operator* op, const double* x, double* y, int nrhs, cudaStream_t s) {
   STBEM_CUDA(cudaMemsetAsync(y, 0, sizeof(double) * op->mesh->n_tet * nrhs, s));
   const int per_sm = op->quad_per_sm > 0 ? op->quad_per_sm : quad_max_per_sm(op);
-  return quad_launch(op, per_sm, op->mesh->n_col * op->mesh->n_col, x, y, nrhs, s);
+  return quad_launch(op, per_sm, op->mesh->n_col * op->mesh->n_col, x, y, nrhs, op->d_tmp, op->tmp_bytes, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -522,20 +586,6 @@ static void batch_grans(const std::vector<bem_operator*>& ops, std::vector<const
   }
 }
 
-int64_t quad_batch_scratch(const std::vector<bem_operator*>& ops) {
-  if (ops.empty()) return 0;
-  int mt, ms;
-  batch_dims(ops, mt, ms);
-  std::vector<const std::vector<uint2>*> gran;
-  std::vector<int64_t> blocks;
-  batch_grans(ops, gran, blocks);
-  const bool fp32 = ops[0]->opts.precision == BEM_PREC_MIXED;
-  int64_t values = 0, least = 0, wanted = 0;
-  for (const bem_operator* op : ops) values += op->nstored * (fp32 ? 4 : 8);
-  stage_scratch(fp32, mt, ms, (int)ops[0]->ctx->sm_count, gran, values, &least, &wanted);
-  return (wanted + 7) / 8;
-}
-
 bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& dev, cudaStream_t s) {
   if (ops.empty()) return BEM_OK;
   for (const bem_operator* op : ops)
@@ -543,10 +593,6 @@ bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& 
       set_error("a batch takes one precision, m_Q and n_theta");
       return BEM_ERR_INVALID_ARG;
     }
-  if (dev.uscratch_len < quad_batch_scratch(ops)) {
-    set_error("batch quadrature scratch too small");
-    return BEM_ERR_INTERNAL;
-  }
   int mt, ms;
   batch_dims(ops, mt, ms);
   int64_t total = 0;
@@ -559,9 +605,14 @@ bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& 
   std::vector<const std::vector<uint2>*> gran;
   std::vector<int64_t> blocks;
   batch_grans(ops, gran, blocks);
+  int64_t least = 0, wanted = 0;
+  stage_scratch(fp32, mt, ms, sms, gran, &least, &wanted);
+  ScratchHold h;
+  st = h.take(ops[0]->ctx->scratch, false, least, wanted, s);
+  if (st != BEM_OK) return st;
   auto launch = [&](int per, int64_t end) {
     return stage_run(first, static_cast<const BlockCtx*>(dev.d_ctx), dev.d_prefix, (int)ops.size(), fp32, sms, gran,
-                     blocks, end, dev.d_uscratch, dev.uscratch_len * 8, per, s);
+                     blocks, end, h.p, h.bytes, per, ops[0]->ctx->side, s);
   };
   int per = occ, how = 0;
   if (ops[0]->ctx->tune_mode) {

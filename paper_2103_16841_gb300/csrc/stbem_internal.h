@@ -6,6 +6,7 @@
 #include <atomic>
 #include <functional>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -49,9 +50,38 @@ struct SurfDev {
 
 }  // namespace stbem
 
+namespace stbem {
+// Quadrature scratch of a context, kept from one assembly to the next (at most
+// the largest that one wanted, 1 GiB) and given back when the context goes or
+// device memory runs short. One assembly holds it at a time; another one that
+// runs beside it (other threads) gets a block of its own, stream-ordered.
+struct Scratch {
+  std::mutex mu;
+  void* p = nullptr;
+  int64_t bytes = 0;
+  bool busy = false;
+  cudaEvent_t done = nullptr;   // the last assembly's work on it
+};
+struct ScratchHold {
+  Scratch* from = nullptr;      // null: a block of its own
+  void* p = nullptr;
+  int64_t bytes = 0;
+  cudaStream_t s = nullptr;
+  ScratchHold() = default;
+  ScratchHold(const ScratchHold&) = delete;
+  ScratchHold& operator=(const ScratchHold&) = delete;
+  // least <= bytes <= wanted; own: never the context's
+  bem_status take(Scratch& c, bool own, int64_t least, int64_t wanted, cudaStream_t stream);
+  ~ScratchHold();
+};
+void scratch_trim(Scratch& c);  // frees it unless an assembly holds it
+}  // namespace stbem
+
 struct bem_context {
   int device = 0;
   cudaStream_t stream = nullptr;
+  cudaStream_t side = nullptr;  // the quadrature's second stream
+  stbem::Scratch scratch;       // of the assemblies on this context
   double sm_count = 0;
   int tune_mode = 0;          // 1: launch shapes timed per shape class (bem_context_set_tuning)
   std::string tune_path;      // text cache of the tuned shapes ("" = process only)
@@ -106,10 +136,10 @@ struct bem_operator {
   double tune_ms[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // sample time per candidate: index = CTAs per SM - 1
   unsigned long long* d_counter = nullptr;  // work counter of the persistent kernels
   // quadrature scratch
-  double* d_tmp = nullptr;
-  int64_t tmp_len = 0;
-  int64_t reserve_len = 0;       // doubles an admission reserves for the scratch
-  int64_t scratch_cap = -1;      // >= 0: bytes the scratch may take beyond that, allocated stream-ordered
+  void* d_tmp = nullptr;         // matrix-free operators only: their products' scratch
+  int64_t tmp_bytes = 0;
+  int64_t reserve_bytes = 0;     // bytes an admission reserves for the scratch
+  int64_t scratch_cap = -1;      // >= 0: bytes the scratch may take beyond that (a server's slot), not the context's
   // made on first use by the products (an operator is used by one host thread at a time)
   mutable float* d_ws = nullptr;        // packed operands of the FP32 / tensor-core products
   mutable int64_t ws_len = 0;
@@ -125,7 +155,7 @@ struct bem_operator {
   mutable bool tcv_stale[2] = {false, false};   // the values were reassembled since the slots were made
   mutable int* d_tc_err = nullptr;         // set when a tensor-core product gave up on a wait
   // optional admission hook, called once the sparsity structure is known
-  // (nstored, nrows_stored, tmp_len set) and before the value arrays are allocated
+  // (nstored, nrows_stored, reserve_bytes set) and before the value arrays are allocated
   std::function<bem_status(const bem_operator*)> admit;
 };
 
@@ -141,14 +171,14 @@ bem_status op_quadrature(bem_operator* op, cudaStream_t s);
 bem_status upload_gauss_stage(const double* x, const double* w, const float* xf, const float* wf, size_t n);
 // most CTAs per SM of the quadrature's persistent stage (at most 4)
 int quad_max_per_sm(const bem_operator* op);
-// least and wanted length of an operator's quadrature scratch, in doubles
+// least and wanted bytes of an operator's quadrature scratch
 void quad_scratch(const bem_operator* op, int64_t* least, int64_t* wanted);
 // the quadrature over the blocks [0, end) of the dense (I, J) order, its
 // persistent stage with per_sm CTAs per SM (assembled, or summed against mf_x)
 bem_status quad_launch(const bem_operator* op, int per_sm, int64_t end, const double* mf_x, double* mf_y, int nrhs,
-                       cudaStream_t s);
+                       void* scratch, int64_t bytes, cudaStream_t s);
 // sets op->quad_per_sm: the context's tuning cache, a timed choice, or the default (stbem_tune.cu)
-bem_status choose_quad_shape(bem_operator* op, cudaStream_t s);
+bem_status choose_quad_shape(bem_operator* op, void* scratch, int64_t bytes, cudaStream_t s);
 // the tuner behind it: the fastest of the candidate launch codes of launch(code, end)
 // over a sample [0, end) of a block queue (the code's meaning is the caller's)
 bem_status tune_launch_shape(const bem_context* ctx, const std::string& key, const std::vector<int>& codes,
@@ -205,8 +235,6 @@ bem_status gmres_solve_layout(const SegLayout& L, const MatvecFn& mv_hi, const M
 bem_status operator_create(bem_context* ctx, const bem_mesh* mesh, const bem_op_opts* opts,
                            std::function<bem_status(const bem_operator*)> admit, bem_operator** out,
                            int64_t scratch_cap = -1);
-// gives the quadrature scratch of an operator created with a scratch_cap back (stream-ordered)
-void operator_release_scratch(bem_operator* op, cudaStream_t s);
 // operator object with its structure arrays allocated (nothing assembled yet)
 bem_status op_structure_alloc(bem_context* ctx, const bem_mesh* mesh, const bem_op_opts* opts,
                               std::unique_ptr<bem_operator>& op);
@@ -215,19 +243,15 @@ bem_status op_structure_alloc(bem_context* ctx, const bem_mesh* mesh, const bem_
 // (and the quadrature scratch when own_scratch)
 bem_status op_layout(bem_operator* op, const int32_t* bw, const int64_t* bnnz, bool first, bool own_scratch,
                      cudaStream_t s);
-// batched pattern and quadrature passes over several operators; the operators
-// share `uscratch` for the quadrature
+// batched pattern and quadrature passes over several operators
 struct BatchDev {
   void* d_ctx = nullptr;                 // BlockCtx[S]
   int64_t* d_prefix = nullptr;           // [S+1] block prefix
   unsigned long long* d_counter = nullptr;
-  double* d_uscratch = nullptr;
-  int64_t uscratch_len = 0;
 };
 bem_status op_outer_points_all(const std::vector<bem_operator*>& ops, cudaStream_t s);
 bem_status op_pattern_batch(const std::vector<bem_operator*>& ops, BatchDev& dev, cudaStream_t s);
 bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& dev, cudaStream_t s);
-int64_t quad_batch_scratch(const std::vector<bem_operator*>& ops);
 size_t block_ctx_size();
 // bytes held by an operator's value arrays, row starts and quadrature scratch
 int64_t operator_value_bytes(const bem_operator* op);

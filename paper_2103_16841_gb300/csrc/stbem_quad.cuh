@@ -186,6 +186,34 @@ struct ColR {            // edge data of a column in precision R
 STBEM_HD inline void sc(float x, float* s, float* c) { sincosf(x, s, c); }
 STBEM_HD inline void sc(double x, double* s, double* c) { sincos(x, s, c); }
 
+// sine and cosine for |x| <= pi / 2: in FP64 the Taylor polynomials at x / 2
+// (|x / 2|^17 / 17! < 5e-17) and the double-angle formulas, without the
+// general function's argument reduction (FP64 instructions are what a node
+// of a conic arc costs)
+STBEM_HD inline void sc_quarter(float x, float* s, float* c) { sincosf(x, s, c); }
+STBEM_HD inline void sc_quarter(double x, double* s, double* c) {
+  const double h = 0.5 * x, z = h * h;
+  double p = -1.0 / 1307674368000.0;
+  p = p * z + 1.0 / 6227020800.0;
+  p = p * z - 1.0 / 39916800.0;
+  p = p * z + 1.0 / 362880.0;
+  p = p * z - 1.0 / 5040.0;
+  p = p * z + 1.0 / 120.0;
+  p = p * z - 1.0 / 6.0;
+  const double sh = h + h * z * p;
+  double q = 1.0 / 20922789888000.0;
+  q = q * z - 1.0 / 87178291200.0;
+  q = q * z + 1.0 / 479001600.0;
+  q = q * z - 1.0 / 3628800.0;
+  q = q * z + 1.0 / 40320.0;
+  q = q * z - 1.0 / 720.0;
+  q = q * z + 1.0 / 24.0;
+  q = q * z - 0.5;
+  const double ch = 1.0 + z * q;
+  *s = 2.0 * sh * ch;
+  *c = 1.0 - 2.0 * sh * sh;
+}
+
 struct ArcRule {
   int nmin, nmax;    // Gauss node bounds per piece
   double tol;        // target relative accuracy of a piece
@@ -254,7 +282,15 @@ STBEM_HD inline R edge_dE(R wa, R dw, R p_s, R d) {
   else dasinh = asinh((wb * ra - wa * rb) / A2);
   R val = p_s * dasinh;
   if (p > R(0) && ad > R(0)) {
-    R dt = edge_T<R>(wb, rb, p, ad) - edge_T<R>(wa, ra, p, ad);
+    R dt;
+    if (sizeof(R) == 8) {
+      // the difference of the two atans by one atan2 of the tangents' subtraction, without their divisions
+      const R na = wa * p * (p * p + wa * wa), da = (ra + ad) * (p * p * ra + wa * wa * ad);
+      const R nb = wb * p * (p * p + wb * wb), db = (rb + ad) * (p * p * rb + wb * wb * ad);
+      dt = atan2(nb * da - na * db, da * db + na * nb);
+    } else {
+      dt = edge_T<R>(wb, rb, p, ad) - edge_T<R>(wa, ra, p, ad);
+    }
     val -= (p_s > R(0) ? ad : -ad) * dt;
   }
   return val;
@@ -436,7 +472,8 @@ STBEM_HD inline float edge_full_mixed(const PtR<float>& T, const ColR<float>& CR
 // fully lit case). FP64 path: everything in FP64. Mixed path: the relative
 // position, the height d, the foot point and the corner distances in FP64
 // (they carry the cancellation between |x - y| and t - tau), the rest in FP32.
-STBEM_HD inline void point_col(const double* x, const ColGeom& G, PointCol& P, bool prec_fp32) {
+// (edges = false, FP64 only: without the whole-edge integrals and Wst)
+STBEM_HD inline void point_col(const double* x, const ColGeom& G, PointCol& P, bool prec_fp32, bool edges = true) {
   P.t = x[0];
   double rel[3] = {x[1] - G.c0[0], x[2] - G.c0[1], x[3] - G.c0[2]};
   double d = rel[0] * G.n[0] + rel[1] * G.n[1] + rel[2] * G.n[2];
@@ -505,7 +542,7 @@ STBEM_HD inline void point_col(const double* x, const ColGeom& G, PointCol& P, b
     D.ws[k] = D.q[k][0] * G.U[k][0] + D.q[k][1] * G.U[k][1];
     if (!(D.ps[k] > 0.0)) in = 0;
     out = fmax(out, -D.ps[k]);
-    D.Efull[k] = edge_dE<double>(D.ws[k], G.L[k], D.ps[k], d);
+    D.Efull[k] = edges ? edge_dE<double>(D.ws[k], G.L[k], D.ps[k], d) : 0.0;
     W += D.Efull[k];
   }
   P.inK = in;
@@ -601,9 +638,10 @@ struct ArcEval {
   R wh[3], ea[3], eb[3];
   R c, d, g0, g1;
   bool use_c;
+  // th: from the middle of a piece of at most half a turn
   STBEM_HD inline R operator()(R th) const {
     R s, co;
-    sc(th, &s, &co);
+    sc_quarter(th, &s, &co);
     R n0 = ca * wh[0] + sa * (co * ea[0] + s * eb[0]);
     R n1 = ca * wh[1] + sa * (co * ea[1] + s * eb[1]);
     R n2 = ca * wh[2] + sa * (co * ea[2] + s * eb[2]);
@@ -643,6 +681,15 @@ STBEM_HD inline void consider_pole(R A0, R Aa, R Ab, R mid, R half, R& best_rho,
     pole_at<R>(th1 + ac, R(0), mid, half, best_rho, best_a, best_b);
     pole_at<R>(th1 - ac, R(0), mid, half, best_rho, best_a, best_b);
   }
+}
+
+// sinh and cosh of the map's nodes; in FP64 both from one expm1 (a node's
+// largest cost on the FP64 pipe)
+STBEM_HD inline void sinh_cosh(float v, float& sh, float& ch) { sh = sinh(v); ch = cosh(v); }
+STBEM_HD inline void sinh_cosh(double v, double& sh, double& ch) {
+  const double t = expm1(v), e = t + 1.0, i = 1.0 / e;
+  sh = 0.5 * (t + t * i);
+  ch = 0.5 * (e + i);
 }
 
 // int_lo^hi I(theta) dtheta. The integrand is a rational trigonometric
@@ -708,8 +755,9 @@ STBEM_HD __noinline__ R arc_piece(const ArcFrame<R>& F, R lo, R hi, const ArcRul
     R mu = R(0.5) * (s1 + s2), et = R(0.5) * (s1 - s2);
     for (int k = 0; k < n; ++k) {
       R v = mu * (R)X[k] - et;
-      R u = a + b * sinh(v);
-      acc += (R)Wt[k] * b * mu * cosh(v) * E(half * u);
+      R sh, ch;
+      sinh_cosh(v, sh, ch);
+      acc += (R)Wt[k] * b * mu * ch * E(half * (a + b * sh));
     }
   } else {
     int n = rule.nmin;
@@ -1029,7 +1077,8 @@ STBEM_HD inline R arc_value(const ArcRec<R>& a, const ArcRule& rule) {
 // 4 pi W_P(x) of a cut face. With `defer` given, arcs with d != 0 (at most
 // three) are appended to defer[*ndefer] instead of integrated, and the
 // return value holds the edge pieces (and any coplanar arc) only.
-template <typename R>
+// LAZY: the whole-edge integrals P.Efull were not formed; a fully lit edge is integrated here.
+template <typename R, bool LAZY = false>
 STBEM_HD __noinline__ double face_cut(const ColR<R>& G, const PtR<R>& P, const FaceCutIn<R>& in,
                                       const ArcRule& rule, ArcRec<R>* defer = nullptr, int* ndefer = nullptr) {
   const R d = P.d, c = in.c;
@@ -1083,8 +1132,8 @@ STBEM_HD __noinline__ double face_cut(const ColR<R>& G, const PtR<R>& P, const F
       }
     }
     if (!has) continue;
-    if (!la_root && !lb_root) total += P.Efull[k];
-    else if (P.far) total += edge_far<R>(P, G, k, la, lb, rule);
+    if (!LAZY && !la_root && !lb_root) total += P.Efull[k];
+    else if (!LAZY && P.far) total += edge_far<R>(P, G, k, la, lb, rule);
     else total += edge_int<R>(P.ws[k] + la * G.L[k], (lb - la) * G.L[k], P.ps[k], d, rule);
     // events relative to xb (O(distance)) and in column coordinates (O(diam K));
     // differences of the latter give arc spans without cancellation
@@ -1240,13 +1289,25 @@ STBEM_HD inline double face_W(const ColGeom& G, const PointCol& P, const FaceGeo
 // operator's 1e-15 rule needs.
 STBEM_HD __noinline__ inline double face_W_fp64(const double* x, const ColGeom& G, const FaceGeom& Fc, int n_theta) {
   PointCol P;
-  point_col(x, G, P, false);
+  point_col(x, G, P, false, false);
   ArcRule r;
   r.nmin = 4;
   r.nmax = n_theta ? n_theta : 32;   // pieces next to a pole (sinh map) take nmax
   r.tol = 1e-10;
   rule_finish(r);
-  return face_W<false>(G, P, Fc, r);
+  double F[3], c = 0.0;
+  const int cls = face_class(G, P, Fc, F, c);
+  if (cls == FACE_DARK) return 0.0;
+  if (cls == FACE_LIT) {
+    double W = 0.0;
+    for (int k = 0; k < 3; ++k) W += edge_dE<double>(P.D.ws[k], G.L[k], P.D.ps[k], P.D.d);
+    return W;
+  }
+  ColR<double> CR;
+  make_colr<double>(G, CR);
+  FaceCutIn<double> in;
+  cut_in_fp64(P, Fc, F, c, in);
+  return face_cut<double, true>(CR, P.D, in, r);
 }
 
 }  // namespace stbem

@@ -334,7 +334,6 @@ bem_status run_job(bem_server* S, bem_context* cx, const Job& J, Done& D, int64_
     return st;
   }
   std::unique_ptr<bem_operator, void (*)(bem_operator*)> op_guard(op, bem_operator_destroy);
-  operator_release_scratch(op, s);   // the slot's share is the next request's
   st = solve_job(S, s, op, J, D);
   if (!caching || (st != BEM_OK && st != BEM_ERR_NOT_CONVERGED)) {
     release(S, reserved, 0);

@@ -70,7 +70,7 @@ template <typename R> struct Types;
 template <> struct Types<float> { typedef ApexF Apex; typedef FaceF Face; };
 template <> struct Types<double> { typedef ApexD Apex; typedef FaceGeom Face; };
 
-enum { CNT_APEX, CNT_ASM, CNT_SLOT, CNT_RAY, CNT_FAR, CNT_ANY, CNT_F64, CNT_N };
+enum { CNT_APEX, CNT_ASM, CNT_SLOT, CNT_RAY, CNT_FAR, CNT_ANY, CNT_COP, CNT_F64, CNT_N };
 
 struct StageArgs {
   BlockCtx one;                  // the operator (S <= 1), or the sizes all operators of a batch share
@@ -80,7 +80,8 @@ struct StageArgs {
   int64_t g0, g1;                // blocks of the chunk (dense order, operators one after the other)
   void* apex;
   void* W;                       // potentials; a queued one holds its apex's index until it is computed
-  uint32_t *q_far, *q_any, *q_64;
+  uint32_t *q_far, *q_any;
+  uint32_t *q_64, *q_64_last;    // FP64 faces: coplanar apexes from the front, the others from the back
   uint2* fmeta;                  // per block and face: first potential, window (first face | faces << 16)
   uint32_t* bits;                // per block and face
   unsigned* cnt;
@@ -91,6 +92,10 @@ struct StageArgs {
 constexpr int kApexThreads = 256;   // >= MAX_COL_SURF: one thread per face in the window scan
 static_assert(kApexThreads >= MAX_COL_SURF, "one thread per face");
 constexpr int kCutThreads = 128;
+constexpr int k64Threads = 128;     // (a warp per CTA: level-3 sphere, 8 slabs 239 ms, four warps 214)
+// scratch of an assembly: 256 MiB / 512 MiB / 1 GiB / 2 GiB gave 308 / 238 / 239 / 236 ms
+// on the level-3 sphere with 8 slabs, 52 / 49 / 45 / 43 ms on the level-2 sphere with 15
+constexpr size_t kScratch = (size_t)1 << 30;
 constexpr int kAsmThreads = 128;
 
 // exclusive sum over the CTA (kApexThreads threads); *total = the sum
@@ -116,14 +121,14 @@ __device__ __forceinline__ unsigned cta_scan(unsigned v, unsigned* s_w, unsigned
   return off + inc - v;
 }
 
-// appends v to a queue; the active lanes take their places with one atomic
-__device__ __forceinline__ void push(uint32_t* q, unsigned* n, uint32_t v) {
+// appends v to a queue (dir: upwards or downwards); the active lanes take their places with one atomic
+__device__ __forceinline__ void push(uint32_t* q, int dir, unsigned* n, uint32_t v) {
   const unsigned m = __activemask(), lane = threadIdx.x & 31;
   const int leader = __ffs(m) - 1;
   unsigned base = 0;
   if ((int)lane == leader) base = atomicAdd(n, (unsigned)__popc(m));
   base = __shfl_sync(m, base, leader);
-  q[base + __popc(m & ((1u << lane) - 1u))] = v;
+  q[dir * (int)(base + __popc(m & ((1u << lane) - 1u)))] = v;
 }
 
 // ---- geometry of an apex against the trial column ----------------------
@@ -402,8 +407,10 @@ __device__ __forceinline__ bool load_cut(const StageArgs& a, uint32_t slot, uint
 
 // FAR: the pairs of apexes in the far field; arcs the chord form refuses go
 // on to the other queue. A value that is not finite is recomputed in FP64.
+// Bound by issue and the latency of the gathers; 80 registers (6 CTAs per SM):
+// level-3 sphere, 8 slabs 211 ms of quadrature against 239 ms with 4 CTAs.
 template <bool FAR>
-__global__ void __launch_bounds__(kCutThreads) k_cut(const StageArgs a) {
+__global__ void __launch_bounds__(kCutThreads, 6) k_cut(const StageArgs a) {
   float* W = static_cast<float*>(a.W);
   const uint32_t* q = FAR ? a.q_far : a.q_any;
   const unsigned n = a.cnt[FAR ? CNT_FAR : CNT_ANY];
@@ -411,7 +418,8 @@ __global__ void __launch_bounds__(kCutThreads) k_cut(const StageArgs a) {
     const uint32_t slot = q[i];
     CutF c;
     if (!load_cut(a, slot, __float_as_uint(W[slot]), c)) {
-      push(a.q_64, &a.cnt[CNT_F64], slot);
+      if (c.T.d == 0.f) push(a.q_64, 1, &a.cnt[CNT_COP], slot);
+      else push(a.q_64_last, -1, &a.cnt[CNT_F64], slot);
       continue;
     }
     ArcRec<float> arc[3];
@@ -428,17 +436,22 @@ __global__ void __launch_bounds__(kCutThreads) k_cut(const StageArgs a) {
         v += arc_value<float>(arc[k], a.one.rule);
       }
     }
-    if (!ok) push(a.q_any, &a.cnt[CNT_ANY], slot);
-    else if (!isfinite(v)) push(a.q_64, &a.cnt[CNT_F64], slot);
+    if (!ok) push(a.q_any, 1, &a.cnt[CNT_ANY], slot);
+    else if (!isfinite(v)) push(a.q_64_last, -1, &a.cnt[CNT_F64], slot);
     else W[slot] = v;
   }
 }
 
-__global__ void __launch_bounds__(kCutThreads) k_cut_fp64(const StageArgs a) {
+// Bound by the FP64 pipe (a warp instruction takes it for 19 cycles) and, where
+// a chunk has few, by their serial chain. Coplanar apexes (closed form, about
+// a fifth of the work of the others' mapped Gauss nodes) have warps of their
+// own.
+__global__ void __launch_bounds__(k64Threads) k_cut_fp64(const StageArgs a) {
   float* W = static_cast<float*>(a.W);
-  const unsigned n = a.cnt[CNT_F64];
+  const unsigned n1 = a.cnt[CNT_F64], n1w = (n1 + 31) / 32 * 32, n = n1w + a.cnt[CNT_COP];
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const uint32_t slot = a.q_64[i];
+    if (i >= n1 && i < n1w) continue;
+    const uint32_t slot = i < n1 ? *(a.q_64_last - i) : a.q_64[i - n1w];
     const ApexF& Y = static_cast<const ApexF*>(a.apex)[__float_as_uint(W[slot])];
     const BlockCtx& B = a.S > 1 ? a.many[Y.seg] : a.one;
     W[slot] = (float)face_W_fp64(B.pts + 4 * (int64_t)Y.pt, B.cols[Y.col],
@@ -647,10 +660,10 @@ int stage_apex_per_sm(bool fp32, int max_tet, int max_surf, int nq) {
   return std::min(occupancy(kern, kApexThreads, smem), 4);
 }
 
-// Scratch of a quadrature over the blocks counted in `gran`: at most kScratch
-// bytes (a chunk), at least the largest run of GRAN blocks.
+// Scratch of a quadrature over the blocks counted in `gran`: at least the
+// largest run of GRAN blocks, at most kScratch bytes.
 void stage_scratch(bool fp32, int max_tet, int max_surf, int sms, const std::vector<const std::vector<uint2>*>& gran,
-                   int64_t value_bytes, int64_t* least, int64_t* wanted) {
+                   int64_t* least, int64_t* wanted) {
   size_t big = 0, all = 0;
   for (const auto* v : gran)
     for (const uint2& c : *v) {
@@ -659,25 +672,39 @@ void stage_scratch(bool fp32, int max_tet, int max_surf, int sms, const std::vec
       all += n;
     }
   const size_t fixed = fixed_bytes(fp32, max_tet, max_surf, sms);
-  const size_t cap = std::min<size_t>(std::max<size_t>(value_bytes / 2, (size_t)64 << 20), (size_t)1 << 30);
-  *least = (int64_t)(fixed + big);
-  *wanted = (int64_t)(fixed + std::max(big, std::min(all, cap)));
+  *least = (int64_t)up256(fixed + big);
+  *wanted = (int64_t)up256(std::max(fixed + big, std::min(2 * fixed + all, kScratch)));
 }
 
-// All stages over the blocks [0, end) of the concatenated operators.
+// All stages over the blocks [0, end) of the concatenated operators. The
+// chunks alternate between two halves of the scratch: the FP64 faces (some
+// thousand per chunk, each a serial chain of most of a millisecond) and the
+// entries of one chunk run on the context's side stream while the caller's
+// stream takes the next chunk's apexes and FP32 faces. Large chunks pay: each
+// kernel of a chunk costs about 10 us of ramp and tail.Level-2
+// sphere, 15 slabs: 94 ms one chunk after the other, 45 ms so; level-3 sphere,
+// 8 slabs: 263 and 214 ms.
 bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* prefix, int S, bool fp32, int sms,
                      const std::vector<const std::vector<uint2>*>& gran, const std::vector<int64_t>& blocks, int64_t end,
-                     void* scratch, int64_t bytes, int per_sm, cudaStream_t s) {
+                     void* scratch, int64_t bytes, int per_sm, cudaStream_t side, cudaStream_t s) {
   const int mt = one.max_tet, ms = one.max_surf, nq = one.nq;
   const size_t fixed = fixed_bytes(fp32, mt, ms, sms);
   unsigned char* base = static_cast<unsigned char*>(scratch);
+  // two halves where the scratch holds the largest run of blocks twice
+  size_t least = 0, all = 0;
+  for (const auto* v : gran)
+    for (const uint2& c : *v) {
+      const size_t n = chunk_bytes(fp32, mt, ms, GRAN, c.x, c.y);
+      least = std::max(least, n);
+      all += n;
+    }
+  const int halves = bytes / 2 / 256 * 256 < (int64_t)(fixed + least) ? 1 : 2;
+  const int64_t half_bytes = bytes / halves / 256 * 256;
   StageArgs a;
   a.one = one;
   a.many = many;
   a.prefix = prefix;
   a.S = S;
-  a.cnt = reinterpret_cast<unsigned*>(base);
-  a.uslab = base + 256;
   a.ucap = (int)(kUBytes / (fp32 ? 4 : 8));
   const size_t sm_apex = fp32 ? apex_smem<float>(mt, ms, nq) : apex_smem<double>(mt, ms, nq);
   const size_t sm_asm = fp32 ? asm_smem<float>(mt, ms) : asm_smem<double>(mt, ms);
@@ -689,45 +716,74 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
   if (fixed > 256) n_asm = std::min(n_asm, sms * 4);   // one slab per CTA
   const int n_far = sms * occupancy((const void*)(fp32 ? (const void*)k_cut<true> : (const void*)k_cut_d), kCutThreads, 0);
   const int n_any = sms * occupancy((const void*)k_cut<false>, kCutThreads, 0);
-  const int n_64 = sms * occupancy((const void*)k_cut_fp64, kCutThreads, 0);
+  const int n_64 = sms * occupancy((const void*)k_cut_fp64, k64Threads, 0);
 
+  struct Events {   // apex and FP32 faces done, entries done, per half
+    cudaEvent_t e[4] = {};
+    ~Events() { for (auto x : e) if (x) cudaEventDestroy(x); }
+  } ev;
+  if (halves == 2)
+    for (auto& x : ev.e) STBEM_CUDA(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+
+  int64_t n_chunk = 0;
   auto flush = [&](int64_t g0, int64_t g1, int64_t rays, int64_t slots) -> bem_status {
     if (rays == 0) return BEM_OK;
     const int64_t nb = g1 - g0;
-    unsigned char* p = base + fixed;
+    const int h = (int)(n_chunk % halves);
+    unsigned char* p = base + h * half_bytes;
+    const cudaStream_t t = halves == 2 ? side : s;   // FP64 faces and entries
+    if (n_chunk >= 2 && halves == 2) STBEM_CUDA(cudaStreamWaitEvent(s, ev.e[2 + h], 0));
+    a.cnt = reinterpret_cast<unsigned*>(p);
+    a.uslab = p + 256;
+    p += fixed;
     auto take = [&](size_t n) { unsigned char* r = p; p += up256(n); return r; };
     a.g0 = g0;
     a.g1 = g1;
     a.apex = take(rays * apex_bytes(fp32));
     a.W = take(slots * (fp32 ? 4 : 8));
     a.q_far = reinterpret_cast<uint32_t*>(take(slots * 4));
-    a.q_any = a.q_64 = nullptr;
+    a.q_any = a.q_64 = a.q_64_last = nullptr;
     if (fp32) {
       a.q_any = reinterpret_cast<uint32_t*>(take(slots * 4));
       a.q_64 = reinterpret_cast<uint32_t*>(take(slots * 4));
+      a.q_64_last = a.q_64 + slots - 1;
     }
     a.fmeta = reinterpret_cast<uint2*>(take(nb * ms * sizeof(uint2)));
     a.bits = reinterpret_cast<uint32_t*>(take(nb * ms * sizeof(uint32_t) * bit_words(mt)));
-    if (p - base > bytes) {
+    if (p - base > (h + 1) * half_bytes) {
       set_error("quadrature scratch too small");
       return BEM_ERR_INTERNAL;
     }
     STBEM_CUDA(cudaMemsetAsync(a.cnt, 0, sizeof(unsigned) * CNT_N, s));
+    auto hand_over = [&]() -> bem_status {
+      if (halves == 1) return BEM_OK;
+      STBEM_CUDA(cudaEventRecord(ev.e[h], s));
+      STBEM_CUDA(cudaStreamWaitEvent(side, ev.e[h], 0));
+      return BEM_OK;
+    };
     if (fp32) {
       k_apex<float><<<n_apex, kApexThreads, sm_apex, s>>>(a);
       k_cut<true><<<n_far, kCutThreads, 0, s>>>(a);
       k_cut<false><<<n_any, kCutThreads, 0, s>>>(a);
-      k_cut_fp64<<<n_64, kCutThreads, 0, s>>>(a);
-      k_assemble<float><<<n_asm, kAsmThreads, sm_asm, s>>>(a);
+      st = hand_over();
+      if (st != BEM_OK) return st;
+      k_cut_fp64<<<n_64, k64Threads, 0, t>>>(a);
+      k_assemble<float><<<n_asm, kAsmThreads, sm_asm, t>>>(a);
     } else {
       k_apex<double><<<n_apex, kApexThreads, sm_apex, s>>>(a);
-      k_cut_d<<<n_far, kCutThreads, 0, s>>>(a);
-      k_assemble<double><<<n_asm, kAsmThreads, sm_asm, s>>>(a);
+      st = hand_over();
+      if (st != BEM_OK) return st;
+      k_cut_d<<<n_far, kCutThreads, 0, t>>>(a);
+      k_assemble<double><<<n_asm, kAsmThreads, sm_asm, t>>>(a);
     }
     STBEM_CUDA(cudaGetLastError());
+    if (halves == 2) STBEM_CUDA(cudaEventRecord(ev.e[2 + h], side));
+    ++n_chunk;
     return BEM_OK;
   };
-  // chunks: runs of granules that fit the scratch
+  // chunks: runs of granules that fit a half; at least four on the mixed path, whose
+  // side stream has other work than the first (FP64 stages all wait for one pipe)
+  const int64_t chunk = std::min<int64_t>(half_bytes, fixed + std::max<int64_t>(least, fp32 ? all / 4 : all));
   int64_t g0 = 0, g1 = 0, rays = 0, slots = 0, off = 0;
   for (size_t o = 0; o < gran.size(); ++o) {
     const int64_t nb = std::min(blocks[o], end - off);
@@ -735,9 +791,9 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
       const uint2 c = (*gran[o])[k];
       const int64_t h0 = off + k * GRAN, h1 = off + std::min<int64_t>(nb, (k + 1) * GRAN);
       if (h1 > g0 && g1 > g0 &&
-          (int64_t)(fixed + chunk_bytes(fp32, mt, ms, h1 - g0, rays + c.x, slots + c.y)) > bytes) {
+          (int64_t)(fixed + chunk_bytes(fp32, mt, ms, h1 - g0, rays + c.x, slots + c.y)) > chunk) {
         st = flush(g0, g1, rays, slots);
-        if (st != BEM_OK) return st;
+        if (st != BEM_OK) break;
         g0 = h0;
         rays = slots = 0;
       }
@@ -745,9 +801,13 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
       rays += c.x;
       slots += c.y;
     }
+    if (st != BEM_OK) break;
     off += blocks[o];
   }
-  return flush(g0, g1, rays, slots);
+  if (st == BEM_OK) st = flush(g0, g1, rays, slots);
+  // the caller's stream goes on when the side stream is done (its last event covers all before it)
+  if (halves == 2 && n_chunk > 0) STBEM_CUDA(cudaStreamWaitEvent(s, ev.e[2 + (n_chunk - 1) % 2], 0));
+  return st;
 }
 
 }  // namespace stbem
