@@ -25,75 +25,99 @@ constexpr int CH = 2048;        // entries per dot-product chunk
 constexpr int TPB = 256;
 
 
-__device__ __forceinline__ int col_of(int64_t idx, int64_t N, int S, const int32_t* seg_of) {
-  const int64_t k = idx / N;
-  const int64_t i = idx - k * N;
-  return (int)(k * S + (S > 1 ? seg_of[i] : 0));
-}
+// The chunks of every column, column by column (ItemTables): item k covers
+// entries [start[k], start[k] + len[k]) of a vector, all of column col[k].
+struct Items {
+  const int64_t* start;
+  const int32_t* len;
+  const int32_t* col;
+  const int32_t* begin;   // [C + 1] items of a column
+  int64_t n;
+};
 
-// partial[i][item] = sum over the item's entries of V_i * w (i < *nvec)
+constexpr int SUB = CH / TPB;   // CTAs of TPB entries per item in the elementwise kernels
+
+// partial[i][item] = sum over the item's entries of V_i * w (i < *nvec).
+// Bound by reading V once. A CTA takes one item and every gridDim.y-th vector:
+// a solve of few columns has some ten items, and one CTA per item read up to
+// restart vectors one after the other with a block reduction for each (with
+// the launches saved below, the solve of 4 right-hand sides on 5,760 panels
+// went from 64 to 50 ms). The sums keep their order.
 __global__ void k_dot_partial(const double* __restrict__ V, int64_t ldv, const int* __restrict__ nvec_p, int nvec_add,
-                              const double* __restrict__ w, const int64_t* __restrict__ it_start,
-                              const int32_t* __restrict__ it_len, int64_t n_items, double* __restrict__ partial) {
-  __shared__ double red[TPB / 32];
+                              const double* __restrict__ w, const Items T, double* __restrict__ partial) {
+  __shared__ double red[2][TPB / 32];
+  const int nvec = (nvec_p ? *nvec_p : 0) + nvec_add;
+  if ((int)blockIdx.y >= nvec) return;
   const int64_t item = blockIdx.x;
-  const int64_t st = it_start[item];
-  const int len = it_len[item];
-  double wv[CH / TPB];
+  const int64_t st = T.start[item];
+  const int len = T.len[item];
+  double wv[SUB];
 #pragma unroll
-  for (int e = 0; e < CH / TPB; ++e) {
+  for (int e = 0; e < SUB; ++e) {
     const int k = threadIdx.x + e * TPB;
     wv[e] = k < len ? w[st + k] : 0.0;
   }
-  const int nvec = (nvec_p ? *nvec_p : 0) + nvec_add;
-  for (int i = 0; i < nvec; ++i) {
+  int buf = 0;
+  for (int i = blockIdx.y; i < nvec; i += gridDim.y, buf ^= 1) {
     const double* v = V + (int64_t)i * ldv + st;
     double sacc = 0.0;
 #pragma unroll
-    for (int e = 0; e < CH / TPB; ++e) {
+    for (int e = 0; e < SUB; ++e) {
       const int k = threadIdx.x + e * TPB;
       if (k < len) sacc += v[k] * wv[e];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sacc;
-    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[buf][threadIdx.x >> 5] = sacc;
+    __syncthreads();   // (the other buffer's readers are past their barrier)
     if (threadIdx.x == 0) {
       double tsum = 0.0;
-      for (int q = 0; q < TPB / 32; ++q) tsum += red[q];
-      partial[(int64_t)i * n_items + item] = tsum;
+      for (int q = 0; q < TPB / 32; ++q) tsum += red[buf][q];
+      partial[(int64_t)i * T.n + item] = tsum;
     }
-    __syncthreads();
   }
 }
 
-// out[c * ldh + i] = sum over the chunks of column c (in order) of partial[i][.]
-__global__ void k_dot_final(const double* __restrict__ partial, int64_t n_items, const int32_t* __restrict__ col_begin,
-                            int C, const int* __restrict__ nvec_p, int nvec_add, double* __restrict__ out, int ldh) {
-  const int nvec = (nvec_p ? *nvec_p : 0) + nvec_add;
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < (int64_t)C * nvec;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(q / nvec), i = (int)(q % nvec);
-    double sacc = 0.0;
-    for (int it = col_begin[c]; it < col_begin[c + 1]; ++it) sacc += partial[(int64_t)i * n_items + it];
-    out[(int64_t)c * ldh + i] = sacc;
-  }
+// sum over the chunks of column c (in order) of partial[i][.]
+__device__ __forceinline__ double column_sum(const double* __restrict__ partial, const Items& T, int c, int i) {
+  double sacc = 0.0;
+  for (int it = T.begin[c]; it < T.begin[c + 1]; ++it) sacc += partial[(int64_t)i * T.n + it];
+  return sacc;
 }
 
-// w += alpha * sum_{i < nvec} h[c][i] V_i   (c the column of each entry)
-__global__ void k_combine(const double* __restrict__ V, int64_t ldv, const double* __restrict__ h, int ldh,
-                          const int* __restrict__ nvec_p, int nvec_add, double alpha, double* __restrict__ w, int64_t N,
-                          int K, int S, const int32_t* __restrict__ seg_of) {
+// out[c] = the squares of column c
+__global__ void k_dot_final(const double* __restrict__ partial, const Items T, int C, double* __restrict__ out) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < C) out[c] = column_sum(partial, T, c, 0);
+}
+
+// w += alpha * sum_{i < nvec} h[c][i] V_i   (c the column of each entry).
+// FINAL: h[c][i] are the sums of the partial dot products (and are kept for
+// the Hessenberg column), so no launch of their own forms them.
+template <bool FINAL>
+__global__ void __launch_bounds__(TPB) k_combine(const double* __restrict__ V, int64_t ldv,
+                                                 const double* __restrict__ partial, double* __restrict__ h, int ldh,
+                                                 const int* __restrict__ nvec_p, int nvec_add, double alpha,
+                                                 double* __restrict__ w, const Items T) {
+  extern __shared__ double hs[];
   const int nvec = (nvec_p ? *nvec_p : 0) + nvec_add;
-  const int64_t total = N * K;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int c = col_of(idx, N, S, seg_of);
-    const double* hc = h + (int64_t)c * ldh;
-    double sacc = 0.0;
-    for (int i = 0; i < nvec; ++i) sacc += hc[i] * V[(int64_t)i * ldv + idx];
-    w[idx] += alpha * sacc;
+  const int64_t item = blockIdx.x / SUB;
+  const int sub = blockIdx.x % SUB, len = T.len[item];
+  if (sub * TPB >= len) return;
+  const int c = T.col[item];
+  for (int i = threadIdx.x; i < nvec; i += TPB) {
+    const double x = FINAL ? column_sum(partial, T, c, i) : h[(int64_t)c * ldh + i];
+    hs[i] = x;
+    if (FINAL && sub == 0 && item == T.begin[c]) h[(int64_t)c * ldh + i] = x;
   }
+  __syncthreads();
+  const int k = sub * TPB + threadIdx.x;
+  if (k >= len) return;
+  const int64_t idx = T.start[item] + k;
+  double sacc = 0.0;
+#pragma unroll 8
+  for (int i = 0; i < nvec; ++i) sacc += hs[i] * V[(int64_t)i * ldv + idx];
+  w[idx] += alpha * sacc;
 }
 
 struct GState {
@@ -115,14 +139,12 @@ struct GState {
   int* iters;        // [C]
 };
 
-__global__ void k_givens(GState G, int C, int m, double tol) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= C) return;
-  const int j = *G.j;
-  if (!G.active[c]) { G.scale[c] = 0.0; return; }
+// The Givens update of column c and its residual estimate; true while it goes on.
+__device__ __forceinline__ int givens_column(const GState& G, int c, int j, int m, double tol, double w2) {
+  if (!G.active[c]) { G.scale[c] = 0.0; return 0; }
   double* Hc = G.H + (int64_t)c * (m + 1) * m + (int64_t)j * (m + 1);
   for (int i = 0; i <= j; ++i) Hc[i] = G.h1[(int64_t)c * (m + 1) + i] + G.h2[(int64_t)c * (m + 1) + i];
-  const double hn = sqrt(fmax(G.hn2[c], 0.0));
+  const double hn = sqrt(fmax(w2, 0.0));
   Hc[j + 1] = hn;
   double* csc = G.cs + (int64_t)c * m;
   double* snc = G.sn + (int64_t)c * m;
@@ -147,22 +169,39 @@ __global__ void k_givens(GState G, int C, int m, double tol) {
   const double rel = fabs(gc[j + 1]) / bn;
   G.relres[c] = rel;
   const bool breakdown = !(hn > 1e-300 * fmax(1.0, bn));
-  if (rel <= tol || breakdown || j + 1 >= m) G.active[c] = 0;
-  G.scale[c] = G.active[c] ? 1.0 / hn : 0.0;
+  const int act = !(rel <= tol || breakdown || j + 1 >= m);
+  G.active[c] = act;
+  G.scale[c] = act ? 1.0 / hn : 0.0;
+  return act;
 }
 
-// V_{j+1} = scale[c] * w and the product operand vj; then j += 1 (last block)
-__global__ void k_next(const double* __restrict__ w, const double* __restrict__ scale, double* __restrict__ V,
-                       int64_t ldv, double* __restrict__ vj, const int* __restrict__ jp, int64_t N, int K, int S,
-                       const int32_t* __restrict__ seg_of) {
-  const int j = *jp;
-  const int64_t total = N * K;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const double v = scale[col_of(idx, N, S, seg_of)] * w[idx];
-    V[(int64_t)(j + 1) * ldv + idx] = v;
-    vj[idx] = v;
+// One thread per column; |w|^2 is summed here. Up to GIV_ONE columns (one CTA)
+// the step index and the number of active columns are updated as well; with
+// more, k_inc does that.
+constexpr int GIV_ONE = 64;
+__global__ void k_givens(GState G, int C, int m, double tol, const double* __restrict__ partial, const Items T) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = *G.j;
+  const int act = c < C ? givens_column(G, c, j, m, tol, column_sum(partial, T, c, 0)) : 0;
+  if (gridDim.x == 1) {
+    const int n = __syncthreads_count(act);   // (and every thread has read j)
+    if (threadIdx.x == 0) {
+      *G.j = j + 1;
+      *G.nactive = n;
+    }
   }
+}
+
+// V_{j+1} = scale[c] * w and the product operand vj (*jp + add = j + 1)
+__global__ void k_next(const double* __restrict__ w, const double* __restrict__ scale, double* __restrict__ V,
+                       int64_t ldv, double* __restrict__ vj, const int* __restrict__ jp, int add, const Items T) {
+  const int64_t item = blockIdx.x / SUB;
+  const int k = blockIdx.x % SUB * TPB + threadIdx.x;
+  if (k >= T.len[item]) return;
+  const int64_t idx = T.start[item] + k;
+  const double v = scale[T.col[item]] * w[idx];
+  V[(int64_t)(jp ? *jp + add : add) * ldv + idx] = v;
+  vj[idx] = v;
 }
 
 // j += inc; nactive = number of active columns
@@ -194,17 +233,6 @@ __global__ void k_cycle_init(GState G, int C, int m, double tol) {
   for (int i = 0; i <= m; ++i) gc[i] = 0.0;
   gc[0] = act ? beta : 0.0;
   G.scale[c] = act ? 1.0 / beta : 0.0;
-}
-
-__global__ void k_scale0(const double* __restrict__ r, const double* __restrict__ scale, double* __restrict__ V0,
-                         double* __restrict__ vj, int64_t N, int K, int S, const int32_t* __restrict__ seg_of) {
-  const int64_t total = N * K;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const double v = scale[col_of(idx, N, S, seg_of)] * r[idx];
-    V0[idx] = v;
-    vj[idx] = v;
-  }
 }
 
 // y = H^{-1} g on the first kdim rows (upper triangular after the rotations)
@@ -266,9 +294,10 @@ struct DA {
 // the uploads are done: the caller synchronizes before they go)
 struct ItemTables {
   std::vector<int64_t> st;
-  std::vector<int32_t> ln, cb;
+  std::vector<int32_t> ln, cl, cb;
   DA<int64_t> d_st;
-  DA<int32_t> d_ln, d_cb;
+  DA<int32_t> d_ln, d_cl, d_cb;
+  Items items() const { return {d_st.p, d_ln.p, d_cl.p, d_cb.p, n}; }
   int64_t n = 0;
   bem_status build(const SegLayout& L, cudaStream_t s) {
     const int C = L.K * L.S;
@@ -281,15 +310,18 @@ struct ItemTables {
         for (int64_t o = 0; o < len; o += CH) {
           st.push_back(off + o);
           ln.push_back((int32_t)std::min<int64_t>(CH, len - o));
+          cl.push_back(c);
         }
       }
     cb[C] = (int32_t)st.size();
     n = (int64_t)st.size();
     G_TRY(d_st.alloc(n, false, s));
     G_TRY(d_ln.alloc(n, false, s));
+    G_TRY(d_cl.alloc(n, false, s));
     G_TRY(d_cb.alloc(C + 1, false, s));
     STBEM_CUDA(cudaMemcpyAsync(d_st.p, st.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, s));
     STBEM_CUDA(cudaMemcpyAsync(d_ln.p, ln.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, s));
+    STBEM_CUDA(cudaMemcpyAsync(d_cl.p, cl.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, s));
     STBEM_CUDA(cudaMemcpyAsync(d_cb.p, cb.data(), sizeof(int32_t) * (C + 1), cudaMemcpyHostToDevice, s));
     return BEM_OK;
   }
@@ -304,9 +336,8 @@ bem_status seg_norms(const SegLayout& L, const double* v, std::vector<double>& o
   DA<double> partial, res;
   G_TRY(partial.alloc(T.n, false, s));
   G_TRY(res.alloc(C, false, s));
-  k_dot_partial<<<(unsigned)std::max<int64_t>(T.n, 1), TPB, 0, s>>>(v, 0, nullptr, 1, v, T.d_st.p, T.d_ln.p, T.n,
-                                                                     partial.p);
-  k_dot_final<<<(unsigned)((C + 63) / 64), 64, 0, s>>>(partial.p, T.n, T.d_cb.p, C, nullptr, 1, res.p, 1);
+  if (T.n > 0) k_dot_partial<<<(unsigned)T.n, TPB, 0, s>>>(v, 0, nullptr, 1, v, T.items(), partial.p);
+  k_dot_final<<<(unsigned)((C + 63) / 64), 64, 0, s>>>(partial.p, T.items(), C, res.p);
   STBEM_CUDA(cudaGetLastError());
   out.resize(C);
   STBEM_CUDA(cudaMemcpyAsync(out.data(), res.p, sizeof(double) * C, cudaMemcpyDeviceToHost, s));
@@ -318,24 +349,12 @@ bem_status seg_norms(const SegLayout& L, const double* v, std::vector<double>& o
 bem_status gmres_device(const SegLayout& L, const MatvecFn& mv, const double* d_b, double* d_x, double tol, int m,
                         int maxit, std::vector<int>& iters, std::vector<double>& relres, std::vector<int>& conv,
                         cudaStream_t s) {
-  const int64_t N = L.N, NN = L.N * L.K;
-  const int K = L.K, S = L.S, C = K * S;
+  const int64_t NN = L.N * L.K;
+  const int C = L.K * L.S;
   ItemTables T;
   G_TRY(T.build(L, s));
   const int64_t n_items = T.n;
-  const int64_t* it_st_p = T.d_st.p;
-  const int32_t* it_ln_p = T.d_ln.p;
-  const int32_t* it_cb_p = T.d_cb.p;
-  DA<int32_t> seg_of;
-  const int32_t* d_seg = nullptr;
-  if (S > 1) {
-    std::vector<int32_t> so(N);
-    for (int sg = 0; sg < S; ++sg)
-      for (int64_t i = L.seg_off[sg]; i < L.seg_off[sg + 1]; ++i) so[i] = sg;
-    G_TRY(seg_of.alloc(N, false, s));
-    STBEM_CUDA(cudaMemcpyAsync(seg_of.p, so.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice, s));
-    d_seg = seg_of.p;
-  }
+  const Items I = T.items();
   // workspace
   DA<double> V, w, vj, r, partial, H, g, cs, sn, h1, h2, hn2, bnorm, rel, scale, y;
   DA<int> ints, active, kdim, it;
@@ -361,10 +380,14 @@ bem_status gmres_device(const SegLayout& L, const MatvecFn& mv, const double* d_
   G_TRY(it.alloc(C, true, s));
   GState G{ints.p, ints.p + 2, H.p, g.p, cs.p, sn.p, h1.p, h2.p, hn2.p, bnorm.p, rel.p, scale.p, y.p,
            active.p, kdim.p, it.p};
-  const unsigned gN = grid_of(NN), gC = (unsigned)((C + 63) / 64);
+  const unsigned gN = grid_of(NN), gC = (unsigned)((C + GIV_ONE - 1) / GIV_ONE);
+  const unsigned gI = (unsigned)n_items, gE = (unsigned)(n_items * SUB);
+  // vectors side by side in the dot products: about eight CTAs per SM
+  const unsigned gV = (unsigned)std::max<int64_t>(1, std::min<int64_t>(m, 8 * 152 / std::max<int64_t>(n_items, 1)));
+  const size_t hbytes = sizeof(double) * (m + 1);
   auto norms2 = [&](const double* v, double* out) -> bem_status {
-    k_dot_partial<<<(unsigned)n_items, TPB, 0, s>>>(v, 0, nullptr, 1, v, it_st_p, it_ln_p, n_items, partial.p);
-    k_dot_final<<<gC, 64, 0, s>>>(partial.p, n_items, it_cb_p, C, nullptr, 1, out, 1);
+    k_dot_partial<<<gI, TPB, 0, s>>>(v, 0, nullptr, 1, v, I, partial.p);
+    k_dot_final<<<gC, 64, 0, s>>>(partial.p, I, C, out);
     STBEM_CUDA(cudaGetLastError());
     return BEM_OK;
   };
@@ -381,15 +404,13 @@ bem_status gmres_device(const SegLayout& L, const MatvecFn& mv, const double* d_
   auto step = [&]() -> bem_status {
     G_TRY(mv(vj.p, w.p, s));
     for (int pass = 0; pass < 2; ++pass) {
-      double* hp = pass == 0 ? h1.p : h2.p;
-      k_dot_partial<<<(unsigned)n_items, TPB, 0, s>>>(V.p, NN, G.j, 1, w.p, it_st_p, it_ln_p, n_items, partial.p);
-      k_dot_final<<<grid_of((int64_t)C * (m + 1)), 256, 0, s>>>(partial.p, n_items, it_cb_p, C, G.j, 1, hp, m + 1);
-      k_combine<<<gN, 256, 0, s>>>(V.p, NN, hp, m + 1, G.j, 1, -1.0, w.p, N, K, S, d_seg);
+      k_dot_partial<<<dim3(gI, gV), TPB, 0, s>>>(V.p, NN, G.j, 1, w.p, I, partial.p);
+      k_combine<true><<<gE, TPB, hbytes, s>>>(V.p, NN, partial.p, pass == 0 ? h1.p : h2.p, m + 1, G.j, 1, -1.0, w.p, I);
     }
-    G_TRY(norms2(w.p, hn2.p));
-    k_givens<<<gC, 64, 0, s>>>(G, C, m, tol);
-    k_next<<<gN, 256, 0, s>>>(w.p, scale.p, V.p, NN, vj.p, G.j, N, K, S, d_seg);
-    k_inc<<<1, 256, 0, s>>>(G.j, 1, active.p, C, G.nactive);
+    k_dot_partial<<<gI, TPB, 0, s>>>(w.p, 0, nullptr, 1, w.p, I, partial.p);
+    k_givens<<<gC, GIV_ONE, 0, s>>>(G, C, m, tol, partial.p, I);
+    if (gC > 1) k_inc<<<1, 256, 0, s>>>(G.j, 1, active.p, C, G.nactive);
+    k_next<<<gE, TPB, 0, s>>>(w.p, scale.p, V.p, NN, vj.p, G.j, 0, I);
     STBEM_CUDA(cudaGetLastError());
     return BEM_OK;
   };
@@ -410,7 +431,7 @@ bem_status gmres_device(const SegLayout& L, const MatvecFn& mv, const double* d_
     k_residual<<<gN, 256, 0, s>>>(d_b, w.p, r.p, NN);
     G_TRY(norms2(r.p, hn2.p));
     k_cycle_init<<<gC, 64, 0, s>>>(G, C, m, tol);
-    k_scale0<<<gN, 256, 0, s>>>(r.p, scale.p, V.p, vj.p, N, K, S, d_seg);
+    k_next<<<gE, TPB, 0, s>>>(r.p, scale.p, V.p, NN, vj.p, nullptr, 0, I);
     k_inc<<<1, 256, 0, s>>>(G.j, 0, active.p, C, G.nactive);
     STBEM_CUDA(cudaGetLastError());
     STBEM_CUDA(cudaMemcpyAsync(&nact, G.nactive, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -455,7 +476,7 @@ bem_status gmres_device(const SegLayout& L, const MatvecFn& mv, const double* d_
     }
     // x += V y
     k_backsolve<<<gC, 64, 0, s>>>(G, C, m);
-    k_combine<<<gN, 256, 0, s>>>(V.p, NN, y.p, m, nullptr, m, 1.0, d_x, N, K, S, d_seg);
+    k_combine<false><<<gE, TPB, hbytes, s>>>(V.p, NN, nullptr, y.p, m, nullptr, m, 1.0, d_x, I);
     STBEM_CUDA(cudaGetLastError());
     if (cancel_requested()) {
       STBEM_CUDA(cudaStreamSynchronize(s));
