@@ -23,6 +23,8 @@ static double __longlong_as_double_host(long long b) {
   return d;
 }
 
+bem_status upload_exp_table();
+
 bem_status upload_gauss_tables() {
   std::vector<double> X(MAX_NTHETA * (MAX_NTHETA + 1) / 2), W(X.size());
   for (int n = 1; n <= MAX_NTHETA; ++n) {
@@ -63,7 +65,8 @@ bem_status upload_gauss_tables() {
   STBEM_CUDA(cudaMemcpyToSymbol(c_gl_w, W.data(), W.size() * sizeof(double)));
   STBEM_CUDA(cudaMemcpyToSymbol(c_gl_xf, Xf.data(), Xf.size() * sizeof(float)));
   STBEM_CUDA(cudaMemcpyToSymbol(c_gl_wf, Wf.data(), Wf.size() * sizeof(float)));
-  return upload_gauss_stage(X.data(), W.data(), Xf.data(), Wf.data(), X.size());
+  const bem_status st = upload_exp_table();
+  return st != BEM_OK ? st : upload_gauss_stage(X.data(), W.data(), Xf.data(), Wf.data(), X.size());
 }
 
 // ---------------------------------------------------------------------------
@@ -764,85 +767,145 @@ bem_status op_pattern_csr(const bem_operator* op, int64_t* d_rowcount, int64_t* 
 
 // ---------------------------------------------------------------------------
 // Right-hand side: b_i = int_K [g(P_lo(y), y) - g(P_hi(y), y)] dA
-// (= -sum_F nu_{F,t} int_F g dS, eq. int_bform with A = Id). K is split into
-// 4^k congruent sub-triangles, k chosen so that a sub-triangle spans at most
-// half the data's length scale (pulse width, or 0.5 for the sin^2 data), and
-// each gets a Duffy-collapsed 8 x 8 Gauss-Legendre rule.
+// (= -sum_F nu_{F,t} int_F g dS, eq. int_bform with A = Id) = S_lo - S_hi, S_F
+// the integral of the data over face F's graph. K is split into 4^k congruent
+// sub-triangles, k chosen so that a sub-triangle spans at most half the
+// data's length scale (pulse width, or 0.5 for the sin^2 data), and each gets
+// a Duffy-collapsed 8 x 8 Gauss-Legendre rule.
 // ---------------------------------------------------------------------------
-__device__ inline double data_g(int kind, const double* prm, double t, const double* x) {
-  if (kind == BEM_DATA_SIN2_UNIFORM) {
-    if (!(t > 0.0 && t < 2.0)) return 0.0;
-    double s = sin(0.5 * STBEM_PI * t);
-    return s * s;
-  }
-  double a = (t - (x[0] * prm[0] + x[1] * prm[1] + x[2] * prm[2]) - prm[3]) / prm[4];
-  return exp(-a * a);
+
+// exp(z), z <= 0, by the table-driven method of P. T. P. Tang (ACM TOMS 15,
+// 1989): z = (128 n + j) ln 2 / 128 + r, exp(z) = 2^n 2^(j/128) (1 + p(r)) with
+// the Taylor polynomial of degree 5 (|r| <= 0.0028: r^6 / 720 < 1e-18), about
+// an ulp. Eleven FP64 instructions where the general function takes some
+// twenty, and the FP64 pipe is what the right-hand side is bound by. Below
+// -708 (denormal results) and for NaN the general function answers.
+__device__ __forceinline__ double exp_neg(double z, const double* __restrict__ tab) {
+  if (!(z > -708.0)) return exp(z);
+  const double magic = 6755399441055744.0;   // 1.5 * 2^52: the sum's low bits are the rounded integer
+  const double kd = __fma_rn(z, 128.0 / 0.693147180559945309417, magic);
+  const int k = __double2loint(kd);
+  const double kf = __dsub_rn(kd, magic);
+  // ln 2 / 128 in two parts, the first with 32 trailing zero bits
+  double r = __fma_rn(kf, -0x1.62e42feep-8, z);
+  r = __fma_rn(kf, -0x1.a39ef35793c76p-40, r);
+  double p = __fma_rn(r, 1.0 / 120.0, 1.0 / 24.0);
+  p = __fma_rn(p, r, 1.0 / 6.0);
+  p = __fma_rn(p, r, 0.5);
+  p = __fma_rn(r * r, p, r);
+  const double t = tab[k & 127];
+  const double v = __fma_rn(t, p, t);
+  return __hiloint2double(__double2hiint(v) + ((k >> 7) << 20), __double2loint(v));
 }
 
-__device__ inline double rhs_subtri(const ColGeom& G, const FaceGeom& Flo, const FaceGeom& Fhi, int kind,
-                                    const double* prm, const double* B0, const double* B1, const double* B2) {
-  const int n = 8;
-  const double* X = gl_x() + n * (n - 1) / 2;
-  const double* Wt = gl_w() + n * (n - 1) / 2;
-  double acc = 0.0;
-  for (int a = 0; a < n; ++a) {
-    double u = 0.5 * (X[a] + 1.0), wu = 0.5 * Wt[a];
-    for (int c = 0; c < n; ++c) {
-      double v = 0.5 * (X[c] + 1.0), wv = 0.5 * Wt[c];
-      double m0 = 1.0 - u, m1 = u * (1.0 - v), m2 = u * v;   // Duffy: Jacobian 2 |sub| u
-      double l[3];
-      for (int k = 0; k < 3; ++k) l[k] = m0 * B0[k] + m1 * B1[k] + m2 * B2[k];
-      double y[3];
-      for (int k = 0; k < 3; ++k) y[k] = l[0] * G.X[0][k] + l[1] * G.X[1][k] + l[2] * G.X[2][k];
-      double tlo = l[0] * Flo.p[0] + l[1] * Flo.p[1] + l[2] * Flo.p[2];
-      double thi = l[0] * Fhi.p[0] + l[1] * Fhi.p[1] + l[2] * Fhi.p[2];
-      acc += wu * wv * u * (data_g(kind, prm, tlo, y) - data_g(kind, prm, thi, y));
+__device__ __constant__ double c_exp2_tab[128];   // 2^(j/128)
+
+bem_status upload_exp_table() {
+  double t[128];
+  for (int j = 0; j < 128; ++j) t[j] = std::exp2(j / 128.0);
+  STBEM_CUDA(cudaMemcpyToSymbol(c_exp2_tab, t, sizeof(t)));
+  return BEM_OK;
+}
+
+constexpr int kRhsThreads = 128;
+
+// S[r][F] by a warp per (face, right-hand side): the 64 nodes of a
+// sub-triangle on the lanes, two each, and a loop over the sub-triangles. The
+// data's argument (t - <y, d> - c) / w, and t, are linear on K: a node costs
+// two FMAs, and S_F serves the panel below and the panel above (a thread per
+// panel formed both its faces at every node from coordinates and left a mesh
+// of 1,920 panels to 15 CTAs). FP64-bound: 64
+// pulses on 30,720 panels 444 -> 72 ms (2.0e9 nodes of 15 FP64 instructions: 58 ms).
+template <int KIND>
+__global__ void __launch_bounds__(kRhsThreads) k_rhs_faces(int64_t n_surf, const SurfDev* __restrict__ surf,
+                                                           const ColGeom* __restrict__ cols, int nrhs,
+                                                           const double* __restrict__ params, double2* __restrict__ S) {
+  __shared__ double tab[128];
+  for (int k = threadIdx.x; k < 128; k += kRhsThreads) tab[k] = c_exp2_tab[k];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  // this lane's nodes: (a, c) = (lane / 8, lane % 8) and (lane / 8 + 4, lane % 8)
+  const double* X = gl_x() + 8 * 7 / 2;
+  const double* Wt = gl_w() + 8 * 7 / 2;
+  double m1[2], m2[2], wn[2];
+  const double v = 0.5 * (X[lane & 7] + 1.0), wv = 0.5 * Wt[lane & 7];
+  for (int h = 0; h < 2; ++h) {
+    const double u = 0.5 * (X[(lane >> 3) + 4 * h] + 1.0), wu = 0.5 * Wt[(lane >> 3) + 4 * h];
+    m1[h] = u * (1.0 - v);
+    m2[h] = u * v;           // Duffy: Jacobian 2 |sub| u
+    wn[h] = wu * wv * u;
+  }
+  const int64_t n = n_surf * nrhs, step = (int64_t)gridDim.x * (kRhsThreads / 32);
+  for (int64_t it = (int64_t)blockIdx.x * (kRhsThreads / 32) + (threadIdx.x >> 5); it < n; it += step) {
+    const int64_t r = it / n_surf, f = it - r * n_surf;
+    const SurfDev& F = surf[f];
+    const ColGeom& G = cols[F.col];
+    const double* prm = KIND == BEM_DATA_PULSE ? params + 5 * r : nullptr;
+    double a[3];   // the argument at the corners
+    for (int k = 0; k < 3; ++k) {
+      a[k] = F.f.p[k];   // (fused: a corner's rounding is common to all nodes of the face)
+      if (KIND == BEM_DATA_PULSE)
+        a[k] = __fma_rn(-G.X[k][0], prm[0], __fma_rn(-G.X[k][1], prm[1], __fma_rn(-G.X[k][2], prm[2], a[k] - prm[3]))) / prm[4];
     }
-  }
-  return acc;
-}
-
-__global__ void k_rhs(int64_t n_tet, const TetDev* tets, const SurfDev* surf, const ColGeom* cols, int kind, int nrhs,
-                      const double* params, double* b) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n_tet) return;
-  const TetDev D = tets[i];
-  const ColGeom& G = cols[D.col];
-  const FaceGeom Flo = surf[D.lo].f, Fhi = surf[D.hi].f;
-  for (int r = 0; r < nrhs; ++r) {
-    const double* prm = params ? params + 5 * r : nullptr;
-    double scale = kind == BEM_DATA_PULSE ? 0.5 * prm[4] : 0.5;
+    const double scale = KIND == BEM_DATA_PULSE ? 0.5 * prm[4] : 0.5;
     int lev = 0;
     while (lev < 4 && G.diam / (double)(1 << lev) > scale) ++lev;
-    int m = 1 << lev;
+    const int m = 1 << lev;
+    const double e1 = (a[1] - a[0]) / m, e2 = (a[2] - a[0]) / m;
     double acc = 0.0;
+    auto add = [&](double base, double d1, double d2) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const double x = base + m1[h] * d1 + m2[h] * d2;
+        double g;
+        if (KIND == BEM_DATA_PULSE) {
+          g = exp_neg(-x * x, tab);
+        } else {
+          g = 0.0;
+          if (x > 0.0 && x < 2.0) {
+            const double sn = sin(0.5 * STBEM_PI * x);
+            g = sn * sn;
+          }
+        }
+        acc += wn[h] * g;
+      }
+    };
     for (int p = 0; p < m; ++p)
       for (int q = 0; p + q < m; ++q) {
-        double a0[3] = {1.0 - (double)(p + q) / m, (double)p / m, (double)q / m};
-        double a1[3] = {1.0 - (double)(p + q + 1) / m, (double)(p + 1) / m, (double)q / m};
-        double a2[3] = {1.0 - (double)(p + q + 1) / m, (double)p / m, (double)(q + 1) / m};
-        acc += rhs_subtri(G, Flo, Fhi, kind, prm, a0, a1, a2);
-        if (p + q + 2 <= m) {
-          double c0[3] = {1.0 - (double)(p + q + 2) / m, (double)(p + 1) / m, (double)(q + 1) / m};
-          acc += rhs_subtri(G, Flo, Fhi, kind, prm, a1, c0, a2);
-        }
+        add(a[0] + p * e1 + q * e2, e1, e2);
+        if (p + q + 2 <= m) add(a[0] + (p + 1) * e1 + q * e2, e2, e2 - e1);
       }
+    // the sum and its rounding error (Knuth's two-sum): b is a small difference of two S
+    double lost = 0.0;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      const double x = __shfl_xor_sync(0xffffffffu, acc, o);
+      lost += __shfl_xor_sync(0xffffffffu, lost, o);
+      const double t = __dadd_rn(acc, x), z = __dsub_rn(t, acc);
+      lost += __dadd_rn(__dsub_rn(acc, __dsub_rn(t, z)), __dsub_rn(x, z));
+      acc = t;
+    }
     // each sub-triangle has area |K| / m^2; Duffy Jacobian 2 |sub| u
-    b[i + n_tet * (int64_t)r] = 2.0 * G.area / ((double)m * m) * acc;
+    if (lane == 0) {
+      const double sc = 2.0 * G.area / ((double)m * m), h = __dmul_rn(sc, acc);
+      S[it] = make_double2(h, __fma_rn(sc, acc, -h) + sc * lost);
+    }
   }
 }
 
-bem_status op_rhs(const bem_operator* op, int kind, int nrhs, const double* d_params, double* d_b, cudaStream_t s) {
-  const bem_mesh* m = op->mesh;
-  k_rhs<<<(unsigned)((m->n_tet + 127) / 128), 128, 0, s>>>(m->n_tet, m->d_tet, m->d_surf, m->d_col, kind, nrhs,
-                                                           d_params, d_b);
-  STBEM_CUDA(cudaGetLastError());
-  return BEM_OK;
+// b[r][i] = S[r][lo(i)] - S[r][hi(i)] (internal panel order)
+__global__ void k_rhs_panels(int64_t n_tet, int64_t n_surf, int nrhs, const TetDev* tets, const double2* S, double* b) {
+  int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (tid >= n_tet * nrhs) return;
+  const int64_t r = tid / n_tet, i = tid - r * n_tet;
+  const TetDev& D = tets[i];
+  const double2 lo = S[r * n_surf + D.lo], hi = S[r * n_surf + D.hi];
+  b[tid] = (lo.x - hi.x) + (lo.y - hi.y);
 }
 
 // Points and weights of the right-hand side rule for arbitrary data: per
 // surface (a face tau = P(y) over K), K split into 4^level congruent
-// triangles in the order of k_rhs (row p, then q; upright, then inverted),
+// triangles in the order of k_rhs_faces (row p, then q; upright, then inverted),
 // each with a Duffy-collapsed ng x ng Gauss-Legendre rule. One thread per
 // (surface, sub-triangle); pts may be null (weights only).
 __global__ void k_rhs_points(int64_t n_surf, const SurfDev* surf, const ColGeom* cols, int level, int ng,
@@ -914,6 +977,28 @@ __global__ void k_rhs_combine(int64_t n_tet, int64_t n_surf, int nrhs, const Tet
   const int64_t r = tid / n_tet, i = tid - r * n_tet;
   const TetDev& D = tets[i];
   b[tid] = S[r * n_surf + D.lo] - S[r * n_surf + D.hi];
+}
+
+bem_status op_rhs(const bem_operator* op, int kind, int nrhs, const double* d_params, double* d_b, cudaStream_t s) {
+  const bem_mesh* m = op->mesh;
+  const int64_t n = m->n_surf * nrhs, nb = m->n_tet * nrhs;
+  double2* S = nullptr;
+  cudaError_t e = cudaMallocAsync((void**)&S, sizeof(double2) * std::max<int64_t>(n, 1), s);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    set_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
+    return e == cudaErrorMemoryAllocation ? BEM_ERR_OUT_OF_MEMORY : BEM_ERR_CUDA;
+  }
+  const unsigned grid = (unsigned)std::min<int64_t>((n + 3) / 4, 152 * 64);
+  if (kind == BEM_DATA_PULSE)
+    k_rhs_faces<BEM_DATA_PULSE><<<grid, kRhsThreads, 0, s>>>(m->n_surf, m->d_surf, m->d_col, nrhs, d_params, S);
+  else
+    k_rhs_faces<BEM_DATA_SIN2_UNIFORM><<<grid, kRhsThreads, 0, s>>>(m->n_surf, m->d_surf, m->d_col, nrhs, d_params, S);
+  k_rhs_panels<<<(unsigned)((nb + 127) / 128), 128, 0, s>>>(m->n_tet, m->n_surf, nrhs, m->d_tet, S, d_b);
+  e = cudaGetLastError();
+  cudaFreeAsync(S, s);
+  STBEM_CUDA(e);
+  return BEM_OK;
 }
 
 bem_status op_rhs_points(const bem_operator* op, int level, int ng, double* d_pts, double* d_wts, cudaStream_t s) {

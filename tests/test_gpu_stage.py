@@ -61,3 +61,20 @@ def test_entries_and_pattern(ctx, surface, level, slabs, T, mq):
     for op in ops.values():
         assert out.size == 0 or np.all(op.entries(out) == 0.0)
         assert op.check()[0] == 0
+
+
+@pytest.mark.parametrize("level,slabs,T,width", [(0, 1, 0.2, 4.0), (0, 3, 2.0, 0.25), (1, 5, 3.0, 0.05), (1, 2, 1.0, 0.5)])
+def test_rhs_over_the_refinement_levels(ctx, level, slabs, T, width):
+    """Right-hand sides from one level (no split of the triangles) to the
+    deepest (4), with pulses far outside the time window (results that
+    underflow) among them, against the oracle: 1e-12 of the largest (the bound
+    of the parity test)."""
+    import paper_2103_16841_gb300 as stb
+    m = inputs.sphere_mesh(level, slabs, T, 0.2, seed=4)
+    op = stb.Operator(ctx, stb.Mesh.from_spacetime(ctx, m), "fp64")
+    prm = inputs.pulse_params(5, seed=3, width=width)
+    prm[3, 3] = 60.0
+    g = op.rhs(stb.DATA_PULSE, prm)
+    r = oracle.Mesh.from_spacetime(m).rhs(stb.DATA_PULSE, prm)
+    assert np.abs(g - r).max() <= 1e-12 * np.abs(r).max()
+    assert np.array_equal(op.rhs(stb.DATA_PULSE, prm), g)
