@@ -230,10 +230,11 @@ bem_status bem_mesh_create(bem_context* ctx, int64_t n_sv, const double* sv_xyz,
     }
   }
   std::vector<int32_t> col_surf_begin(n_col + 1, 0);
-  int max_tets = 0, max_surf = 0;
+  int max_tets = 0, max_surf = 0, col_gcd = 0;
   for (int64_t c = 0; c < n_col; ++c) {
     col_surf_begin[c + 1] = col_surf_begin[c] + (int)scols[c].size();
     max_tets = std::max(max_tets, col_tet_begin[c + 1] - col_tet_begin[c]);
+    col_gcd = std::gcd(col_gcd, col_tet_begin[c + 1] - col_tet_begin[c]);
     max_surf = std::max(max_surf, (int)scols[c].size());
   }
   if (max_tets > MAX_COL_TETS || max_surf > MAX_COL_SURF) {
@@ -277,7 +278,7 @@ bem_status bem_mesh_create(bem_context* ctx, int64_t n_sv, const double* sv_xyz,
   std::unique_ptr<bem_mesh> m(new bem_mesh());
   m->ctx = ctx;
   m->n_tet = n_tet; m->n_col = n_col; m->n_surf = n_surf;
-  m->max_col_tets = max_tets; m->max_col_surf = max_surf;
+  m->max_col_tets = max_tets; m->max_col_surf = max_surf; m->col_gcd = col_gcd;
   m->perm = perm; m->iperm = iperm;
   m->col_tet_begin = col_tet_begin; m->col_surf_begin = col_surf_begin;
   m->coord_scale = std::max(scale, 1e-300);

@@ -91,6 +91,7 @@ struct bem_mesh {
   bem_context* ctx = nullptr;
   int64_t n_tet = 0, n_col = 0, n_surf = 0;
   int max_col_tets = 0, max_col_surf = 0;
+  int col_gcd = 1;              // divides the number of panels of every column
   std::vector<int32_t> perm;    // internal -> caller panel id
   std::vector<int32_t> iperm;   // caller -> internal
   std::vector<int32_t> col_tet_begin, col_surf_begin;  // [n_col+1]
@@ -212,7 +213,8 @@ struct BatchMatvec {
   int32_t* d_cseg = nullptr;
   int32_t* d_ccol = nullptr;
   int64_t n_cta = 0, N = 0;
-  int rows_pad = 32, groups = 1;
+  int col_gcd = 1, max_rows = 1;   // of the columns of all operators
+  int64_t max_cols = 1;
   bool fp64_values = false;
   float* d_xf = nullptr;
   int64_t xf_len = 0;

@@ -1206,7 +1206,7 @@ STBEM_HD __noinline__ double face_cut(const ColR<R>& G, const PtR<R>& P, const F
 
 #ifdef __CUDACC__
 // ---------------------------------------------------------------------------
-// FP32 pairs (double-float, about 2^-45 relative): the geometry of an apex
+// FP32 pairs (double-float, about 2^-48 relative): the geometry of an apex
 // against a column off the FP64 pipe, which on sm_103a has 1/76 of the FP32
 // rate. Error-free sums (Knuth) and products (fma), after Dekker 1971; the
 // intrinsics keep the compiler from contracting them.
@@ -1230,14 +1230,14 @@ __device__ __forceinline__ F2 f2_neg(F2 a) { return {-a.h, -a.l}; }
 __device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
   const float p = __fmul_rn(a.h, b.h);
   float e = __fmaf_rn(a.h, b.h, -p);
-  e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e));
+  e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.l, b.l, e)));
   return f2_fast(p, e);
 }
 __device__ __forceinline__ F2 f2_sqrt(F2 a) {
   if (!(a.h > 0.f)) return {0.f, 0.f};
   const float s = __fsqrt_rn(a.h), p = __fmul_rn(s, s);
   const float r = __fadd_rn(__fsub_rn(__fsub_rn(a.h, p), __fmaf_rn(s, s, -p)), a.l);   // a - s^2
-  return f2_fast(s, __fdividef(r, 2.f * s));
+  return f2_fast(s, __fdiv_rn(r, 2.f * s));
 }
 
 // D0 where it cancels (see cut_in_mixed), from FP32 pairs

@@ -78,3 +78,24 @@ def test_rhs_over_the_refinement_levels(ctx, level, slabs, T, width):
     r = oracle.Mesh.from_spacetime(m).rhs(stb.DATA_PULSE, prm)
     assert np.abs(g - r).max() <= 1e-12 * np.abs(r).max()
     assert np.array_equal(op.rhs(stb.DATA_PULSE, prm), g)
+
+
+@pytest.mark.parametrize("level,slabs", [(0, 1), (0, 2), (0, 3), (1, 4), (0, 64), (1, 21)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_products_over_the_column_sizes(ctx, level, slabs, precision):
+    """Products for column sizes of every divisor (rows per thread 1, 2, 4), one
+    slot to many, a cluster of CTAs per column, and ragged groups of right-hand
+    sides, against the exported matrix: FP64 accumulation within n 2^-53, FP32
+    within (n + 2) 2^-24 of |A| |x| (n the row's entries; the classical bound of a
+    sum in any order)."""
+    import paper_2103_16841_gb300 as stb
+    m = inputs.sphere_mesh(level, slabs, 2.0, 0.2, seed=5)
+    op = stb.Operator(ctx, stb.Mesh.from_spacetime(ctx, m), precision)
+    A = op.export_dense()
+    row = (A != 0).sum(axis=1)
+    for nrhs in (1, 3, 4, 5, 9):
+        x = np.random.default_rng(nrhs).normal(size=(nrhs, m.n_tet))
+        ref, mag = x @ A.T, np.abs(x) @ np.abs(A).T
+        for dtype, u in (("fp64", 2.0 ** -53), ("fp32", 2.0 ** -24)):
+            y = op.matvec(torch.tensor(x, device="cuda"), dtype=dtype).cpu().numpy()
+            assert np.all(np.abs(y - ref) <= (2 * row + 4) * u * mag + 1e-300), (nrhs, dtype)
