@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
   __shared__ BlockCtx B;
   __shared__ __align__(16) ColF G;
   __shared__ unsigned s_w[kApexThreads / 32], s_base[4];
-  __shared__ int s_seg, s_wmax;
+  __shared__ int s_seg;
   const int tid = threadIdx.x, nq = a.one.nq, max_surf = a.one.max_surf, words = bit_words(a.one.max_tet);
   const BlockPtr P = block_ptr(smem, a.one.max_tet, max_surf, nq);
   Face* Fs = reinterpret_cast<Face*>(smem + (bits_smem(a.one.max_tet, max_surf, nq) + 15) / 16 * 16);
@@ -245,7 +245,6 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
       cur = s_seg;
       b -= a.prefix[cur];
     }
-    if (tid == 0) s_wmax = 0;
     __syncthreads();
     if (B.bw[b] == 0) continue;
     const int64_t I = b / B.n_col, J = b % B.n_col;
@@ -264,7 +263,6 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
     // windows of the faces, their places among the chunk's potentials
     int slo = 0, nsw = 0;
     if (tid < C.nsI) bits_surfaces(P.bits + tid * words, words, P.pan, slo, nsw);
-    if (nsw) atomicMax(&s_wmax, nsw);
     unsigned total;
     const unsigned ex = cta_scan((unsigned)(nsw * nq) | (nsw ? 1u << 24 : 0u), s_w, &total);
     const int nact = (int)(total >> 24);
@@ -282,10 +280,9 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
     }
     for (int k = tid; k < C.nsI * words; k += kApexThreads) a.bits[(g - a.g0) * max_surf * words + k] = P.bits[k];
     __syncthreads();
-    const int wmax = s_wmax, nr = nact * nq;
+    const int nr = nact * nq, lane = tid & 31;
     R* W = static_cast<R*>(a.W);
-    for (int r0 = 0; r0 < nr; r0 += kApexThreads) {
-      const int r = r0 + tid;
+    for (int r = tid; r - lane < nr; r += kApexThreads) {   // (whole warps)
       const bool on = r < nr;
       int n = 0, first = 0;
       uint32_t slot0 = 0;
@@ -311,6 +308,7 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
         }
       }
       bool any = false;
+      const int wmax = __reduce_max_sync(0xffffffffu, n);
       for (int s0 = 0; s0 < wmax; s0 += 64) {
         unsigned long long mask = 0;
         const int s1 = min(n, s0 + 64);
@@ -318,7 +316,12 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
           int cls;
           R F[3];
           if constexpr (FP32) {
-            cls = face_class_mixed(T, M, Fs[first + s], F);
+            // one FP32 sum settles what is far from the cone: the pairs' sums differ from
+            // it by less than the filter's margin
+            const FaceF& Fc = Fs[first + s];
+            const float mx = fmaxf(fmaxf(Fc.p_hi[0] + M.rho_hi[0], Fc.p_hi[1] + M.rho_hi[1]), Fc.p_hi[2] + M.rho_hi[2]);
+            cls = mx < -B.margin ? (int)FACE_LIT : Fc.pmin_hi + M.rlot_hi > B.margin ? (int)FACE_DARK
+                                                                                    : face_class_mixed(T, M, Fc, F);
           } else {
             double c;
             cls = face_class(B.cols[J], T, Fs[first + s], F, c);
@@ -327,15 +330,24 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
           else W[slot0 + s * nq] = cls == FACE_LIT ? Wst : R(0);
         }
         any |= mask != 0;
+        // places in the queues: a scan over the warp and one atomic per queue
         const unsigned cnt = (unsigned)__popcll(mask);
-        unsigned tot;
-        const unsigned at = cta_scan(far ? cnt : cnt << 16, s_w, &tot);
-        if (tid == 0) {
-          if (tot & 0xffffu) s_base[0] = atomicAdd(&a.cnt[CNT_FAR], tot & 0xffffu);
-          if (tot >> 16) s_base[2] = atomicAdd(&a.cnt[CNT_ANY], tot >> 16);
+        const unsigned mine = far ? cnt : cnt << 16;
+        unsigned at = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned u = __shfl_up_sync(0xffffffffu, at, o);
+          if (lane >= o) at += u;
         }
-        __syncthreads();
-        uint32_t* q = far ? a.q_far + s_base[0] + (at & 0xffffu) : a.q_any + s_base[2] + (at >> 16);
+        unsigned base_far = 0, base_any = 0;
+        if (lane == 31) {
+          if (at & 0xffffu) base_far = atomicAdd(&a.cnt[CNT_FAR], at & 0xffffu);
+          if (at >> 16) base_any = atomicAdd(&a.cnt[CNT_ANY], at >> 16);
+        }
+        base_far = __shfl_sync(0xffffffffu, base_far, 31);
+        base_any = __shfl_sync(0xffffffffu, base_any, 31);
+        at -= mine;
+        uint32_t* q = far ? a.q_far + base_far + (at & 0xffffu) : a.q_any + base_any + (at >> 16);
         while (mask) {
           const int s = s0 + __ffsll((long long)mask) - 1;
           mask &= mask - 1;
@@ -344,7 +356,6 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
           if constexpr (FP32) W[slot] = __uint_as_float(ray0 + r);
           else W[slot] = __hiloint2double(0, (int)(ray0 + r));
         }
-        __syncthreads();   // s_base is rewritten by the next round
       }
       if (any) {
         Apex Y;
@@ -405,17 +416,172 @@ __device__ __forceinline__ bool load_cut(const StageArgs& a, uint32_t slot, uint
   return true;
 }
 
-// FAR: the pairs of apexes in the far field; arcs the chord form refuses go
-// on to the other queue. A value that is not finite is recomputed in FP64.
-// Bound by issue and the latency of the gathers; 80 registers (6 CTAs per SM):
-// level-3 sphere, 8 slabs 211 ms of quadrature against 239 ms with 4 CTAs.
-template <bool FAR>
-__global__ void __launch_bounds__(kCutThreads, 6) k_cut(const StageArgs a) {
+// The crossings of the conic with edge k (as in face_cut): the lit part [la, lb]
+// of the edge and which ends are crossings; false: no lit part.
+__device__ __forceinline__ bool edge_lit(const CutF& c, int k, float& la, float& lb, bool& la_root, bool& lb_root) {
+  const int k1 = (k + 1) % 3;
+  const float Fa = c.in.F[k], Fb = c.in.F[k1];
+  la = 0.f;
+  lb = 1.f;
+  la_root = lb_root = false;
+  if (Fa < 0.f && Fb < 0.f) return true;
+  const float a0 = c.in.a0[k], a1 = c.in.a1[k], L = c.R.L[k];
+  const float Ex = c.R.U[k][0] * L, Ey = c.R.U[k][1] * L;
+  const float A2 = L * L - a1 * a1;
+  const float B2 = 2.f * ((c.T.q[k][0] * Ex + c.T.q[k][1] * Ey) + a0 * a1);
+  const float C2 = Fa * (c.T.rs[k] + a0);
+  // both roots, or one where the edge is parallel to the cone (r1 then fails every test below)
+  float r0 = 2.f, r1 = 2.f;
+  if (fabsf(A2) <= 1e-6f * (L * L + a1 * a1)) {
+    if (B2 != 0.f) r0 = -C2 / B2;
+  } else {
+    const float disc = B2 * B2 - 4.f * A2 * C2;
+    if (disc >= 0.f) {
+      const float sq = sqrtf(disc);
+      const float qq = -0.5f * (B2 + (B2 >= 0.f ? sq : -sq));
+      if (qq != 0.f) { r0 = qq / A2; r1 = C2 / qq; }
+      else r0 = 0.f;
+    }
+  }
+  const float slack = 1e-5f;
+  const bool ok0 = a0 - a1 * r0 > 0.f && r0 >= -slack && r0 <= 1.f + slack;
+  const bool ok1 = a0 - a1 * r1 > 0.f && r1 >= -slack && r1 <= 1.f + slack;
+  r0 = fminf(1.f, fmaxf(0.f, r0));
+  r1 = fminf(1.f, fmaxf(0.f, r1));
+  const float lo = ok0 ? (ok1 ? fminf(r0, r1) : r0) : r1, hi = ok0 ? (ok1 ? fmaxf(r0, r1) : r0) : r1;
+  if (Fa < 0.f) {           // exit on this edge
+    if (ok0 || ok1) { lb = hi; lb_root = true; }
+    return true;
+  }
+  if (Fb < 0.f) {           // entry on this edge
+    if (ok0 || ok1) { la = lo; la_root = true; }
+    return true;
+  }
+  if (ok0 && ok1 && hi > lo) {
+    la = lo; lb = hi; la_root = lb_root = true;
+    return true;
+  }
+  return false;
+}
+
+// (a function of its own for the same reason as whole_edge)
+__device__ __noinline__ bool chord_arc(const float* xb, float d, float C, float far_rho, const float* g, const float* A,
+                                       const float* D, const ArcRule& rule, float& out) {
+  return arc_far<float>(xb, d, C, far_rho, g, A, D, rule, out);
+}
+
+// The far field's cut faces (nine tenths of them on a fine sphere): a lit set
+// with one exit and one entry, so one arc and at most two edges with a crossing,
+// taken in registers; the edges' Gauss rules run in two converged turns (first
+// and second crossed edge) instead of three divergent ones. What has other
+// events, or an arc the chord form refuses, goes on to the other queue. The
+// arithmetic is face_cut's and arc_far's. Bound by issue and the latency of
+// the gathers: level-3 sphere, 8 slabs 193 -> 149 ms of quadrature against the
+// general code in this kernel (with the warp-wide queue places of k_apex), level-2
+// sphere, 32 slabs 106 -> 87 ms.
+__global__ void __launch_bounds__(kCutThreads, 6) k_cut_far(const StageArgs a) {
   float* W = static_cast<float*>(a.W);
-  const uint32_t* q = FAR ? a.q_far : a.q_any;
-  const unsigned n = a.cnt[FAR ? CNT_FAR : CNT_ANY];
+  const unsigned n = a.cnt[CNT_FAR];
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const uint32_t slot = q[i];
+    const uint32_t slot = a.q_far[i];
+    CutF c;
+    if (!load_cut(a, slot, __float_as_uint(W[slot]), c)) {
+      if (c.T.d == 0.f) push(a.q_64, 1, &a.cnt[CNT_COP], slot);
+      else push(a.q_64_last, -1, &a.cnt[CNT_F64], slot);
+      continue;
+    }
+    float t[3] = {0.f, 0.f, 0.f}, h2[2] = {0.f, 0.f};   // edge terms; the crossed edges' lit ranges
+    float l2[2] = {0.f, 0.f};
+    int k2[2] = {-1, -1}, n_exit = 0, n_entry = 0;
+    float A[2] = {0.f, 0.f}, E[2] = {0.f, 0.f};          // exit and entry, column coordinates
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      float la, lb;
+      bool ra, rb;
+      if (!edge_lit(c, k, la, lb, ra, rb)) continue;
+      if (!ra && !rb) {
+        t[k] = c.T.Efull[k];
+        continue;
+      }
+      const int z = k2[0] < 0 ? 0 : 1;   // (a third crossed edge has other events: not taken here)
+      if (z == 0) { k2[0] = k; l2[0] = la; h2[0] = lb; }
+      else { k2[1] = k; l2[1] = la; h2[1] = lb; }
+      const float Ux = c.R.U[k][0], Uy = c.R.U[k][1], L = c.R.L[k];
+      if (ra) { ++n_entry; E[0] = c.R.Q[k][0] + la * Ux * L; E[1] = c.R.Q[k][1] + la * Uy * L; }
+      if (rb) { ++n_exit; A[0] = c.R.Q[k][0] + lb * Ux * L; A[1] = c.R.Q[k][1] + lb * Uy * L; }
+    }
+    if (n_exit + n_entry == 0) {
+      const float G2 = c.in.g[0] * c.in.g[0] + c.in.g[1] * c.in.g[1];
+      if (!(G2 < 1.f && c.in.c > 0.f && c.in.D0 > 0.f)) W[slot] = 0.f;   // no closed ellipse: nothing lit
+      else push(a.q_any, 1, &a.cnt[CNT_ANY], slot);
+      continue;
+    }
+    if (n_exit != 1 || n_entry != 1) {
+      push(a.q_any, 1, &a.cnt[CNT_ANY], slot);
+      continue;
+    }
+    // the crossed edges
+    float m2[2], hh[2];
+#pragma unroll 1
+    for (int z = 0; z < 2; ++z) {
+      const int k = k2[z];
+      m2[z] = hh[z] = 0.f;
+      if (k < 0) continue;
+      const float la = l2[z], lb = h2[z];
+      const float h = 0.5f * (lb - la);
+      if (!(h > 0.f)) continue;
+      const float mid = 0.5f * (la + lb);
+      const float L = k == 0 ? c.R.L[0] : k == 1 ? c.R.L[1] : c.R.L[2];
+      const float ps = k == 0 ? c.T.ps[0] : k == 1 ? c.T.ps[1] : c.T.ps[2];
+      const float ws = k == 0 ? c.T.ws[0] : k == 1 ? c.T.ws[1] : c.T.ws[2];
+      const float Ux = k == 0 ? c.R.U[0][0] : k == 1 ? c.R.U[1][0] : c.R.U[2][0];
+      const float Uy = k == 0 ? c.R.U[0][1] : k == 1 ? c.R.U[1][1] : c.R.U[2][1];
+      const float Qx = k == 0 ? c.R.Q[0][0] : k == 1 ? c.R.Q[1][0] : c.R.Q[2][0];
+      const float Qy = k == 0 ? c.R.Q[0][1] : k == 1 ? c.R.Q[1][1] : c.R.Q[2][1];
+      const float q0x = -c.T.xb[0], q0y = -c.T.xb[1];
+      const int nn = gauss_order<float>((-ws / L - mid) / h, fabsf(ps) / (L * h), a.one.rule.ltol_f, 3, 10);
+      const float* X = gl_nodes<float>(nn);
+      const float* Wt = gl_weights<float>(nn);
+      const float ex = Ux * L, ey = Uy * L, d2 = c.T.d * c.T.d;
+      float acc = 0.f;
+      for (int g = 0; g < nn; ++g) {
+        const float lam = mid + h * X[g];
+        const float ux = Qx + lam * ex, uy = Qy + lam * ey;
+        const float qx = q0x + ux, qy = q0y + uy, q2 = qx * qx + qy * qy;
+        const float r = sqrtf(q2 + d2);
+        const float del = (ux * (2.f * q0x + ux) + uy * (2.f * q0y + uy)) / (r + c.T.C);
+        acc += Wt[g] * del / q2;
+      }
+      m2[z] = acc * ps * L;
+      hh[z] = h;
+    }
+    float v = 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (k == k2[0]) v = __fadd_rn(v, __fmul_rn(m2[0], hh[0]));
+      else if (k == k2[1]) v = __fadd_rn(v, __fmul_rn(m2[1], hh[1]));
+      else v += t[k];
+    }
+    const float D[2] = {E[0] - A[0], E[1] - A[1]};
+    float arc = 0.f;
+    if (!chord_arc(c.T.xb, c.T.d, c.T.C, c.T.far_rho, c.in.g, A, D, a.one.rule, arc)) {
+      push(a.q_any, 1, &a.cnt[CNT_ANY], slot);
+      continue;
+    }
+    v += arc;
+    if (!isfinite(v)) push(a.q_64_last, -1, &a.cnt[CNT_F64], slot);
+    else W[slot] = v;
+  }
+}
+
+// The other cut faces: near apexes, several arcs, whole ellipses. A value that
+// is not finite is recomputed in FP64. Bound by issue with about half of the
+// lanes at work; 80 registers (6 CTAs per SM).
+__global__ void __launch_bounds__(kCutThreads, 6) k_cut_any(const StageArgs a) {
+  float* W = static_cast<float*>(a.W);
+  const unsigned n = a.cnt[CNT_ANY];
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t slot = a.q_any[i];
     CutF c;
     if (!load_cut(a, slot, __float_as_uint(W[slot]), c)) {
       if (c.T.d == 0.f) push(a.q_64, 1, &a.cnt[CNT_COP], slot);
@@ -425,19 +591,8 @@ __global__ void __launch_bounds__(kCutThreads, 6) k_cut(const StageArgs a) {
     ArcRec<float> arc[3];
     int na = 0;
     float v = (float)face_cut<float>(c.R, c.T, c.in, a.one.rule, arc, &na);
-    bool ok = true;
-    for (int k = 0; k < na; ++k) {
-      if (FAR) {
-        float t = 0.f;
-        ok = ok && arc[k].far && arc_far<float>(arc[k].xb, arc[k].d, arc[k].C, arc[k].far_rho, arc[k].g, arc[k].A,
-                                                arc[k].dAB, a.one.rule, t);
-        v += t;
-      } else {
-        v += arc_value<float>(arc[k], a.one.rule);
-      }
-    }
-    if (!ok) push(a.q_any, 1, &a.cnt[CNT_ANY], slot);
-    else if (!isfinite(v)) push(a.q_64_last, -1, &a.cnt[CNT_F64], slot);
+    for (int k = 0; k < na; ++k) v += arc_value<float>(arc[k], a.one.rule);
+    if (!isfinite(v)) push(a.q_64_last, -1, &a.cnt[CNT_F64], slot);
     else W[slot] = v;
   }
 }
@@ -714,8 +869,8 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
   const int n_apex = sms * std::max(1, std::min(per_sm, stage_apex_per_sm(fp32, mt, ms, nq)));
   int n_asm = sms * occupancy(k_asm, kAsmThreads, sm_asm);
   if (fixed > 256) n_asm = std::min(n_asm, sms * 4);   // one slab per CTA
-  const int n_far = sms * occupancy((const void*)(fp32 ? (const void*)k_cut<true> : (const void*)k_cut_d), kCutThreads, 0);
-  const int n_any = sms * occupancy((const void*)k_cut<false>, kCutThreads, 0);
+  const int n_far = sms * occupancy((const void*)(fp32 ? (const void*)k_cut_far : (const void*)k_cut_d), kCutThreads, 0);
+  const int n_any = sms * occupancy((const void*)k_cut_any, kCutThreads, 0);
   const int n_64 = sms * occupancy((const void*)k_cut_fp64, k64Threads, 0);
 
   struct Events {   // apex and FP32 faces done, entries done, per half
@@ -763,8 +918,8 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
     };
     if (fp32) {
       k_apex<float><<<n_apex, kApexThreads, sm_apex, s>>>(a);
-      k_cut<true><<<n_far, kCutThreads, 0, s>>>(a);
-      k_cut<false><<<n_any, kCutThreads, 0, s>>>(a);
+      k_cut_far<<<n_far, kCutThreads, 0, s>>>(a);
+      k_cut_any<<<n_any, kCutThreads, 0, s>>>(a);
       st = hand_over();
       if (st != BEM_OK) return st;
       k_cut_fp64<<<n_64, k64Threads, 0, t>>>(a);
