@@ -618,7 +618,7 @@ void bem_operator_destroy(bem_operator* op) {
   cudaFree(op->d_boff); cudaFree(op->d_rsoff); cudaFree(op->d_rs); cudaFree(op->d_val);
   cudaFree(op->d_val32); cudaFree(op->d_tmp); cudaFree(op->d_counter);
   cudaFree(op->d_ws); cudaFree(op->d_pv);
-  cudaFree(op->d_tc_colptr); cudaFree(op->d_tc_blk); cudaFree(op->d_tc_err);
+  cudaFree(op->d_tc_gptr); cudaFree(op->d_tc_gtb); cudaFree(op->d_tc_rs); cudaFree(op->d_tc_blk); cudaFree(op->d_tc_err);
   cudaFree(op->d_tcv[0]); cudaFree(op->d_tcv[1]);
   delete op;
 }

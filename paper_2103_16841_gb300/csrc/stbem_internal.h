@@ -146,7 +146,11 @@ struct bem_operator {
   mutable int64_t ws_len = 0;
   mutable double* d_pv = nullptr;       // caller-order <-> internal-order vectors of the products
   mutable int64_t pv_len = 0;           // (stream-ordered allocation, grown on demand)
-  mutable int32_t* d_tc_colptr = nullptr;  // tensor-core product: non-empty blocks per test column
+  mutable int32_t* d_tc_gptr = nullptr;    // tensor-core product: non-empty blocks per row group,
+  mutable int32_t* d_tc_gtb = nullptr;     // first row per group, row starts in the groups' row order
+  mutable int32_t* d_tc_rs = nullptr;
+  mutable int64_t tc_groups = 0, tc_nrows = 0;
+  mutable int tc_rows = 0;                 // most rows of a group
   mutable void* d_tc_blk = nullptr;        // (TcBlk records, trial columns ascending)
   mutable int64_t tc_nblk = 0;
   mutable int tc_span[2] = {0, 0};         // widest band union of a block from a BF16 / TF32 chunk boundary

@@ -23,7 +23,17 @@
 //   assembled values, BF16 or TF32-rounded, about 1.1-1.25 x their bytes).
 //   Building a block's A tile is then a copy of whole chunks.
 //
-// One CTA per test column I, six warps:
+// The MMA's 128 rows hold as many consecutive test columns as fit ("row
+// groups": five columns of 24 panels), so "block" below is a row group against
+// a trial column: its rows' row starts and chunk slots are kept in the group's
+// order. Per block the pipeline costs about a microsecond whatever its size,
+// and a column of 24 panels used a fifth of the tile. The blocks of a group are
+// shared by PARTS CTAs, whose sums are added at the end, where groups are few.
+// Level-3 sphere, 8 slabs: BF16 with 13 right-hand sides 2.26 -> 0.61 ms, TF32
+// with 64 2.59 -> 1.01 ms; level-2 sphere, 32 slabs (a column per group, two
+// parts), 64 right-hand sides: TF32 0.78 -> 0.64 ms, BF16 0.49 -> 0.41 ms.
+//
+// One CTA per (row group, part), six warps:
 //   warps 0-3  build the A tile of each block (thread = row: its slots to
 //              their chunk positions, the previous band's other chunks
 //              cleared) in shared memory (k_spmm_tc) or in tensor memory with
@@ -58,16 +68,16 @@
 
 namespace stbem {
 
-// One non-empty block of a test column, in the order of its trial columns.
+// One non-empty block of a row group, in the order of its trial columns.
 struct TcBlk {
   int32_t je;          // end of trial column J (internal panel index)
-  int32_t W;           // band width
-  int32_t nt;          // rows (panels of column I)
+  int32_t W;           // widest band of its columns
+  int32_t nt;          // rows (panels of the group's columns)
   int32_t cmin;        // union of the rows' bands [cmin, cend), clipped to J
   int32_t cend;
-  int32_t pad;
-  int64_t vo;          // value offset in the assembled storage
-  int64_t ro;          // row-start offset
+  int32_t t0;          // first row
+  int64_t J;           // trial column
+  int64_t ro;          // row-start offset (the groups' row order)
   int64_t vc[2];       // offset of the block's chunk slots (16-byte units): BF16, TF32
   int64_t pad2;
 };
@@ -94,21 +104,27 @@ constexpr uint32_t kMetaOff = 896;
 // chunk slots of a row's band of width W (E values per chunk)
 __host__ __device__ constexpr int tc_slots(int W, int E) { return (W + 2 * E - 2) / E; }
 
-__global__ void k_tc_meta(int64_t nb, const int32_t* __restrict__ bI, const int32_t* __restrict__ bJ,
-                          const int64_t* __restrict__ vc16, const int64_t* __restrict__ vc32, int64_t n_col,
-                          const int32_t* __restrict__ ctb, const int32_t* __restrict__ bw,
-                          const int64_t* __restrict__ boff, const int64_t* __restrict__ rsoff,
-                          const int32_t* __restrict__ rs, TcBlk* __restrict__ out, int* __restrict__ span) {
+// Block records (warp per block) and the row starts in the groups' row order.
+// Rows whose own column has no values in the block get an empty band at the
+// block's first panel.
+__global__ void k_tc_meta(int64_t nb, const int32_t* __restrict__ bG, const int32_t* __restrict__ bJ,
+                          const int32_t* __restrict__ bW, const int64_t* __restrict__ ro_, const int64_t* __restrict__ vc16,
+                          const int64_t* __restrict__ vc32, int64_t n_col, const int32_t* __restrict__ gtb,
+                          const int32_t* __restrict__ ctb, const TetDev* __restrict__ tets, const int32_t* __restrict__ bw,
+                          const int64_t* __restrict__ rsoff, const int32_t* __restrict__ rs, TcBlk* __restrict__ out,
+                          int32_t* __restrict__ prs, int* __restrict__ span) {
   const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (k >= nb) return;
-  const int64_t I = bI[k], J = bJ[k], b = I * n_col + J;
-  const int nt = ctb[I + 1] - ctb[I];
-  const int W = bw[b];
-  const int64_t ro = rsoff[b];
+  const int64_t J = bJ[k], ro = ro_[k];
+  const int t0 = gtb[bG[k]], nt = gtb[bG[k] + 1] - t0;
   int lo = INT_MAX, hi = INT_MIN;
   for (int r = lane; r < nt; r += 32) {
-    const int s = rs[ro + r];
+    const int I = tets[t0 + r].col;
+    const int64_t b = I * n_col + J;
+    const int W = bw[b];
+    if (W <= 0) continue;
+    const int s = rs[rsoff[b] + (t0 + r - ctb[I])];
     lo = min(lo, s);
     hi = max(hi, s + W);
   }
@@ -117,17 +133,22 @@ __global__ void k_tc_meta(int64_t nb, const int32_t* __restrict__ bI, const int3
     lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
     hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
   }
+  for (int r = lane; r < nt; r += 32) {
+    const int I = tets[t0 + r].col;
+    const int64_t b = I * n_col + J;
+    prs[ro + r] = bw[b] > 0 ? rs[rsoff[b] + (t0 + r - ctb[I])] : lo;
+  }
   if (lane == 0) {
     const int je = ctb[J + 1];
     hi = min(hi, je);
     TcBlk t;
     t.je = je;
-    t.W = W;
+    t.W = bW[k];
     t.nt = nt;
     t.cmin = lo;
     t.cend = hi;
-    t.pad = 0;
-    t.vo = boff[b];
+    t.t0 = t0;
+    t.J = J;
     t.ro = ro;
     t.vc[0] = vc16[k];
     t.vc[1] = vc32[k];
@@ -143,7 +164,9 @@ __global__ void k_tc_meta(int64_t nb, const int32_t* __restrict__ bI, const int3
 // row's band (and in column J), zeros elsewhere; BF16 or TF32-rounded FP32.
 template <bool TF32, typename V>
 __global__ void k_tc_pack_vals(int64_t nb, const TcBlk* __restrict__ blk, const V* __restrict__ val,
-                               const int32_t* __restrict__ rs, uint4* __restrict__ out) {
+                               const int32_t* __restrict__ prs, int64_t n_col, const int32_t* __restrict__ ctb,
+                               const TetDev* __restrict__ tets, const int32_t* __restrict__ bw,
+                               const int64_t* __restrict__ boff, uint4* __restrict__ out) {
   constexpr int E = TF32 ? 4 : 8;
   const int lane = threadIdx.x & 31;
   for (int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; k < nb;
@@ -152,25 +175,29 @@ __global__ void k_tc_pack_vals(int64_t nb, const TcBlk* __restrict__ blk, const 
     const int S = tc_slots(b.W, E), nt = b.nt;
     for (int idx = lane; idx < S * nt; idx += 32) {
       const int j = idx / nt, r = idx - j * nt;
-      const int st = rs[b.ro + r];
+      const int st = prs[b.ro + r];
       const int base = (st / E) * E + j * E;
+      // the row's own column: its band width, values and rows
+      const int I = tets[b.t0 + r].col;
+      const int64_t ib = I * n_col + b.J;
+      const int Wr = bw[ib], ntr = ctb[I + 1] - ctb[I];
+      const V* vr = val + boff[ib] + (b.t0 + r - ctb[I]);
+      auto at = [&](int col) {
+        const int w = col - st;
+        return (w >= 0 && w < Wr && col < b.je) ? (float)vr[(int64_t)w * ntr] : 0.f;
+      };
       uint32_t wv[4];
 #pragma unroll
       for (int h = 0; h < 4; ++h) {
         if (TF32) {
-          const int col = base + h, w = col - st;
-          const float v = (w >= 0 && w < b.W && col < b.je) ? (float)val[b.vo + (int64_t)w * nt + r] : 0.f;
           uint32_t t;
-          asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(t) : "f"(v));
+          asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(t) : "f"(at(base + h)));
           wv[h] = t;
         } else {
           uint32_t p = 0;
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int col = base + 2 * h + e, w = col - st;
-            const float v = (w >= 0 && w < b.W && col < b.je) ? (float)val[b.vo + (int64_t)w * nt + r] : 0.f;
-            p |= (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v)) << (16 * e);
-          }
+          for (int e = 0; e < 2; ++e)
+            p |= (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(at(base + 2 * h + e))) << (16 * e);
           wv[h] = p;
         }
       }
@@ -202,18 +229,19 @@ __global__ void k_pack_xc(const double* __restrict__ x, int64_t n_tet, int nr, i
 }
 
 struct TcArgs {
-  const int32_t* ctb;
-  const int32_t* colptr;   // [n_col + 1] into blk
+  const int32_t* gtb;      // [groups + 1] first row of a group
+  const int32_t* gptr;     // [groups + 1] into blk
   const TcBlk* blk;
   const uint4* vals;       // chunk slots of the product's type
   const int32_t* rs;       // row starts (16 bytes of tail room)
-  double* y;               // [nr][n_tet] (internal order)
+  double* y;               // [parts][nr][n_tet] (internal order)
   int64_t n_tet;
   int nr, N;               // right-hand sides of the pass, MMA N (multiple of 16)
   int nkc;                 // chunk capacity of a stage's A and B tiles (even)
   uint32_t v_bytes;        // capacity of a stage's value buffer (multiple of 1024)
   int stages;
   uint32_t tmem_cols;
+  int parts;               // CTAs that share a group's blocks
   int* err;                // set to 1 when a wait ran out of budget
 };
 
@@ -227,9 +255,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_spmm_tc(const TcArgs a, const _
   constexpr int ROWS = MT * 128;
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t I = blockIdx.x;
-  const int t0 = a.ctb[I], nt = a.ctb[I + 1] - t0;
-  const int b0 = a.colptr[I], nb = a.colptr[I + 1] - b0;
+  const int g = blockIdx.x / a.parts, part = blockIdx.x - g * a.parts;
+  const int t0 = a.gtb[g], nt = a.gtb[g + 1] - t0;
+  const int nbg = a.gptr[g + 1] - a.gptr[g];
+  const int b0 = a.gptr[g] + (int)((int64_t)nbg * part / a.parts);
+  const int nb = a.gptr[g] + (int)((int64_t)nbg * (part + 1) / a.parts) - b0;
+  double* y = a.y + (int64_t)part * a.nr * a.n_tet;
   const int ST = a.stages, N = a.N;
   const uint32_t a_bytes = (uint32_t)a.nkc * ROWS * 16, b_bytes = (uint32_t)a.nkc * N * 16;
   const uint32_t stage_bytes = a_bytes + b_bytes + a.v_bytes + kRsBytes;
@@ -338,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_spmm_tc(const TcArgs a, const _
             const int n = c + j;
             if (n < a.nr) {
               const double o = nb == 0 ? 0.0 : bad ? __longlong_as_double(0x7ff8000000000000LL) : (double)v[j];
-              a.y[(int64_t)n * a.n_tet + t0 + r] = o;
+              y[(int64_t)n * a.n_tet + t0 + r] = o;
             }
           }
         }
@@ -421,9 +452,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_spmm_tm(const TcArgs a, const _
   constexpr int E = TF32 ? 4 : 8;         // elements per 16-byte chunk
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t I = blockIdx.x;
-  const int t0 = a.ctb[I], nt = a.ctb[I + 1] - t0;
-  const int b0 = a.colptr[I], nb = a.colptr[I + 1] - b0;
+  const int g = blockIdx.x / a.parts, part = blockIdx.x - g * a.parts;
+  const int t0 = a.gtb[g], nt = a.gtb[g + 1] - t0;
+  const int nbg = a.gptr[g + 1] - a.gptr[g];
+  const int b0 = a.gptr[g] + (int)((int64_t)nbg * part / a.parts);
+  const int nb = a.gptr[g] + (int)((int64_t)nbg * (part + 1) / a.parts) - b0;
+  double* y = a.y + (int64_t)part * a.nr * a.n_tet;
   const int ST = a.stages, N = a.N, NKC = a.nkc;
   const uint32_t b_bytes = (uint32_t)NKC * N * 16;
   const uint32_t stage_bytes = b_bytes + a.v_bytes + kRsBytes;
@@ -539,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_spmm_tm(const TcArgs a, const _
             const int n = c + j;
             if (n < a.nr) {
               const double o = nb == 0 ? 0.0 : bad ? __longlong_as_double(0x7ff8000000000000LL) : (double)v[j];
-              a.y[(int64_t)n * a.n_tet + t0 + r] = o;
+              y[(int64_t)n * a.n_tet + t0 + r] = o;
             }
           }
         }
@@ -626,9 +660,19 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// Block records of the operator (made once; an operator's sparsity
-// structure never changes): the non-empty blocks of each test column, their
-// band unions and the offsets of their chunk slots in both types.
+// y = the sum of the parts, in order
+__global__ void k_tc_sum(const double* __restrict__ part, double* __restrict__ y, int64_t n, int parts) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    double s = 0.0;
+    for (int p = 0; p < parts; ++p) s += part[p * n + i];
+    y[i] = s;
+  }
+}
+
+// Row groups and block records of the operator (made once; an operator's
+// sparsity structure never changes): the non-empty blocks of each group, their
+// band unions, the offsets of their chunk slots in both types, and the row
+// starts in the groups' row order.
 bem_status ensure_tc_meta(const bem_operator* op, cudaStream_t s) {
   if (op->d_tc_blk) return BEM_OK;
   const bem_mesh* m = op->mesh;
@@ -636,76 +680,92 @@ bem_status ensure_tc_meta(const bem_operator* op, cudaStream_t s) {
   std::vector<int32_t> hbw(nc * nc);
   STBEM_CUDA(cudaMemcpyAsync(hbw.data(), op->d_bw, sizeof(int32_t) * nc * nc, cudaMemcpyDeviceToHost, s));
   STBEM_CUDA(cudaStreamSynchronize(s));
-  std::vector<int32_t> colptr(nc + 1, 0), bI, bJ;
-  std::vector<int64_t> vc16, vc32;
-  int64_t o16 = 0, o32 = 0, cap16 = 0, cap32 = 0;
-  for (int64_t I = 0; I < nc; ++I) {
-    const int64_t nt = m->col_tet_begin[I + 1] - m->col_tet_begin[I];
+  // consecutive columns to at most 128 rows (one M tile); a taller column is a group of its own
+  std::vector<int32_t> gcol{0}, gtb{0};
+  int max_rows = 0;
+  for (int64_t I = 0; I < nc;) {
+    int64_t e = I + 1;
+    while (e < nc && m->col_tet_begin[e + 1] - m->col_tet_begin[I] <= 128) ++e;
+    max_rows = std::max(max_rows, m->col_tet_begin[e] - m->col_tet_begin[I]);
+    gcol.push_back((int32_t)e);
+    gtb.push_back(m->col_tet_begin[e]);
+    I = e;
+  }
+  const int64_t ng = (int64_t)gcol.size() - 1;
+  std::vector<int32_t> ptr(ng + 1, 0), bG, bJ, bW, wmax(nc);
+  std::vector<int64_t> ro, vc16, vc32;
+  int64_t orow = 0, o16 = 0, o32 = 0, cap16 = 0, cap32 = 0;
+  for (int64_t g = 0; g < ng; ++g) {
+    const int64_t nt = gtb[g + 1] - gtb[g];
+    std::fill(wmax.begin(), wmax.end(), 0);
+    for (int64_t I = gcol[g]; I < gcol[g + 1]; ++I)
+      for (int64_t J = 0; J < nc; ++J) wmax[J] = std::max(wmax[J], hbw[I * nc + J]);
     for (int64_t J = 0; J < nc; ++J) {
-      const int W = hbw[I * nc + J];
+      const int W = wmax[J];
       if (W <= 0) continue;
-      bI.push_back((int32_t)I);
+      bG.push_back((int32_t)g);
       bJ.push_back((int32_t)J);
+      bW.push_back(W);
+      ro.push_back(orow);
       vc16.push_back(o16);
       vc32.push_back(o32);
+      orow += nt;
       o16 += tc_slots(W, 8) * nt;
       o32 += tc_slots(W, 4) * nt;
       cap16 = std::max<int64_t>(cap16, tc_slots(W, 8) * nt * 16);
       cap32 = std::max<int64_t>(cap32, tc_slots(W, 4) * nt * 16);
     }
-    colptr[I + 1] = (int32_t)bI.size();
+    ptr[g + 1] = (int32_t)bG.size();
   }
-  const int64_t nb = (int64_t)bI.size();
-  int32_t *d_ptr = nullptr, *d_I = nullptr, *d_J = nullptr;
-  int64_t *d_v16 = nullptr, *d_v32 = nullptr;
-  int* d_span = nullptr;
-  void* d_blk = nullptr;
-  auto cleanup = [&]() {
-    cudaFree(d_I); cudaFree(d_J); cudaFree(d_v16); cudaFree(d_v32); cudaFree(d_span);
-  };
+  const int64_t nb = (int64_t)bG.size();
+  struct Arrays {   // freed on every way out unless released
+    void* p[11] = {};
+    ~Arrays() { for (void* q : p) cudaFree(q); }
+  } A;
   const size_t nb1 = (size_t)std::max<int64_t>(nb, 1);
-  if (cudaMalloc(&d_ptr, sizeof(int32_t) * (nc + 1)) != cudaSuccess ||
-      cudaMalloc(&d_blk, sizeof(TcBlk) * nb1) != cudaSuccess || cudaMalloc(&d_I, sizeof(int32_t) * nb1) != cudaSuccess ||
-      cudaMalloc(&d_J, sizeof(int32_t) * nb1) != cudaSuccess || cudaMalloc(&d_v16, sizeof(int64_t) * nb1) != cudaSuccess ||
-      cudaMalloc(&d_v32, sizeof(int64_t) * nb1) != cudaSuccess || cudaMalloc(&d_span, sizeof(int) * 2) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(d_ptr); cudaFree(d_blk);
-    cleanup();
-    set_error("out of device memory (tensor-core product tables)");
-    return BEM_ERR_OUT_OF_MEMORY;
-  }
+  const size_t bytes[11] = {sizeof(int32_t) * (ng + 1), sizeof(int32_t) * (ng + 1), sizeof(TcBlk) * nb1,
+                            sizeof(int32_t) * (size_t)(orow + 4) /* whole 16-byte granules are copied */, sizeof(int32_t) * nb1,
+                            sizeof(int32_t) * nb1, sizeof(int32_t) * nb1, sizeof(int64_t) * nb1, sizeof(int64_t) * nb1,
+                            sizeof(int64_t) * nb1, sizeof(int) * 2};
+  for (int k = 0; k < 11; ++k)
+    if (cudaMalloc(&A.p[k], bytes[k]) != cudaSuccess) {
+      cudaGetLastError();
+      A.p[k] = nullptr;
+      set_error("out of device memory (tensor-core product tables)");
+      return BEM_ERR_OUT_OF_MEMORY;
+    }
   int hspan[2] = {0, 0};
-  cudaMemcpyAsync(d_ptr, colptr.data(), sizeof(int32_t) * (nc + 1), cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(d_span, hspan, sizeof(hspan), cudaMemcpyHostToDevice, s);
+  const void* src[11] = {ptr.data(), gtb.data(), nullptr, nullptr, bG.data(), bJ.data(), bW.data(),
+                         ro.data(), vc16.data(), vc32.data(), hspan};
+  for (int k = 0; k < 11; ++k)
+    if (src[k] && (nb > 0 || k < 2 || k == 10)) STBEM_CUDA(cudaMemcpyAsync(A.p[k], src[k], bytes[k], cudaMemcpyHostToDevice, s));
   if (nb > 0) {
-    cudaMemcpyAsync(d_I, bI.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(d_J, bJ.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(d_v16, vc16.data(), sizeof(int64_t) * nb, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(d_v32, vc32.data(), sizeof(int64_t) * nb, cudaMemcpyHostToDevice, s);
     const int64_t threads = nb * 32;
-    k_tc_meta<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(nb, d_I, d_J, d_v16, d_v32, nc, m->d_col_tet_begin,
-                                                                op->d_bw, op->d_boff, op->d_rsoff, op->d_rs,
-                                                                static_cast<TcBlk*>(d_blk), d_span);
+    k_tc_meta<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(
+        nb, (const int32_t*)A.p[4], (const int32_t*)A.p[5], (const int32_t*)A.p[6], (const int64_t*)A.p[7],
+        (const int64_t*)A.p[8], (const int64_t*)A.p[9], nc, (const int32_t*)A.p[1], m->d_col_tet_begin, m->d_tet, op->d_bw,
+        op->d_rsoff, op->d_rs, (TcBlk*)A.p[2], (int32_t*)A.p[3], (int*)A.p[10]);
+    STBEM_CUDA(cudaGetLastError());
   }
-  cudaMemcpyAsync(hspan, d_span, sizeof(hspan), cudaMemcpyDeviceToHost, s);
-  const cudaError_t e = cudaStreamSynchronize(s);
-  cleanup();
-  if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) {
-    cudaFree(d_ptr); cudaFree(d_blk);
-    set_error(std::string("tensor-core product tables: ") + cudaGetErrorString(e));
-    return BEM_ERR_CUDA;
-  }
+  STBEM_CUDA(cudaMemcpyAsync(hspan, A.p[10], sizeof(hspan), cudaMemcpyDeviceToHost, s));
+  STBEM_CUDA(cudaStreamSynchronize(s));
   if (!op->d_tc_err) {
     if (cudaMalloc(&op->d_tc_err, sizeof(int)) != cudaSuccess) {
       cudaGetLastError();
-      cudaFree(d_ptr); cudaFree(d_blk);
+      op->d_tc_err = nullptr;
       set_error("out of device memory (tensor-core product flag)");
       return BEM_ERR_OUT_OF_MEMORY;
     }
-    cudaMemsetAsync(op->d_tc_err, 0, sizeof(int), s);
+    STBEM_CUDA(cudaMemsetAsync(op->d_tc_err, 0, sizeof(int), s));
   }
-  op->d_tc_colptr = d_ptr;
-  op->d_tc_blk = d_blk;
+  op->d_tc_gptr = (int32_t*)A.p[0];
+  op->d_tc_gtb = (int32_t*)A.p[1];
+  op->d_tc_blk = A.p[2];
+  op->d_tc_rs = (int32_t*)A.p[3];
+  for (int k = 0; k < 4; ++k) A.p[k] = nullptr;
+  op->tc_groups = ng;
+  op->tc_rows = max_rows;
+  op->tc_nrows = orow;
   op->tc_nblk = nb;
   op->tc_span[0] = hspan[0];
   op->tc_span[1] = hspan[1];
@@ -732,20 +792,25 @@ bem_status ensure_tc_vals(const bem_operator* op, bool tf32, cudaStream_t s) {
   const TcBlk* blk = static_cast<const TcBlk*>(op->d_tc_blk);
   uint4* out = static_cast<uint4*>(op->d_tcv[t]);
   const unsigned grid = (unsigned)std::min<int64_t>((op->tc_nblk * 32 + 255) / 256, 152 * 32);
-  if (tf32) k_tc_pack_vals<true, float><<<grid, 256, 0, s>>>(op->tc_nblk, blk, op->d_val32, op->d_rs, out);
-  else if (op->d_val32) k_tc_pack_vals<false, float><<<grid, 256, 0, s>>>(op->tc_nblk, blk, op->d_val32, op->d_rs, out);
-  else k_tc_pack_vals<false, double><<<grid, 256, 0, s>>>(op->tc_nblk, blk, op->d_val, op->d_rs, out);
+  const bem_mesh* m = op->mesh;
+  auto pack = [&](auto kern, auto* val) {
+    kern<<<grid, 256, 0, s>>>(op->tc_nblk, blk, val, op->d_tc_rs, m->n_col, m->d_col_tet_begin, m->d_tet, op->d_bw, op->d_boff,
+                              out);
+  };
+  if (tf32) pack(k_tc_pack_vals<true, float>, op->d_val32);
+  else if (op->d_val32) pack(k_tc_pack_vals<false, float>, op->d_val32);
+  else pack(k_tc_pack_vals<false, double>, op->d_val);
   STBEM_CUDA(cudaGetLastError());
   return BEM_OK;
 }
 
 // kind 0: A tiles in shared memory (k_spmm_tc); kind 1: in tensor memory (k_spmm_tm)
 template <bool TF32, int MT>
-bem_status launch_tc(int kind, const TcArgs& a, const CUtensorMap& map, size_t smem, int64_t n_col, cudaStream_t s) {
+bem_status launch_tc(int kind, const TcArgs& a, const CUtensorMap& map, size_t smem, int64_t n_cta, cudaStream_t s) {
   const void* kern = kind ? (const void*)k_spmm_tm<TF32, MT> : (const void*)k_spmm_tc<TF32, MT>;
   TRY_STATUS(ensure_smem_attr(kern, smem));
-  if (kind) k_spmm_tm<TF32, MT><<<(unsigned)n_col, kThreads, smem, s>>>(a, map);
-  else k_spmm_tc<TF32, MT><<<(unsigned)n_col, kThreads, smem, s>>>(a, map);
+  if (kind) k_spmm_tm<TF32, MT><<<(unsigned)n_cta, kThreads, smem, s>>>(a, map);
+  else k_spmm_tc<TF32, MT><<<(unsigned)n_cta, kThreads, smem, s>>>(a, map);
   STBEM_CUDA(cudaGetLastError());
   return BEM_OK;
 }
@@ -753,7 +818,7 @@ bem_status launch_tc(int kind, const TcArgs& a, const CUtensorMap& map, size_t s
 }  // namespace
 
 int64_t tc_table_bytes(const bem_operator* op) {
-  int64_t b = op->d_tc_blk ? op->tc_nblk * (int64_t)sizeof(TcBlk) + (op->mesh->n_col + 1) * 4 : 0;
+  int64_t b = op->d_tc_blk ? op->tc_nblk * (int64_t)sizeof(TcBlk) + (op->tc_groups + 1) * 8 + op->tc_nrows * 4 : 0;
   for (int t = 0; t < 2; ++t)
     if (op->d_tcv[t]) b += op->tcv_len[t] * 16;
   return b;
@@ -780,7 +845,19 @@ bem_status op_spmm_tc(const bem_operator* op, const double* x, double* y, int nr
   const int E = bf16 ? 8 : 4;
   const int N = std::max(16, (nrhs + 15) / 16 * 16);
   const int64_t nchunks = (n + E - 1) / E;
-  TRY_STATUS(ensure_ws(op, nchunks * N * 4));   // 16 bytes per (chunk, rhs)
+  // parts: some four CTAs per SM in all, of at least eight blocks each. The
+  // tensor cores' FP32 accumulation truncates, so a row's sum cut in parts
+  // comes out closer to the exact one, by an amount that grows with the row:
+  // the level-3 sphere with 8 slabs (11,300 values per row) moves by 1.2e-5 in
+  // BF16 and 1.9e-5 in TF32 with two parts, the level-2 sphere with 32 slabs
+  // (5,300) by 4e-6 and 6e-6. Long rows are therefore cut in two at most, or
+  // left whole, to stay within 1.3e-5 of the uncut sum.
+  const int64_t per_group = op->tc_nblk / std::max<int64_t>(op->tc_groups, 1), per_row = op->nstored / n;
+  const int most = per_row > 8000 ? (bf16 ? 2 : 1) : per_row > 3000 ? 2 : 8;
+  int parts = 1;
+  while (parts < most && op->tc_groups * parts < 4 * 152 && per_group >= 16 * parts) parts *= 2;
+  const int64_t xc_len = nchunks * N * 4;       // 16 bytes per (chunk, rhs)
+  TRY_STATUS(ensure_ws(op, xc_len + (parts > 1 ? 2 * parts * n * nrhs : 0)));
   void* Xc = op->d_ws;
   if (bf16) k_pack_xc<false><<<grid_for(nchunks * N * E), 256, 0, s>>>(x, n, nrhs, N, nchunks, Xc);
   else k_pack_xc<true><<<grid_for(nchunks * N * E), 256, 0, s>>>(x, n, nrhs, N, nchunks, Xc);
@@ -801,7 +878,7 @@ bem_status op_spmm_tc(const bem_operator* op, const double* x, double* y, int nr
     set_error("tensor-core product: tensor map rejected (" + std::to_string((int)r) + ")");
     return BEM_ERR_CUDA;
   }
-  const int MT = m->max_col_tets > 128 ? 2 : 1;
+  const int MT = op->tc_rows > 128 ? 2 : 1;
   const int span = std::max(op->tc_span[bf16 ? 0 : 1], 1);
   const int nkc = 2 * ((span + 2 * E - 1) / (2 * E));
   // value slots of the largest block; a multiple of 1024 bytes keeps every
@@ -819,12 +896,13 @@ bem_status op_spmm_tc(const bem_operator* op, const double* x, double* y, int nr
     smem_max = (size_t)v;
   }
   TcArgs a;
-  a.ctb = m->d_col_tet_begin;
-  a.colptr = op->d_tc_colptr;
+  a.gtb = op->d_tc_gtb;
+  a.gptr = op->d_tc_gptr;
   a.blk = static_cast<const TcBlk*>(op->d_tc_blk);
   a.vals = static_cast<const uint4*>(op->d_tcv[bf16 ? 0 : 1]);
-  a.rs = op->d_rs;
-  a.y = y;
+  a.rs = op->d_tc_rs;
+  a.parts = parts;
+  a.y = parts > 1 ? reinterpret_cast<double*>(op->d_ws + xc_len) : y;
   a.n_tet = n;
   a.nr = nrhs;
   a.N = N;
@@ -846,11 +924,17 @@ bem_status op_spmm_tc(const bem_operator* op, const double* x, double* y, int nr
     a.stages = st;
     a.tmem_cols = pow2(cols_of(kind, st));
     const size_t smem = st * (stage_b + (kind ? 0 : stage_a)) + tail;
+    const int64_t n_cta = op->tc_groups * parts;
     if (bf16)
-      return MT == 1 ? launch_tc<false, 1>(kind, a, map, smem, m->n_col, s)
-                     : launch_tc<false, 2>(kind, a, map, smem, m->n_col, s);
-    return MT == 1 ? launch_tc<true, 1>(kind, a, map, smem, m->n_col, s)
-                   : launch_tc<true, 2>(kind, a, map, smem, m->n_col, s);
+      return MT == 1 ? launch_tc<false, 1>(kind, a, map, smem, n_cta, s) : launch_tc<false, 2>(kind, a, map, smem, n_cta, s);
+    return MT == 1 ? launch_tc<true, 1>(kind, a, map, smem, n_cta, s) : launch_tc<true, 2>(kind, a, map, smem, n_cta, s);
+  };
+  // the product with a shape, and the sum of its parts
+  auto product = [&](int kind, int st) -> bem_status {
+    TRY_STATUS(launch(kind, st));
+    if (parts > 1) k_tc_sum<<<grid_for(n * nrhs), 256, 0, s>>>(a.y, y, n * nrhs, parts);
+    STBEM_CUDA(cudaGetLastError());
+    return BEM_OK;
   };
   // launch shape: where the A tiles live and the pipeline depth (1 to 6
   // stages; with the stage size they fix the CTAs per SM), timed once per
@@ -864,12 +948,12 @@ bem_status op_spmm_tc(const bem_operator* op, const double* x, double* y, int nr
     set_error("tensor-core product: the widest block does not fit in shared or tensor memory");
     return BEM_ERR_UNSUPPORTED;
   }
-  const auto key = std::make_tuple(m->n_col, m->max_col_tets, op->tc_span[bf16 ? 0 : 1], op->tcv_cap[bf16 ? 0 : 1], N,
+  const auto key = std::make_tuple(op->tc_groups * 16 + parts, op->tc_rows, op->tc_span[bf16 ? 0 : 1], op->tcv_cap[bf16 ? 0 : 1], N,
                                    (int)bf16, op->ctx->device);
   {
     std::lock_guard<std::mutex> lk(g_tc_mu);
     auto it = g_tc_shape.find(key);
-    if (it != g_tc_shape.end()) return launch(it->second.first, it->second.second);
+    if (it != g_tc_shape.end()) return product(it->second.first, it->second.second);
   }
   cudaEvent_t e0, e1;
   STBEM_CUDA(cudaEventCreate(&e0));
@@ -901,7 +985,7 @@ bem_status op_spmm_tc(const bem_operator* op, const double* x, double* y, int nr
     std::lock_guard<std::mutex> lk(g_tc_mu);
     g_tc_shape[key] = best_c;
   }
-  return launch(best_c.first, best_c.second);
+  return product(best_c.first, best_c.second);
 }
 
 namespace {

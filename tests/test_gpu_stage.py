@@ -99,3 +99,23 @@ def test_products_over_the_column_sizes(ctx, level, slabs, precision):
         for dtype, u in (("fp64", 2.0 ** -53), ("fp32", 2.0 ** -24)):
             y = op.matvec(torch.tensor(x, device="cuda"), dtype=dtype).cpu().numpy()
             assert np.all(np.abs(y - ref) <= (2 * row + 4) * u * mag + 1e-300), (nrhs, dtype)
+
+
+@pytest.mark.parametrize("level,slabs", [(0, 1), (0, 14), (0, 42), (0, 43), (0, 64), (1, 3), (1, 16), (2, 2)])
+@pytest.mark.parametrize("dtype", ["tf32", "bf16"])
+def test_tensor_core_products_over_the_row_groups(ctx, level, slabs, dtype):
+    """Tensor-core products with one to many columns per 128-row tile, tiles
+    that are full, nearly full and exceeded (129 rows: two tiles), and groups
+    split over several CTAs, row by row within the rounding of the operands and
+    of an FP32 sum: (2 u + 2 u^2 + (n + 2) 2^-24) |A| |x|."""
+    import paper_2103_16841_gb300 as stb
+    m = inputs.sphere_mesh(level, slabs, 2.0, 0.2, seed=8)
+    op = stb.Operator(ctx, stb.Mesh.from_spacetime(ctx, m), "mixed")
+    A = op.export_dense()
+    u = {"tf32": 2.0 ** -11, "bf16": 2.0 ** -8}[dtype]
+    for nrhs in (1, 17, 64):
+        x = np.random.default_rng(nrhs).normal(size=(nrhs, m.n_tet))
+        y = op.matvec(torch.tensor(x, device="cuda"), dtype=dtype).cpu().numpy()
+        bound = (2 * u + 2 * u * u + ((A != 0).sum(axis=1) + 2) * 2.0 ** -24) * (np.abs(x) @ np.abs(A).T) + 1e-300
+        assert (np.abs(y - x @ A.T) / bound).max() <= 1.0, nrhs
+    assert op.check()[0] == 0
