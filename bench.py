@@ -313,22 +313,22 @@ def run_ours(args):
     roof = None
     inner_per_s = n_inner / (quad_ms / 1e3)
     if prof and "fp32_flops_per_inner" in prof:
-        # executed flops per inner integral of the quadrature kernel, from an ncu
-        # capture of the same kernel on a mesh whose values exceed L2 (level-3
-        # sphere, 8 slabs), times this run's inner integrals, over the kernel's
-        # CUDA-event time; peaks measured on this GPU in this run
+        # executed flops per inner integral of the quadrature's stages, from an ncu
+        # capture of every stage launch of one assembly (profiles/quad_stages.md),
+        # times this run's inner integrals, over the quadrature's CUDA-event time;
+        # peaks measured on this GPU in this run
         f32 = prof["fp32_flops_per_inner"] * n_inner / (quad_ms / 1e3) / 1e12
         f64 = prof["fp64_flops_per_inner"] * n_inner / (quad_ms / 1e3) / 1e12
         traffic = prof["dram_bytes_per_inner"] * n_inner if prof.get("dram_bytes_per_inner") else None
         roof = {"bound": "alu", "achieved": round(f32, 3), "peak": round(alu["fp32_tflops"], 2), "unit": "TFLOP/s",
                 "frac": round(f32 / alu["fp32_tflops"], 4), "traffic": traffic,
-                "kernel": "k_quad_blocks<mixed>",
+                "kernel": "quadrature stages (k_apex, k_cut_far, k_cut_any, k_cut_fp64, k_assemble)",
                 "fp64": {"achieved": round(f64, 4), "peak": round(alu["fp64_tflops"], 3), "unit": "TFLOP/s",
                          "frac": round(f64 / alu["fp64_tflops"], 4)},
                 "inner_integrals_per_launch": n_inner,
                 "note": "achieved = executed FP32 (FP64) flops per inner integral from ncu (SASS op counters, "
-                        "FFMA counted 2) on the level-3 sphere with 8 slabs x inner integrals of this launch / "
-                        "its CUDA-event time; peak = FMA rate measured on this GPU in this run (bem_alu_peaks; "
+                        "FFMA counted 2) over all stages on a small sphere x inner integrals of this assembly / "
+                        "the quadrature's CUDA-event time; peak = FMA rate measured on this GPU in this run (bem_alu_peaks; "
                         "152 SMs x 128 lanes x 2 x 2.07 GHz = 80.5 TFLOP/s nominal)"}
     cb = cpu_baseline(m, seconds=args.cpu_seconds) if args.cpu_seconds > 0 else None
     vbytes = st["stored"] * (4 if prec == "mixed" else 12)  # FP32 values; FP64 operators also keep FP64
@@ -596,9 +596,9 @@ def serving_leg(ctx, args):
 
 
 def load_profile_summary():
-    """Per-pair FP32 work and DRAM traffic of the quadrature kernel from the
-    committed ncu summary (profiles/quad_kernel_mixed.json)."""
-    p = os.path.join(ROOT, "profiles", "quad_kernel_mixed.json")
+    """FP32 work and DRAM traffic per inner integral of the quadrature from the
+    committed ncu summary (profiles/quad_stages.json)."""
+    p = os.path.join(ROOT, "profiles", "quad_stages.json")
     try:
         return json.load(open(p))
     except Exception:
