@@ -348,7 +348,9 @@ def run_ours(args):
                 "includes": "mesh upload, assembly, RHS, GMRES(FP32 inner + FP64 refinement, tol 1e-8), "
                             "density to host",
                 "solve": solve_info},
-        "gpu_launches": 3 * args.steps,
+        # at least: outer points, pattern, and the quadrature's stages (five, or three in
+        # FP64) of its chunks, four or more in mixed precision
+        "gpu_launches": (2 + (5 * 4 if prec == "mixed" else 3)) * args.steps,
         "clocks": clk.summary(),
         "roofline": roof,
         "cpu_baseline": cb,
