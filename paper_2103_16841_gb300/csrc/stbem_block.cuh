@@ -19,12 +19,10 @@ static_assert(sizeof(PanelF) == 48, "PanelF layout");
 
 // FP32 image of a column: corners, frame and centroid ball
 struct ColF {
-  float Xh[3][3], Xl[3][3];            // corners as FP32 pairs
-  float nh[3], nl[3], e1h[3], e1l[3], e2h[3], e2l[3];
+  float Xh[3][3];
   ColR<float> R;
   float ctr[3], rad;
 };
-static_assert(sizeof(ColF) % 16 == 0, "ColF is copied in 16-byte pieces");
 static_assert(sizeof(FaceF) == 48, "FaceF is copied in 16-byte pieces");
 
 struct BlockCtx {
@@ -43,7 +41,6 @@ struct BlockCtx {
   const PanelF* panf;
   const double* pts;
   const float4* ptsf;          // outer points (t, x, y, z) rounded to FP32
-  const float4* ptsl;          // and the remainders: pts = ptsf + ptsl as FP32 pairs
   const double* trange;
   int32_t* bw;
   int64_t* bnnz;

@@ -121,12 +121,7 @@ __global__ void k_col_f32(int64_t n_col, const ColGeom* cols, ColF* out) {
   const ColGeom& G = cols[c];
   ColF F;
   for (int k = 0; k < 3; ++k)
-    for (int i = 0; i < 3; ++i) split2(G.X[k][i], F.Xh[k][i], F.Xl[k][i]);
-  for (int i = 0; i < 3; ++i) {
-    split2(G.n[i], F.nh[i], F.nl[i]);
-    split2(G.e1[i], F.e1h[i], F.e1l[i]);
-    split2(G.e2[i], F.e2h[i], F.e2l[i]);
-  }
+    for (int i = 0; i < 3; ++i) F.Xh[k][i] = (float)G.X[k][i];
   make_colr<float>(G, F.R);
   for (int i = 0; i < 3; ++i) F.ctr[i] = (float)G.ctr[i];
   F.rad = (float)G.rad;
@@ -181,7 +176,7 @@ bem_status mesh_device_geometry(bem_mesh* m, const double* d_sv_xyz, const int32
 // id) and x = (A + xi1 (B - A)) + xi2 (C - A) without fused operations.
 // ---------------------------------------------------------------------------
 __global__ void k_outer_points(int64_t n_surf, int mq, const ColGeom* cols, const SurfDev* surf, double* pts,
-                               float* ptsf, float* ptsl, double* trange) {
+                               float* ptsf, double* trange) {
   int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (s >= n_surf) return;
   const SurfDev S = surf[s];
@@ -202,8 +197,7 @@ __global__ void k_outer_points(int64_t n_surf, int mq, const ColGeom* cols, cons
         for (int d = 0; d < 4; ++d) {
           double p = __dadd_rn(A[d], __dmul_rn(x1, __dsub_rn(B[d], A[d])));
           out[4 * n + d] = __dadd_rn(p, __dmul_rn(x2, __dsub_rn(C[d], A[d])));
-          const int64_t o = (int64_t)s * nq * 4 + 4 * n + d;
-          split2(out[4 * n + d], ptsf[o], ptsl[o]);
+          ptsf[(int64_t)s * nq * 4 + 4 * n + d] = (float)out[4 * n + d];
         }
         tlo = fmin(tlo, out[4 * n]);
         thi = fmax(thi, out[4 * n]);
@@ -218,7 +212,7 @@ bem_status op_outer_points(bem_operator* op, cudaStream_t s) {
   const bem_mesh* m = op->mesh;
   int th = 128;
   k_outer_points<<<(unsigned)((m->n_surf + th - 1) / th), th, 0, s>>>(m->n_surf, op->mq, m->d_col, m->d_surf,
-                                                                      op->d_pts, op->d_ptsf, op->d_ptsl, op->d_pts_trange);
+                                                                      op->d_pts, op->d_ptsf, op->d_pts_trange);
   STBEM_CUDA(cudaGetLastError());
   return BEM_OK;
 }
@@ -379,7 +373,7 @@ static BlockCtx make_ctx(const bem_operator* op) {
   B.facef = static_cast<const FaceF*>(m->d_facef);
   B.col_tet_begin = m->d_col_tet_begin; B.col_surf_begin = m->d_col_surf_begin;
   B.surf = m->d_surf; B.tets = m->d_tet; B.pts = op->d_pts; B.ptsf = reinterpret_cast<const float4*>(op->d_ptsf);
-  B.ptsl = reinterpret_cast<const float4*>(op->d_ptsl); B.trange = op->d_pts_trange;
+  B.trange = op->d_pts_trange;
   B.bw = op->d_bw; B.bnnz = op->d_bnnz; B.boff = op->d_boff; B.rsoff = op->d_rsoff; B.rs = op->d_rs;
   B.val = op->d_val; B.val32 = op->d_val32;
   B.max_surf = m->max_col_surf; B.max_tet = m->max_col_tets;

@@ -115,7 +115,6 @@ struct bem_operator {
   int mq = 3, nq = 9, n_theta = 12;
   double* d_pts = nullptr;       // [n_surf][nq][4] outer points
   float* d_ptsf = nullptr;       // the same rounded to FP32 (the sparsity filter's inputs)
-  float* d_ptsl = nullptr;       // and the remainders (FP32 pairs)
   double* d_pts_trange = nullptr;// [n_surf][2] min / max time of the outer points
   int32_t* d_bw = nullptr;       // [n_col*n_col] band width per column block
   int64_t* d_bnnz = nullptr;     // [n_col*n_col] pattern entries per block

@@ -151,7 +151,7 @@ struct PointCol {        // apex x against one column
 // per face, FP32 view for the mixed path: corner times as FP32 pairs
 struct FaceF {
   float p_hi[3], p_lo[3];
-  float g[2], g_lo[2];
+  float g[2], pad[2];
   float pmin_hi, pmin_lo;
 };
 
@@ -175,7 +175,8 @@ STBEM_HD inline void make_facef(const FaceGeom& F, FaceF& o) {
     if (F.p[k] < F.p[km]) km = k;
   }
   o.pmin_hi = o.p_hi[km]; o.pmin_lo = o.p_lo[km];
-  for (int i = 0; i < 2; ++i) split2(F.g[i], o.g[i], o.g_lo[i]);
+  o.g[0] = (float)F.g[0]; o.g[1] = (float)F.g[1];
+  o.pad[0] = o.pad[1] = 0.f;
 }
 
 template <typename R>
@@ -1016,7 +1017,7 @@ STBEM_HD inline void cut_in_fp64(const PointCol& P, const FaceGeom& Fc, const do
 // about 3 % of the cut faces) its two terms cancel, and c (an O(1) difference
 // formed in FP32 pairs, but with <g, xb> in FP32) loses the relative accuracy
 // D0 needs; there the caller replaces it by the value from the apex's FP64
-// geometry (d0_fp64) or from FP32 pairs (d0_pairs).
+// geometry (d0_fp64).
 STBEM_HD inline void cut_in_mixed(const PtR<float>& T, const ConeM& M, const FaceF& Fc, const float* F, float c,
                                   FaceCutIn<float>& o) {
   for (int k = 0; k < 3; ++k) {
@@ -1031,9 +1032,8 @@ STBEM_HD inline void cut_in_mixed(const PtR<float>& T, const ConeM& M, const Fac
   o.D0 = c * c - T.d * T.d * (1.f - (Fc.g[0] * Fc.g[0] + Fc.g[1] * Fc.g[1]));
 }
 STBEM_HD inline bool d0_cancels(const FaceCutIn<float>& in) { return fabsf(in.D0) < 0.05f * in.c * in.c; }
-STBEM_HD inline float d0_fp64(const PointCol& P, const FaceGeom& F64) {
-  const double c64 = P.t - (F64.p[0] + (F64.g[0] * P.D.xb[0] + F64.g[1] * P.D.xb[1]));
-  const double d64 = P.D.d;
+STBEM_HD inline float d0_fp64(double t, const double* xb, double d64, const FaceGeom& F64) {
+  const double c64 = t - (F64.p[0] + (F64.g[0] * xb[0] + F64.g[1] * xb[1]));
   return (float)(c64 * c64 - d64 * d64 * (1.0 - (F64.g[0] * F64.g[0] + F64.g[1] * F64.g[1])));
 }
 
@@ -1204,54 +1204,6 @@ STBEM_HD __noinline__ double face_cut(const ColR<R>& G, const PtR<R>& P, const F
   return (double)total;
 }
 
-#ifdef __CUDACC__
-// ---------------------------------------------------------------------------
-// FP32 pairs (double-float, about 2^-48 relative): the geometry of an apex
-// against a column off the FP64 pipe, which on sm_103a has 1/76 of the FP32
-// rate. Error-free sums (Knuth) and products (fma), after Dekker 1971; the
-// intrinsics keep the compiler from contracting them.
-// ---------------------------------------------------------------------------
-struct F2 { float h, l; };
-__device__ __forceinline__ F2 f2_fast(float a, float b) {   // |a| >= |b|
-  const float s = __fadd_rn(a, b);
-  return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ F2 f2_sum(float a, float b) {
-  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
-  F2 s = f2_sum(a.h, b.h);
-  const F2 t = f2_sum(a.l, b.l);
-  s = f2_fast(s.h, __fadd_rn(s.l, t.h));
-  return f2_fast(s.h, __fadd_rn(s.l, t.l));
-}
-__device__ __forceinline__ F2 f2_neg(F2 a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = __fmaf_rn(a.h, b.h, -p);
-  e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.l, b.l, e)));
-  return f2_fast(p, e);
-}
-__device__ __forceinline__ F2 f2_sqrt(F2 a) {
-  if (!(a.h > 0.f)) return {0.f, 0.f};
-  const float s = __fsqrt_rn(a.h), p = __fmul_rn(s, s);
-  const float r = __fadd_rn(__fsub_rn(__fsub_rn(a.h, p), __fmaf_rn(s, s, -p)), a.l);   // a - s^2
-  return f2_fast(s, __fdiv_rn(r, 2.f * s));
-}
-
-// D0 where it cancels (see cut_in_mixed), from FP32 pairs
-__device__ __forceinline__ float d0_pairs(F2 d, const F2* xb, F2 nt, const FaceF& Fc) {
-  const F2 g0 = {Fc.g[0], Fc.g_lo[0]}, g1 = {Fc.g[1], Fc.g_lo[1]};
-  F2 c = f2_add(F2{Fc.p_hi[0], Fc.p_lo[0]}, nt);                      // -(t - P(xb))
-  c = f2_add(c, f2_add(f2_mul(g0, xb[0]), f2_mul(g1, xb[1])));
-  const F2 gg = f2_add(f2_mul(g0, g0), f2_mul(g1, g1));
-  const F2 om = f2_add(F2{1.f, 0.f}, f2_neg(gg));
-  const F2 D = f2_add(f2_mul(c, c), f2_neg(f2_mul(f2_mul(d, d), om)));
-  return D.h + D.l;
-}
-#endif
-
 // 4 pi W_P(x) in one call (used by the kernel-level entry point and checks)
 template <bool FP32>
 STBEM_HD inline double face_W(const ColGeom& G, const PointCol& P, const FaceGeom& Fc, const ArcRule& rule) {
@@ -1268,7 +1220,7 @@ STBEM_HD inline double face_W(const ColGeom& G, const PointCol& P, const FaceGeo
     make_colr<float>(G, CR);
     FaceCutIn<float> in;
     cut_in_mixed(P.F, P.M, Ff, F, c, in);
-    if (d0_cancels(in)) in.D0 = d0_fp64(P, Fc);
+    if (d0_cancels(in)) in.D0 = d0_fp64(P.t, P.D.xb, P.D.d, Fc);
     return face_cut<float>(CR, P.F, in, rule);
   }
   double F[3], c = 0.0;

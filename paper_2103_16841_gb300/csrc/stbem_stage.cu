@@ -25,7 +25,7 @@
 // active, every warp held the registers and shared memory of the largest
 // phase (8 to 16 warps per SM), and the phases' code did not fit the
 // instruction caches. Queues fill the lanes, and each stage has its own
-// register budget and occupancy. The intermediate data are about 150 bytes
+// register budget and occupancy. The intermediate data are about 170 bytes
 // per (face, outer point), written and read once.
 #include <cuda_runtime.h>
 
@@ -49,16 +49,16 @@ namespace {
 
 // One apex (face, outer point) against a trial column, as the cut stages need it.
 struct alignas(16) ApexF {
-  float xbh[2], xbl[2];          // foot point, FP32 pairs
-  float dh, dl, far_rho;
-  int far;
+  float xb[2], d, far_rho;
   float rs[3], E[3];             // corner distances, whole-edge integrals
   float rho_hi[3], rho_lo[3], nt_hi, nt_lo;
+  int far;
   uint32_t slot0;                // potential of the window's first face
   int32_t surf0;                 // and that face
-  int32_t col, pt, seg, pad;
+  int32_t col, pt, seg;
+  double xb64[2], d64;           // where the conic's size cancels (d0_cancels)
 };
-static_assert(sizeof(ApexF) == 112, "ApexF layout");
+static_assert(sizeof(ApexF) == 128, "ApexF layout");
 struct alignas(16) ApexD {
   double t, d, xb[2], rs[3], E[3];
   uint32_t slot0;
@@ -153,56 +153,98 @@ __device__ __noinline__ float whole_edge(const PtR<float>& T, const ColR<float>&
   return edge_full_mixed(T, R, k);
 }
 
-// The mixed path: what cancels between |x - y| and t - tau (relative
-// position, height, foot point, corner distances) in FP32 pairs, the rest in
-// FP32. The same values came from FP64 before, whose pipe (1/76 of the FP32
-// rate) was the kernel's busiest unit.
-__device__ __forceinline__ void apex_geometry(const float4 xh, const float4 xl, const ColF& G, PtR<float>& T, ConeM& M,
-                                              F2& d, F2* xb, float& Wst) {
-  const F2 nt = {-xh.x, -xl.x}, x[3] = {{xh.y, xl.y}, {xh.z, xl.z}, {xh.w, xl.w}};
-  F2 rel[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) rel[i] = f2_add(x[i], F2{-G.Xh[0][i], -G.Xl[0][i]});
-  auto dot = [&](const float* h, const float* l) {
-    return f2_add(f2_add(f2_mul(rel[0], F2{h[0], l[0]}), f2_mul(rel[1], F2{h[1], l[1]})), f2_mul(rel[2], F2{h[2], l[2]}));
-  };
-  d = dot(G.nh, G.nl);
-  if (fabsf(d.h) < 1e-13f * G.R.diam) d = F2{0.f, 0.f};
-  xb[0] = dot(G.e1h, G.e1l);
-  xb[1] = dot(G.e2h, G.e2l);
-  T.d = d.h;
-  T.xb[0] = xb[0].h;
-  T.xb[1] = xb[1].h;
-#pragma unroll
+// Positions of a test column against a trial column, mixed path: what the
+// outer points of all its faces share, since a point's position depends on its
+// node alone (only its time depends on the face). Relative position, height,
+// foot point and corner distances are formed in FP64: they carry the
+// cancellation between |x - y| and t - tau, and their FP32 roundings decide
+// between forms of a face's integral that differ by 1e-6 (formed in FP32 pairs,
+// some 50 of 30 million entries of the level-2 sphere with 15 slabs came out
+// by up to 1e-6 apart). One array per quantity, [nq] each.
+struct Positions {
+  double *r[3], *rlo, *xb64[2], *d64;
+  float *xb[2], *d, *far_rho, *rs[3], *E[3];
+  int* far;
+};
+constexpr size_t kPosBytes = 7 * sizeof(double) + 10 * sizeof(float) + sizeof(int);
+__device__ __forceinline__ Positions positions(unsigned char* smem, int nq) {
+  Positions P;
+  double* d = reinterpret_cast<double*>(smem);
+  auto next64 = [&] { double* p = d; d += nq; return p; };
+  for (int k = 0; k < 3; ++k) P.r[k] = next64();
+  P.rlo = next64();
+  P.xb64[0] = next64(); P.xb64[1] = next64(); P.d64 = next64();
+  float* f = reinterpret_cast<float*>(d);
+  auto next32 = [&] { float* p = f; f += nq; return p; };
+  P.xb[0] = next32(); P.xb[1] = next32(); P.d = next32(); P.far_rho = next32();
+  for (int k = 0; k < 3; ++k) P.rs[k] = next32();
+  for (int k = 0; k < 3; ++k) P.E[k] = next32();
+  P.far = reinterpret_cast<int*>(f);
+  return P;
+}
+// position q in registers (T.far, T.ps and T.ws are not set)
+__device__ __forceinline__ void take_position(const Positions& P, int q, const ColR<float>& R, PtR<float>& T) {
+  T.d = P.d[q];
+  T.xb[0] = P.xb[0][q];
+  T.xb[1] = P.xb[1][q];
   for (int k = 0; k < 3; ++k) {
-    F2 v[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      v[i] = k == 0 ? rel[i] : f2_add(x[i], F2{-G.Xh[k][i], -G.Xl[k][i]});
-      v[i] = f2_mul(v[i], v[i]);
-    }
-    const F2 r = f2_sqrt(f2_add(f2_add(v[0], v[1]), v[2]));
-    T.rs[k] = r.h;
-    const F2 rho = f2_add(r, nt);
-    M.rho_hi[k] = rho.h;
-    M.rho_lo[k] = rho.l;
+    T.rs[k] = P.rs[k][q];
+    T.q[k][0] = R.Q[k][0] - T.xb[0];
+    T.q[k][1] = R.Q[k][1] - T.xb[1];
   }
-  frame_points(T, G.R);
-  float out = 0.f;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) out = fmaxf(out, -T.ps[k]);
-  T.far = out >= FAR_RHO * G.R.diam;
   T.C = T.rs[0];
-  T.far_rho = out;
-  const F2 o2 = {out, 0.f};
-  const F2 rl = f2_add(f2_sqrt(f2_add(f2_mul(d, d), f2_mul(o2, o2))), nt);
-  M.nt_hi = nt.h;
-  M.nt_lo = nt.l;
-  M.rlot_hi = rl.h;
-  M.rlot_lo = rl.l;
-#pragma unroll 1
-  for (int k = 0; k < 3; ++k) T.Efull[k] = whole_edge(T, G.R, k);
-  Wst = (T.Efull[0] + T.Efull[1]) + T.Efull[2];
+}
+
+// x: [nq] outer points of a face of the test column (all threads; ends with a barrier)
+__device__ __forceinline__ void column_positions(const double* x, int nq, const ColGeom& G, const ColR<float>& R,
+                                                 const Positions& P) {
+  // a warp takes the frames or the distances, not both
+  const int frames = (nq + 31) / 32 * 32;
+  for (int it = threadIdx.x; it < frames + 3 * nq; it += blockDim.x) {
+    if (it < frames) {
+      if (it >= nq) continue;
+      const double* y = x + 4 * it;
+      const double rel[3] = {y[1] - G.c0[0], y[2] - G.c0[1], y[3] - G.c0[2]};
+      double d = rel[0] * G.n[0] + rel[1] * G.n[1] + rel[2] * G.n[2];
+      if (fabs(d) < 1e-13 * G.diam) d = 0.0;
+      const double xb0 = rel[0] * G.e1[0] + rel[1] * G.e1[1] + rel[2] * G.e1[2];
+      const double xb1 = rel[0] * G.e2[0] + rel[1] * G.e2[1] + rel[2] * G.e2[2];
+      PtR<float> T;
+      T.xb[0] = (float)xb0;
+      T.xb[1] = (float)xb1;
+      frame_points(T, R);
+      float out = 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) out = fmaxf(out, -T.ps[k]);
+      P.d64[it] = d;
+      P.xb64[0][it] = xb0;
+      P.xb64[1][it] = xb1;
+      P.rlo[it] = sqrt(d * d + (double)out * (double)out);
+      P.d[it] = (float)d;
+      P.xb[0][it] = T.xb[0];
+      P.xb[1][it] = T.xb[1];
+      P.far_rho[it] = out;
+      P.far[it] = out >= FAR_RHO * R.diam;
+    } else {
+      const int q = (it - frames) / 3, k = (it - frames) - 3 * q;
+      const double* y = x + 4 * q;
+      const double dx = y[1] - G.X[k][0], dy = y[2] - G.X[k][1], dz = y[3] - G.X[k][2];
+      const double r = sqrt(dx * dx + dy * dy + dz * dz);
+      P.r[k][q] = r;
+      P.rs[k][q] = (float)r;
+    }
+  }
+  __syncthreads();
+  for (int it = threadIdx.x; it < 3 * nq; it += blockDim.x) {
+    const int q = it / 3, k = it - 3 * q;
+    PtR<float> T;
+    take_position(P, q, R, T);
+    frame_points(T, R);
+    T.far = P.far[q];
+    T.far_rho = P.far_rho[q];
+    P.E[k][q] = whole_edge(T, R, k);
+  }
+  __syncthreads();
 }
 
 // ---- k_apex ------------------------------------------------------------
@@ -211,6 +253,7 @@ template <typename R>
 size_t apex_smem(int max_tet, int max_surf, int nq) {
   size_t s = bits_smem(max_tet, max_surf, nq);
   s = (s + 15) / 16 * 16 + sizeof(typename Types<R>::Face) * max_surf;
+  if (sizeof(R) == 4) s += (kPosBytes * nq + 7) / 8 * 8;
   return s + sizeof(uint2) * max_surf + sizeof(uint16_t) * ((max_surf + 7) / 8 * 8);
 }
 
@@ -222,13 +265,15 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ BlockSm C;
   __shared__ BlockCtx B;
-  __shared__ __align__(16) ColF G;
+  __shared__ __align__(16) ColR<float> G;
   __shared__ unsigned s_w[kApexThreads / 32], s_base[4];
   __shared__ int s_seg;
   const int tid = threadIdx.x, nq = a.one.nq, max_surf = a.one.max_surf, words = bit_words(a.one.max_tet);
   const BlockPtr P = block_ptr(smem, a.one.max_tet, max_surf, nq);
   Face* Fs = reinterpret_cast<Face*>(smem + (bits_smem(a.one.max_tet, max_surf, nq) + 15) / 16 * 16);
-  uint2* fm = reinterpret_cast<uint2*>(Fs + max_surf);
+  unsigned char* after = reinterpret_cast<unsigned char*>(Fs + max_surf);
+  const Positions X = positions(after, nq);
+  uint2* fm = reinterpret_cast<uint2*>(after + (FP32 ? (kPosBytes * nq + 7) / 8 * 8 : 0));
   uint16_t* act = reinterpret_cast<uint16_t*>(fm + max_surf);
   if (tid == 0 && a.S <= 1) B = a.one;
   int cur = a.S > 1 ? -1 : 0;
@@ -255,8 +300,10 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
     if constexpr (FP32) {
       const uint4* src = reinterpret_cast<const uint4*>(B.facef + C.surfJ);
       for (int k = tid; k < 3 * C.nsJ; k += kApexThreads) reinterpret_cast<uint4*>(Fs)[k] = src[k];
-      const uint4* cs = reinterpret_cast<const uint4*>(B.colf + J);
-      for (int k = tid; k < (int)(sizeof(ColF) / 16); k += kApexThreads) reinterpret_cast<uint4*>(&G)[k] = cs[k];
+      const float* cs = reinterpret_cast<const float*>(&B.colf[J].R);
+      for (int k = tid; k < (int)(sizeof(G) / 4); k += kApexThreads) reinterpret_cast<float*>(&G)[k] = cs[k];
+      __syncthreads();
+      column_positions(B.pts + 4 * (int64_t)C.surfI * nq, nq, B.cols[J], G, X);
     } else {
       for (int k = tid; k < C.nsJ; k += kApexThreads) Fs[k] = B.surf[C.surfJ + k].f;
     }
@@ -286,22 +333,27 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
       const bool on = r < nr;
       int n = 0, first = 0;
       uint32_t slot0 = 0;
-      int pt = 0;
+      int pt = 0, q = 0;
+      double t = 0.0;
       typename std::conditional<FP32, PtR<float>, PointCol>::type T;
       ConeM M;
-      F2 d2 = {0.f, 0.f}, xb2[2] = {{0.f, 0.f}, {0.f, 0.f}};
       R Wst = R(0);
       bool far = true;
       if (on) {
-        const int k = r / nq, q = r - k * nq, f = act[k];
+        const int k = r / nq, f = act[k];
+        q = r - k * nq;
         const uint2 m = fm[f];
         first = (int)(m.y & 0xffffu);
         n = (int)(m.y >> 16);
         slot0 = m.x + q;
         pt = (C.surfI + f) * nq + q;
         if constexpr (FP32) {
-          apex_geometry(B.ptsf[pt], B.ptsl[pt], G, T, M, d2, xb2, Wst);
-          far = T.far;
+          take_position(X, q, G, T);
+          t = B.pts[4 * (int64_t)pt];
+          for (int c = 0; c < 3; ++c) split2(X.r[c][q] - t, M.rho_hi[c], M.rho_lo[c]);
+          split2(X.rlo[q] - t, M.rlot_hi, M.rlot_lo);
+          Wst = (X.E[0][q] + X.E[1][q]) + X.E[2][q];
+          far = X.far[q];
         } else {
           point_col(B.pts + 4 * (int64_t)pt, B.cols[J], T, false);
           Wst = T.Wst;
@@ -347,12 +399,12 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
         base_far = __shfl_sync(0xffffffffu, base_far, 31);
         base_any = __shfl_sync(0xffffffffu, base_any, 31);
         at -= mine;
-        uint32_t* q = far ? a.q_far + base_far + (at & 0xffffu) : a.q_any + base_any + (at >> 16);
+        uint32_t* to = far ? a.q_far + base_far + (at & 0xffffu) : a.q_any + base_any + (at >> 16);
         while (mask) {
           const int s = s0 + __ffsll((long long)mask) - 1;
           mask &= mask - 1;
           const uint32_t slot = slot0 + s * nq;
-          *q++ = slot;
+          *to++ = slot;
           if constexpr (FP32) W[slot] = __uint_as_float(ray0 + r);
           else W[slot] = __hiloint2double(0, (int)(ray0 + r));
         }
@@ -360,13 +412,13 @@ __global__ void __launch_bounds__(kApexThreads, sizeof(R) == 4 ? 4 : 2) k_apex(c
       if (any) {
         Apex Y;
         if constexpr (FP32) {
-          for (int i = 0; i < 2; ++i) { Y.xbh[i] = xb2[i].h; Y.xbl[i] = xb2[i].l; }
-          Y.dh = d2.h; Y.dl = d2.l; Y.far_rho = T.far_rho; Y.far = T.far;
+          for (int i = 0; i < 2; ++i) { Y.xb[i] = T.xb[i]; Y.xb64[i] = X.xb64[i][q]; }
+          Y.d = T.d; Y.d64 = X.d64[q]; Y.far_rho = X.far_rho[q]; Y.far = far;
           for (int k = 0; k < 3; ++k) {
-            Y.rs[k] = T.rs[k]; Y.E[k] = T.Efull[k]; Y.rho_hi[k] = M.rho_hi[k]; Y.rho_lo[k] = M.rho_lo[k];
+            Y.rs[k] = T.rs[k]; Y.E[k] = X.E[k][q]; Y.rho_hi[k] = M.rho_hi[k]; Y.rho_lo[k] = M.rho_lo[k];
           }
-          Y.nt_hi = M.nt_hi; Y.nt_lo = M.nt_lo;
-          Y.pt = pt; Y.pad = 0;
+          split2(-t, Y.nt_hi, Y.nt_lo);
+          Y.pt = pt;
         } else {
           Y.t = T.t; Y.d = T.D.d; Y.xb[0] = T.D.xb[0]; Y.xb[1] = T.D.xb[1];
           for (int k = 0; k < 3; ++k) { Y.rs[k] = T.D.rs[k]; Y.E[k] = T.D.Efull[k]; }
@@ -388,14 +440,15 @@ struct CutF {
   FaceCutIn<float> in;
 };
 __device__ __forceinline__ bool load_cut(const StageArgs& a, uint32_t slot, uint32_t ray, CutF& c) {
-  const ApexF Y = static_cast<const ApexF*>(a.apex)[ray];
+  const ApexF& Y = static_cast<const ApexF*>(a.apex)[ray];
   const BlockCtx& B = a.S > 1 ? a.many[Y.seg] : a.one;
-  const FaceF Fc = B.facef[Y.surf0 + (int)(slot - Y.slot0) / a.one.nq];
+  const int surf = Y.surf0 + (int)(slot - Y.slot0) / a.one.nq;
+  const FaceF Fc = B.facef[surf];
   c.R = B.colf[Y.col].R;
   PtR<float>& T = c.T;
   ConeM M;
-  T.d = Y.dh;
-  T.xb[0] = Y.xbh[0]; T.xb[1] = Y.xbh[1];
+  T.d = Y.d;
+  T.xb[0] = Y.xb[0]; T.xb[1] = Y.xb[1];
   T.far = Y.far;
   T.far_rho = Y.far_rho;
   for (int k = 0; k < 3; ++k) {
@@ -409,10 +462,7 @@ __device__ __forceinline__ bool load_cut(const StageArgs& a, uint32_t slot, uint
   const float cc = face_c_mixed(T, M, Fc, c.R.diam);
   if (near_singular_mixed(cc, T.d, c.R.diam)) return false;
   cut_in_mixed(T, M, Fc, F, cc, c.in);
-  if (d0_cancels(c.in)) {
-    const F2 xb[2] = {{Y.xbh[0], Y.xbl[0]}, {Y.xbh[1], Y.xbl[1]}};
-    c.in.D0 = d0_pairs(F2{Y.dh, Y.dl}, xb, F2{Y.nt_hi, Y.nt_lo}, Fc);
-  }
+  if (d0_cancels(c.in)) c.in.D0 = d0_fp64(B.pts[4 * (int64_t)Y.pt], Y.xb64, Y.d64, B.surf[surf].f);
   return true;
 }
 
