@@ -685,11 +685,12 @@ STBEM_HD inline void consider_pole(R A0, R Aa, R Ab, R mid, R half, R& best_rho,
 }
 
 // sinh and cosh of the map's nodes; in FP64 both from one expm1 (a node's
-// largest cost on the FP64 pipe)
+// largest cost on the FP64 pipe) of |v|: expm1(v) + 1 of a negative v would
+// keep 2^-53 absolutely, e^|v| too little (v reaches -28 next to a pole)
 STBEM_HD inline void sinh_cosh(float v, float& sh, float& ch) { sh = sinh(v); ch = cosh(v); }
 STBEM_HD inline void sinh_cosh(double v, double& sh, double& ch) {
-  const double t = expm1(v), e = t + 1.0, i = 1.0 / e;
-  sh = 0.5 * (t + t * i);
+  const double t = expm1(fabs(v)), e = t + 1.0, i = 1.0 / e;
+  sh = copysign(0.5 * (t + t * i), v);
   ch = 0.5 * (e + i);
 }
 
