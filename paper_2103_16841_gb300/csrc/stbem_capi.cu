@@ -88,7 +88,7 @@ bem_status bem_context_create(int device, bem_context** out) {
   std::unique_ptr<bem_context> ctx(new bem_context());
   ctx->device = device;
   STBEM_CUDA(cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking));
-  STBEM_CUDA(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
+  STBEM_CUDA(cudaStreamCreateWithFlags(&ctx->scratch.side, cudaStreamNonBlocking));
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   ctx->sm_count = sms;
@@ -103,7 +103,7 @@ bem_status bem_context_create(int device, bem_context** out) {
 void bem_context_destroy(bem_context* ctx) {
   if (!ctx) return;
   if (ctx->stream) cudaStreamDestroy(ctx->stream);
-  if (ctx->side) cudaStreamDestroy(ctx->side);
+  if (ctx->scratch.side) cudaStreamDestroy(ctx->scratch.side);
   scratch_trim(ctx->scratch);
   if (ctx->scratch.done) cudaEventDestroy(ctx->scratch.done);
   delete ctx;
@@ -413,6 +413,7 @@ bem_status stbem::op_layout(bem_operator* op, const int32_t* bw, const int64_t* 
       unsigned char* p = nullptr;
       TRY(dalloc(&p, (size_t)op->tmp_bytes));
       op->d_tmp = p;
+      STBEM_CUDA(cudaStreamCreateWithFlags(&op->side, cudaStreamNonBlocking));
     }
   } else if ((!op->opts.matrix_free && vo != op->nstored) || nnz != op->nnz) {
     set_error("reassembly changed the sparsity structure");
@@ -615,6 +616,7 @@ void bem_operator_destroy(bem_operator* op) {
   if (!op) return;
   cudaFree(op->d_pts); cudaFree(op->d_ptsf); cudaFree(op->d_gran); cudaFree(op->d_pts_trange); cudaFree(op->d_bw); cudaFree(op->d_bnnz);
   cudaFree(op->d_boff); cudaFree(op->d_rsoff); cudaFree(op->d_rs); cudaFree(op->d_val);
+  if (op->side) cudaStreamDestroy(op->side);
   cudaFree(op->d_val32); cudaFree(op->d_tmp); cudaFree(op->d_counter);
   cudaFree(op->d_ws); cudaFree(op->d_pv);
   cudaFree(op->d_tc_gptr); cudaFree(op->d_tc_gtb); cudaFree(op->d_tc_rs); cudaFree(op->d_tc_blk); cudaFree(op->d_tc_err);

@@ -423,46 +423,50 @@ void quad_scratch(const bem_operator* op, int64_t* least, int64_t* wanted) {
 }
 
 bem_status quad_launch(const bem_operator* op, int per_sm, int64_t end, const double* mf_x, double* mf_y, int nrhs,
-                       void* scratch, int64_t bytes, cudaStream_t s) {
+                       void* scratch, int64_t bytes, cudaStream_t side, cudaStream_t s) {
   BlockCtx B = make_ctx(op);
   const int64_t nb = op->mesh->n_col * op->mesh->n_col;
   B.mf_x = mf_x;
   B.mf_y = mf_y;
   B.mf_nrhs = nrhs;
   return stage_run(B, nullptr, nullptr, 1, op->opts.precision == BEM_PREC_MIXED, (int)op->ctx->sm_count,
-                   {&op->h_gran}, {nb}, std::min(end, nb), scratch, bytes, per_sm, op->ctx->side, s);
+                   {&op->h_gran}, {nb}, std::min(end, nb), scratch, bytes, per_sm, side, s);
 }
 
-bem_status ScratchHold::take(Scratch& c, bool own, int64_t least, int64_t wanted, cudaStream_t stream) {
+bem_status ScratchHold::take(Scratch& c, bool own_block, int64_t least, int64_t wanted, cudaStream_t stream) {
   s = stream;
-  if (!own) {
+  {
     std::lock_guard<std::mutex> lk(c.mu);
     if (!c.busy) {
-      if (c.bytes < wanted) {
-        cudaFree(c.p);   // (waits for the work on it)
-        c.p = nullptr;
-        c.bytes = 0;
-        if (cudaMalloc(&c.p, wanted) == cudaSuccess) {
-          c.bytes = wanted;
-        } else {
-          cudaGetLastError();
+      c.busy = true;
+      from = &c;
+      side = c.side;
+      if (!own_block) {
+        if (c.bytes < wanted) {
+          cudaFree(c.p);   // (waits for the work on it)
           c.p = nullptr;
+          c.bytes = 0;
+          if (cudaMalloc(&c.p, wanted) == cudaSuccess) {
+            c.bytes = wanted;
+          } else {
+            cudaGetLastError();
+            c.p = nullptr;
+          }
         }
-      }
-      if (!c.done && cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        c.done = nullptr;
-      }
-      if (c.p && c.done) {
-        STBEM_CUDA(cudaStreamWaitEvent(s, c.done, 0));
-        c.busy = true;
-        from = &c;
-        p = c.p;
-        bytes = c.bytes;
-        return BEM_OK;
+        if (!c.done && cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming) != cudaSuccess) {
+          cudaGetLastError();
+          c.done = nullptr;
+        }
+        if (c.p && c.done) {
+          STBEM_CUDA(cudaStreamWaitEvent(s, c.done, 0));
+          p = c.p;
+          bytes = c.bytes;
+          return BEM_OK;
+        }
       }
     }
   }
+  own = true;
   for (int64_t n = wanted;; n = std::max(least, n / 4)) {
     if (cudaMallocAsync(&p, n, s) == cudaSuccess) {
       bytes = n;
@@ -477,13 +481,11 @@ bem_status ScratchHold::take(Scratch& c, bool own, int64_t least, int64_t wanted
 }
 
 ScratchHold::~ScratchHold() {
-  if (from) {
-    std::lock_guard<std::mutex> lk(from->mu);
-    cudaEventRecord(from->done, s);
-    from->busy = false;
-  } else if (p) {
-    cudaFreeAsync(p, s);
-  }
+  if (own && p) cudaFreeAsync(p, s);
+  if (!from) return;
+  std::lock_guard<std::mutex> lk(from->mu);
+  if (!own && p) cudaEventRecord(from->done, s);
+  from->busy = false;
 }
 
 void scratch_trim(Scratch& c) {
@@ -502,9 +504,9 @@ bem_status op_quadrature(bem_operator* op, cudaStream_t s) {
   ScratchHold h;
   bem_status st = h.take(op->ctx->scratch, capped, least, wanted, s);
   if (st != BEM_OK) return st;
-  st = choose_quad_shape(op, h.p, h.bytes, s);
+  st = choose_quad_shape(op, h.p, h.bytes, h.side, s);
   if (st != BEM_OK) return st;
-  return quad_launch(op, op->quad_per_sm, op->mesh->n_col * op->mesh->n_col, nullptr, nullptr, 0, h.p, h.bytes, s);
+  return quad_launch(op, op->quad_per_sm, op->mesh->n_col * op->mesh->n_col, nullptr, nullptr, 0, h.p, h.bytes, h.side, s);
 }
 
 // Matrix-free product y = A x (internal order, [nrhs][n_tet]): the quadrature
@@ -512,7 +514,7 @@ bem_status op_quadrature(bem_operator* op, cudaStream_t s) {
 bem_status op_matvec_free(const bem_operator* op, const double* x, double* y, int nrhs, cudaStream_t s) {
   STBEM_CUDA(cudaMemsetAsync(y, 0, sizeof(double) * op->mesh->n_tet * nrhs, s));
   const int per_sm = op->quad_per_sm > 0 ? op->quad_per_sm : quad_max_per_sm(op);
-  return quad_launch(op, per_sm, op->mesh->n_col * op->mesh->n_col, x, y, nrhs, op->d_tmp, op->tmp_bytes, s);
+  return quad_launch(op, per_sm, op->mesh->n_col * op->mesh->n_col, x, y, nrhs, op->d_tmp, op->tmp_bytes, op->side, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -609,7 +611,7 @@ bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& 
   if (st != BEM_OK) return st;
   auto launch = [&](int per, int64_t end) {
     return stage_run(first, static_cast<const BlockCtx*>(dev.d_ctx), dev.d_prefix, (int)ops.size(), fp32, sms, gran,
-                     blocks, end, h.p, h.bytes, per, ops[0]->ctx->side, s);
+                     blocks, end, h.p, h.bytes, per, h.side, s);
   };
   int per = occ, how = 0;
   if (ops[0]->ctx->tune_mode) {

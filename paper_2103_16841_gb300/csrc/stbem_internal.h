@@ -51,27 +51,32 @@ struct SurfDev {
 }  // namespace stbem
 
 namespace stbem {
-// Quadrature scratch of a context, kept from one assembly to the next (at most
-// the largest that one wanted, 1 GiB) and given back when the context goes or
-// device memory runs short. One assembly holds it at a time; another one that
-// runs beside it (other threads) gets a block of its own, stream-ordered.
+// Quadrature scratch of a context and the second stream of its assemblies. The
+// memory is kept from one assembly to the next (at most the largest that one
+// wanted, 1 GiB) and given back when the context goes or device memory runs
+// short. One assembly holds both at a time; another one that runs beside it
+// (other threads) gets a block of its own, stream-ordered, and no second
+// stream. Only assemblies take it, and they are never captured: a stream that
+// has joined a capture must not meet other work.
 struct Scratch {
   std::mutex mu;
   void* p = nullptr;
   int64_t bytes = 0;
   bool busy = false;
+  cudaStream_t side = nullptr;
   cudaEvent_t done = nullptr;   // the last assembly's work on it
 };
 struct ScratchHold {
-  Scratch* from = nullptr;      // null: a block of its own
+  Scratch* from = nullptr;      // null: another assembly has the context's
   void* p = nullptr;
   int64_t bytes = 0;
-  cudaStream_t s = nullptr;
+  bool own = false;             // p is a block of its own
+  cudaStream_t s = nullptr, side = nullptr;   // side: null where there is none
   ScratchHold() = default;
   ScratchHold(const ScratchHold&) = delete;
   ScratchHold& operator=(const ScratchHold&) = delete;
-  // least <= bytes <= wanted; own: never the context's
-  bem_status take(Scratch& c, bool own, int64_t least, int64_t wanted, cudaStream_t stream);
+  // least <= bytes <= wanted; own_block: never the context's memory
+  bem_status take(Scratch& c, bool own_block, int64_t least, int64_t wanted, cudaStream_t stream);
   ~ScratchHold();
 };
 void scratch_trim(Scratch& c);  // frees it unless an assembly holds it
@@ -80,7 +85,6 @@ void scratch_trim(Scratch& c);  // frees it unless an assembly holds it
 struct bem_context {
   int device = 0;
   cudaStream_t stream = nullptr;
-  cudaStream_t side = nullptr;  // the quadrature's second stream
   stbem::Scratch scratch;       // of the assemblies on this context
   double sm_count = 0;
   int tune_mode = 0;          // 1: launch shapes timed per shape class (bem_context_set_tuning)
@@ -137,6 +141,7 @@ struct bem_operator {
   unsigned long long* d_counter = nullptr;  // work counter of the persistent kernels
   // quadrature scratch
   void* d_tmp = nullptr;         // matrix-free operators only: their products' scratch
+  cudaStream_t side = nullptr;   // and second stream (captured with them, so no one else's)
   int64_t tmp_bytes = 0;
   int64_t reserve_bytes = 0;     // bytes an admission reserves for the scratch
   int64_t scratch_cap = -1;      // >= 0: bytes the scratch may take beyond that (a server's slot), not the context's
@@ -178,11 +183,12 @@ int quad_max_per_sm(const bem_operator* op);
 // least and wanted bytes of an operator's quadrature scratch
 void quad_scratch(const bem_operator* op, int64_t* least, int64_t* wanted);
 // the quadrature over the blocks [0, end) of the dense (I, J) order, its
-// persistent stage with per_sm CTAs per SM (assembled, or summed against mf_x)
+// persistent stage with per_sm CTAs per SM (assembled, or summed against mf_x);
+// side: a second stream that nothing else uses meanwhile, or null
 bem_status quad_launch(const bem_operator* op, int per_sm, int64_t end, const double* mf_x, double* mf_y, int nrhs,
-                       void* scratch, int64_t bytes, cudaStream_t s);
+                       void* scratch, int64_t bytes, cudaStream_t side, cudaStream_t s);
 // sets op->quad_per_sm: the context's tuning cache, a timed choice, or the default (stbem_tune.cu)
-bem_status choose_quad_shape(bem_operator* op, void* scratch, int64_t bytes, cudaStream_t s);
+bem_status choose_quad_shape(bem_operator* op, void* scratch, int64_t bytes, cudaStream_t side, cudaStream_t s);
 // the tuner behind it: the fastest of the candidate launch codes of launch(code, end)
 // over a sample [0, end) of a block queue (the code's meaning is the caller's)
 bem_status tune_launch_shape(const bem_context* ctx, const std::string& key, const std::vector<int>& codes,

@@ -884,11 +884,12 @@ void stage_scratch(bool fp32, int max_tet, int max_surf, int sms, const std::vec
 // All stages over the blocks [0, end) of the concatenated operators. The
 // chunks alternate between two halves of the scratch: the FP64 faces (some
 // thousand per chunk, each a serial chain of most of a millisecond) and the
-// entries of one chunk run on the context's side stream while the caller's
-// stream takes the next chunk's apexes and FP32 faces. Large chunks pay: each
-// kernel of a chunk costs about 10 us of ramp and tail.Level-2
+// entries of one chunk run on the side stream (where there is one) while the
+// caller's stream takes the next chunk's apexes and FP32 faces. Large chunks
+// pay: each kernel of a chunk costs about 10 us of ramp and tail. Level-2
 // sphere, 15 slabs: 94 ms one chunk after the other, 45 ms so; level-3 sphere,
-// 8 slabs: 263 and 214 ms.
+// 8 slabs: 263 and 214 ms. On every way out the caller's stream waits for the
+// side stream.
 bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* prefix, int S, bool fp32, int sms,
                      const std::vector<const std::vector<uint2>*>& gran, const std::vector<int64_t>& blocks, int64_t end,
                      void* scratch, int64_t bytes, int per_sm, cudaStream_t side, cudaStream_t s) {
@@ -903,7 +904,7 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
       least = std::max(least, n);
       all += n;
     }
-  const int halves = bytes / 2 / 256 * 256 < (int64_t)(fixed + least) ? 1 : 2;
+  const int halves = !side || bytes / 2 / 256 * 256 < (int64_t)(fixed + least) ? 1 : 2;
   const int64_t half_bytes = bytes / halves / 256 * 256;
   StageArgs a;
   a.one = one;
@@ -931,6 +932,7 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
     for (auto& x : ev.e) STBEM_CUDA(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
 
   int64_t n_chunk = 0;
+  bool forked = false;   // the side stream has work of this run
   auto flush = [&](int64_t g0, int64_t g1, int64_t rays, int64_t slots) -> bem_status {
     if (rays == 0) return BEM_OK;
     const int64_t nb = g1 - g0;
@@ -964,6 +966,7 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
       if (halves == 1) return BEM_OK;
       STBEM_CUDA(cudaEventRecord(ev.e[h], s));
       STBEM_CUDA(cudaStreamWaitEvent(side, ev.e[h], 0));
+      forked = true;
       return BEM_OK;
     };
     if (fp32) {
@@ -1010,8 +1013,11 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
     off += blocks[o];
   }
   if (st == BEM_OK) st = flush(g0, g1, rays, slots);
-  // the caller's stream goes on when the side stream is done (its last event covers all before it)
-  if (halves == 2 && n_chunk > 0) STBEM_CUDA(cudaStreamWaitEvent(s, ev.e[2 + (n_chunk - 1) % 2], 0));
+  // the caller's stream goes on when the side stream is done
+  if (forked) {
+    STBEM_CUDA(cudaEventRecord(ev.e[2], side));
+    STBEM_CUDA(cudaStreamWaitEvent(s, ev.e[2], 0));
+  }
   return st;
 }
 

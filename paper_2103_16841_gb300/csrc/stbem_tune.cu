@@ -142,7 +142,7 @@ bem_status tune_launch_shape(const bem_context* ctx, const std::string& key, con
 
 // Candidates: the occupancy and the one or two CTA counts below it; code =
 // CTAs per SM - 1.
-bem_status choose_quad_shape(bem_operator* op, void* scratch, int64_t bytes, cudaStream_t s) {
+bem_status choose_quad_shape(bem_operator* op, void* scratch, int64_t bytes, cudaStream_t side, cudaStream_t s) {
   if (op->quad_per_sm > 0) return BEM_OK;
   if (op->ctx->tune_mode == 0 || op->opts.matrix_free) {
     op->quad_per_sm = quad_max_per_sm(op);
@@ -155,7 +155,9 @@ bem_status choose_quad_shape(bem_operator* op, void* scratch, int64_t bytes, cud
   // sample: 1/32 of the dense block order, at least 16 test columns
   const int64_t nblk = op->mesh->n_col * op->mesh->n_col;
   const int64_t end = std::min(nblk, std::max(nblk / 32, 16 * op->mesh->n_col));
-  auto launch = [&](int code, int64_t e) { return quad_launch(op, code + 1, e, nullptr, nullptr, 0, scratch, bytes, s); };
+  auto launch = [&](int code, int64_t e) {
+    return quad_launch(op, code + 1, e, nullptr, nullptr, 0, scratch, bytes, side, s);
+  };
   int best = 0;
   const bem_status st = tune_launch_shape(op->ctx, shape_class(op), codes, end, launch, s, &best, &op->quad_tuned,
                                           op->tune_ms);
