@@ -274,7 +274,20 @@ static bem_status mv_launch(K kern, int64_t n_cols, unsigned groups, unsigned c,
   return BEM_OK;
 }
 
-// One launch, a layer of the grid per group of NR right-hand sides; x packed [group][n][NR] (PACKED) or [nrhs][n].
+// Right-hand sides [r0, r0 + k) in launches of at most as many groups of nr as a grid has layers
+constexpr int kMaxLayers = 65535;
+template <typename F>
+static bem_status in_layers(int nr, int r0, int k, F launch) {
+  for (const int end = r0 + k; r0 < end;) {
+    const int n = std::min<int64_t>(end - r0, (int64_t)kMaxLayers * nr);
+    const bem_status st = launch(r0, n);
+    if (st != BEM_OK) return st;
+    r0 += n;
+  }
+  return BEM_OK;
+}
+
+// A layer of the grid per group of NR right-hand sides; x packed [group][n][NR] (PACKED) or [nrhs][n].
 template <typename V, typename Acc, typename XT, bool PACKED>
 static bem_status spmv_launch(const bem_operator* op, const V* val, const XT* x, double* y, int nrhs, cudaStream_t s) {
   const bem_mesh* m = op->mesh;
@@ -282,11 +295,13 @@ static bem_status spmv_launch(const bem_operator* op, const V* val, const XT* x,
   return with_shape(vec_width<V, Acc>(m->col_gcd), nrhs, [&](auto vec, auto nrc) -> bem_status {
     constexpr int VEC = sizeof(Acc) == 8 ? 1 : decltype(vec)::value, NR = decltype(nrc)::value;
     const unsigned c = mv_cluster(m->n_col, m->n_col, kMvThreads * VEC / m->max_col_tets);
-    auto launch = [&](auto kern, int nr, int r0, int k) {   // k right-hand sides from r0 on, nr at a time
-      return mv_launch(kern, m->n_col, (unsigned)((k + nr - 1) / nr), c, sizeof(Acc) * kMvThreads * VEC * nr, s, m->n_col,
-                       (const int32_t*)m->d_col_tet_begin, (const int32_t*)op->d_bw, (const int64_t*)op->d_boff,
-                       (const int64_t*)op->d_rsoff, (const int32_t*)op->d_rs, val, x + (int64_t)r0 * n,
-                       y + (int64_t)r0 * n, n, k);
+    auto launch = [&](auto kern, int nr, int first, int count) {   // nr right-hand sides at a time
+      return in_layers(nr, first, count, [&](int r0, int k) {
+        return mv_launch(kern, m->n_col, (unsigned)((k + nr - 1) / nr), c, sizeof(Acc) * kMvThreads * VEC * nr, s, m->n_col,
+                         (const int32_t*)m->d_col_tet_begin, (const int32_t*)op->d_bw, (const int64_t*)op->d_boff,
+                         (const int64_t*)op->d_rsoff, (const int32_t*)op->d_rs, val, x + (int64_t)r0 * n,
+                         y + (int64_t)r0 * n, n, k);
+      });
     };
     // a last vector alone takes the kernel for one (where x is not packed)
     const int alone = !PACKED && NR > 1 && nrhs % NR == 1 ? 1 : 0;
@@ -398,9 +413,11 @@ bem_status BatchMatvec::apply(const double* x, double* y, int K, int arith, cuda
       constexpr int VEC = sizeof(Acc) == 8 ? 1 : decltype(vec)::value, NR = decltype(nrc)::value;
       constexpr bool PACKED = decltype(packed)::value;
       const unsigned c = mv_cluster(n_cta, max_cols, kMvThreads * VEC / max_rows);
-      auto launch = [&](auto kern, int nr, int r0, int k) {
-        return mv_launch(kern, n_cta, (unsigned)((k + nr - 1) / nr), c, sizeof(Acc) * kMvThreads * VEC * nr, s, sg,
-                         (const int32_t*)d_cseg, (const int32_t*)d_ccol, xin + (int64_t)r0 * N, y + (int64_t)r0 * N, N, k);
+      auto launch = [&](auto kern, int nr, int first, int count) {
+        return in_layers(nr, first, count, [&](int r0, int k) {
+          return mv_launch(kern, n_cta, (unsigned)((k + nr - 1) / nr), c, sizeof(Acc) * kMvThreads * VEC * nr, s, sg,
+                           (const int32_t*)d_cseg, (const int32_t*)d_ccol, xin + (int64_t)r0 * N, y + (int64_t)r0 * N, N, k);
+        });
       };
       const int alone = !PACKED && NR > 1 && K % NR == 1 ? 1 : 0;
       bem_status st = launch(k_matvec_batch<V, Acc, XT, NR, VEC, PACKED>, NR, 0, K - alone);
