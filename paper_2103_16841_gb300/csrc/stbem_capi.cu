@@ -397,7 +397,7 @@ bem_status stbem::op_layout(bem_operator* op, const int32_t* bw, const int64_t* 
                                                 16 * m->n_tet);
     }
     if (op->opts.matrix_free) op->nstored = 0;
-    if (op->admit) TRY(op->admit(op));
+    if (op->admit) TRY(op->admit(op, bw));
     if (!op->opts.matrix_free) {
       // mixed-precision values carry FP32 accuracy: FP32 storage only
       if (op->opts.precision == BEM_PREC_FP64) TRY(dalloc_room(op->ctx, &op->d_val, (size_t)vo));
@@ -523,7 +523,7 @@ bem_status bem_operator_create(bem_context* ctx, const bem_mesh* mesh, const bem
 }  // extern "C"
 
 bem_status stbem::operator_create(bem_context* ctx, const bem_mesh* mesh, const bem_op_opts* opts,
-                                  std::function<bem_status(const bem_operator*)> admit, bem_operator** out,
+                                  std::function<bem_status(const bem_operator*, const int32_t*)> admit, bem_operator** out,
                                   int64_t scratch_cap) {
   if (!ctx || !mesh || !out) { set_error("bem_operator_create: invalid argument"); return BEM_ERR_INVALID_ARG; }
   *out = nullptr;

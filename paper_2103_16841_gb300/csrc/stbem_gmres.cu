@@ -329,6 +329,15 @@ struct ItemTables {
 
 }  // namespace
 
+int64_t gmres_bytes(int64_t n, int nrhs, int restart, bool refined) {
+  const int64_t K = nrhs, m = restart, items = K * ((n + CH - 1) / CH);
+  // V, w, vj, r, and the refinement's r, dx, Ax
+  int64_t b = 8 * n * K * (m + 4 + (refined ? 3 : 0));
+  b += items * (8 * (m + 1) + 16) + 4 * (K + 1);                       // partial sums, item tables
+  b += K * (8 * ((m + 1) * m + 3 * (m + 1) + 3 * m + 4) + 3 * 4) + 16;   // GState
+  return b + 32 * 512;                                                 // granules of the allocations
+}
+
 bem_status seg_norms(const SegLayout& L, const double* v, std::vector<double>& out, cudaStream_t s) {
   const int C = L.K * L.S;
   ItemTables T;

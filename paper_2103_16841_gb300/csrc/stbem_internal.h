@@ -164,8 +164,10 @@ struct bem_operator {
   mutable bool tcv_stale[2] = {false, false};   // the values were reassembled since the slots were made
   mutable int* d_tc_err = nullptr;         // set when a tensor-core product gave up on a wait
   // optional admission hook, called once the sparsity structure is known
-  // (nstored, nrows_stored, reserve_bytes set) and before the value arrays are allocated
-  std::function<bem_status(const bem_operator*)> admit;
+  // (nstored, nrows_stored, reserve_bytes set) and before the value arrays are allocated;
+  // bw: the blocks' band widths on the host
+  std::function<bem_status(const bem_operator*, const int32_t* bw)> admit;
+  mutable struct { int64_t groups = 0, nblk = 0, nrows = 0, slots[2] = {0, 0}; } tc_plan;   // sizes admitted (tc_bytes)
 };
 
 namespace stbem {
@@ -244,7 +246,7 @@ bem_status gmres_solve_layout(const SegLayout& L, const MatvecFn& mv_hi, const M
                               double* d_x, const bem_solve_opts* o, bem_solve_info* info, cudaStream_t s);
 // operator creation with an admission hook (see bem_operator::admit)
 bem_status operator_create(bem_context* ctx, const bem_mesh* mesh, const bem_op_opts* opts,
-                           std::function<bem_status(const bem_operator*)> admit, bem_operator** out,
+                           std::function<bem_status(const bem_operator*, const int32_t*)> admit, bem_operator** out,
                            int64_t scratch_cap = -1);
 // operator object with its structure arrays allocated (nothing assembled yet)
 bem_status op_structure_alloc(bem_context* ctx, const bem_mesh* mesh, const bem_op_opts* opts,
@@ -264,6 +266,14 @@ bem_status op_outer_points_all(const std::vector<bem_operator*>& ops, cudaStream
 bem_status op_pattern_batch(const std::vector<bem_operator*>& ops, BatchDev& dev, cudaStream_t s);
 bem_status op_quadrature_batch(const std::vector<bem_operator*>& ops, BatchDev& dev, cudaStream_t s);
 size_t block_ctx_size();
+// bytes of the tensor-core product's tables and chunk slots of one type while they
+// are made (bw: the blocks' band widths; needed the first time only)
+int64_t tc_bytes(const bem_operator* op, const int32_t* bw, bool bf16);
+// bytes of the workspace of a product with nrhs right-hand sides (tensor-core types: after tc_bytes)
+int64_t matvec_ws_bytes(const bem_operator* op, int arith, int nrhs);
+int64_t packed_len(int64_t n, int nrhs);
+// bytes of gmres_solve's vectors and tables beside the products' workspace
+int64_t gmres_bytes(int64_t n, int nrhs, int restart, bool refined);
 // bytes held by an operator's value arrays, row starts and quadrature scratch
 int64_t operator_value_bytes(const bem_operator* op);
 // arithmetic of a product (values equal to BEM_DTYPE_*)

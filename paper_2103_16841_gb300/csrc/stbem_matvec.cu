@@ -317,7 +317,7 @@ static void pack_x(const double* x, float* out, int64_t n, int nrhs, cudaStream_
 }
 
 // FP32 numbers of the packed x of nrhs vectors of n entries
-static int64_t packed_len(int64_t n, int nrhs) { return nrhs == 1 ? n : n * ((nrhs + 3) / 4) * 4; }
+int64_t packed_len(int64_t n, int nrhs) { return nrhs == 1 ? n : n * ((nrhs + 3) / 4) * 4; }
 
 bem_status op_matvec(const bem_operator* op, const double* x, double* y, int nrhs, int arith, cudaStream_t s) {
   // matrix-free operators: the operator's own precision, whatever `arith` asks

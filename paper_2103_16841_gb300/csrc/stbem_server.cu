@@ -183,18 +183,15 @@ int64_t structure_bytes(const bem_mesh* m) {
          m->n_surf * (int64_t)(sizeof(SurfDev) + (MAX_NQ * 4 + 2) * 8 + MAX_NQ * 4 * 4) + nb * (4 + 8 + 8 + 8);
 }
 
-// operator values + solver workspace for nrhs right-hand sides
-int64_t admission_bytes(const bem_operator* op, const bem_server_opts& o, int nrhs) {
-  const int64_t n = op->mesh->n_tet;
-  int64_t b = operator_value_bytes(op);
-  b += n * (int64_t)nrhs * 8 * (o.restart + 1 + 8);  // Krylov basis, b, x, r, w, dx, Ax, permutations
+// operator values + solver workspace for nrhs right-hand sides (bw: the blocks'
+// band widths, null for an operator that was admitted before). The integrals of
+// the right-hand sides over the faces go before the solve's vectors come.
+int64_t admission_bytes(const bem_operator* op, const int32_t* bw, const bem_server_opts& o, int nrhs) {
+  int64_t b = operator_value_bytes(op) + 3 * 8 * op->mesh->n_tet * (int64_t)nrhs;   // b, x, the density
+  b += gmres_bytes(op->mesh->n_tet, nrhs, o.restart, o.inner_dtype != BEM_DTYPE_FP64);
   if (o.inner_dtype == BEM_DTYPE_TF32 || o.inner_dtype == BEM_DTYPE_BF16)
-    b += (n + 1) * (int64_t)std::min(nrhs, 64) * 8 * 2;
-  if (o.inner_dtype == BEM_DTYPE_FP32) b += n * (int64_t)nrhs * 4;
-  // chunk slots of the tensor-core product: at most two 16-byte slots per block row beyond the values
-  if (o.inner_dtype == BEM_DTYPE_TF32) b += op->nstored * 4 + op->nrows_stored * 32;
-  if (o.inner_dtype == BEM_DTYPE_BF16) b += op->nstored * 2 + op->nrows_stored * 32;
-  return b;
+    b += tc_bytes(op, bw, o.inner_dtype == BEM_DTYPE_BF16);
+  return b + matvec_ws_bytes(op, o.inner_dtype, nrhs);
 }
 
 // Right-hand side, solve and density of a request on an assembled operator
@@ -288,7 +285,7 @@ bem_status run_job(bem_server* S, bem_context* cx, const Job& J, Done& D, int64_
     }
   } mark{S, key, builder};
   if (hit) {
-    const int64_t need = admission_bytes(hit->op, S->o, nrhs) - operator_value_bytes(hit->op);
+    const int64_t need = admission_bytes(hit->op, nullptr, S->o, nrhs) - operator_value_bytes(hit->op);
     bem_status st = acquire(S, J.ticket, need);
     if (st == BEM_OK) {
       reserved = need;
@@ -323,8 +320,8 @@ bem_status run_job(bem_server* S, bem_context* cx, const Job& J, Done& D, int64_
   bem_operator* op = nullptr;
   const uint64_t ticket = J.ticket;
   bem_server_opts so_srv = S->o;
-  st = operator_create(cx, mesh, &oo, [&, ticket, nrhs](const bem_operator* o2) -> bem_status {
-        const int64_t need = admission_bytes(o2, so_srv, nrhs);
+  st = operator_create(cx, mesh, &oo, [&, ticket, nrhs](const bem_operator* o2, const int32_t* bw) -> bem_status {
+        const int64_t need = admission_bytes(o2, bw, so_srv, nrhs);
         bem_status a = acquire(S, ticket, need);
         if (a == BEM_OK) reserved = need;
         return a;

@@ -669,6 +669,94 @@ __global__ void k_tc_sum(const double* __restrict__ part, double* __restrict__ y
   }
 }
 
+// Row groups of a mesh and their non-empty blocks, from the blocks' band widths
+struct TcLayout {
+  std::vector<int32_t> gcol{0}, gtb{0};   // [groups + 1] first column and row of a group
+  std::vector<int32_t> ptr, bG, bJ, bW;   // blocks of a group; group, trial column and widest band of a block
+  std::vector<int64_t> ro, vc16, vc32;    // its row starts and chunk slots (16 bytes each)
+  int64_t nrows = 0, slots[2] = {0, 0}, cap[2] = {0, 0};   // in all, and most slot bytes of a block
+  int max_rows = 0;
+  int64_t groups() const { return (int64_t)gcol.size() - 1; }
+};
+TcLayout tc_layout(const bem_mesh* m, const int32_t* bw) {
+  TcLayout L;
+  const int64_t nc = m->n_col;
+  // consecutive columns to at most 128 rows (one M tile); a taller column is a group of its own
+  for (int64_t I = 0; I < nc;) {
+    int64_t e = I + 1;
+    while (e < nc && m->col_tet_begin[e + 1] - m->col_tet_begin[I] <= 128) ++e;
+    L.max_rows = std::max(L.max_rows, m->col_tet_begin[e] - m->col_tet_begin[I]);
+    L.gcol.push_back((int32_t)e);
+    L.gtb.push_back(m->col_tet_begin[e]);
+    I = e;
+  }
+  L.ptr.assign(L.groups() + 1, 0);
+  std::vector<int32_t> wmax(nc);
+  for (int64_t g = 0; g < L.groups(); ++g) {
+    const int64_t nt = L.gtb[g + 1] - L.gtb[g];
+    std::fill(wmax.begin(), wmax.end(), 0);
+    for (int64_t I = L.gcol[g]; I < L.gcol[g + 1]; ++I)
+      for (int64_t J = 0; J < nc; ++J) wmax[J] = std::max(wmax[J], bw[I * nc + J]);
+    for (int64_t J = 0; J < nc; ++J) {
+      const int W = wmax[J];
+      if (W <= 0) continue;
+      L.bG.push_back((int32_t)g);
+      L.bJ.push_back((int32_t)J);
+      L.bW.push_back(W);
+      L.ro.push_back(L.nrows);
+      L.vc16.push_back(L.slots[0]);
+      L.vc32.push_back(L.slots[1]);
+      L.nrows += nt;
+      for (int t = 0; t < 2; ++t) {
+        const int64_t n = tc_slots(W, t ? 4 : 8) * nt;
+        L.slots[t] += n;
+        L.cap[t] = std::max(L.cap[t], n * 16);
+      }
+    }
+    L.ptr[g + 1] = (int32_t)L.bG.size();
+  }
+  return L;
+}
+
+// device arrays of the tables: group blocks, group rows, block records and row
+// starts, which stay; the blocks' group, trial column, band, row starts and slots
+// of both types, and the spans, which do not
+constexpr int kTcArrays = 11;
+void tc_array_bytes(int64_t groups, int64_t nblk, int64_t nrows, size_t* bytes) {
+  const size_t nb = (size_t)std::max<int64_t>(nblk, 1), i4 = sizeof(int32_t), i8 = sizeof(int64_t);
+  const size_t b[kTcArrays] = {i4 * (groups + 1), i4 * (groups + 1), sizeof(TcBlk) * nb,
+                               i4 * (size_t)(nrows + 4) /* whole 16-byte granules are copied */, i4 * nb, i4 * nb, i4 * nb,
+                               i8 * nb, i8 * nb, i8 * nb, sizeof(int) * 2};
+  std::copy(b, b + kTcArrays, bytes);
+}
+
+// CTAs that share a group's blocks: some four CTAs per SM in all, of at least
+// eight blocks each. The
+// tensor cores' FP32 accumulation truncates, so a row's sum cut in parts
+// comes out closer to the exact one, by an amount that grows with the row:
+// the level-3 sphere with 8 slabs (11,300 values per row) moves by 1.2e-5 in
+// BF16 and 1.9e-5 in TF32 with two parts, the level-2 sphere with 32 slabs
+// (5,300) by 4e-6 and 6e-6. Long rows are therefore cut in two at most, or
+// left whole, to stay within 1.3e-5 of the uncut sum.
+int tc_parts(int64_t groups, int64_t nblk, int64_t per_row, bool bf16) {
+  const int64_t per_group = nblk / std::max<int64_t>(groups, 1);
+  const int most = per_row > 8000 ? (bf16 ? 2 : 1) : per_row > 3000 ? 2 : 8;
+  int parts = 1;
+  while (parts < most && groups * parts < 4 * 152 && per_group >= 16 * parts) parts *= 2;
+  return parts;
+}
+
+// MMA N of a pass
+int tc_n(int nrhs) { return std::max(16, (nrhs + 15) / 16 * 16); }
+// FP32 numbers of the packed x (16 bytes per chunk and right-hand side) and of the parts' sums
+int64_t tc_xc_len(int64_t n, int nrhs, bool bf16) {
+  const int E = bf16 ? 8 : 4;
+  return (n + E - 1) / E * tc_n(nrhs) * 4;
+}
+int64_t tc_ws_len(int64_t n, int nrhs, int parts, bool bf16) {
+  return tc_xc_len(n, nrhs, bf16) + (parts > 1 ? 2 * parts * n * nrhs : 0);
+}
+
 // Row groups and block records of the operator (made once; an operator's
 // sparsity structure never changes): the non-empty blocks of each group, their
 // band unions, the offsets of their chunk slots in both types, and the row
@@ -680,54 +768,15 @@ bem_status ensure_tc_meta(const bem_operator* op, cudaStream_t s) {
   std::vector<int32_t> hbw(nc * nc);
   STBEM_CUDA(cudaMemcpyAsync(hbw.data(), op->d_bw, sizeof(int32_t) * nc * nc, cudaMemcpyDeviceToHost, s));
   STBEM_CUDA(cudaStreamSynchronize(s));
-  // consecutive columns to at most 128 rows (one M tile); a taller column is a group of its own
-  std::vector<int32_t> gcol{0}, gtb{0};
-  int max_rows = 0;
-  for (int64_t I = 0; I < nc;) {
-    int64_t e = I + 1;
-    while (e < nc && m->col_tet_begin[e + 1] - m->col_tet_begin[I] <= 128) ++e;
-    max_rows = std::max(max_rows, m->col_tet_begin[e] - m->col_tet_begin[I]);
-    gcol.push_back((int32_t)e);
-    gtb.push_back(m->col_tet_begin[e]);
-    I = e;
-  }
-  const int64_t ng = (int64_t)gcol.size() - 1;
-  std::vector<int32_t> ptr(ng + 1, 0), bG, bJ, bW, wmax(nc);
-  std::vector<int64_t> ro, vc16, vc32;
-  int64_t orow = 0, o16 = 0, o32 = 0, cap16 = 0, cap32 = 0;
-  for (int64_t g = 0; g < ng; ++g) {
-    const int64_t nt = gtb[g + 1] - gtb[g];
-    std::fill(wmax.begin(), wmax.end(), 0);
-    for (int64_t I = gcol[g]; I < gcol[g + 1]; ++I)
-      for (int64_t J = 0; J < nc; ++J) wmax[J] = std::max(wmax[J], hbw[I * nc + J]);
-    for (int64_t J = 0; J < nc; ++J) {
-      const int W = wmax[J];
-      if (W <= 0) continue;
-      bG.push_back((int32_t)g);
-      bJ.push_back((int32_t)J);
-      bW.push_back(W);
-      ro.push_back(orow);
-      vc16.push_back(o16);
-      vc32.push_back(o32);
-      orow += nt;
-      o16 += tc_slots(W, 8) * nt;
-      o32 += tc_slots(W, 4) * nt;
-      cap16 = std::max<int64_t>(cap16, tc_slots(W, 8) * nt * 16);
-      cap32 = std::max<int64_t>(cap32, tc_slots(W, 4) * nt * 16);
-    }
-    ptr[g + 1] = (int32_t)bG.size();
-  }
-  const int64_t nb = (int64_t)bG.size();
+  const TcLayout L = tc_layout(m, hbw.data());
+  const int64_t ng = L.groups(), nb = (int64_t)L.bG.size();
   struct Arrays {   // freed on every way out unless released
-    void* p[11] = {};
+    void* p[kTcArrays] = {};
     ~Arrays() { for (void* q : p) cudaFree(q); }
   } A;
-  const size_t nb1 = (size_t)std::max<int64_t>(nb, 1);
-  const size_t bytes[11] = {sizeof(int32_t) * (ng + 1), sizeof(int32_t) * (ng + 1), sizeof(TcBlk) * nb1,
-                            sizeof(int32_t) * (size_t)(orow + 4) /* whole 16-byte granules are copied */, sizeof(int32_t) * nb1,
-                            sizeof(int32_t) * nb1, sizeof(int32_t) * nb1, sizeof(int64_t) * nb1, sizeof(int64_t) * nb1,
-                            sizeof(int64_t) * nb1, sizeof(int) * 2};
-  for (int k = 0; k < 11; ++k)
+  size_t bytes[kTcArrays];
+  tc_array_bytes(ng, nb, L.nrows, bytes);
+  for (int k = 0; k < kTcArrays; ++k)
     if (cudaMalloc(&A.p[k], bytes[k]) != cudaSuccess) {
       cudaGetLastError();
       A.p[k] = nullptr;
@@ -735,9 +784,9 @@ bem_status ensure_tc_meta(const bem_operator* op, cudaStream_t s) {
       return BEM_ERR_OUT_OF_MEMORY;
     }
   int hspan[2] = {0, 0};
-  const void* src[11] = {ptr.data(), gtb.data(), nullptr, nullptr, bG.data(), bJ.data(), bW.data(),
-                         ro.data(), vc16.data(), vc32.data(), hspan};
-  for (int k = 0; k < 11; ++k)
+  const void* src[kTcArrays] = {L.ptr.data(), L.gtb.data(), nullptr, nullptr, L.bG.data(), L.bJ.data(), L.bW.data(),
+                                L.ro.data(), L.vc16.data(), L.vc32.data(), hspan};
+  for (int k = 0; k < kTcArrays; ++k)
     if (src[k] && (nb > 0 || k < 2 || k == 10)) STBEM_CUDA(cudaMemcpyAsync(A.p[k], src[k], bytes[k], cudaMemcpyHostToDevice, s));
   if (nb > 0) {
     const int64_t threads = nb * 32;
@@ -764,15 +813,15 @@ bem_status ensure_tc_meta(const bem_operator* op, cudaStream_t s) {
   op->d_tc_rs = (int32_t*)A.p[3];
   for (int k = 0; k < 4; ++k) A.p[k] = nullptr;
   op->tc_groups = ng;
-  op->tc_rows = max_rows;
-  op->tc_nrows = orow;
+  op->tc_rows = L.max_rows;
+  op->tc_nrows = L.nrows;
   op->tc_nblk = nb;
   op->tc_span[0] = hspan[0];
   op->tc_span[1] = hspan[1];
-  op->tcv_len[0] = o16;
-  op->tcv_len[1] = o32;
-  op->tcv_cap[0] = cap16;
-  op->tcv_cap[1] = cap32;
+  for (int t = 0; t < 2; ++t) {
+    op->tcv_len[t] = L.slots[t];
+    op->tcv_cap[t] = L.cap[t];
+  }
   return BEM_OK;
 }
 
@@ -817,6 +866,26 @@ bem_status launch_tc(int kind, const TcArgs& a, const CUtensorMap& map, size_t s
 
 }  // namespace
 
+int64_t tc_bytes(const bem_operator* op, const int32_t* bw, bool bf16) {
+  if (!op->tc_plan.groups) {
+    const TcLayout L = tc_layout(op->mesh, bw);
+    op->tc_plan = {L.groups(), (int64_t)L.bG.size(), L.nrows, {L.slots[0], L.slots[1]}};
+  }
+  size_t a[kTcArrays];
+  tc_array_bytes(op->tc_plan.groups, op->tc_plan.nblk, op->tc_plan.nrows, a);
+  int64_t b = sizeof(int) + 16 * std::max<int64_t>(op->tc_plan.slots[bf16 ? 0 : 1], 1);
+  for (size_t x : a) b += (int64_t)x;
+  return b;
+}
+
+int64_t matvec_ws_bytes(const bem_operator* op, int arith, int nrhs) {
+  const int64_t n = op->mesh->n_tet;
+  if (arith == MV_FP32) return 4 * packed_len(n, nrhs);
+  if (arith != MV_TF32 && arith != MV_BF16) return 0;
+  const bool bf16 = arith == MV_BF16;
+  return 4 * tc_ws_len(n, std::min(nrhs, 64), tc_parts(op->tc_plan.groups, op->tc_plan.nblk, op->nstored / n, bf16), bf16);
+}
+
 int64_t tc_table_bytes(const bem_operator* op) {
   int64_t b = op->d_tc_blk ? op->tc_nblk * (int64_t)sizeof(TcBlk) + (op->tc_groups + 1) * 8 + op->tc_nrows * 4 : 0;
   for (int t = 0; t < 2; ++t)
@@ -843,21 +912,11 @@ bem_status op_spmm_tc(const bem_operator* op, const double* x, double* y, int nr
     return BEM_ERR_UNSUPPORTED;
   }
   const int E = bf16 ? 8 : 4;
-  const int N = std::max(16, (nrhs + 15) / 16 * 16);
+  const int N = tc_n(nrhs);
   const int64_t nchunks = (n + E - 1) / E;
-  // parts: some four CTAs per SM in all, of at least eight blocks each. The
-  // tensor cores' FP32 accumulation truncates, so a row's sum cut in parts
-  // comes out closer to the exact one, by an amount that grows with the row:
-  // the level-3 sphere with 8 slabs (11,300 values per row) moves by 1.2e-5 in
-  // BF16 and 1.9e-5 in TF32 with two parts, the level-2 sphere with 32 slabs
-  // (5,300) by 4e-6 and 6e-6. Long rows are therefore cut in two at most, or
-  // left whole, to stay within 1.3e-5 of the uncut sum.
-  const int64_t per_group = op->tc_nblk / std::max<int64_t>(op->tc_groups, 1), per_row = op->nstored / n;
-  const int most = per_row > 8000 ? (bf16 ? 2 : 1) : per_row > 3000 ? 2 : 8;
-  int parts = 1;
-  while (parts < most && op->tc_groups * parts < 4 * 152 && per_group >= 16 * parts) parts *= 2;
-  const int64_t xc_len = nchunks * N * 4;       // 16 bytes per (chunk, rhs)
-  TRY_STATUS(ensure_ws(op, xc_len + (parts > 1 ? 2 * parts * n * nrhs : 0)));
+  const int parts = tc_parts(op->tc_groups, op->tc_nblk, op->nstored / n, bf16);
+  const int64_t xc_len = tc_xc_len(n, nrhs, bf16);
+  TRY_STATUS(ensure_ws(op, tc_ws_len(n, nrhs, parts, bf16)));
   void* Xc = op->d_ws;
   if (bf16) k_pack_xc<false><<<grid_for(nchunks * N * E), 256, 0, s>>>(x, n, nrhs, N, nchunks, Xc);
   else k_pack_xc<true><<<grid_for(nchunks * N * E), 256, 0, s>>>(x, n, nrhs, N, nchunks, Xc);
