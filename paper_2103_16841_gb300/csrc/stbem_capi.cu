@@ -409,7 +409,9 @@ bem_status stbem::op_layout(bem_operator* op, const int32_t* bw, const int64_t* 
     if (own_scratch && op->opts.matrix_free) {
       int64_t least = 0, wanted = 0;
       quad_scratch(op, &least, &wanted);
-      op->tmp_bytes = std::max(least, std::min(wanted, std::max<int64_t>(4 * vo, (int64_t)64 << 20)));
+      // a sixteenth of what the values would take, or 64 MiB
+      const int64_t values = (op->opts.precision == BEM_PREC_FP64 ? 8 : 4) * vo;
+      op->tmp_bytes = std::max(least, std::min(wanted, std::max<int64_t>(values / 16, (int64_t)64 << 20)));
       unsigned char* p = nullptr;
       TRY(dalloc(&p, (size_t)op->tmp_bytes));
       op->d_tmp = p;
@@ -508,6 +510,7 @@ bem_status assemble(bem_operator* op, cudaStream_t s, bool first) {
 }  // namespace
 
 int64_t stbem::operator_value_bytes(const bem_operator* op) {
+  if (op->opts.matrix_free) return op->tmp_bytes;
   int64_t b = 0;
   if (op->opts.precision == BEM_PREC_FP64) b += 8 * op->nstored;
   if (op->opts.store_fp32 || op->opts.precision == BEM_PREC_MIXED) b += 4 * op->nstored;
@@ -872,6 +875,7 @@ bem_status bem_matvec(const bem_operator* op, const double* x_dev, double* y_dev
   double* xi = op->d_pv;
   double* yi = op->d_pv + nn;
   TRY(permute(m->d_perm, x_dev, xi, m->n_tet, nrhs, true, s));
+  FreeScratch scratch(op, s);
   TRY(op_matvec(op, xi, yi, nrhs, false, s));
   TRY(permute(m->d_perm, yi, y_dev, m->n_tet, nrhs, false, s));
   return BEM_OK;
@@ -890,6 +894,7 @@ bem_status bem_matvec_dtype(const bem_operator* op, const double* x_dev, double*
   double* xi = op->d_pv;
   double* yi = op->d_pv + nn;
   TRY(permute(m->d_perm, x_dev, xi, m->n_tet, nrhs, true, s));
+  FreeScratch scratch(op, s);
   TRY(op_matvec(op, xi, yi, nrhs, dtype, s));
   TRY(permute(m->d_perm, yi, y_dev, m->n_tet, nrhs, false, s));
   return BEM_OK;

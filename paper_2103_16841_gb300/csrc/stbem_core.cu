@@ -433,39 +433,54 @@ bem_status quad_launch(const bem_operator* op, int per_sm, int64_t end, const do
                    {&op->h_gran}, {nb}, std::min(end, nb), scratch, bytes, per_sm, side, s);
 }
 
-bem_status ScratchHold::take(Scratch& c, bool own_block, int64_t least, int64_t wanted, cudaStream_t stream) {
-  s = stream;
-  {
-    std::lock_guard<std::mutex> lk(c.mu);
-    if (!c.busy) {
-      c.busy = true;
-      from = &c;
-      side = c.side;
-      if (!own_block) {
-        if (c.bytes < wanted) {
-          cudaFree(c.p);   // (waits for the work on it)
-          c.p = nullptr;
-          c.bytes = 0;
-          if (cudaMalloc(&c.p, wanted) == cudaSuccess) {
-            c.bytes = wanted;
-          } else {
-            cudaGetLastError();
-            c.p = nullptr;
-          }
-        }
-        if (!c.done && cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming) != cudaSuccess) {
-          cudaGetLastError();
-          c.done = nullptr;
-        }
-        if (c.p && c.done) {
-          STBEM_CUDA(cudaStreamWaitEvent(s, c.done, 0));
-          p = c.p;
-          bytes = c.bytes;
-          return BEM_OK;
-        }
-      }
+// takes the context's second stream and, with `memory`, its scratch (true if there is that
+// much), unless they are held, or in use by unfinished work of another stream
+bool ScratchHold::claim(Scratch& c, bool memory, int64_t wanted) {
+  std::lock_guard<std::mutex> lk(c.mu);
+  if (c.busy) return false;
+  if (!c.done && cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    c.done = nullptr;
+    return false;
+  }
+  if (c.last != s && cudaEventQuery(c.done) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  c.busy = true;
+  from = &c;
+  side = c.side;
+  if (!memory) return false;
+  if (c.bytes < wanted) {
+    cudaFree(c.p);   // (waits for the work on it)
+    c.p = nullptr;
+    c.bytes = 0;
+    if (cudaMalloc(&c.p, wanted) == cudaSuccess) {
+      c.bytes = wanted;
+    } else {
+      cudaGetLastError();
+      c.p = nullptr;
     }
   }
+  if (!c.p || cudaStreamWaitEvent(s, c.done, 0) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  p = c.p;
+  bytes = c.bytes;
+  return true;
+}
+
+bool ScratchHold::take_idle(Scratch& c, int64_t wanted, cudaStream_t stream) {
+  s = stream;
+  if (claim(c, true, wanted)) return true;
+  release();
+  return false;
+}
+
+bem_status ScratchHold::take(Scratch& c, bool own_block, int64_t least, int64_t wanted, cudaStream_t stream) {
+  s = stream;
+  if (claim(c, !own_block, wanted)) return BEM_OK;
   own = true;
   for (int64_t n = wanted;; n = std::max(least, n / 4)) {
     if (cudaMallocAsync(&p, n, s) == cudaSuccess) {
@@ -480,12 +495,17 @@ bem_status ScratchHold::take(Scratch& c, bool own_block, int64_t least, int64_t 
   return BEM_ERR_OUT_OF_MEMORY;
 }
 
-ScratchHold::~ScratchHold() {
+void ScratchHold::release() {
   if (own && p) cudaFreeAsync(p, s);
-  if (!from) return;
-  std::lock_guard<std::mutex> lk(from->mu);
-  if (!own && p) cudaEventRecord(from->done, s);
-  from->busy = false;
+  if (from) {
+    std::lock_guard<std::mutex> lk(from->mu);
+    cudaEventRecord(from->done, s);
+    from->last = s;
+    from->busy = false;
+  }
+  from = nullptr;
+  p = nullptr;
+  side = nullptr;
 }
 
 void scratch_trim(Scratch& c) {
@@ -509,12 +529,31 @@ bem_status op_quadrature(bem_operator* op, cudaStream_t s) {
   return quad_launch(op, op->quad_per_sm, op->mesh->n_col * op->mesh->n_col, nullptr, nullptr, 0, h.p, h.bytes, h.side, s);
 }
 
+FreeScratch::FreeScratch(const bem_operator* o, cudaStream_t s) {
+  if (!o->opts.matrix_free || o->held) return;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return;
+  }
+  int64_t least = 0, wanted = 0;
+  quad_scratch(o, &least, &wanted);
+  if (wanted <= o->tmp_bytes || !h.take_idle(o->ctx->scratch, wanted, s)) return;
+  op = o;
+  op->held = &h;
+}
+
 // Matrix-free product y = A x (internal order, [nrhs][n_tet]): the quadrature
-// pass with the entries summed against x instead of stored.
+// pass with the entries summed against x instead of stored. An operator's own
+// scratch (op_layout) is for captured products and calls beside another holder of
+// the context's: level-3 sphere, 8 slabs 149 ms with the context's 1 GiB, 806
+// with its own 87 MB; level-2 sphere, 15 slabs 33 ms and 144 with 64 MiB.
 bem_status op_matvec_free(const bem_operator* op, const double* x, double* y, int nrhs, cudaStream_t s) {
   STBEM_CUDA(cudaMemsetAsync(y, 0, sizeof(double) * op->mesh->n_tet * nrhs, s));
   const int per_sm = op->quad_per_sm > 0 ? op->quad_per_sm : quad_max_per_sm(op);
-  return quad_launch(op, per_sm, op->mesh->n_col * op->mesh->n_col, x, y, nrhs, op->d_tmp, op->tmp_bytes, op->side, s);
+  const int64_t nb = op->mesh->n_col * op->mesh->n_col;
+  if (op->held) return quad_launch(op, per_sm, nb, x, y, nrhs, op->held->p, op->held->bytes, op->held->side, s);
+  return quad_launch(op, per_sm, nb, x, y, nrhs, op->d_tmp, op->tmp_bytes, op->side, s);
 }
 
 // ---------------------------------------------------------------------------

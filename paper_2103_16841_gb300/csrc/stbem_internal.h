@@ -54,20 +54,22 @@ namespace stbem {
 // Quadrature scratch of a context and the second stream of its assemblies. The
 // memory is kept from one assembly to the next (at most the largest that one
 // wanted, 1 GiB) and given back when the context goes or device memory runs
-// short. One assembly holds both at a time; another one that runs beside it
-// (other threads) gets a block of its own, stream-ordered, and no second
-// stream. Only assemblies take it, and they are never captured: a stream that
-// has joined a capture must not meet other work.
+// short. One assembly, or one product or solve of a matrix-free operator, holds
+// both at a time; an assembly that runs beside it (other threads) gets a block
+// of its own, stream-ordered, and no second stream. What is captured under a
+// caller's capture takes neither, and a solve holds them while its graph lives:
+// a stream that has joined a capture must not meet other work.
 struct Scratch {
   std::mutex mu;
   void* p = nullptr;
   int64_t bytes = 0;
   bool busy = false;
   cudaStream_t side = nullptr;
-  cudaEvent_t done = nullptr;   // the last assembly's work on it
+  cudaEvent_t done = nullptr;   // the last holder's work on them,
+  cudaStream_t last = nullptr;  // on this stream
 };
 struct ScratchHold {
-  Scratch* from = nullptr;      // null: another assembly has the context's
+  Scratch* from = nullptr;      // null: another holder has the context's
   void* p = nullptr;
   int64_t bytes = 0;
   bool own = false;             // p is a block of its own
@@ -77,7 +79,12 @@ struct ScratchHold {
   ScratchHold& operator=(const ScratchHold&) = delete;
   // least <= bytes <= wanted; own_block: never the context's memory
   bem_status take(Scratch& c, bool own_block, int64_t least, int64_t wanted, cudaStream_t stream);
-  ~ScratchHold();
+  bool take_idle(Scratch& c, int64_t wanted, cudaStream_t stream);   // the context's, unless it is held
+  void release();
+  ~ScratchHold() { release(); }
+
+ private:
+  bool claim(Scratch& c, bool memory, int64_t wanted);
 };
 void scratch_trim(Scratch& c);  // frees it unless an assembly holds it
 }  // namespace stbem
@@ -140,9 +147,12 @@ struct bem_operator {
   double tune_ms[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // sample time per candidate: index = CTAs per SM - 1
   unsigned long long* d_counter = nullptr;  // work counter of the persistent kernels
   // quadrature scratch
-  void* d_tmp = nullptr;         // matrix-free operators only: their products' scratch
-  cudaStream_t side = nullptr;   // and second stream (captured with them, so no one else's)
+  // matrix-free operators only: scratch and second stream (captured with the products, so no
+  // one else's) where the context's are not to be had, and the context's while a call holds them
+  void* d_tmp = nullptr;
+  cudaStream_t side = nullptr;
   int64_t tmp_bytes = 0;
+  mutable const stbem::ScratchHold* held = nullptr;
   int64_t reserve_bytes = 0;     // bytes an admission reserves for the scratch
   int64_t scratch_cap = -1;      // >= 0: bytes the scratch may take beyond that (a server's slot), not the context's
   // made on first use by the products (an operator is used by one host thread at a time)
@@ -201,6 +211,14 @@ std::string batch_shape_class(const bem_context* ctx, int prec, int nq, int n_th
 // raise a kernel's dynamic shared-memory limit to at least `bytes` (never lowers it)
 bem_status ensure_smem_attr(const void* kern, size_t bytes);
 // matrix-free product (internal order): the quadrature pass summed against x
+// the context's scratch for the products of a matrix-free operator during a call, if it is
+// idle and the stream is not under capture
+struct FreeScratch {
+  const bem_operator* op = nullptr;
+  ScratchHold h;
+  FreeScratch(const bem_operator* o, cudaStream_t s);
+  ~FreeScratch() { if (op) op->held = nullptr; }
+};
 bem_status op_matvec_free(const bem_operator* op, const double* x, double* y, int nrhs, cudaStream_t s);
 // Layout of the vectors of a batched GMRES: K vectors of length N ([K][N]);
 // entries [seg_off[s], seg_off[s+1]) of a vector belong to segment s (one

@@ -125,6 +125,7 @@ bem_status gmres_solve_layout(const SegLayout& L, const MatvecFn& mv_hi, const M
 
 bem_status gmres_solve(bem_operator* op, const double* d_b, double* d_x, int nrhs, const bem_solve_opts* o,
                        bem_solve_info* info, cudaStream_t s) {
+  FreeScratch scratch(op, s);
   SegLayout L;
   L.N = op->mesh->n_tet;
   L.K = nrhs;
@@ -142,6 +143,7 @@ bem_status gmres_solve(bem_operator* op, const double* d_b, double* d_x, int nrh
 
 bem_status gmres_solve_two(const bem_operator* hi_op, bem_operator* lo_op, const double* d_b, double* d_x,
                            int nrhs, const bem_solve_opts* o, bem_solve_info* info, cudaStream_t s) {
+  FreeScratch hi_scratch(hi_op, s), lo_scratch(lo_op, s);
   SegLayout L;
   L.N = lo_op->mesh->n_tet;
   L.K = nrhs;
