@@ -234,6 +234,7 @@ struct TcArgs {
   const TcBlk* blk;
   const uint4* vals;       // chunk slots of the product's type
   const int32_t* rs;       // row starts (16 bytes of tail room)
+  const double* x;         // [nr][n_tet] (internal order)
   double* y;               // [parts][nr][n_tet] (internal order)
   int64_t n_tet;
   int nr, N;               // right-hand sides of the pass, MMA N (multiple of 16)
@@ -245,11 +246,51 @@ struct TcArgs {
   int* err;                // set to 1 when a wait ran out of budget
 };
 
+template <bool TF32>
+__device__ __forceinline__ float tc_rounded(float v) {
+  if (!TF32) return __bfloat162float(__float2bfloat16_rn(v));
+  uint32_t t;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(t) : "f"(v));
+  return __uint_as_float(t);
+}
+
+// Row r's sum for right-hand side n in FP32 from the values that it has. The
+// MMA multiplies a tile's zeros too, so one Inf or NaN in x makes NaN in all
+// rows of a group with a block there; a sum that is not finite is formed again
+// this way, and rows without a value at that panel keep theirs.
+template <bool TF32>
+__device__ float tc_row_sum(const TcBlk* __restrict__ blk, int nb, const uint4* __restrict__ vals,
+                                         const int32_t* __restrict__ rs, const double* __restrict__ x, int nt, int r) {
+  constexpr int E = TF32 ? 4 : 8;
+  float acc = 0.f;
+  for (int k = 0; k < nb; ++k) {
+    const TcBlk& b = blk[k];
+    const int base = rs[b.ro + r] / E * E, S = tc_slots(b.W, E);
+    for (int j = 0; j < S; ++j) {
+      const uint4 q = vals[b.vc[TF32 ? 1 : 0] + (int64_t)j * nt + r];
+      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+      for (int e = 0; e < E; ++e) {
+        const float v = TF32 ? __uint_as_float(w[e]) : __uint_as_float(e & 1 ? w[e >> 1] & 0xffff0000u : w[e >> 1] << 16);
+        if (v != 0.f) acc += v * tc_rounded<TF32>((float)x[base + j * E + e]);
+      }
+    }
+  }
+  return acc;
+}
+
+template <bool TF32>
+__device__ __noinline__ void tc_again(const TcArgs& a, int b0, int nb, int t0, int nt, int r, int c, double* __restrict__ y) {
+  for (int n = c; n < min(c + 16, a.nr); ++n) {
+    double& o = y[(int64_t)n * a.n_tet + t0 + r];
+    if (!isfinite(o)) o = tc_row_sum<TF32>(a.blk + b0, nb, a.vals, a.rs, a.x + (int64_t)n * a.n_tet, nt, r);
+  }
+}
+
 // Per stage in shared memory: the A tile, the B tile (X rows), the block's
 // value slots, its row starts (bulk copy from the 16-byte granule holding
 // the first one) and its record (written by the loader).
 template <bool TF32, int MT>
-__global__ void __launch_bounds__(kThreads, 1) k_spmm_tc(const TcArgs a, const __grid_constant__ CUtensorMap tmx) {
+__global__ void __launch_bounds__(kThreads, 1) k_spmm_tc(const __grid_constant__ TcArgs a, const __grid_constant__ CUtensorMap tmx) {
   using namespace tc;
   constexpr int E = TF32 ? 4 : 8;         // elements per 16-byte chunk
   constexpr int ROWS = MT * 128;
@@ -364,14 +405,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_spmm_tc(const TcArgs a, const _
         float v[16];
         tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(mt * N + c), v);
         if (r < nt) {
+          bool again = false;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const int n = c + j;
             if (n < a.nr) {
               const double o = nb == 0 ? 0.0 : bad ? __longlong_as_double(0x7ff8000000000000LL) : (double)v[j];
               y[(int64_t)n * a.n_tet + t0 + r] = o;
+              again |= !isfinite(v[j]);
             }
           }
+          if (again && nb > 0 && !bad) tc_again<TF32>(a, b0, nb, t0, nt, r, c, y);
         }
       }
     }
@@ -447,7 +491,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_spmm_tc(const TcArgs a, const _
 // read by the MMA straight from tensor memory; shared memory then holds only
 // the B tiles, value slots and row starts, so more stages fit.
 template <bool TF32, int MT>
-__global__ void __launch_bounds__(kThreads, 1) k_spmm_tm(const TcArgs a, const __grid_constant__ CUtensorMap tmx) {
+__global__ void __launch_bounds__(kThreads, 1) k_spmm_tm(const __grid_constant__ TcArgs a, const __grid_constant__ CUtensorMap tmx) {
   using namespace tc;
   constexpr int E = TF32 ? 4 : 8;         // elements per 16-byte chunk
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -568,14 +612,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_spmm_tm(const TcArgs a, const _
         float v[16];
         tmem_ld16(tmem + lanes + (uint32_t)(mt * N + c), v);
         if (r < nt) {
+          bool again = false;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const int n = c + j;
             if (n < a.nr) {
               const double o = nb == 0 ? 0.0 : bad ? __longlong_as_double(0x7ff8000000000000LL) : (double)v[j];
               y[(int64_t)n * a.n_tet + t0 + r] = o;
+              again |= !isfinite(v[j]);
             }
           }
+          if (again && nb > 0 && !bad) tc_again<TF32>(a, b0, nb, t0, nt, r, c, y);
         }
       }
     }
@@ -961,6 +1008,7 @@ bem_status op_spmm_tc(const bem_operator* op, const double* x, double* y, int nr
   a.vals = static_cast<const uint4*>(op->d_tcv[bf16 ? 0 : 1]);
   a.rs = op->d_tc_rs;
   a.parts = parts;
+  a.x = x;
   a.y = parts > 1 ? reinterpret_cast<double*>(op->d_ws + xc_len) : y;
   a.n_tet = n;
   a.nr = nrhs;
