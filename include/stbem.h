@@ -83,7 +83,10 @@ enum { BEM_DATA_SIN2_UNIFORM = 0, BEM_DATA_PULSE = 1 };
 /* ------------------------------------------------------------------ */
 
 /* Binds CUDA device `device` (usually 0) and creates the streams the library
- * uses. Fails with BEM_ERR_CUDA when no device is usable. */
+ * uses. Fails with BEM_ERR_CUDA when no device is usable. A context keeps the
+ * quadrature scratch of its largest assembly (at most 1 GiB of device memory)
+ * until it is destroyed, or until an allocation of the library finds too
+ * little memory. */
 bem_status bem_context_create(int device, bem_context** out);
 void bem_context_destroy(bem_context* ctx);
 /* Thread-local text of the last failure in this thread ("" if none). */

@@ -40,7 +40,7 @@ namespace {
 
 template <typename T>
 bem_status balloc(T** p, int64_t n) {
-  if (cudaMalloc((void**)p, sizeof(T) * std::max<int64_t>(n, 1)) != cudaSuccess) {
+  if (device_alloc((void**)p, sizeof(T) * std::max<int64_t>(n, 1)) != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
     set_error("out of device memory (batch)");

@@ -30,22 +30,12 @@ namespace {
 template <typename T>
 bem_status dalloc(T** p, size_t n) {
   if (n == 0) n = 1;
-  cudaError_t e = cudaMalloc((void**)p, n * sizeof(T));
+  cudaError_t e = device_alloc((void**)p, n * sizeof(T));
   if (e != cudaSuccess) {
     set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? BEM_ERR_OUT_OF_MEMORY : BEM_ERR_CUDA;
   }
   return BEM_OK;
-}
-
-// the same, giving the context's quadrature scratch back when memory runs short
-template <typename T>
-bem_status dalloc_room(bem_context* ctx, T** p, size_t n) {
-  const bem_status st = dalloc(p, n);
-  if (st != BEM_ERR_OUT_OF_MEMORY) return st;
-  cudaGetLastError();
-  scratch_trim(ctx->scratch);
-  return dalloc(p, n);
 }
 
 template <typename T>
@@ -96,12 +86,14 @@ bem_status bem_context_create(int device, bem_context** out) {
     TRY(upload_gauss_tables());
     g_tables_ready = true;
   }
+  contexts_add(ctx.get());
   *out = ctx.release();
   return BEM_OK;
 }
 
 void bem_context_destroy(bem_context* ctx) {
   if (!ctx) return;
+  contexts_remove(ctx);
   if (ctx->stream) cudaStreamDestroy(ctx->stream);
   if (ctx->scratch.side) cudaStreamDestroy(ctx->scratch.side);
   scratch_trim(ctx->scratch);
@@ -400,10 +392,10 @@ bem_status stbem::op_layout(bem_operator* op, const int32_t* bw, const int64_t* 
     if (op->admit) TRY(op->admit(op, bw));
     if (!op->opts.matrix_free) {
       // mixed-precision values carry FP32 accuracy: FP32 storage only
-      if (op->opts.precision == BEM_PREC_FP64) TRY(dalloc_room(op->ctx, &op->d_val, (size_t)vo));
+      if (op->opts.precision == BEM_PREC_FP64) TRY(dalloc(&op->d_val, (size_t)vo));
       // (8 floats of tail room: the tensor-core product copies whole 16-byte granules)
       if (op->opts.store_fp32 || op->opts.precision == BEM_PREC_MIXED)
-        TRY(dalloc_room(op->ctx, &op->d_val32, (size_t)vo + 8));
+        TRY(dalloc(&op->d_val32, (size_t)vo + 8));
       TRY(dalloc(&op->d_rs, (size_t)ro + 4));   // (tail room as for the values)
     }
     if (own_scratch && op->opts.matrix_free) {
@@ -806,7 +798,7 @@ static bem_status ensure_pv(const bem_operator* op, int64_t nn, cudaStream_t s) 
   if (op->d_pv) STBEM_CUDA(cudaFreeAsync(op->d_pv, s));
   op->d_pv = nullptr;
   op->pv_len = 0;
-  cudaError_t e = cudaMallocAsync((void**)&op->d_pv, sizeof(double) * 2 * nn, s);
+  cudaError_t e = device_alloc_async((void**)&op->d_pv, sizeof(double) * 2 * nn, s);
   if (e != cudaSuccess) {
     op->d_pv = nullptr;
     set_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));

@@ -159,9 +159,9 @@ bem_status mesh_device_geometry(bem_mesh* m, const double* d_sv_xyz, const int32
   k_surf_geom<<<(unsigned)((m->n_surf + th - 1) / th), th, 0, s>>>(m->n_surf, m->d_col, d_surf_p, d_surf_col,
                                                                    m->d_surf);
   k_tet_ball<<<(unsigned)((m->n_tet + th - 1) / th), th, 0, s>>>(m->n_tet, d_tet_vx, m->d_tet);
-  STBEM_CUDA(cudaMalloc(&m->d_colf, sizeof(ColF) * m->n_col));
-  STBEM_CUDA(cudaMalloc(&m->d_facef, sizeof(FaceF) * m->n_surf));
-  STBEM_CUDA(cudaMalloc(&m->d_panf, sizeof(PanelF) * m->n_tet));
+  STBEM_CUDA(device_alloc(&m->d_colf, sizeof(ColF) * m->n_col));
+  STBEM_CUDA(device_alloc(&m->d_facef, sizeof(FaceF) * m->n_surf));
+  STBEM_CUDA(device_alloc(&m->d_panf, sizeof(PanelF) * m->n_tet));
   k_face_f32<<<(unsigned)((m->n_surf + th - 1) / th), th, 0, s>>>(m->n_surf, m->d_surf,
                                                                   static_cast<FaceF*>(m->d_facef));
   k_col_f32<<<(unsigned)((m->n_col + th - 1) / th), th, 0, s>>>(m->n_col, m->d_col, static_cast<ColF*>(m->d_colf));
@@ -483,7 +483,7 @@ bem_status ScratchHold::take(Scratch& c, bool own_block, int64_t least, int64_t 
   if (claim(c, !own_block, wanted)) return BEM_OK;
   own = true;
   for (int64_t n = wanted;; n = std::max(least, n / 4)) {
-    if (cudaMallocAsync(&p, n, s) == cudaSuccess) {
+    if (device_alloc_async(&p, n, s) == cudaSuccess) {
       bytes = n;
       return BEM_OK;
     }
@@ -514,6 +514,51 @@ void scratch_trim(Scratch& c) {
   cudaFree(c.p);
   c.p = nullptr;
   c.bytes = 0;
+}
+
+namespace {
+std::mutex g_contexts_mu;
+std::vector<bem_context*> g_contexts;
+
+// gives back the idle scratch of the current device's contexts; false: there was none
+bool trim_idle() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  bool some = false;
+  std::lock_guard<std::mutex> lk(g_contexts_mu);
+  for (bem_context* c : g_contexts) {
+    if (c->device != dev) continue;
+    {
+      std::lock_guard<std::mutex> l2(c->scratch.mu);
+      some = some || (c->scratch.p && !c->scratch.busy);
+    }
+    scratch_trim(c->scratch);
+  }
+  return some;
+}
+
+template <typename F>
+cudaError_t with_room(F alloc) {
+  const cudaError_t e = alloc();
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  return trim_idle() ? alloc() : e;
+}
+}  // namespace
+
+void contexts_add(bem_context* c) {
+  std::lock_guard<std::mutex> lk(g_contexts_mu);
+  g_contexts.push_back(c);
+}
+void contexts_remove(bem_context* c) {
+  std::lock_guard<std::mutex> lk(g_contexts_mu);
+  g_contexts.erase(std::remove(g_contexts.begin(), g_contexts.end(), c), g_contexts.end());
+}
+cudaError_t device_alloc(void** p, size_t bytes) {
+  return with_room([&] { return cudaMalloc(p, bytes); });
+}
+cudaError_t device_alloc_async(void** p, size_t bytes, cudaStream_t s) {
+  return with_room([&] { return cudaMallocAsync(p, bytes, s); });
 }
 
 bem_status op_quadrature(bem_operator* op, cudaStream_t s) {
@@ -691,7 +736,7 @@ __global__ void k_value_scan(const V* v, int64_t n, unsigned long long* bad, uns
 
 bem_status op_value_scan(const bem_operator* op, int64_t* nbad, double* maxabs, cudaStream_t s) {
   unsigned long long* d;
-  STBEM_CUDA(cudaMalloc(&d, 2 * sizeof(unsigned long long)));
+  STBEM_CUDA(device_alloc((void**)&d, 2 * sizeof(unsigned long long)));
   STBEM_CUDA(cudaMemsetAsync(d, 0, 2 * sizeof(unsigned long long), s));
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -1018,7 +1063,7 @@ bem_status op_rhs(const bem_operator* op, int kind, int nrhs, const double* d_pa
   const bem_mesh* m = op->mesh;
   const int64_t n = m->n_surf * nrhs, nb = m->n_tet * nrhs;
   double2* S = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&S, sizeof(double2) * std::max<int64_t>(n, 1), s);
+  cudaError_t e = device_alloc_async((void**)&S, sizeof(double2) * std::max<int64_t>(n, 1), s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     set_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));

@@ -50,6 +50,7 @@ struct SurfDev {
 
 }  // namespace stbem
 
+struct bem_context;
 namespace stbem {
 // Quadrature scratch of a context and the second stream of its assemblies. The
 // memory is kept from one assembly to the next (at most the largest that one
@@ -86,7 +87,14 @@ struct ScratchHold {
  private:
   bool claim(Scratch& c, bool memory, int64_t wanted);
 };
-void scratch_trim(Scratch& c);  // frees it unless an assembly holds it
+void scratch_trim(Scratch& c);  // frees it unless it is held
+
+// Device memory for everything else: where it is short, the idle scratch of the
+// device's contexts is given back and the call repeated.
+cudaError_t device_alloc(void** p, size_t bytes);
+cudaError_t device_alloc_async(void** p, size_t bytes, cudaStream_t s);
+void contexts_add(bem_context* c);
+void contexts_remove(bem_context* c);
 }  // namespace stbem
 
 struct bem_context {

@@ -219,7 +219,7 @@ bem_status ensure_ws(const bem_operator* op, int64_t floats) {
   if (op->d_ws) cudaFree(op->d_ws);
   op->d_ws = nullptr;
   op->ws_len = 0;
-  if (cudaMalloc(&op->d_ws, sizeof(float) * floats) != cudaSuccess) {
+  if (device_alloc((void**)&op->d_ws, sizeof(float) * floats) != cudaSuccess) {
     cudaGetLastError();
     set_error("out of device memory (matvec workspace)");
     return BEM_ERR_OUT_OF_MEMORY;
@@ -382,9 +382,9 @@ bem_status BatchMatvec::init(const std::vector<bem_operator*>& o, cudaStream_t s
     N += op->mesh->n_tet;
   }
   n_cta = (int64_t)cseg.size();
-  if (cudaMalloc(&d_segs, sizeof(MvSeg) * std::max(S, 1)) != cudaSuccess ||
-      cudaMalloc(&d_cseg, sizeof(int32_t) * std::max<int64_t>(n_cta, 1)) != cudaSuccess ||
-      cudaMalloc(&d_ccol, sizeof(int32_t) * std::max<int64_t>(n_cta, 1)) != cudaSuccess) {
+  if (device_alloc((void**)&d_segs, sizeof(MvSeg) * std::max(S, 1)) != cudaSuccess ||
+      device_alloc((void**)&d_cseg, sizeof(int32_t) * std::max<int64_t>(n_cta, 1)) != cudaSuccess ||
+      device_alloc((void**)&d_ccol, sizeof(int32_t) * std::max<int64_t>(n_cta, 1)) != cudaSuccess) {
     cudaGetLastError();
     set_error("out of device memory (batch matvec tables)");
     return BEM_ERR_OUT_OF_MEMORY;
@@ -430,7 +430,7 @@ bem_status BatchMatvec::apply(const double* x, double* y, int K, int arith, cuda
       if (d_xf) cudaFree(d_xf);
       d_xf = nullptr;
       xf_len = 0;
-      if (cudaMalloc(&d_xf, sizeof(float) * packed_len(N, K)) != cudaSuccess) {
+      if (device_alloc((void**)&d_xf, sizeof(float) * packed_len(N, K)) != cudaSuccess) {
         cudaGetLastError();
         set_error("out of device memory (batch matvec workspace)");
         return BEM_ERR_OUT_OF_MEMORY;

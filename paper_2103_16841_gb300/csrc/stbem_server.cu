@@ -61,7 +61,7 @@ struct DBuf {
   ~DBuf() { if (p) cudaFreeAsync(p, st); }
   bem_status alloc(int64_t n, cudaStream_t s) {
     st = s;
-    if (cudaMallocAsync((void**)&p, sizeof(T) * std::max<int64_t>(n, 1), s) != cudaSuccess) {
+    if (device_alloc_async((void**)&p, sizeof(T) * std::max<int64_t>(n, 1), s) != cudaSuccess) {
       cudaGetLastError();
       p = nullptr;
       set_error("out of device memory");

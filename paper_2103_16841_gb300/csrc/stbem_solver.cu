@@ -39,7 +39,7 @@ struct Dev {
   ~Dev() { if (p) cudaFreeAsync(p, st); }
   cudaError_t alloc(int64_t n, cudaStream_t s) {
     st = s;
-    return cudaMallocAsync((void**)&p, sizeof(double) * n, s);
+    return device_alloc_async((void**)&p, sizeof(double) * n, s);
   }
 };
 

@@ -824,7 +824,7 @@ bem_status ensure_tc_meta(const bem_operator* op, cudaStream_t s) {
   size_t bytes[kTcArrays];
   tc_array_bytes(ng, nb, L.nrows, bytes);
   for (int k = 0; k < kTcArrays; ++k)
-    if (cudaMalloc(&A.p[k], bytes[k]) != cudaSuccess) {
+    if (device_alloc((void**)&A.p[k], bytes[k]) != cudaSuccess) {
       cudaGetLastError();
       A.p[k] = nullptr;
       set_error("out of device memory (tensor-core product tables)");
@@ -846,7 +846,7 @@ bem_status ensure_tc_meta(const bem_operator* op, cudaStream_t s) {
   STBEM_CUDA(cudaMemcpyAsync(hspan, A.p[10], sizeof(hspan), cudaMemcpyDeviceToHost, s));
   STBEM_CUDA(cudaStreamSynchronize(s));
   if (!op->d_tc_err) {
-    if (cudaMalloc(&op->d_tc_err, sizeof(int)) != cudaSuccess) {
+    if (device_alloc((void**)&op->d_tc_err, sizeof(int)) != cudaSuccess) {
       cudaGetLastError();
       op->d_tc_err = nullptr;
       set_error("out of device memory (tensor-core product flag)");
@@ -877,7 +877,7 @@ bem_status ensure_tc_vals(const bem_operator* op, bool tf32, cudaStream_t s) {
   const int t = tf32 ? 1 : 0;
   if (op->d_tcv[t] && !op->tcv_stale[t]) return BEM_OK;
   if (!op->d_tcv[t] &&
-      cudaMalloc(&op->d_tcv[t], sizeof(uint4) * (size_t)std::max<int64_t>(op->tcv_len[t], 1)) != cudaSuccess) {
+      device_alloc((void**)&op->d_tcv[t], sizeof(uint4) * (size_t)std::max<int64_t>(op->tcv_len[t], 1)) != cudaSuccess) {
     cudaGetLastError();
     op->d_tcv[t] = nullptr;
     set_error("out of device memory (tensor-core product values)");
@@ -1130,7 +1130,7 @@ extern "C" bem_status bem_selftest_bounded_wait(bem_context* ctx, double* waited
   STBEM_CUDA(cudaSetDevice(ctx->device));
   int* d_flag = nullptr;
   long long* d_cyc = nullptr;
-  if (cudaMalloc(&d_flag, sizeof(int)) != cudaSuccess || cudaMalloc(&d_cyc, sizeof(long long)) != cudaSuccess) {
+  if (device_alloc((void**)&d_flag, sizeof(int)) != cudaSuccess || device_alloc((void**)&d_cyc, sizeof(long long)) != cudaSuccess) {
     cudaGetLastError();
     cudaFree(d_flag);
     set_error("out of device memory");

@@ -1,0 +1,50 @@
+"""Device memory short while a context keeps its quadrature scratch."""
+import gc
+
+import numpy as np
+import pytest
+
+from paper_2103_16841_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("call", ["solve", "tf32", "matrix_free"])
+def test_idle_scratch_is_given_back(call):
+    """An assembly of 14,400 panels leaves 1 GiB of scratch with its context. With
+    less than that free elsewhere, a solve whose basis takes 0.7 GB (32 right-hand
+    sides, 200 steps), a TF32 product with its tables and slots (0.2 GB) and another
+    operator all find room."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2103_16841_gb300 as stb
+    gc.collect()
+    ctx = stb.Context(0)
+    mesh = stb.Mesh.from_spacetime(ctx, inputs.sphere_mesh(2, 15, 4.0, 0.2, seed=1))
+    op = stb.Operator(ctx, mesh, "mixed")
+    b = np.random.default_rng(0).normal(size=(mesh.n_tet, 32))
+    x = torch.tensor(np.ascontiguousarray(b.T), device="cuda")
+
+    def solve(restart):
+        return op.solve(b, tol=1e-14, restart=restart, maxit=2, inner="fp64", allow_unconverged=True)[0]
+
+    small = solve(2)                       # (kernels and small buffers are there)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    left = {"solve": 500, "tf32": 64, "matrix_free": 32}[call] << 20
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - left, dtype=torch.uint8, device="cuda")
+    try:
+        if call == "solve":
+            assert np.isfinite(solve(200)).all()
+        elif call == "tf32":
+            y = torch.empty_like(x[:1])
+            op.matvec(x[:1].contiguous(), y, dtype="tf32")
+            torch.cuda.synchronize()
+            assert bool(torch.isfinite(y).all())
+        else:
+            stb.Operator(ctx, mesh, "mixed", matrix_free=True).close()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.isfinite(small).all()
