@@ -539,10 +539,13 @@ bool trim_idle() {
 
 template <typename F>
 cudaError_t with_room(F alloc) {
-  const cudaError_t e = alloc();
-  if (e != cudaErrorMemoryAllocation) return e;
-  cudaGetLastError();
-  return trim_idle() ? alloc() : e;
+  cudaError_t e = alloc();
+  if (e == cudaSuccess) return e;
+  cudaGetLastError();   // (a later launch's check must not see it)
+  if (e != cudaErrorMemoryAllocation || !trim_idle()) return e;
+  e = alloc();
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 }  // namespace
 

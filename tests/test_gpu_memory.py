@@ -48,3 +48,25 @@ def test_idle_scratch_is_given_back(call):
         del hold
         torch.cuda.empty_cache()
     assert np.isfinite(small).all()
+
+
+def test_calls_after_one_that_found_no_memory():
+    """A refused call leaves nothing behind that a later launch would report."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2103_16841_gb300 as stb
+    ctx = stb.Context(0)
+    mesh = stb.Mesh.from_spacetime(ctx, inputs.sphere_mesh(2, 15, 4.0, 0.2, seed=1))
+    op = stb.Operator(ctx, stb.Mesh.from_spacetime(ctx, inputs.sphere_mesh(0, 1, 0.5, 0.2, seed=2)), "mixed")
+    prm = inputs.pulse_params(3, seed=3)
+    want = op.rhs(stb.DATA_PULSE, prm)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (64 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(stb._lib.BemError):
+            stb.Operator(ctx, mesh, "mixed")
+        assert np.array_equal(op.rhs(stb.DATA_PULSE, prm), want)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
