@@ -1062,22 +1062,31 @@ __global__ void k_rhs_combine(int64_t n_tet, int64_t n_surf, int nrhs, const Tet
   b[tid] = S[r * n_surf + D.lo] - S[r * n_surf + D.hi];
 }
 
+// The face integrals of as many right-hand sides as 64 MiB hold at a time: the
+// workspace stays small beside b, and four million (face, right-hand side) pairs
+// fill the device many times over.
 bem_status op_rhs(const bem_operator* op, int kind, int nrhs, const double* d_params, double* d_b, cudaStream_t s) {
   const bem_mesh* m = op->mesh;
-  const int64_t n = m->n_surf * nrhs, nb = m->n_tet * nrhs;
+  const int64_t room = ((int64_t)64 << 20) / (sizeof(double2) * std::max<int64_t>(m->n_surf, 1));
+  const int most = (int)std::min<int64_t>(nrhs, std::max<int64_t>(room, 1));
   double2* S = nullptr;
-  cudaError_t e = device_alloc_async((void**)&S, sizeof(double2) * std::max<int64_t>(n, 1), s);
+  cudaError_t e = device_alloc_async((void**)&S, sizeof(double2) * std::max<int64_t>(m->n_surf * most, 1), s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     set_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? BEM_ERR_OUT_OF_MEMORY : BEM_ERR_CUDA;
   }
-  const unsigned grid = (unsigned)std::min<int64_t>((n + 3) / 4, 152 * 64);
-  if (kind == BEM_DATA_PULSE)
-    k_rhs_faces<BEM_DATA_PULSE><<<grid, kRhsThreads, 0, s>>>(m->n_surf, m->d_surf, m->d_col, nrhs, d_params, S);
-  else
-    k_rhs_faces<BEM_DATA_SIN2_UNIFORM><<<grid, kRhsThreads, 0, s>>>(m->n_surf, m->d_surf, m->d_col, nrhs, d_params, S);
-  k_rhs_panels<<<(unsigned)((nb + 127) / 128), 128, 0, s>>>(m->n_tet, m->n_surf, nrhs, m->d_tet, S, d_b);
+  for (int r0 = 0; r0 < nrhs; r0 += most) {
+    const int k = std::min(most, nrhs - r0);
+    const int64_t nb = m->n_tet * k;
+    const unsigned grid = (unsigned)std::min<int64_t>((m->n_surf * k + 3) / 4, 152 * 64);
+    const double* prm = d_params ? d_params + 5 * (int64_t)r0 : nullptr;
+    if (kind == BEM_DATA_PULSE)
+      k_rhs_faces<BEM_DATA_PULSE><<<grid, kRhsThreads, 0, s>>>(m->n_surf, m->d_surf, m->d_col, k, prm, S);
+    else
+      k_rhs_faces<BEM_DATA_SIN2_UNIFORM><<<grid, kRhsThreads, 0, s>>>(m->n_surf, m->d_surf, m->d_col, k, prm, S);
+    k_rhs_panels<<<(unsigned)((nb + 127) / 128), 128, 0, s>>>(m->n_tet, m->n_surf, k, m->d_tet, S, d_b + r0 * m->n_tet);
+  }
   e = cudaGetLastError();
   cudaFreeAsync(S, s);
   STBEM_CUDA(e);

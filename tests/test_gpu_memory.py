@@ -50,6 +50,28 @@ def test_idle_scratch_is_given_back(call):
     assert np.isfinite(small).all()
 
 
+def test_right_hand_sides_in_a_small_workspace():
+    """220,000 right-hand sides of 60 panels with 400 MB free: 0.22 GB for them in
+    both panel orders and their parameters, and no workspace of 0.28 GB beside
+    that. The same bits as in pieces."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2103_16841_gb300 as stb
+    ctx = stb.Context(0)
+    op = stb.Operator(ctx, stb.Mesh.from_spacetime(ctx, inputs.sphere_mesh(0, 1, 0.5, 0.2, seed=2)), "mixed")
+    prm = inputs.pulse_params(220000, seed=3, width=4.0)
+    pieces = [op.rhs(stb.DATA_PULSE, prm[i:i + 40000]) for i in range(0, len(prm), 40000)]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (400 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        b = op.rhs(stb.DATA_PULSE, prm)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.array_equal(b, np.concatenate(pieces, axis=1))
+
+
 def test_calls_after_one_that_found_no_memory():
     """A refused call leaves nothing behind that a later launch would report."""
     if not torch.cuda.is_available():
