@@ -9,7 +9,8 @@
 // class times every candidate on a sample of the block queue (the first
 // blocks of the dense (I, J) order; their values are rewritten by the full
 // pass that follows) and keeps the fastest. A shape class is the device
-// (name, SM count), the precision, m_Q^2, the rule order, the largest column
+// (name, SM count), the stage that is tuned ("apex": choices made for another
+// kernel, by an older build, are not taken), the precision, m_Q^2, the rule order, the largest column
 // sizes and the number of columns to within a factor of two. Choices are
 // kept for the process and, with a cache path, in a text file, one line per
 // class: "stbem-tune-v2 <class> <code>", code = CTAs per SM - 1 (a batch's
@@ -47,7 +48,7 @@ std::string shape_class(const bem_operator* op) {
   const bem_mesh* m = op->mesh;
   const int cols_log2 = (int)std::floor(std::log2((double)std::max<int64_t>(m->n_col, 1)));
   std::ostringstream k;
-  k << name << "|sm" << (int)op->ctx->sm_count << "|p" << op->opts.precision << "|q" << op->nq << "|t"
+  k << name << "|sm" << (int)op->ctx->sm_count << "|apex|p" << op->opts.precision << "|q" << op->nq << "|t"
     << op->n_theta << "|r" << m->max_col_tets << "|f" << m->max_col_surf << "|c" << cols_log2;
   return k.str();
 }
@@ -62,7 +63,7 @@ std::string batch_shape_class(const bem_context* ctx, int prec, int nq, int n_th
   for (char& c : name)
     if (c == ' ' || c == '|') c = '_';
   std::ostringstream k;
-  k << name << "|sm" << (int)ctx->sm_count << "|batch|p" << prec << "|q" << nq << "|t" << n_theta << "|r" << max_tet
+  k << name << "|sm" << (int)ctx->sm_count << "|apex|batch|p" << prec << "|q" << nq << "|t" << n_theta << "|r" << max_tet
     << "|f" << max_surf << "|o" << (int)std::floor(std::log2((double)std::max<int64_t>(n_ops, 1))) << "|b"
     << (int)std::floor(std::log2((double)std::max<int64_t>(n_blocks, 1)));
   return k.str();
