@@ -436,6 +436,13 @@ bem_status quad_launch(const bem_operator* op, int per_sm, int64_t end, const do
 // takes the context's second stream and, with `memory`, its scratch (true if there is that
 // much), unless they are held, or in use by unfinished work of another stream
 bool ScratchHold::claim(Scratch& c, bool memory, int64_t wanted) {
+  // queries and allocations here concern no stream under capture, so another thread's
+  // capture (global mode) is none of their business
+  struct Relaxed {
+    cudaStreamCaptureMode m = cudaStreamCaptureModeRelaxed;
+    Relaxed() { cudaThreadExchangeStreamCaptureMode(&m); }
+    ~Relaxed() { cudaThreadExchangeStreamCaptureMode(&m); }
+  } relaxed;
   std::lock_guard<std::mutex> lk(c.mu);
   if (c.busy) return false;
   if (!c.done && cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming) != cudaSuccess) {

@@ -77,3 +77,54 @@ def test_assemblies_of_several_threads(ctx):
     for t in ts:
         t.join()
     assert not bad, bad
+
+
+def test_matrix_free_product_beside_a_capture():
+    """Another thread's product, for which the context's scratch (given back
+    meanwhile) is allocated again, while this one captures (global mode): the
+    capture stays valid and the product is the assembled matrix's, within
+    (2 n + 4) 2^-53 of |A| |x|."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2103_16841_gb300 as stb
+    ctx = stb.Context(0)
+    mesh = stb.Mesh.from_spacetime(ctx, inputs.sphere_mesh(1, 9, 4.0, 0.2, seed=7))
+    large = stb.Mesh.from_spacetime(ctx, inputs.sphere_mesh(3, 8, 4.0, 0.2, seed=1))
+    free = stb.Operator(ctx, mesh, "mixed", matrix_free=True)
+    x = torch.randn(mesh.n_tet, dtype=torch.float64, device="cuda")
+    out, y = torch.empty_like(x), torch.zeros_like(x)
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+    free.matvec(x, y, stream=other)        # (its kernels and vectors are there)
+    torch.mul(x, 2.0, out=out)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (64 << 20), dtype=torch.uint8, device="cuda")
+    with pytest.raises(stb._lib.BemError):
+        stb.Operator(ctx, large, "mixed")
+    del hold
+    torch.cuda.empty_cache()
+    y.zero_()
+    torch.cuda.synchronize()
+    bad = []
+
+    def work():
+        try:
+            free.matvec(x, y, stream=other)
+        except Exception as e:
+            bad.append(repr(e))
+
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(mine):
+        g.capture_begin()
+        torch.mul(x, 3.0, out=out)
+        t = threading.Thread(target=work)
+        t.start()
+        t.join()
+        g.capture_end()
+    g.replay()
+    torch.cuda.synchronize()
+    assert not bad, bad
+    assert torch.equal(out, 3.0 * x)
+    A, xs = stb.Operator(ctx, mesh, "mixed").export_dense(), x.cpu().numpy()
+    bound = (2 * (A != 0).sum(axis=1) + 4) * 2.0 ** -53 * (np.abs(A) @ np.abs(xs)) + 1e-300
+    assert (np.abs(y.cpu().numpy() - A @ xs) <= bound).all()
