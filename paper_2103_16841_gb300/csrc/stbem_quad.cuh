@@ -272,6 +272,21 @@ STBEM_HD inline R edge_T(R w, R r, R p, R ad) {
 }
 
 template <typename R>
+STBEM_HD __noinline__ R edge_dT(R wa, R ra, R wb, R rb, R p, R ad) {   // (rare: kept out of the callers' code)
+  return edge_T<R>(wb, rb, p, ad) - edge_T<R>(wa, ra, p, ad);
+}
+
+// 2^-900 <= v < 2^900 of a positive v, by its exponent (no FP64 instruction)
+STBEM_HD inline bool in_mid_range(double v) {
+#ifdef __CUDA_ARCH__
+  const unsigned e = ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
+  return e - 123u < 1800u;
+#else
+  return v >= 0x1p-900 && v < 0x1p900;
+#endif
+}
+
+template <typename R>
 STBEM_HD inline R edge_dE(R wa, R dw, R p_s, R d) {
   R p = fabs(p_s), ad = fabs(d);
   R A2 = p_s * p_s + d * d;
@@ -288,7 +303,9 @@ STBEM_HD inline R edge_dE(R wa, R dw, R p_s, R d) {
       // the difference of the two atans by one atan2 of the tangents' subtraction, without their divisions
       const R na = wa * p * (p * p + wa * wa), da = (ra + ad) * (p * p * ra + wa * wa * ad);
       const R nb = wb * p * (p * p + wb * wb), db = (rb + ad) * (p * p * rb + wb * wb * ad);
-      dt = atan2(nb * da - na * db, da * db + na * nb);
+      const R dd = da * db;   // eighth powers of lengths: not where they leave the range of numbers
+      if (in_mid_range((double)dd)) dt = atan2(nb * da - na * db, dd + na * nb);
+      else dt = edge_dT<R>(wa, ra, wb, rb, p, ad);
     } else {
       dt = edge_T<R>(wb, rb, p, ad) - edge_T<R>(wa, ra, p, ad);
     }

@@ -14,6 +14,9 @@ SRC = r"""
 extern "C" void sinh_cosh_of(int n, const double* v, double* sh, double* ch) {
   for (int k = 0; k < n; ++k) stbem::sinh_cosh(v[k], sh[k], ch[k]);
 }
+extern "C" void edge_of(int n, const double* p, double* out) {
+  for (int k = 0; k < n; ++k) out[k] = stbem::edge_dE<double>(p[4 * k], p[4 * k + 1], p[4 * k + 2], p[4 * k + 3]);
+}
 """
 
 
@@ -40,3 +43,20 @@ def test_sinh_and_cosh_of_the_nodes(lib):
     w = v.astype(np.longdouble)
     assert np.all(np.abs(sh - np.sinh(w)) <= 8 * 2.0 ** -53 * np.abs(np.sinh(w)))
     assert np.all(np.abs(ch - np.cosh(w)) <= 8 * 2.0 ** -53 * np.cosh(w))
+
+
+@pytest.mark.parametrize("power", [-240, -130, -110, 110, 130, 240])
+def test_edge_integrals_in_any_unit(lib, power):
+    """The integral of an edge is a length: with all lengths times a power of two it
+    is the same number times that. Terms of at most the edge's length cancel, each
+    within a few 2^-53: 32 x 2^-53 of the terms."""
+    rng = np.random.default_rng(1)
+    n = 2000
+    q = np.stack((rng.normal(size=n), 10 ** rng.uniform(-2, 0.5, n), rng.normal(size=n), rng.normal(size=n)), 1)
+    s = 2.0 ** power
+    a, b = np.zeros(n), np.zeros(n)
+    for v, out in ((q, a), (q * s, b)):
+        v = np.ascontiguousarray(v)
+        lib.edge_of(n, ctypes.c_void_p(v.ctypes.data), ctypes.c_void_p(out.ctypes.data))
+    terms = np.abs(q[:, 2]) * np.arcsinh(np.abs(q[:, 0]) + q[:, 1] + 1.0) + np.pi * np.abs(q[:, 3])
+    assert np.all(np.abs(b / s - a) <= 32 * 2.0 ** -53 * terms)
