@@ -350,7 +350,7 @@ void bem_mesh_destroy(bem_mesh* m) {
   if (!m) return;
   cudaFree(m->d_col); cudaFree(m->d_col_tet_begin); cudaFree(m->d_col_surf_begin);
   cudaFree(m->d_surf); cudaFree(m->d_tet); cudaFree(m->d_perm);
-  cudaFree(m->d_colf); cudaFree(m->d_facef); cudaFree(m->d_panf);
+  cudaFree(m->d_images);
   delete m;
 }
 

@@ -70,18 +70,38 @@ bem_status upload_gauss_tables() {
 }
 
 // ---------------------------------------------------------------------------
-// Staging: column frames, face gradients, panel balls
+// Staging: column frames, face gradients, panel balls, and their FP32 images
+// (in the same kernels and one allocation: mesh creation is some launches long)
 // ---------------------------------------------------------------------------
-__global__ void k_col_geom(int64_t n_col, const double* sv_xyz, const int32_t* corner_sv, ColGeom* out) {
+__device__ __forceinline__ void col_f32(const ColGeom& G, ColF& F) {
+  for (int k = 0; k < 3; ++k)
+    for (int i = 0; i < 3; ++i) F.Xh[k][i] = (float)G.X[k][i];
+  make_colr<float>(G, F.R);
+  for (int i = 0; i < 3; ++i) F.ctr[i] = (float)G.ctr[i];
+  F.rad = (float)G.rad;
+}
+__device__ __forceinline__ void panel_f32(const TetDev& D, int s0, PanelF& F) {
+  for (int k = 0; k < 4; ++k) F.vt[k] = (float)D.vt[k];
+  for (int k = 0; k < 5; ++k) F.ball[k] = (float)D.ball[k];
+  F.tmin = (float)D.tmin;
+  F.pmax = (float)D.pmax;
+  F.lo = (uint8_t)(D.lo - s0);
+  F.hi = (uint8_t)(D.hi - s0);
+  F.dup = (uint8_t)D.dup;
+  F.pad = 0;
+}
+
+__global__ void k_col_geom(int64_t n_col, const double* sv_xyz, const int32_t* corner_sv, ColGeom* out, ColF* outf) {
   int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (c >= n_col) return;
   const int32_t* s = corner_sv + 3 * c;
   make_colgeom(sv_xyz + 3 * s[0], sv_xyz + 3 * s[1], sv_xyz + 3 * s[2], out[c]);
+  col_f32(out[c], outf[c]);
 }
 
 // surf_p [n_surf][3] corner times; surf_col [n_surf]
 __global__ void k_surf_geom(int64_t n_surf, const ColGeom* cols, const double* surf_p, const int32_t* surf_col,
-                            SurfDev* out) {
+                            SurfDev* out, FaceF* outf) {
   int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (s >= n_surf) return;
   SurfDev S;
@@ -90,12 +110,13 @@ __global__ void k_surf_geom(int64_t n_surf, const ColGeom* cols, const double* s
   for (int k = 0; k < 3; ++k) S.f.p[k] = surf_p[3 * s + k];
   face_gradient(cols[S.col], S.f);
   out[s] = S;
+  make_facef(S.f, outf[s]);
 }
 
 // tet_vx [n_tet][4][4]: the panel's vertices (t,x,y,z) in the caller's order;
 // the 4D ball is formed in that order with the fixed operation order of the
 // sparsity contract: centre (((X0+X1)+X2)+X3)/4, radius max_v |X_v - c|.
-__global__ void k_tet_ball(int64_t n_tet, const double* tet_vx, TetDev* tets) {
+__global__ void k_tet_ball(int64_t n_tet, const double* tet_vx, TetDev* tets, const int32_t* col_surf_begin, PanelF* outf) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n_tet) return;
   const double* X = tet_vx + 16 * i;
@@ -112,61 +133,25 @@ __global__ void k_tet_ball(int64_t n_tet, const double* tet_vx, TetDev* tets) {
   }
   for (int d = 0; d < 4; ++d) tets[i].ball[d] = c[d];
   tets[i].ball[4] = mx;
-}
-
-// FP32 images of the columns, faces and panels
-__global__ void k_col_f32(int64_t n_col, const ColGeom* cols, ColF* out) {
-  int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= n_col) return;
-  const ColGeom& G = cols[c];
-  ColF F;
-  for (int k = 0; k < 3; ++k)
-    for (int i = 0; i < 3; ++i) F.Xh[k][i] = (float)G.X[k][i];
-  make_colr<float>(G, F.R);
-  for (int i = 0; i < 3; ++i) F.ctr[i] = (float)G.ctr[i];
-  F.rad = (float)G.rad;
-  out[c] = F;
-}
-__global__ void k_face_f32(int64_t n_surf, const SurfDev* surf, FaceF* out) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n_surf) return;
-  FaceF F;
-  make_facef(surf[i].f, F);
-  out[i] = F;
-}
-__global__ void k_panel_f32(int64_t n_tet, const TetDev* tets, const int32_t* col_surf_begin, PanelF* out) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n_tet) return;
-  const TetDev& D = tets[i];
-  const int s0 = col_surf_begin[D.col];
-  PanelF F;
-  for (int k = 0; k < 4; ++k) F.vt[k] = (float)D.vt[k];
-  for (int k = 0; k < 5; ++k) F.ball[k] = (float)D.ball[k];
-  F.tmin = (float)D.tmin;
-  F.pmax = (float)D.pmax;
-  F.lo = (uint8_t)(D.lo - s0);
-  F.hi = (uint8_t)(D.hi - s0);
-  F.dup = (uint8_t)D.dup;
-  F.pad = 0;
-  out[i] = F;
+  panel_f32(tets[i], col_surf_begin[tets[i].col], outf[i]);
 }
 
 bem_status mesh_device_geometry(bem_mesh* m, const double* d_sv_xyz, const int32_t* d_col_corner_sv,
                                 const double* d_tet_vx, const int32_t* d_surf_col, const double* d_surf_p) {
   cudaStream_t s = m->ctx->stream;
   int th = 128;
-  k_col_geom<<<(unsigned)((m->n_col + th - 1) / th), th, 0, s>>>(m->n_col, d_sv_xyz, d_col_corner_sv, m->d_col);
+  auto up = [](size_t n) { return (n + 255) / 256 * 256; };
+  const size_t nc = up(sizeof(ColF) * m->n_col), nf = up(sizeof(FaceF) * m->n_surf), np = sizeof(PanelF) * m->n_tet;
+  STBEM_CUDA(device_alloc(&m->d_images, nc + nf + np));
+  m->d_colf = m->d_images;
+  m->d_facef = static_cast<unsigned char*>(m->d_images) + nc;
+  m->d_panf = static_cast<unsigned char*>(m->d_images) + nc + nf;
+  k_col_geom<<<(unsigned)((m->n_col + th - 1) / th), th, 0, s>>>(m->n_col, d_sv_xyz, d_col_corner_sv, m->d_col,
+                                                                 static_cast<ColF*>(m->d_colf));
   k_surf_geom<<<(unsigned)((m->n_surf + th - 1) / th), th, 0, s>>>(m->n_surf, m->d_col, d_surf_p, d_surf_col,
-                                                                   m->d_surf);
-  k_tet_ball<<<(unsigned)((m->n_tet + th - 1) / th), th, 0, s>>>(m->n_tet, d_tet_vx, m->d_tet);
-  STBEM_CUDA(device_alloc(&m->d_colf, sizeof(ColF) * m->n_col));
-  STBEM_CUDA(device_alloc(&m->d_facef, sizeof(FaceF) * m->n_surf));
-  STBEM_CUDA(device_alloc(&m->d_panf, sizeof(PanelF) * m->n_tet));
-  k_face_f32<<<(unsigned)((m->n_surf + th - 1) / th), th, 0, s>>>(m->n_surf, m->d_surf,
-                                                                  static_cast<FaceF*>(m->d_facef));
-  k_col_f32<<<(unsigned)((m->n_col + th - 1) / th), th, 0, s>>>(m->n_col, m->d_col, static_cast<ColF*>(m->d_colf));
-  k_panel_f32<<<(unsigned)((m->n_tet + th - 1) / th), th, 0, s>>>(m->n_tet, m->d_tet, m->d_col_surf_begin,
-                                                                  static_cast<PanelF*>(m->d_panf));
+                                                                   m->d_surf, static_cast<FaceF*>(m->d_facef));
+  k_tet_ball<<<(unsigned)((m->n_tet + th - 1) / th), th, 0, s>>>(m->n_tet, d_tet_vx, m->d_tet, m->d_col_surf_begin,
+                                                                 static_cast<PanelF*>(m->d_panf));
   STBEM_CUDA(cudaGetLastError());
   return BEM_OK;
 }

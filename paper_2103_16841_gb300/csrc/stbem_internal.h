@@ -122,7 +122,8 @@ struct bem_mesh {
   stbem::SurfDev* d_surf = nullptr;
   stbem::TetDev* d_tet = nullptr;
   int32_t* d_perm = nullptr;    // internal -> caller
-  void* d_colf = nullptr;       // FP32 images of the columns, faces and panels (ColF, FaceF, PanelF)
+  void* d_images = nullptr;     // FP32 images, one allocation:
+  void* d_colf = nullptr;       // of the columns, faces and panels (ColF, FaceF, PanelF)
   void* d_facef = nullptr;
   void* d_panf = nullptr;
 };
