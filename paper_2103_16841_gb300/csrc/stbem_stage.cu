@@ -856,6 +856,17 @@ size_t fixed_bytes(bool fp32, int max_tet, int max_surf, int sms) {
   return 256 + (u > kUBytes ? up256(u * sms * 4) : 0);
 }
 
+// Intermediate data of a chunk where the scratch holds two of them, of `all` bytes:
+// at least four chunks on the mixed path, whose side stream has other work than the
+// first (FP64 stages all wait for one pipe), but not below 256 MiB: every chunk pays
+// the serial chain of its FP64 faces. Reassembly of the level-0 sphere with 2 slabs
+// 945 -> 343 us (625 before the stages), level-1, 5 slabs 2.9 -> 2.0 ms (64 and 128
+// MiB: 2.7 and 2.5); nothing changes where the whole takes 1 GiB and more.
+int64_t chunk_part(bool fp32, int64_t all) {
+  const int64_t small = (int64_t)256 << 20;
+  return fp32 ? std::max(all / 4, std::min(all, small)) : all;
+}
+
 }  // namespace
 
 int stage_apex_per_sm(bool fp32, int max_tet, int max_surf, int nq) {
@@ -878,7 +889,9 @@ void stage_scratch(bool fp32, int max_tet, int max_surf, int sms, const std::vec
     }
   const size_t fixed = fixed_bytes(fp32, max_tet, max_surf, sms);
   *least = (int64_t)up256(fixed + big);
-  *wanted = (int64_t)up256(std::max(fixed + big, std::min(2 * fixed + all, kScratch)));
+  // two chunks, or all of it in one pass
+  const size_t room = 2 * fixed + std::max<size_t>(all, fp32 ? 2 * chunk_part(fp32, (int64_t)all) : 0);
+  *wanted = (int64_t)up256(std::max(fixed + big, std::min(room + 512, kScratch)));
 }
 
 // All stages over the blocks [0, end) of the concatenated operators. The
@@ -989,15 +1002,8 @@ bem_status stage_run(const BlockCtx& one, const BlockCtx* many, const int64_t* p
     ++n_chunk;
     return BEM_OK;
   };
-  // chunks: runs of granules that fit a half; at least four on the mixed path, whose
-  // side stream has other work than the first (FP64 stages all wait for one pipe), but
-  // not below 128 MiB: every chunk pays the serial chain of its FP64 faces.
-  // Reassembly of the level-0 sphere with 2 slabs 945 -> 343 us (625 before the
-  // stages), level-1, 5 slabs 2.9 -> 2.5 ms; nothing changes where the whole
-  // takes 512 MiB and more.
-  const int64_t kSmall = (int64_t)128 << 20;
-  const int64_t part = fp32 ? std::max<int64_t>((int64_t)all / 4, std::min<int64_t>(all, kSmall)) : (int64_t)all;
-  const int64_t chunk = std::min<int64_t>(half_bytes, fixed + std::max<int64_t>(least, part));
+  // chunks: runs of granules that fit a half
+  const int64_t chunk = std::min<int64_t>(half_bytes, fixed + std::max<int64_t>(least, chunk_part(fp32, all)));
   int64_t g0 = 0, g1 = 0, rays = 0, slots = 0, off = 0;
   for (size_t o = 0; o < gran.size(); ++o) {
     const int64_t nb = std::min(blocks[o], end - off);
