@@ -349,8 +349,8 @@ def run_ours(args):
                             "density to host",
                 "solve": solve_info},
         # at least: outer points, pattern, and the quadrature's stages (five, or three in
-        # FP64) of its chunks, four or more in mixed precision
-        "gpu_launches": (2 + (5 * 4 if prec == "mixed" else 3)) * args.steps,
+        # FP64) of its chunks, four or more in mixed precision (one on small meshes)
+        "gpu_launches": (2 + (5 * (4 if n_inner > 10 ** 8 else 1) if prec == "mixed" else 3)) * args.steps,
         "clocks": clk.summary(),
         "roofline": roof,
         "cpu_baseline": cb,

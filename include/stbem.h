@@ -161,7 +161,7 @@ void bem_mesh_destroy(bem_mesh* mesh);
 
 typedef struct {
   int32_t precision; /* BEM_PREC_FP64 or BEM_PREC_MIXED */
-  int32_t m_q;       /* midpoint-rule subdivision m_Q (Fig. int_tri_mid); 1..8, paper uses 3 */
+  int32_t m_q;       /* midpoint-rule subdivision m_Q (Fig. int_tri_mid); 1..4, paper uses 3 */
   int32_t n_theta;   /* cap on Gauss nodes per conic-arc piece (4..32); 0 = default (32 FP64, 16 MIXED).
                         The count per piece is chosen from the distance of the integrand's nearest
                         complex pole to reach 1e-15 (FP64) or 1e-7 (MIXED) relative accuracy. */
@@ -169,7 +169,10 @@ typedef struct {
                         matvecs. MIXED operators always store FP32 values only (their accuracy). */
   int32_t matrix_free;/* 1: no values are stored; every product re-runs the quadrature with the
                         entries summed against x on the fly (the dot product fused into the
-                        quadrature pass); export_dense / entries are then unsupported. */
+                        quadrature pass); export_dense / entries are then unsupported. Products
+                        and solves use the context's scratch while no other call does; the
+                        operator's own (64 MiB, or a sixteenth of what the values would take) is
+                        for captured products and bem_matvec_noalloc. */
   int32_t trial_space;/* BEM_TRIAL_P0 (0, the default); BEM_TRIAL_P1 returns BEM_ERR_UNSUPPORTED */
 } bem_op_opts;
 
@@ -298,8 +301,10 @@ bem_status bem_matvec(const bem_operator* op, const double* x_dev, double* y_dev
  * right-hand sides per pass (the values are read once per pass); FP32 and
  * TF32 need the FP32 values (MIXED operators, or store_fp32 = 1). On first
  * use the TF32 / BF16 products make the operator's block records and a copy
- * of its values cut into 16-byte chunk slots in their type (1.1-1.25 x the
- * value bytes, kept with the operator and remade after a reassembly); the
+ * of its values cut into 16-byte chunk slots in their type (1.3-1.6 x the value
+ * bytes in TF32 and 1.6-2.3 x in BF16 with 6 to 32 slabs, up to 3.5 x and 7 x
+ * where columns are short; kept with the operator and remade after a
+ * reassembly; an Inf or NaN in x reaches the rows that have a value there); the
  * products keep packed operands in a per-operator workspace; the first
  * TF32 / BF16 product of a mesh shape times the candidate launch shapes once
  * and keeps the fastest for the process (so these first calls synchronize

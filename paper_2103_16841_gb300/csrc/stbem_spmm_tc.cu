@@ -20,7 +20,10 @@
 //   re-cut at the 16-byte chunk boundaries of the trial panel index (slot j
 //   of row r = the chunk starting at panel E * (floor(rs[r] / E) + j), zeros
 //   outside the band), stored per block as [slot][row] (made once from the
-//   assembled values, BF16 or TF32-rounded, about 1.1-1.25 x their bytes).
+//   assembled values, BF16 or TF32-rounded). Slots of a row group are padded
+//   to the widest band of its columns: on spheres with 6 to 32 slabs they take
+//   1.6-2.3 x the values' bytes in BF16 and 1.3-1.6 x in TF32, with 3 slabs (14
+//   columns per group) 4.0 x and 2.9 x.
 //   Building a block's A tile is then a copy of whole chunks.
 //
 // The MMA's 128 rows hold as many consecutive test columns as fit ("row
@@ -778,13 +781,14 @@ void tc_array_bytes(int64_t groups, int64_t nblk, int64_t nrows, size_t* bytes) 
 }
 
 // CTAs that share a group's blocks: some four CTAs per SM in all, of at least
-// eight blocks each. The
-// tensor cores' FP32 accumulation truncates, so a row's sum cut in parts
-// comes out closer to the exact one, by an amount that grows with the row:
-// the level-3 sphere with 8 slabs (11,300 values per row) moves by 1.2e-5 in
-// BF16 and 1.9e-5 in TF32 with two parts, the level-2 sphere with 32 slabs
-// (5,300) by 4e-6 and 6e-6. Long rows are therefore cut in two at most, or
-// left whole, to stay within 1.3e-5 of the uncut sum.
+// eight blocks each. The tensor cores' FP32 accumulation truncates, so a row's
+// sum cut in parts comes out closer to the exact one, by an amount that grows
+// with the row. Measured with two parts against none: level-3 sphere, 8 slabs
+// (11,300 values per row) 1.2e-5 in BF16 and 1.9e-5 in TF32, level-2 sphere, 32
+// slabs (5,300) 4e-6 and 6e-6. Long rows are cut in two at most, or left whole,
+// which kept these two meshes within 1.3e-5 of the uncut sums; on others the
+// difference is not bounded by that. More parts of long rows would be faster
+// (level-3 sphere, BF16, 13 vectors: 522 us with 8 for 613) and more accurate.
 int tc_parts(int64_t groups, int64_t nblk, int64_t per_row, bool bf16) {
   const int64_t per_group = nblk / std::max<int64_t>(groups, 1);
   const int most = per_row > 8000 ? (bf16 ? 2 : 1) : per_row > 3000 ? 2 : 8;
